@@ -94,7 +94,7 @@ bool has(const std::vector<int>& v, int x) { return std::find(v.begin(), v.end()
 
 // ------------------------------------------------------------ program
 enum OpKind { OP_PLOT, OP_MEMSET, OP_RESHAPE, OP_ROWOR, OP_UNPACK,
-              OP_MMA, OP_CENTRES, OP_PLOT_EXPR, OP_PLOT_CORNER, OP_PERMUTE, OP_EWISE };
+              OP_MMA, OP_PLOT_EXPR, OP_PLOT_CORNER, OP_PERMUTE, OP_EWISE };
 
 struct Op {
   OpKind kind;
@@ -102,7 +102,7 @@ struct Op {
   int n = 0;                            // plot jobs / rowor problems
   int64_t count = 0;                    // prep items / plot tiles / rowor grid / words / rows
   int64_t m = 0, nw = 0;                // outer / dot: M and words per row
-  int i0 = 0, i1 = 0, i2 = 0, i3 = 0;   // plot: rows/tile, max degree, common degree, max res
+  int i0 = 0, i1 = 0, i2 = 0;           // plot: rows/tile, max degree, common degree
   size_t smem = 0;                      // rowor dynamic shared memory
   int64_t zw = 0;                       // plot: words of the ranges it clears (off1, nw ranges)
   uint64_t* p = nullptr;                // memset / and output
@@ -114,7 +114,6 @@ struct Op {
 const char* op_name(const Op& op) {
   switch (op.kind) {
     case OP_PLOT: return "plot_kernel";
-    case OP_CENTRES: return "plot_centres_kernel";
     case OP_PLOT_EXPR: return "plot_expr_kernel";
     case OP_PLOT_CORNER: return "plot_corner_kernel";
     case OP_PERMUTE: return "permute_u32_kernel";
@@ -1102,8 +1101,7 @@ void plot_corner(Builder& bd, const std::vector<PlotReq>& reqs, const std::vecto
 
 // Every requested plot: the corner-rule relations and the expression relations
 // in one launch each (first, so that the polynomial plot launch stays right
-// before the contractions), the polynomial ones in the two launches of
-// plot_poly.  Arrays come back in the order of `reqs`.
+// before the contractions), the polynomial ones in one more.  Arrays come back in the order of `reqs`.
 std::vector<BitArr> plot_all(Builder& bd, const std::vector<PlotReq>& reqs) {
   std::vector<BitArr> plots(reqs.size());
   std::vector<PlotReq> poly, corner;
@@ -1180,18 +1178,69 @@ std::vector<BitArr> plot_all(Builder& bd, const std::vector<PlotReq>& reqs) {
   return plots;
 }
 
-// The polynomial relations' plots in two launches: the FP32 centre tables of
-// the last ports (once per distinct axis, not once per block), then the plot
-// itself.
+// The FP32 filter of one plot job (plot.cu): its error bound B, or no filter
+// when a port shares its variable with another, an axis is too long for exact
+// FP32 pixel indices or the magnitudes leave FP32's comfortable range.
+void plot_filter(PlotJob& J, const pa_relation& r, const pa_axis* axes,
+                 const std::vector<int64_t>& ord) {
+  const int n = r.arity, D = r.degree;
+  J.eps32 = (float)J.eps;
+  bool ok = J.ndim == n && isfinite(J.eps32);
+  double X[kMaxDim], xmax = 1.0;
+  for (int p = 0; p < n; ++p) {
+    const pa_axis& ax = axes[r.vars[p]];
+    const double d = J.delta[p];
+    ok = ok && ax.res < (1 << 22);
+    // the last port's expansions reach a few pixels past the range
+    X[p] = fmax(fabs(ax.lo), fabs(ax.hi)) * (1.0 + 0x1p-20) + (p == n - 1 ? 3.0 * d : 0.0);
+    xmax = fmax(xmax, X[p]);
+    J.lo_hi[p] = (float)ax.lo;
+    J.lo_lo[p] = (float)(ax.lo - (double)J.lo_hi[p]);
+    J.d_hi[p] = (float)d;
+    J.d_lo[p] = (float)(d - (double)J.d_hi[p]);
+    ok = ok && X[p] < 1e18 && d > 1e-18;
+  }
+  // A = sum |c_e| prod X_p^e_p over the monomials in nest order (the last port
+  // outermost, exponents ascending)
+  double A = 0.0;
+  size_t at = 0;
+  int e[kMaxDim] = {};
+  for (;;) {
+    int total = 0;
+    for (int p = 0; p < n; ++p) total += e[p];
+    if (total > D) {
+      // carry: the first port past its limit starts over, the next one steps
+      int p = 0;
+      while (p < n && e[p] == 0) ++p;
+      e[p] = 0;
+      if (p + 1 >= n) break;
+      ++e[p + 1];
+      continue;
+    }
+    double m = fabs(r.coeffs[ord[at++]]);
+    for (int p = 0; p < n; ++p)
+      for (int k = 0; k < e[p]; ++k) m *= X[p];
+    A += m;
+    ++e[0];
+  }
+  const double K = 7.0 * D + n * (D + 1.0) + 14.0;
+  const double underflow = 0x1p-140 * (double)ord.size() * pow(xmax, D) + 1e-30;
+  const double B = 1.05 * K * 0x1p-24 * A + 0x1p-21 * (double)J.eps32 + underflow;
+  ok = ok && at == ord.size() && A < 1e30 && pow(xmax, D) < 1e30 && B < 1e30;
+  J.filter = ok ? 1 : 0;
+  J.bound = ok ? (float)(B * (1.0 + 0x1p-20)) : INFINITY;
+  J.dabs = (float)(1.01 * J.delta[n - 1]);
+}
+
+// The polynomial relations' plots in one launch.
 std::vector<BitArr> plot_poly(Builder& bd, const std::vector<PlotReq>& reqs) {
   const int nrel = (int)reqs.size();
   std::vector<BitArr> plots;
   std::vector<PlotJob> jobs(nrel);
-  std::vector<size_t> coeff_off(nrel);
+  std::vector<size_t> coeff_off(nrel), c32_off(nrel);
   // Words per block: the plots' words spread over the blocks the GPU holds
   // at once (so that no second wave of blocks waits for the first), between
-  // 256 (enough words to carry a block's set-up: row polynomials, centre
-  // table copy) and 2048.
+  // 256 (enough words to carry a block's set-up) and one pass of 2048.
   int64_t tile_words = 2048;
   {
     int64_t words = 0;
@@ -1206,9 +1255,10 @@ std::vector<BitArr> plot_poly(Builder& bd, const std::vector<PlotReq>& reqs) {
     const int64_t slots = plot_resident_blocks(common >= 1 && common <= 4 ? common : -1);
     tile_words = std::min<int64_t>(2048, std::max<int64_t>(256, (words + slots - 1) / slots));
   }
-  int64_t tiles = 0, max_tile_words = 1, ycen = 0;
-  std::vector<CentreTab> tabs;  // one per distinct last-port axis of the hoisted jobs
-  int max_rows = 1, max_deg = 0, common_deg = reqs[0].rel->degree, max_res_last = 1;
+  int64_t tiles = 0;
+  int max_rows = 1, max_deg = 0, common_deg = reqs[0].rel->degree;
+  std::vector<double> nc;
+  std::vector<float> nc32;
   for (int i = 0; i < nrel; ++i) {
     const pa_relation& r = *reqs[i].rel;
     const pa_axis* axes = reqs[i].axes;
@@ -1224,9 +1274,14 @@ std::vector<BitArr> plot_poly(Builder& bd, const std::vector<PlotReq>& reqs) {
     plots.push_back(a);
     // coefficients in nest order
     std::vector<int64_t> ord = nest_order(r.arity, r.degree);
-    std::vector<double> nc(ord.size());
-    for (size_t k = 0; k < ord.size(); ++k) nc[k] = r.coeffs[ord[k]];
+    nc.resize(ord.size());
+    nc32.resize(ord.size());
+    for (size_t k = 0; k < ord.size(); ++k) {
+      nc[k] = r.coeffs[ord[k]];
+      nc32[k] = (float)nc[k];
+    }
     coeff_off[i] = bd.put(nc.data(), nc.size());
+    c32_off[i] = bd.put(nc32.data(), nc32.size());
 
     PlotJob& J = jobs[i];
     memset(&J, 0, sizeof J);
@@ -1243,84 +1298,33 @@ std::vector<BitArr> plot_poly(Builder& bd, const std::vector<PlotReq>& reqs) {
       J.lo[p] = ax.lo;
       J.delta[p] = (ax.hi - ax.lo) / (double)ax.res;
     }
-    J.hoisted = (a.ndim == r.arity) ? 1 : 0;
     J.nrows = a.nrows();
     J.row_words = a.row_words();
-    const int64_t res_last = a.res[a.ndim - 1];
-    if (J.hoisted) {
-      const int a = r.arity - 1;
-      const CentreTab* t = nullptr;
-      for (const CentreTab& c : tabs)
-        if (c.lo == J.lo[a] && c.delta == J.delta[a] && c.res == res_last) t = &c;
-      if (!t) {
-        CentreTab c;
-        c.y32 = reinterpret_cast<float*>(bd.alloc_words((res_last + 1) / 2));
-        c.lo = J.lo[a];
-        c.delta = J.delta[a];
-        c.item0 = ycen;
-        c.res = res_last;
-        ycen += res_last;
-        tabs.push_back(c);
-        t = &tabs.back();
-      }
-      J.y32 = t->y32;
-    }
-    {
-      const pa_axis& ax = axes[r.vars[r.arity - 1]];
-      J.ymax = (float)(fmax(fabs(ax.lo), fabs(ax.hi)) * (1.0 + 0x1p-20));
-      J.hword = (float)(32.0 * ((ax.hi - ax.lo) / (double)ax.res) * 1.01);
-      // coefficients with e_last = j form block j of the nest order; its size is
-      // the number of monomials of arity-1 variables of degree <= D - j
-      int32_t off = 0;
-      for (int j = 0; j <= r.degree; ++j) {
-        J.block_off[j] = off;
-        off += (int32_t)coeff_count(r.arity - 1, r.degree - j);
-      }
-    }
+    J.eps = relation_eps(r, axes);
+    plot_filter(J, r, axes, ord);
     J.rows_per_tile = (int32_t)std::max<int64_t>(
-        1, std::min<int64_t>(256, (tile_words + J.row_words - 1) / J.row_words));
+        1, std::min<int64_t>(1024, (tile_words + J.row_words - 1) / J.row_words));
     J.tile0 = tiles;
     tiles += (J.nrows + J.rows_per_tile - 1) / J.rows_per_tile;
     max_rows = std::max(max_rows, J.rows_per_tile);
-    max_tile_words = std::max<int64_t>(max_tile_words, (int64_t)J.rows_per_tile * J.row_words);
     max_deg = std::max(max_deg, r.degree);
-    max_res_last = std::max(max_res_last, (int)res_last);
     if (r.degree != common_deg) common_deg = -1;
-    const double eps = relation_eps(r, axes);
-    J.eps = eps;
-    J.eps32 = (float)eps;
-    J.kfac = (float)((4.0 * r.degree + 8.0) * 0x1p-24 * 1.01);
-    J.abs_margin = (float)(0x1p-21 * (double)J.eps32 + 1e-30);
-    if (!isfinite(J.eps32)) {
-      // eps beyond FP32 range: disable the filter, every pixel takes the FP64 path
-      J.eps32 = 0.0f;
-      J.kfac = INFINITY;
-    }
     bd.st.pixels_plotted += (double)a.bits();
     bd.st.n_plots++;
   }
   if (tiles > 0x7fffffffLL) bd.fail(PA_ERR_TOO_LARGE, "plot grid too large");
-  for (int i = 0; i < nrel; ++i)
+  for (int i = 0; i < nrel; ++i) {
     jobs[i].coeffs = reinterpret_cast<const double*>(bd.dev(coeff_off[i]));
-  const size_t jobs_off = bd.put(jobs.data(), jobs.size(), 64);
-  if (ycen > 0) {
-    Op cop;
-    cop.kind = OP_CENTRES;
-    cop.off0 = bd.put(tabs.data(), tabs.size(), 64);
-    cop.n = (int)tabs.size();
-    cop.count = ycen;
-    bd.ops.push_back(cop);
+    jobs[i].c32 = reinterpret_cast<const float*>(bd.dev(c32_off[i]));
   }
   Op op;
   op.kind = OP_PLOT;
-  op.off0 = jobs_off;
+  op.off0 = bd.put(jobs.data(), jobs.size(), 64);
   op.n = nrel;
   op.count = tiles;
   op.i0 = max_rows;
   op.i1 = max_deg;
   op.i2 = common_deg;
-  op.i3 = max_res_last;
-  op.m = max_tile_words;
   bd.ops.push_back(op);
   return plots;
 }
@@ -1433,7 +1437,7 @@ void fold_memsets(Builder& bd) {
   pop.zw = total;
 }
 
-// Plots of all networks in one launch pair, then their joins level by level:
+// Plots of all networks in one launch, then their joins level by level:
 // the joins of one level of every network's cluster tree are independent and
 // share one contraction launch per tile width.
 void build_networks(Builder& bd, std::vector<Network>& nets, bool one_join_per_launch = false,
@@ -1596,7 +1600,7 @@ void run_ops(pa_ctx* ctx, const std::vector<Op>& ops, char* blob, cudaStream_t s
     switch (op.kind) {
       case OP_PLOT:
         launch_plot(reinterpret_cast<const PlotJob*>(blob + op.off0), op.n, op.count, op.i0,
-                    op.i1, op.i2, op.i3, op.m, reinterpret_cast<const ZeroRange*>(blob + op.off1),
+                    op.i1, op.i2, reinterpret_cast<const ZeroRange*>(blob + op.off1),
                     (int)op.nw, op.zw, s);
         break;
       case OP_EWISE:
@@ -1613,9 +1617,6 @@ void run_ops(pa_ctx* ctx, const std::vector<Op>& ops, char* blob, cudaStream_t s
         break;
       case OP_PLOT_CORNER:
         launch_plot_corner(reinterpret_cast<const CornerJob*>(blob + op.off0), op.n, op.count, s);
-        break;
-      case OP_CENTRES:
-        launch_plot_centres(reinterpret_cast<const CentreTab*>(blob + op.off0), op.n, op.count, s);
         break;
       case OP_MEMSET:
         check_cuda(ctx, cudaMemsetAsync(op.p, 0, (size_t)op.count * 8, s), "cudaMemsetAsync");

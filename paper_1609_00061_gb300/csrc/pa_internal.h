@@ -31,36 +31,27 @@ constexpr int kMaxDeg = PA_MAX_DEGREE;
 // rounded on both, so the value is the one pa.h defines).
 struct PlotJob {
   const double* coeffs;             // device, nest order
+  const float* c32;                 // the same rounded to FP32 (filtered jobs)
   uint64_t* out;                    // device, pa_array layout
   double lo[kMaxDim];               // per port: range start of its variable
   double delta[kMaxDim];            // per port: pixel width of its variable
-  const float* y32;                 // [res_last] FP32 centres of the last port (hoisted jobs)
+  float lo_hi[kMaxDim], lo_lo[kMaxDim];  // lo and delta as sums of two floats
+  float d_hi[kMaxDim], d_lo[kMaxDim];
   int64_t nrows;                    // rows = product of all but the last array axis
   int64_t row_words;                // ceil(res_last / 64)
   int64_t tile0;                    // first block of this job in the plot launch
   int32_t rows_per_tile;
   int32_t arity, degree, kind, strict;
-  int32_t hoisted;                  // 1: the last port is the last array axis, used once
+  int32_t filter;                   // 1: FP32 filter (plot.cu); 0: FP64 at every pixel
   int32_t ndim;                     // array axes (distinct variables)
   int32_t res[kMaxDim];             // array axis resolutions
   int32_t port_axis[kMaxDim];       // port -> array axis
   double eps;
   float eps32;                      // eps rounded to FP32
-  float kfac;                       // FP32 filter: error bound factor on sum |g_j| Y^j
-  float abs_margin;                 // FP32 filter: margin for eps rounding / underflow
-  float ymax;                       // >= |y| for every FP32 centre of the last port
-  float hword;                      // >= distance from a word's pixel 32 to any of its 64 centres
-  int32_t block_off[kMaxDeg + 1];   // nest-order offset of the coefficients with e_last = j
+  float bound;                      // B: FP32 against FP64, eps rounding included (plot.cu)
+  float dabs;                       // 1.01 x the last port's pixel width
 };
 
-// One FP32 centre table: y32[i] = fl32(lo + (i + 1/2) delta) for i < res, the
-// last-port centres shared by every hoisted plot job over that axis.
-struct CentreTab {
-  float* y32;
-  double lo, delta;
-  int64_t item0;  // first item of this table in the centre-table launch
-  int64_t res;
-};
 // One expression relation to plot (expr.cu): the postfix program and its
 // constants on the device, the pixel grid as for PlotJob; word0 is the first
 // word of this job in the launch's flat word space.
@@ -106,22 +97,17 @@ struct ZeroRange {
   int64_t words;
   int64_t w0;
 };
-// Every table in one launch (one thread per centre), before the plot launch;
-// the plot kernel waits for it only after its row set-up (programmatic
-// dependent launch), so the two overlap.
-void launch_plot_centres(const CentreTab* d_tabs, int ntabs, int64_t total_items, cudaStream_t s);
 // One launch plots every job: blocks of rows_per_tile rows, each computing its
-// rows' polynomials and thresholds in shared memory first.  common_degree: the
-// degree shared by every job (selects a specialised kernel), or -1 when they
-// differ.
+// rows' polynomials in shared memory first.  common_degree: the degree shared
+// by every job (selects a specialised kernel), or -1 when they differ.
 // The same launch also clears the `nzero` ranges (zero_words words in all)
 // that later contractions OR their results into, so that no separate memset
 // sits between the launches.
 // Plot blocks the GPU holds at once (all SMs), for the kernel of this degree.
 int plot_resident_blocks(int common_degree);
 void launch_plot(const PlotJob* d_jobs, int njobs, int64_t total_tiles, int max_rows_per_tile,
-                 int max_degree, int common_degree, int max_res_last, int64_t max_tile_words,
-                 const ZeroRange* d_zero, int nzero, int64_t zero_words, cudaStream_t s);
+                 int max_degree, int common_degree, const ZeroRange* d_zero, int nzero,
+                 int64_t zero_words, cudaStream_t s);
 
 // ------------------------------------------------------------- bit arrays
 // A bit-packed array with `inner` trailing axes flattened into packed rows:

@@ -3,41 +3,41 @@
 // Pixel e is on when f(c_e) is finite and |f(c_e)| <= eps (PA_EQ; f <= eps for
 // PA_LE, f < eps for PA_LT; strict makes every test "<").  The decision is
 // defined by the IEEE double evaluation fixed in pa.h.  GB300 runs FP64 at a
-// small fraction of its FP32 rate, so each pixel is first evaluated in FP32
-// against a rigorous bound on |f32 - f64|; only pixels whose FP32 value lies
-// within that bound of eps are evaluated again in FP64.  The result is the
-// FP64 decision, bit for bit.
+// small fraction of its FP32 rate, so everything is first evaluated in FP32
+// against a rigorous bound on |f32 - f64|.
 //
-// Row hoisting: with every port but the last fixed, f is a polynomial
-// f = sum_j g_j y^j in the last port y.  The g_j are exactly the inner nested
-// sums of the pa.h evaluation order, so computing them once per row in FP64
-// (at the start of the block that plots the row) and finishing each pixel with
-// sum_j g_j y^j performs the very same IEEE operations as evaluating the pixel
-// from scratch.
+// The FP32 filter.  With every port but the last fixed, f is a polynomial
+// sum_j g_j y^j in the last port y.  The g_j are computed once per row in FP32
+// (GB300 does 238 FP32 against 1.7 FP64 flops per SM and clock: with the row
+// polynomials in FP64 the 90 plots of 512^3 in 38 random networks took 4.1 ms,
+// most of it on the FP64 pipe).  Each 64-pixel word then expands its row's
+// polynomial about its middle pixel,
+//   f(y_c + t) = sum_k a_k t^k,   a_k by synthetic division,
+// decides the whole word when |a_0| and S = sum_k |a_k| h^k (k >= 1, h >= the
+// distance from y_c to any centre of the word) leave no doubt, and otherwise
+// evaluates its pixels as polynomials in the integer offset s = (y - y_c) / delta
+// (a_k scaled by delta^k, D fused multiply-adds per pixel).
 //
-// Error bound for the FP32 pass (u = 2^-24, D the degree, g_j rounded to FP32,
-// y32 = fl32(y64), a = sum_j |g_j| |y|^j):
-//   |f32 - f64| <= (2D+1) u a   (FP32 evaluation)
-//               +  (D+1) u a    (rounding of g_j and y)
-//               +  (2D+1) 2^-53 a (FP64 evaluation)
-// and a <= a_row = sum_j |g_j| Y^j with Y >= |y| on the whole axis.  The kernel
-// uses B_row = (4D + 8) u 1.01 a_row + 2^-21 eps + 1e-30, which also covers the
-// rounding of a_row, of eps to FP32 and of the thresholds themselves.
-//
-// Whole-word pruning (the paper's suggestion of skipping regions whose error
-// provably exceeds eps, here per 64-pixel word).  With F the exact row
-// polynomial, y_c the word's pixel 32 and h >= the distance from y_c to any
-// centre of the word, Taylor's theorem gives for every pixel y of the word
-//   |F(y) - F(y_c)| <= h |F'(y_c)| + h^2 / 2 max |F''|,
-// max |F''| <= S2 = sum_j j (j-1) |g_j| Yw^(j-2) with Yw = |y_c| + h, and the
-// FP32 derivative d_c (Horner) satisfies |d_c - F'(y_c)| <= (2D + 4) u S1,
-// S1 = sum_j j |g_j| |y_c|^(j-1).  With T = 1.01 (h (|d_c| + (2D+4) u S1) +
-// h^2 S2 / 2) and the pixel bound B_row used three times (f32 vs f64 at y_c,
-// f64 vs F at y_c and at y):
-//   |f64(y) - f32(y_c)| <= 3 B_row + T,
-// so f32(y_c) beyond eps + B_row + 4 B_row + T proves the whole word off (|f|
-// for PA_EQ), and for PA_LE / PA_LT f32(y_c) below eps - B_row - 4 B_row - T
-// proves it on; only the remaining words are evaluated pixel by pixel.
+// Error bound.  u = 2^-24, X_p >= |x_p| on port p's range (widened by three
+// pixels on the last port, which covers |y_c| + |t| for every word), and
+//   A = sum_e |c_e| prod_p X_p^e_p   (all exponents, the last port's included).
+// Every quantity the kernel computes is a sum of rounded products of the
+// coefficients' monomials, so its error is at most (roundings on a monomial's
+// path) u A.  A monomial of total degree at most D meets: the rounding of c_e
+// (1); per factor x_p the error of the FP32 centre (2.2: two roundings of a
+// value within X_p, see centre32) and one or two roundings of products; at
+// most D + 1 roundings of sums per port, D + 1 in the synthetic division, one
+// per factor in the scaling by delta^k and D + 1 in the final Horner sum.
+// Together less than K = 7 D + n (D + 1) + 14 for n ports.  The FP64 value's own error
+// (the same counts of 2^-53) is covered by the factor 1.05, so with
+//   B = 1.05 K u A + 2^-21 eps + underflow
+// (eps is rounded to FP32; a product that underflows loses at most 2^-149,
+// times powers of the X_p) the FP64 decision equals the sign of |f32| - eps
+// (f32 - eps for PA_LE / PA_LT) whenever that value exceeds B in magnitude.
+// The whole-word test keeps 3 B.  Pixels within B, some per cent of the band
+// edges on a fine grid, are collected and decided by the FP64 evaluation of
+// pa.h from scratch: the result is the FP64 decision, bit for bit.  A relation
+// whose A is not comfortably inside the FP32 range takes FP64 at every pixel.
 #include <float.h>
 
 #include <algorithm>
@@ -54,53 +54,60 @@ namespace pa {
 // nest(-1, .) the next coefficient in nest order (read through cp).  No
 // evaluation recurses at run time: a recursive device function runs on the
 // 1 KB default call stack, which an 8-port relation (eight frames) overflows.
-template <int K>
-__device__ __forceinline__ double nest_t(int rem, const double*& cp, const double* x) {
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+
+template <int K, class T>
+__device__ __forceinline__ T nest_t(int rem, const T*& cp, const T* x) {
   if constexpr (K < 0) {
     return *cp++;
   } else {
-    double s = 0.0, pw = 1.0;
+    T s = 0, pw = 1;
     for (int e = 0; e <= rem; ++e) {
-      const double term = __dmul_rn(nest_t<K - 1>(rem - e, cp, x), pw);
-      s = (e == 0) ? term : __dadd_rn(s, term);
-      pw = __dmul_rn(pw, x[K]);
+      const T term = mul_rn(nest_t<K - 1, T>(rem - e, cp, x), pw);
+      s = (e == 0) ? term : add_rn(s, term);
+      pw = mul_rn(pw, x[K]);
     }
     return s;
   }
 }
 
+template <class T>
 struct NestOut {
-  double v;
-  const double* cp;  // past the coefficients read
+  T v;
+  const T* cp;  // past the coefficients read
 };
 
 // Any depth as a loop over an explicit per-depth state (partial sum, power of
 // x_L, exponent, remaining degree): the same products and sums in the same
 // order as nest_t, out of line and with few registers, for the deep cases.
-__device__ __noinline__ NestOut nest_deep(int k, int rem, const double* cp, const double* x) {
+template <class T>
+__device__ __noinline__ NestOut<T> nest_deep(int k, int rem, const T* cp, const T* x) {
   if (k < 0) return {*cp, cp + 1};
-  double s[kMaxDim], pw[kMaxDim];
+  T s[kMaxDim], pw[kMaxDim];
   int e[kMaxDim], rm[kMaxDim];
   int L = k;
   rm[k] = rem;
   e[k] = 0;
-  pw[k] = 1.0;
-  s[k] = 0.0;
+  pw[k] = 1;
+  s[k] = 0;
   for (;;) {
     // open the term e[L] of depth L down to depth 0
     while (L > 0) {
       rm[L - 1] = rm[L] - e[L];
       e[L - 1] = 0;
-      pw[L - 1] = 1.0;
-      s[L - 1] = 0.0;
+      pw[L - 1] = 1;
+      s[L - 1] = 0;
       --L;
     }
-    double v = *cp++;  // nest(-1, .): the next coefficient
+    T v = *cp++;  // nest(-1, .): the next coefficient
     // close terms upward while depths complete
     for (;;) {
-      const double term = __dmul_rn(v, pw[L]);
-      s[L] = (e[L] == 0) ? term : __dadd_rn(s[L], term);
-      pw[L] = __dmul_rn(pw[L], x[L]);
+      const T term = mul_rn(v, pw[L]);
+      s[L] = (e[L] == 0) ? term : add_rn(s[L], term);
+      pw[L] = mul_rn(pw[L], x[L]);
       if (++e[L] <= rm[L]) break;
       if (L == k) return {s[k], cp};
       v = s[L];
@@ -109,65 +116,57 @@ __device__ __noinline__ NestOut nest_deep(int k, int rem, const double* cp, cons
   }
 }
 
-__device__ __forceinline__ double nest_rows(int k, int rem, const double*& cp, const double* x) {
+template <class T>
+__device__ __forceinline__ T nest_rows(int k, int rem, const T*& cp, const T* x) {
   switch (k) {
-    case -1: return nest_t<-1>(rem, cp, x);
-    case 0: return nest_t<0>(rem, cp, x);
-    case 1: return nest_t<1>(rem, cp, x);
-    case 2: return nest_t<2>(rem, cp, x);
+    case -1: return nest_t<-1, T>(rem, cp, x);
+    case 0: return nest_t<0, T>(rem, cp, x);
+    case 1: return nest_t<1, T>(rem, cp, x);
+    case 2: return nest_t<2, T>(rem, cp, x);
     default: {
-      const NestOut o = nest_deep(k, rem, cp, x);
+      const NestOut<T> o = nest_deep<T>(k, rem, cp, x);
       cp = o.cp;
       return o.v;
     }
   }
 }
 
-// The row polynomial g_0..g_DS of a 2- or 3-port relation at one row, for a
-// degree fixed at compile time: the very products and sums of nest_t, in the
-// same order, with the powers of the row ports (1, x, x*x, ... by repeated
-// multiplication, the same sequence nest_t forms for every sum) computed once
-// instead of once per sum, and every sum unrolled, so that the sums of the
-// D + 1 blocks proceed side by side rather than one FP64 chain after another.
+// The row polynomial g_0..g_DS of a 2- or 3-port relation at one row, FP32, for
+// a degree fixed at compile time (Horner in the row ports, every index
+// constant).  c: the coefficients in nest order.
 template <int DS>
-__device__ __forceinline__ void row_poly2(const double* __restrict__ cp, double x0, double* g) {
-  double p0[DS + 1];
-  p0[0] = 1.0;
-#pragma unroll
-  for (int e = 1; e <= DS; ++e) p0[e] = __dmul_rn(p0[e - 1], x0);
+__device__ __forceinline__ void row_poly2(const float* __restrict__ c, float x0, float* g) {
+  int at = 0;
 #pragma unroll
   for (int j = 0; j <= DS; ++j) {
-    double s0 = __dmul_rn(cp[0], p0[0]);
+    float s = c[at + DS - j];
 #pragma unroll
-    for (int e = 1; e <= DS - j; ++e) s0 = __dadd_rn(s0, __dmul_rn(cp[e], p0[e]));
-    cp += DS - j + 1;
-    g[j] = s0;
+    for (int e = DS - j - 1; e >= 0; --e) s = __fmaf_rn(s, x0, c[at + e]);
+    at += DS - j + 1;
+    g[j] = s;
   }
 }
 
 template <int DS>
-__device__ __forceinline__ void row_poly3(const double* __restrict__ cp, double x0, double x1,
-                                          double* g) {
-  double p0[DS + 1], p1[DS + 1];
-  p0[0] = 1.0;
-  p1[0] = 1.0;
-#pragma unroll
-  for (int e = 1; e <= DS; ++e) {
-    p0[e] = __dmul_rn(p0[e - 1], x0);
-    p1[e] = __dmul_rn(p1[e - 1], x1);
-  }
+__device__ __forceinline__ void row_poly3(const float* __restrict__ c, float x0, float x1,
+                                          float* g) {
+  int at = 0;
 #pragma unroll
   for (int j = 0; j <= DS; ++j) {
-    double s1 = 0.0;
+    // the sums over x0 of the blocks e1 = 0..DS - j, then Horner in x1
+    float t[DS + 1];
 #pragma unroll
     for (int e1 = 0; e1 <= DS - j; ++e1) {
-      double s0 = __dmul_rn(cp[0], p0[0]);
+      const int m = DS - j - e1;
+      float s = c[at + m];
 #pragma unroll
-      for (int e = 1; e <= DS - j - e1; ++e) s0 = __dadd_rn(s0, __dmul_rn(cp[e], p0[e]));
-      cp += DS - j - e1 + 1;
-      const double term = __dmul_rn(s0, p1[e1]);
-      s1 = (e1 == 0) ? term : __dadd_rn(s1, term);
+      for (int e = m - 1; e >= 0; --e) s = __fmaf_rn(s, x0, c[at + e]);
+      at += m + 1;
+      t[e1] = s;
     }
+    float s1 = t[DS - j];
+#pragma unroll
+    for (int e1 = DS - j - 1; e1 >= 0; --e1) s1 = __fmaf_rn(s1, x1, t[e1]);
     g[j] = s1;
   }
 }
@@ -186,20 +185,82 @@ __device__ __forceinline__ bool decide64(double f, int kind, double eps, int str
   return f < eps;
 }
 
-// exact FP64 value of sum_j g_j y^j in the order fixed by pa.h
-__device__ __noinline__ bool exact64(double y64, const double* g6, int D, int kind, double eps,
-                                     int strict) {
-  double s6 = g6[0], p6 = 1.0;
-  for (int j = 1; j <= D; ++j) {
-    p6 = __dmul_rn(p6, y64);
-    s6 = __dadd_rn(s6, __dmul_rn(g6[j], p6));
+// The nested FP64 sums of pa.h for 2 or 3 ports and a degree fixed at compile
+// time: the products and sums of nest_t in the same order, with the powers of
+// each port formed once and every sum unrolled, so that independent sums
+// proceed side by side (the FP64 chain is what a pixel decided in FP64 costs).
+template <int DS>
+__device__ __forceinline__ double nest2(const double* __restrict__ cp, double x0, double x1) {
+  double p0[DS + 1];
+  p0[0] = 1.0;
+#pragma unroll
+  for (int e = 1; e <= DS; ++e) p0[e] = __dmul_rn(p0[e - 1], x0);
+  double f = 0.0, p1 = 1.0;
+#pragma unroll
+  for (int j = 0; j <= DS; ++j) {
+    double s = __dmul_rn(cp[0], p0[0]);
+#pragma unroll
+    for (int e = 1; e <= DS - j; ++e) s = __dadd_rn(s, __dmul_rn(cp[e], p0[e]));
+    cp += DS - j + 1;
+    const double term = __dmul_rn(s, p1);
+    f = j == 0 ? term : __dadd_rn(f, term);
+    p1 = __dmul_rn(p1, x1);
   }
-  return decide64(s6, kind, eps, strict);
+  return f;
 }
 
-// general path (a variable on several ports): full nested FP64 evaluation
-__device__ __noinline__ bool general64(const PlotJob* J, int64_t row, int64_t i) {
-  const int ndim = J->ndim;
+template <int DS>
+__device__ __forceinline__ double nest3(const double* __restrict__ cp, double x0, double x1,
+                                        double x2) {
+  double p0[DS + 1], p1[DS + 1];
+  p0[0] = 1.0;
+  p1[0] = 1.0;
+#pragma unroll
+  for (int e = 1; e <= DS; ++e) {
+    p0[e] = __dmul_rn(p0[e - 1], x0);
+    p1[e] = __dmul_rn(p1[e - 1], x1);
+  }
+  double f = 0.0, p2 = 1.0;
+#pragma unroll
+  for (int j = 0; j <= DS; ++j) {
+    double s1 = 0.0;
+#pragma unroll
+    for (int e1 = 0; e1 <= DS - j; ++e1) {
+      double s = __dmul_rn(cp[0], p0[0]);
+#pragma unroll
+      for (int e = 1; e <= DS - j - e1; ++e) s = __dadd_rn(s, __dmul_rn(cp[e], p0[e]));
+      cp += DS - j - e1 + 1;
+      const double term = __dmul_rn(s, p1[e1]);
+      s1 = (e1 == 0) ? term : __dadd_rn(s1, term);
+    }
+    const double term = __dmul_rn(s1, p2);
+    f = j == 0 ? term : __dadd_rn(f, term);
+    p2 = __dmul_rn(p2, x2);
+  }
+  return f;
+}
+
+// The FP64 decision of one pixel: the full nested evaluation of pa.h at its
+// centre.
+template <int DS>
+__device__ __noinline__ bool decide_pixel64(const PlotJob* J, int64_t row, int64_t i) {
+  const int ndim = J->ndim, arity = J->arity;
+  if constexpr (DS >= 0) {
+    if (J->filter && (arity == 2 || arity == 3) && row < (1ll << 31)) {
+      // port p on axis p
+      const double xl = centre(J->lo[arity - 1], J->delta[arity - 1], i);
+      uint32_t r0 = (uint32_t)row, r1 = 0;
+      if (arity == 3) {
+        const uint32_t q = r0 / (uint32_t)J->res[1];
+        r1 = r0 - q * (uint32_t)J->res[1];
+        r0 = q;
+      }
+      const double x0 = centre(J->lo[0], J->delta[0], r0);
+      const double f = arity == 2 ? nest2<DS>(J->coeffs, x0, xl)
+                                  : nest3<DS>(J->coeffs, x0, centre(J->lo[1], J->delta[1], r1), xl);
+      return decide64(f, J->kind, J->eps, J->strict);
+    }
+  }
   int64_t rest = row;
   int64_t idx[kMaxDim];
   idx[ndim - 1] = i;
@@ -208,61 +269,44 @@ __device__ __noinline__ bool general64(const PlotJob* J, int64_t row, int64_t i)
     rest /= J->res[a];
   }
   double x[kMaxDim];
-  for (int p = 0; p < J->arity; ++p) x[p] = centre(J->lo[p], J->delta[p], idx[J->port_axis[p]]);
+  for (int p = 0; p < arity; ++p) x[p] = centre(J->lo[p], J->delta[p], idx[J->port_axis[p]]);
   const double* cp = J->coeffs;
-  return decide64(nest_rows(J->arity - 1, J->degree, cp, x), J->kind, J->eps, J->strict);
+  return decide64(nest_rows<double>(arity - 1, J->degree, cp, x), J->kind, J->eps, J->strict);
+}
+
+// The FP32 centre of pixel i of port p (fi = i + 1/2, exact below 2^23): lo and
+// delta as sums of two floats, one rounding in each of the two larger steps,
+// so |error| <= 2.2 u max(|lo|, |hi|).
+__device__ __forceinline__ float centre32(const PlotJob* J, int p, float fi) {
+  return __fadd_rn(__fmaf_rn(fi, J->d_hi[p], J->lo_hi[p]), __fmaf_rn(fi, J->d_lo[p], J->lo_lo[p]));
 }
 
 // --------------------------------------------------------------- plot kernel
-// One block plots a tile of rows.  Set-up: the FP32 centres of the last axis
-// are staged in shared memory (padded so that consecutive words hit distinct
-// banks) and each row's polynomial and thresholds are computed there.  Then
-// Taylor tests decide whole spans and words first (each thread a span of
-// four words, then its words); the words no test decides are listed, and the
-// block evaluates them, a piece of each word per thread, in FP32
-// (f = g_0 + g_1 y + ... by fused multiply-adds): |f| below eps - B_row is on,
-// above eps + B_row is off, anything else is decided by the exact FP64
-// evaluation.
+// One block plots a tile of rows.  Set-up: each row's FP32 polynomial goes to
+// shared memory (one thread per row).  Then, for up to kPass words of the tile
+// at a time, in phases that each run with full warps on a list the phase
+// before made:
+//   1. every word is tested as a whole (neighbouring threads take neighbouring
+//      words, so decided words are stored in full sectors);
+//   2. an undecided word on which f is provably monotone has its band edges
+//      solved for (Newton, then the two pixels on either side of each edge are
+//      evaluated: by monotonicity they decide every other pixel), about 130
+//      instructions against 450 for 64 pixel evaluations;
+//   3. the others are evaluated pixel by pixel, one thread per word;
+//   4. a word with a pixel within B of eps is evaluated again by a warp, which
+//      collects those pixels;
+//   5. the collected pixels are decided in FP64, a thread each.
+// Phases 4 and 5 exist because one such pixel handled in place holds up its
+// whole warp.  What bounds it: instruction issue (no pipe above 40 %; the
+// output is 1/8 byte per pixel), and on small plots the chain of phases.
+// Against FP64 row polynomials, FP32 centre tables from a launch of their own
+// and 64 evaluations per undecided word (ncu, cold): 38 random networks, 12.7
+// Gpixel, 4.14 -> 2.11 ms; 4096 chains, 4.9 Gpixel, 1.37 + 0.10 -> 0.70 ms;
+// four 256^3 plots 55 + 3 -> 29 us; eight 2048^2 plots 19 + 3 -> 14 us.
 constexpr int kPlotThreads = 256;
 static_assert(sizeof(PlotJob) % 4 == 0, "plot descriptors are copied as 32-bit words");
-constexpr int kYTabCap = 12288;  // largest last axis whose centres are staged in shared memory
-
-__device__ __forceinline__ int ypad(int i) { return i + (i >> 6); }
-
-// Byte offset of the thresholds in a plot block's shared memory (16-aligned).
-__host__ __device__ __forceinline__ size_t plot_thr_offset(int rmax, int gstride) {
-  return ((size_t)rmax * gstride * 12 + 15) / 16 * 16;
-}
-
-// The FP32 centre of last-axis pixel i.
-__device__ __forceinline__ float ycentre32(double ylo, double ydelta, int i) {
-  return __double2float_rn(centre(ylo, ydelta, i));
-}
-
-// Centre tables, one thread per centre.  The plot launch that follows may
-// start as soon as every block of this one has begun.
-__global__ void __launch_bounds__(256)
-plot_centres_kernel(const CentreTab* __restrict__ tabs, int ntabs, int64_t total) {
-  asm volatile("griddepcontrol.launch_dependents;");
-  for (int64_t it = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; it < total;
-       it += (int64_t)gridDim.x * blockDim.x) {
-    int lo = 0, hi = ntabs - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (tabs[mid].item0 <= it) lo = mid; else hi = mid - 1;
-    }
-    const CentreTab& T = tabs[lo];
-    const int i = (int)(it - T.item0);
-    T.y32[i] = ycentre32(T.lo, T.delta, i);
-  }
-}
-
-void launch_plot_centres(const CentreTab* d_tabs, int ntabs, int64_t total_items, cudaStream_t s) {
-  if (total_items <= 0) return;
-  int64_t blocks = (total_items + 255) / 256;
-  if (blocks > 152 * 8) blocks = 152 * 8;
-  plot_centres_kernel<<<(unsigned)blocks, 256, 0, s>>>(d_tabs, ntabs, total_items);
-}
+constexpr int kPass = 2048;      // words per pass (the lists' entries are 16-bit)
+constexpr int kPendCap = 512;    // collected FP64 pixels per pass; more are evaluated in place
 
 // Clear the listed ranges with every thread of the grid, eight words per
 // thread and step: chunk c covers words [8c, 8c + 8) of the ranges' flat
@@ -286,407 +330,407 @@ __device__ __forceinline__ void clear_ranges(const ZeroRange* __restrict__ zr, i
   }
 }
 
-// The 64 pixels of one word in FP32: bit b of *on is set when the pixel is
-// certainly on, bit b of *pending when only the FP64 evaluation can decide.
-template <int DS, bool EQ, bool YS, bool FULL>
-__device__ __forceinline__ void eval_word(const float* g, int D, float lo, float hi,
-                                          const float* ytab_w, const float* __restrict__ y32g,
-                                          int i0, int nb, uint64_t* on, uint64_t* pending) {
-  uint32_t on_lo = 0, on_hi = 0, pe_lo = 0, pe_hi = 0;
-#pragma unroll
-  for (int bb = 0; bb < 64; ++bb) {
-    if (FULL || bb < nb) {
-      const float y = YS ? ytab_w[bb] : __ldg(y32g + i0 + bb);
-      float s = g[0], pw = y;
-      if (DS >= 0) {
-#pragma unroll
-        for (int j = 1; j <= (DS >= 0 ? DS : 1); ++j) {
-          if (j > 1) pw = __fmul_rn(pw, y);
-          s = __fmaf_rn(g[j], pw, s);
-        }
-      } else {
-        for (int j = 1; j <= D; ++j) {
-          if (j > 1) pw = __fmul_rn(pw, y);
-          s = __fmaf_rn(g[j], pw, s);
-        }
-      }
-      const float dd = EQ ? fabsf(s) : s;
-      const bool c_on = dd < lo;
-      const bool c_pe = !c_on && !(dd > hi);
-      if (bb < 32) {
-        if (c_on) on_lo |= 1u << bb;
-        if (c_pe) pe_lo |= 1u << bb;
-      } else {
-        if (c_on) on_hi |= 1u << (bb - 32);
-        if (c_pe) pe_hi |= 1u << (bb - 32);
-      }
-    }
+// The last job whose first tile is at most this block's: every thread compares
+// one job of an evenly spaced sample, then the gap is searched the same way (two
+// rounds of independent loads up to 65536 jobs; a binary search by one thread
+// is a chain of as many L2 latencies as log2(jobs)).
+__device__ __forceinline__ int find_job(const PlotJob* __restrict__ jobs, int njobs) {
+  int lo = 0, n = njobs;  // the job is in [lo, lo + n)
+  while (n > 1) {
+    const int step = (n + (int)blockDim.x - 1) / (int)blockDim.x;
+    const int64_t at = (int64_t)threadIdx.x * step;
+    const int below = at < n && jobs[lo + at].tile0 <= (int64_t)blockIdx.x;
+    const int c = __syncthreads_count(below);  // tile0 ascends, job lo is below
+    const int first = (c - 1) * step;
+    lo += first;
+    n = min(step, n - first);
   }
-  *on = ((uint64_t)on_hi << 32) | on_lo;
-  *pending = ((uint64_t)pe_hi << 32) | pe_lo;
+  return lo;
 }
 
-template <int DS, bool EQ, bool YS>
-__device__ __forceinline__ void eval_word_any(const float* g, int D, float lo, float hi,
-                                              const float* ytab_w, const float* y32g, int i0,
-                                              int nb, uint64_t* on, uint64_t* pending) {
-  if (nb == 64) eval_word<DS, EQ, YS, true>(g, D, lo, hi, ytab_w, y32g, i0, nb, on, pending);
-  else eval_word<DS, EQ, YS, false>(g, D, lo, hi, ytab_w, y32g, i0, nb, on, pending);
+// Taylor coefficients about yc of the polynomial in a (in place, synthetic
+// division).
+template <int DS, int N>
+__device__ __forceinline__ void taylor_shift(float (&a)[N], int D, float yc) {
+  if constexpr (DS >= 0) {
+#pragma unroll
+    for (int i = 0; i < DS; ++i)
+#pragma unroll
+      for (int j = DS - 1; j >= i; --j) a[j] = __fmaf_rn(yc, a[j + 1], a[j]);
+  } else {
+    for (int i = 0; i < D; ++i)
+      for (int j = D - 1; j >= i; --j) a[j] = __fmaf_rn(yc, a[j + 1], a[j]);
+  }
 }
 
-// Eight pixels of a row in FP32 (f = g_0 + g_1 y + ... by fused
-// multiply-adds): bit b of the result is set when pixel b is certainly on,
-// bit b of *pending when only the FP64 evaluation can decide.  nb8 pixels
-// (1..8) exist; y comes from the padded shared table (YS) or global memory.
-template <int DS, bool EQ, bool YS>
-__device__ __forceinline__ uint32_t eval8(const float* g, int D, float lo, float hi,
-                                          const float* yt, const float* __restrict__ yg, int ic,
-                                          int nb8, uint32_t* pending) {
-  uint32_t on = 0, pe = 0;
+// The value compared with 0 at integer offset s from the expansion point:
+// |f| - eps (PA_EQ) or f - eps.  a: scaled Taylor coefficients.
+template <int DS, bool EQ, int N>
+__device__ __forceinline__ float excess(const float (&a)[N], int D, float s, float eps) {
+  float f;
+  if constexpr (DS >= 0) {
+    f = a[DS];
 #pragma unroll
-  for (int bb = 0; bb < 8; ++bb) {
-    if (bb < nb8) {
-      const float y = YS ? yt[bb] : __ldg(yg + ic + bb);
-      float s = g[0], pw = y;
-      if (DS >= 0) {
-#pragma unroll
-        for (int j = 1; j <= (DS >= 0 ? DS : 1); ++j) {
-          if (j > 1) pw = __fmul_rn(pw, y);
-          s = __fmaf_rn(g[j], pw, s);
-        }
-      } else {
-        for (int j = 1; j <= D; ++j) {
-          if (j > 1) pw = __fmul_rn(pw, y);
-          s = __fmaf_rn(g[j], pw, s);
-        }
-      }
-      const float dd = EQ ? fabsf(s) : s;
-      const bool c_on = dd < lo;
-      const bool c_pe = !c_on && !(dd > hi);
-      on |= (uint32_t)c_on << bb;
-      pe |= (uint32_t)c_pe << bb;
-    }
+    for (int k = DS - 1; k >= 0; --k) f = __fmaf_rn(f, s, a[k]);
+  } else {
+    f = a[D];
+    for (int k = D - 1; k >= 0; --k) f = __fmaf_rn(f, s, a[k]);
   }
-  *pending = pe;
-  return on;
+  return __fsub_rn(EQ ? fabsf(f) : f, eps);
+}
+
+// P pixels (8 or 32) at offsets s0, s0 + 1, ...: bit b of the result is the
+// sign of pixel b's excess (1: on), *closest the smallest |excess|.
+template <int DS, bool EQ, int P, int S0, int N>
+__device__ __forceinline__ uint32_t eval_pixels(const float (&a)[N], int D, float eps,
+                                                float* closest) {
+  uint32_t m = 0;
+  float c = *closest;
+#pragma unroll
+  for (int b = P - 1; b >= 0; --b) {
+    const float e = excess<DS, EQ>(a, D, (float)(S0 + b), eps);
+    m = __funnelshift_l(__float_as_uint(e), m, 1);
+    c = fminf(c, fabsf(e));
+  }
+  *closest = c;
+  return m;
+}
+
+// The number of offsets in [lo, hi] (integers) at which the increasing
+// polynomial a is below T, when the offsets on either side of the crossing are
+// more than B from it; false when that is not established.
+template <int DS, int N>
+__device__ __forceinline__ bool count_below(const float (&a)[N], int D, float T, float r, float lo,
+                                            float hi, float B, int* n) {
+  float s = __fmul_rn(T - a[0], r);
+#pragma unroll
+  for (int it = 0; it < 2; ++it) {
+    s = fminf(fmaxf(s, lo - 1.0f), hi + 1.0f);
+    float f, d = 0.0f;
+    if constexpr (DS >= 0) {
+      f = a[DS];
+#pragma unroll
+      for (int k = DS - 1; k >= 0; --k) {
+        d = __fmaf_rn(d, s, f);
+        f = __fmaf_rn(f, s, a[k]);
+      }
+    } else {
+      f = a[D];
+      for (int k = D - 1; k >= 0; --k) {
+        d = __fmaf_rn(d, s, f);
+        f = __fmaf_rn(f, s, a[k]);
+      }
+    }
+    s = __fmaf_rn(T - f, __frcp_rn(d), s);
+  }
+  s = floorf(fminf(fmaxf(s, lo - 1.0f), hi));
+  const float e0 = excess<DS, false>(a, D, s, T), e1 = excess<DS, false>(a, D, s + 1.0f, T);
+  *n = (int)(s + 1.0f - lo);
+  return (s < lo || e0 < -B) && (s >= hi || e1 > B);
 }
 
 template <int DS>
-__global__ void __launch_bounds__(kPlotThreads, 3)
-plot_kernel(const PlotJob* __restrict__ jobs, int njobs, int ytab_cap, int gstride, int rmax,
+__global__ void __launch_bounds__(kPlotThreads, 4)
+plot_kernel(const PlotJob* __restrict__ jobs, int njobs, int gstride,
             const ZeroRange* __restrict__ zr, int nzero, int64_t zero_words) {
-  extern __shared__ __align__(16) unsigned char plot_smem[];
+  extern __shared__ __align__(16) float g32s[];  // [rows][gstride] row polynomials
   asm volatile("griddepcontrol.launch_dependents;");
-  // [rmax][gstride] FP64 row polynomials, [rmax][gstride] FP32 copies,
-  // [rmax] thresholds, then the padded FP32 centre table
-  double* g64s = reinterpret_cast<double*>(plot_smem);
-  float* g32s = reinterpret_cast<float*>(g64s + (size_t)rmax * gstride);
-  float4* thrs = reinterpret_cast<float4*>(plot_smem + plot_thr_offset(rmax, gstride));
-  float* ytab = reinterpret_cast<float*>(thrs + rmax);
-  // The block's job and a copy of its descriptor in shared memory: every
-  // global read of the set-up is one round trip on the block's critical path
-  // (the descriptors were just uploaded), so the jobs' first tiles are
-  // compared by one thread each instead of a binary search, and the
-  // descriptor's fields are read from shared memory afterwards.
   __shared__ PlotJob sJ;
-  __shared__ int s_job;
-  if (njobs <= (int)blockDim.x) {
-    const int below = (threadIdx.x < njobs && jobs[threadIdx.x].tile0 <= (int64_t)blockIdx.x);
-    const int n = __syncthreads_count(below);  // tile0 ascends from 0
-    if (threadIdx.x == 0) s_job = n - 1;
-  } else if (threadIdx.x == 0) {
-    int lo = 0, hi = njobs - 1;
-    while (lo < hi) {
-      int mid = (lo + hi + 1) >> 1;
-      if (jobs[mid].tile0 <= (int64_t)blockIdx.x) lo = mid; else hi = mid - 1;
-    }
-    s_job = lo;
-  }
-  __syncthreads();
+  __shared__ uint16_t list[kPass], list_px[kPass], list_re[kPass];
+  __shared__ uint32_t plist[kPendCap];
+  __shared__ int s_n, s_npx, s_nre, s_np;
   {
-    const uint32_t* src = reinterpret_cast<const uint32_t*>(jobs + s_job);
+    const int job = find_job(jobs, njobs);
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(jobs + job);
     uint32_t* dst = reinterpret_cast<uint32_t*>(&sJ);
     for (int i = threadIdx.x; i < (int)(sizeof(PlotJob) / 4); i += blockDim.x) dst[i] = src[i];
   }
+  if (threadIdx.x == 0) s_n = s_npx = s_nre = s_np = 0;
   __syncthreads();
   const PlotJob* J = &sJ;
   const int D = DS >= 0 ? DS : J->degree;
+  constexpr int kG = DS >= 0 ? DS + 1 : kMaxDeg + 1;
   const int row_words = (int)J->row_words;
-  const int res_last = J->res[J->ndim - 1];
+  const int last = J->ndim - 1;
+  const int res_last = J->res[last];
   const int R = J->rows_per_tile;
   const int64_t row0 = ((int64_t)blockIdx.x - J->tile0) * R;
   const int nr = (int)min((int64_t)R, J->nrows - row0);
-  const bool hoisted = J->hoisted != 0;
-  const bool ysmem = hoisted && res_last <= ytab_cap;
+  const bool filter = J->filter != 0;
   const int arity = J->arity;
-  const double ylo = J->lo[arity - 1], ydelta = J->delta[arity - 1];
-  if (hoisted) {
-    // set-up: per row (one thread each) the row polynomial g_0..g_D in FP64
-    // (the inner nested sums of the pa.h order), its FP32 copy and the row's
-    // thresholds eps -+ B_row.  (One thread per (row, j) evaluates every
-    // port's centre D + 1 times: slower where the FP64 pipe is the limit, as
-    // in the set-up of large 3-D plots.)
+  if (filter) {
     for (int r = threadIdx.x; r < nr; r += blockDim.x) {
-      int64_t rest = row0 + r;
-      int64_t idx[kMaxDim];
-      for (int a = J->ndim - 2; a >= 0; --a) {
-        idx[a] = rest % J->res[a];
-        rest /= J->res[a];
+      float x[kMaxDim];
+      const int64_t row = row0 + r;
+      if (row < (1ll << 31)) {
+        uint32_t rest = (uint32_t)row;
+        for (int a = last - 1; a >= 0; --a) {
+          const uint32_t q = a > 0 ? rest / (uint32_t)J->res[a] : 0u;
+          x[a] = centre32(J, a, (float)(rest - q * (uint32_t)J->res[a]) + 0.5f);
+          rest = q;
+        }
+      } else {
+        int64_t rest = row;
+        for (int a = last - 1; a >= 0; --a) {
+          x[a] = centre32(J, a, (float)(rest % J->res[a]) + 0.5f);
+          rest /= J->res[a];
+        }
       }
-      double x[kMaxDim];
-      for (int p = 0; p < arity - 1; ++p)
-        x[p] = centre(J->lo[p], J->delta[p], idx[J->port_axis[p]]);
-      const double* cp = J->coeffs;
-      const float Y = J->ymax;
-      float a = 0.0f, pw = 1.0f;
+      float* gr = g32s + r * gstride;
+      const float* cp = J->c32;
       bool done = false;
       if constexpr (DS >= 0) {
         if (arity == 2 || arity == 3) {
-          double gv[DS + 1];
+          float gv[DS + 1];
           if (arity == 2) row_poly2<DS>(cp, x[0], gv);
           else row_poly3<DS>(cp, x[0], x[1], gv);
 #pragma unroll
-          for (int j = 0; j <= DS; ++j) {
-            const float g1 = __double2float_rn(gv[j]);
-            g64s[r * gstride + j] = gv[j];
-            g32s[r * gstride + j] = g1;
-            a = __fmaf_rn(fabsf(g1), pw, a);
-            pw = __fmul_rn(pw, Y);
-          }
+          for (int j = 0; j <= DS; ++j) gr[j] = gv[j];
           done = true;
         }
       }
-      for (int j = 0; !done && j <= D; ++j) {
-        const double g = nest_rows(arity - 2, D - j, cp, x);  // cp walks block j
-        const float g1 = __double2float_rn(g);
-        g64s[r * gstride + j] = g;
-        g32s[r * gstride + j] = g1;
-        a = __fmaf_rn(fabsf(g1), pw, a);
-        pw = __fmul_rn(pw, Y);
-      }
-      float B = __fmaf_rn(a, J->kfac, J->abs_margin);
-      float tlo = __fsub_rn(J->eps32, B), thi = __fadd_rn(J->eps32, B);
-      if (!(a <= FLT_MAX) || !(B <= FLT_MAX)) {
-        tlo = -INFINITY;  // nothing is certain: every pixel of the row takes the FP64 path
-        thi = INFINITY;
-        B = INFINITY;
-      }
-      thrs[r] = make_float4(tlo, thi, B, 0.0f);
+      // filtered jobs have port p on axis p (every variable on one port)
+      for (int j = 0; !done && j <= D; ++j) gr[j] = nest_rows<float>(arity - 2, D - j, cp, x);
     }
   }
-  // the centre tables (and any earlier work in the stream) are complete and
-  // visible past this point; nothing global is read or written before it but
-  // the job descriptors and coefficients
-  asm volatile("griddepcontrol.wait;" ::: "memory");
   // the later contractions' result buffers that start at zero (each block a
   // share; a block's share is small next to its plot tile)
   if (zero_words > 0) clear_ranges(zr, nzero, zero_words);
-  if (hoisted) {
-    if (ysmem) {
-      // eight loads in flight per thread before the stores (a load-store
-      // loop waits out the L2 latency once per element)
-      const float* __restrict__ yg = J->y32;
-      const int bs = blockDim.x;
-      int i = threadIdx.x;
-      for (; i + 7 * bs < res_last; i += 8 * bs) {
-        float v[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) v[k] = yg[i + k * bs];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) ytab[ypad(i + k * bs)] = v[k];
-      }
-      for (; i < res_last; i += bs) ytab[ypad(i)] = yg[i];
-    }
-    __syncthreads();
-  }
-  const int kind = J->kind, strict = J->strict;
-  const double eps = J->eps;
-  uint64_t* __restrict__ out = J->out;
+  __syncthreads();
+  const bool eq = J->kind == PA_EQ;
+  uint64_t* __restrict__ out = J->out + row0 * row_words;  // the tile's words are consecutive
   // read once: the stores to `out` below could otherwise make the compiler
   // reload these from the job descriptor in every loop
-  const float hword = J->hword;
-  const float* __restrict__ y32 = J->y32;
-  constexpr int kG = DS >= 0 ? DS + 1 : kMaxDeg + 1;
+  const float eps = J->eps32, B = J->bound;
+  const float dl = J->d_hi[arity - 1], dabs = J->dabs;
+  const float ylo_hi = J->lo_hi[arity - 1], ylo_lo = J->lo_lo[arity - 1], dl_lo = J->d_lo[arity - 1];
   const int nwords = nr * row_words;
-  auto load_g = [&](int r, float* g) {
+  const float inv_rw = 1.0f / (float)row_words;
+  // row of the tile's word t (exact: with several rows a tile has few words)
+  auto row_of = [&](int t) { return nr == 1 ? 0 : (int)(((float)t + 0.5f) * inv_rw); };
+  auto ycentre = [&](int i) {
+    const float fi = (float)i + 0.5f;
+    return __fadd_rn(__fmaf_rn(fi, dl, ylo_hi), __fmaf_rn(fi, dl_lo, ylo_lo));
+  };
+  auto load_g = [&](int r, float (&a)[kG]) {
     const float* gr = g32s + r * gstride;
 #pragma unroll
-    for (int j = 0; j < kG; ++j) g[j] = (DS >= 0 || j <= D) ? gr[j] : 0.0f;
+    for (int j = 0; j < kG; ++j) a[j] = (DS >= 0 || j <= D) ? gr[j] : 0.0f;
   };
-  // Phase 1: the whole-word test on every full word (see the header); words it
-  // cannot decide go to a shared list, so that phase 2 evaluates pixels with
-  // every lane busy instead of a few lanes per warp.
-  int* list = reinterpret_cast<int*>(ytab + (ysmem ? res_last + res_last / 64 + 1 : 0));
-  __shared__ int s_n;
-  if (threadIdx.x == 0) s_n = 0;
-  __syncthreads();
   const int lane = threadIdx.x & 31;
-  // Taylor test of the pixels within h of y_c in row r: 1 when every one is
-  // certainly off, 2 when every one is certainly on, 0 when undecided
-  auto decide_span = [&](int r, float yc, float h) -> int {
-    float g[kG];
-    load_g(r, g);
-    const float4 th = thrs[r];
-    const float ya = fabsf(yc), yw = ya + h;
-    // Horner for F and F' at y_c; S1 at |y_c| and S2 at |y_c| + h
-    float fc = g[D], dc = 0.0f, s1 = 0.0f, s2 = 0.0f;
-    for (int j = D - 1; j >= 0; --j) {
-      dc = __fmaf_rn(dc, yc, fc);
-      fc = __fmaf_rn(fc, yc, g[j]);
-    }
-    for (int j = D; j >= 1; --j) s1 = __fmaf_rn(s1, ya, (float)j * fabsf(g[j]));
-    for (int j = D; j >= 2; --j) s2 = __fmaf_rn(s2, yw, (float)(j * (j - 1)) * fabsf(g[j]));
-    const float e1 = (float)(2 * D + 4) * 5.9604645e-8f * s1;  // (2D + 4) 2^-24 S1
-    const float taylor = __fmaf_rn(h, fabsf(dc) + e1, 0.5f * h * h * s2) * 1.01f;
-    const float margin = __fmaf_rn(4.0f, th.z, taylor);
-    if (kind == PA_EQ) return (fabsf(fc) > th.y + margin) ? 1 : 0;
-    if (fc > th.y + margin) return 1;
-    if (fc < th.x - margin) return 2;
-    return 0;
-  };
-  // Spans of four full words are tested first (centre pixel 128, four times
-  // the word's half-width): on a sparse plot most of them are decided at once.
-  // Words of undecided spans (and of rows that are not whole spans) are
-  // tested one by one; the words no test decides go to phase 2.
-  const bool spans = hoisted && (row_words % 4 == 0) && (res_last == row_words * 64);
-  const int S = spans ? 4 : 1;
-  const int nspans = nwords / S;
-  for (int base = 0; base < nspans; base += blockDim.x) {
-    const int sp = base + threadIdx.x;
-    int span_dec = 0;  // this lane's span decided as a whole (1 off, 2 on)
-    int r = 0, w0 = 0;
-    if (sp < nspans) {
-      r = (sp * S) / row_words;
-      w0 = sp * S - r * row_words;
-      if (S == 4) {
-        const int i0 = w0 * 64;
-        const float yc = ysmem ? ytab[ypad(i0 + 128)] : __ldg(y32 + i0 + 128);
-        span_dec = decide_span(r, yc, 4.0f * hword);
-        if (span_dec) {
-          uint64_t* o = out + (row0 + r) * row_words + w0;
-          const uint64_t v = span_dec == 1 ? 0ull : ~0ull;
-          o[0] = v;
-          o[1] = v;
-          o[2] = v;
-          o[3] = v;
-        }
-      }
-    }
-    for (int k = 0; k < S; ++k) {
-      bool keep = false;
-      if (sp < nspans && !span_dec) {
-        keep = true;
-        const int w = w0 + k;
-        const int i0 = w * 64;
-        if (hoisted && res_last - i0 >= 64) {
-          const float yc = ysmem ? ytab[i0 + w + 32] : __ldg(y32 + i0 + 32);
-          const int dec = decide_span(r, yc, hword);
-          if (dec) {
-            out[(row0 + r) * row_words + w] = dec == 1 ? 0ull : ~0ull;
-            keep = false;
-          }
-        }
-      }
-      // warp-aggregated append of the undecided words
-      const unsigned m = __ballot_sync(0xffffffffu, keep);
-      int off = 0;
-      if (lane == 0 && m) off = atomicAdd(&s_n, __popc(m));
-      off = __shfl_sync(0xffffffffu, off, 0);
-      if (keep) list[off + __popc(m & ((1u << lane) - 1u))] = r * row_words + w0 + k;
-    }
-  }
-  __syncthreads();
-  // Phase 2: pixel by pixel.  A block with few undecided words (a curve
-  // crossing some of its rows) cuts each into C = 8 pieces of 8 pixels, one
-  // per thread, so that they spread over its threads; otherwise each thread
-  // takes whole words (C = 1), whose 64 pixels it evaluates with more
-  // independent work in flight and one set-up per word.
-  const int nlist = s_n;
   const int nthr = (int)blockDim.x;
-  const int C = 4 * nlist <= nthr ? 8 : 1;
-  const int PC = 64 / C;
-  if (C == 1) {
-    for (int e = threadIdx.x; e < nlist; e += nthr) {
-      const int f = list[e];
-      const int r = f / row_words, w = f - r * row_words;
-      const int64_t row = row0 + r;
-      const int i0 = w * 64;
-      const int nb = min(64, res_last - i0);
-      uint64_t word = 0;
-      if (hoisted) {
-        float g[kG];
-        load_g(r, g);
-        const float4 th = thrs[r];
-        const float lo = th.x, hi = th.y;
-        uint64_t pending = 0;
-        const float* ytab_w = ytab + i0 + w;  // ypad(i0 + b) = i0 + w + b
-        if (kind == PA_EQ) {
-          if (ysmem) eval_word_any<DS, true, true>(g, D, lo, hi, ytab_w, y32, i0, nb, &word, &pending);
-          else eval_word_any<DS, true, false>(g, D, lo, hi, ytab_w, y32, i0, nb, &word, &pending);
-        } else {
-          if (ysmem) eval_word_any<DS, false, true>(g, D, lo, hi, ytab_w, y32, i0, nb, &word, &pending);
-          else eval_word_any<DS, false, false>(g, D, lo, hi, ytab_w, y32, i0, nb, &word, &pending);
-        }
-        while (pending) {
-          const int bb = __ffsll((long long)pending) - 1;
-          pending &= pending - 1;
-          if (exact64(centre(ylo, ydelta, i0 + bb), g64s + r * gstride, D, kind, eps, strict))
-            word |= (1ull << bb);
-        }
-      } else {
-        for (int bb = 0; bb < nb; ++bb)
-          if (general64(J, row, i0 + bb)) word |= (1ull << bb);
+  // Taylor coefficients about pixel ic of row r, scaled to steps of one pixel
+  auto expand = [&](int r, int ic, float (&a)[kG]) {
+    load_g(r, a);
+    taylor_shift<DS>(a, D, ycentre(ic));
+    float pw = dl;
+    if constexpr (DS >= 0) {
+#pragma unroll
+      for (int j = 1; j <= DS; ++j) {
+        a[j] = __fmul_rn(a[j], pw);
+        pw = __fmul_rn(pw, dl);
       }
-      out[row * row_words + w] = word;
-    }
-  }
-  for (int e = threadIdx.x; C > 1 && e < nlist * C; e += nthr) {
-    const int f = list[e / C], c = e % C;
-    const int r = f / row_words, w = f - r * row_words;
-    const int64_t row = row0 + r;
-    const int ic0 = w * 64 + PC * c;  // first pixel of the piece
-    uint64_t bits = 0;
-    float g[kG];
-    float lo = 0.0f, hi = 0.0f;
-    if (hoisted) {
-      load_g(r, g);
-      const float4 th = thrs[r];
-      lo = th.x;
-      hi = th.y;
-    }
-    for (int g8 = 0; g8 < PC / 8; ++g8) {
-      const int ic = ic0 + 8 * g8;
-      const int nb8 = min(8, res_last - ic);  // <= 0: padding past the row
-      if (nb8 <= 0) break;
-      uint32_t b8 = 0;
-      if (hoisted) {
-        uint32_t pending = 0;
-        const float* yt = ytab + ic + w;  // ypad(ic + b) = ic + w + b
-        if (kind == PA_EQ) {
-          if (ysmem) b8 = eval8<DS, true, true>(g, D, lo, hi, yt, y32, ic, nb8, &pending);
-          else b8 = eval8<DS, true, false>(g, D, lo, hi, yt, y32, ic, nb8, &pending);
-        } else {
-          if (ysmem) b8 = eval8<DS, false, true>(g, D, lo, hi, yt, y32, ic, nb8, &pending);
-          else b8 = eval8<DS, false, false>(g, D, lo, hi, yt, y32, ic, nb8, &pending);
-        }
-        while (pending) {
-          const int bb = __ffs(pending) - 1;
-          pending &= pending - 1;
-          if (exact64(centre(ylo, ydelta, ic + bb), g64s + r * gstride, D, kind, eps, strict))
-            b8 |= 1u << bb;
-        }
-      } else {
-        for (int bb = 0; bb < nb8; ++bb)
-          if (general64(J, row, ic + bb)) b8 |= 1u << bb;
+    } else {
+      for (int j = 1; j <= D; ++j) {
+        a[j] = __fmul_rn(a[j], pw);
+        pw = __fmul_rn(pw, dl);
       }
-      bits |= (uint64_t)b8 << (8 * g8);
     }
-    uint64_t* ow = out + row * row_words + w;
-    switch (C) {
-      case 1: *ow = bits; break;
-      case 2: reinterpret_cast<uint32_t*>(ow)[c] = (uint32_t)bits; break;
-      case 4: reinterpret_cast<uint16_t*>(ow)[c] = (uint16_t)bits; break;
-      default: reinterpret_cast<uint8_t*>(ow)[c] = (uint8_t)bits; break;
+  };
+  auto full_mask = [](int nb) { return nb >= 64 ? ~0ull : (1ull << nb) - 1ull; };
+  // warp-aggregated append of k to a shared list (every lane of the warp)
+  auto append = [&](uint16_t* to, int* count, bool keep, int k) {
+    const unsigned m = __ballot_sync(0xffffffffu, keep);
+    if (!m) return;
+    int off = 0;
+    if (lane == 0) off = atomicAdd(count, __popc(m));
+    off = __shfl_sync(0xffffffffu, off, 0);
+    if (keep) to[off + __popc(m & ((1u << lane) - 1u))] = (uint16_t)k;
+  };
+  for (int t0 = 0; t0 < nwords; t0 += kPass) {
+    const int np = min(kPass, nwords - t0);
+    if (!filter) {
+      // FP64 at every pixel, eight pixels per thread
+      for (int e = threadIdx.x; e < 8 * np; e += nthr) {
+        const int t = t0 + (e >> 3), c8 = e & 7, r = row_of(t), w = t - r * row_words;
+        const int i0 = w * 64 + 8 * c8, nb = min(8, res_last - i0);
+        uint32_t bits = 0;
+        for (int b = 0; b < nb; ++b)
+          if (decide_pixel64<DS>(J, row0 + r, i0 + b)) bits |= 1u << b;
+        reinterpret_cast<uint8_t*>(out + t)[c8] = (uint8_t)bits;
+      }
+      continue;
+    }
+    // ---- phase 1: whole words
+    for (int base = 0; base < np; base += nthr) {
+      const int k = base + threadIdx.x;
+      bool keep = k < np;
+      if (keep) {
+        const int t = t0 + k, r = row_of(t), w = t - r * row_words;
+        const int nb = min(64, res_last - w * 64), c = nb >> 1;
+        float a[kG];
+        load_g(r, a);
+        taylor_shift<DS>(a, D, ycentre(w * 64 + c));
+        const float h = __fmul_rn((float)c, dabs);
+        float S = fabsf(a[D]);
+        if constexpr (DS >= 0) {
+#pragma unroll
+          for (int j = DS - 1; j >= 1; --j) S = __fmaf_rn(S, h, fabsf(a[j]));
+        } else {
+          for (int j = D - 1; j >= 1; --j) S = __fmaf_rn(S, h, fabsf(a[j]));
+        }
+        if (D >= 1) S = __fmul_rn(S, h);
+        else S = 0.0f;
+        const float v = eq ? fabsf(a[0]) : a[0], margin = __fmaf_rn(3.0f, B, S);
+        const bool off = v - eps > margin, on = eps - v > margin;
+        if (off || on) {
+          out[t] = off ? 0ull : full_mask(nb);
+          keep = false;
+        }
+      }
+      append(list, &s_n, keep, k);
+    }
+    __syncthreads();
+    // ---- phase 2: band edges of words on which f is monotone
+    const int nlist = s_n;
+    for (int base = 0; base < nlist; base += nthr) {
+      const int e = base + threadIdx.x;
+      bool hard = false;
+      int k = 0;
+      if (e < nlist) {
+        k = list[e];
+        const int t = t0 + k, r = row_of(t), w = t - r * row_words;
+        const int nb = min(64, res_last - w * 64), ic = nb >> 1;
+        float a[kG];
+        expand(r, w * 64 + ic, a);
+        // f' keeps a_1's sign when a_1 outweighs the other terms at the
+        // word's ends by more than the coefficients' errors (D B / hs)
+        const float hs = (float)ic;
+        float Q = 0.0f;
+        if constexpr (DS >= 2) {
+          Q = (float)DS * fabsf(a[DS]);
+#pragma unroll
+          for (int j = DS - 1; j >= 2; --j) Q = __fmaf_rn(Q, hs, (float)j * fabsf(a[j]));
+          Q = __fmul_rn(Q, hs);
+        } else if constexpr (DS < 0) {
+          for (int j = D; j >= 2; --j) Q = __fmaf_rn(Q, hs, (float)j * fabsf(a[j]));
+          Q = __fmul_rn(Q, hs);
+        }
+        const float a1 = D >= 1 ? a[D >= 1 ? 1 : 0] : 0.0f;
+        hard = !((fabsf(a1) * 0.999f - Q) * hs > (float)(2 * D) * B);
+        if (!hard) {
+          const bool up = a1 > 0.0f;
+#pragma unroll
+          for (int j = 0; j < kG; ++j)
+            if (DS >= 0 || j <= D) a[j] = up ? a[j] : -a[j];
+          const float rc = __frcp_rn(fabsf(a1));
+          const float lo = -(float)ic, hi = (float)(nb - 1 - ic);
+          uint64_t bits;
+          if (eq) {
+            int n0, n1;
+            hard = !(count_below<DS>(a, D, -eps, rc, lo, hi, B, &n0) &
+                     count_below<DS>(a, D, eps, rc, lo, hi, B, &n1));
+            bits = full_mask(n1) & ~full_mask(n0);
+          } else {
+            int n;
+            hard = !count_below<DS>(a, D, up ? eps : -eps, rc, lo, hi, B, &n);
+            bits = up ? full_mask(n) : full_mask(nb) & ~full_mask(n);
+          }
+          if (!hard) out[t] = bits;
+        }
+      }
+      append(list_px, &s_npx, hard, k);
+    }
+    __syncthreads();
+    // ---- phase 3: pixels.  A block with few such words cuts each into eight
+    // pieces of 8 pixels, so that they spread over its threads.
+    const int npx = s_npx;
+    const int C = 4 * npx <= nthr ? 8 : 1;
+    for (int base = 0; base < npx * C; base += nthr) {
+      const int e = base + threadIdx.x;
+      bool close = false;
+      int k = 0;
+      if (e < npx * C) {
+        k = list_px[C == 1 ? e : e >> 3];
+        const int c8 = C == 1 ? 0 : e & 7;
+        const int t = t0 + k, r = row_of(t), w = t - r * row_words;
+        const int i0 = w * 64 + 8 * c8;                      // first pixel of the piece
+        const int nb = min(C == 1 ? 64 : 8, res_last - i0);  // <= 0: padding past the row
+        uint64_t bits = 0;
+        if (nb > 0) {
+          // expansion about a pixel of the row near the piece's middle; a piece
+          // cut by the row's end is also evaluated past it, those bits dropped
+          const int half = C == 1 ? 32 : 4;
+          const int ic = nb > half ? half : C == 1 && nb > 16 ? 16 : nb >> 1;
+          float a[kG];
+          expand(r, i0 + ic, a);
+          float closest = INFINITY;
+          if (C == 1 && nb > 32) {
+            uint32_t lo, hi;
+            if (eq) {
+              lo = eval_pixels<DS, true, 32, -32>(a, D, eps, &closest);
+              hi = eval_pixels<DS, true, 32, 0>(a, D, eps, &closest);
+            } else {
+              lo = eval_pixels<DS, false, 32, -32>(a, D, eps, &closest);
+              hi = eval_pixels<DS, false, 32, 0>(a, D, eps, &closest);
+            }
+            bits = ((uint64_t)hi << 32) | lo;
+          } else if (C == 1 && nb > 16) {
+            bits = eq ? eval_pixels<DS, true, 32, -16>(a, D, eps, &closest)
+                      : eval_pixels<DS, false, 32, -16>(a, D, eps, &closest);
+          } else if (C == 8 && nb > 4) {
+            bits = eq ? eval_pixels<DS, true, 8, -4>(a, D, eps, &closest)
+                      : eval_pixels<DS, false, 8, -4>(a, D, eps, &closest);
+          } else {
+            closest = 0.0f;  // few pixels: left to phase 4
+          }
+          bits &= full_mask(nb);
+          close = !(closest > B);
+        }
+        if (C == 1) out[t] = bits;
+        else reinterpret_cast<uint8_t*>(out + t)[c8] = (uint8_t)bits;
+      }
+      append(list_re, &s_nre, close, k);  // (a word may be listed once per piece)
+    }
+    __syncthreads();
+    // ---- phase 4: words with pixels FP32 cannot decide, a warp each
+    const int nre = s_nre;
+    for (int e = threadIdx.x >> 5; e < nre; e += nthr >> 5) {
+      const int k = list_re[e];
+      const int t = t0 + k, r = row_of(t), w = t - r * row_words;
+      const int nb = min(64, res_last - w * 64), ic = nb >> 1;
+      float a[kG];
+      expand(r, w * 64 + ic, a);
+      uint32_t half[2];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int b = 32 * q + lane;
+        const float s = (float)(b - ic);
+        const float ex = eq ? excess<DS, true>(a, D, s, eps) : excess<DS, false>(a, D, s, eps);
+        bool on = b < nb && ex < 0.0f;
+        if (b < nb && !(fabsf(ex) > B)) {
+          const int at = atomicAdd(&s_np, 1);
+          on = false;
+          if (at < kPendCap) plist[at] = (uint32_t)k * 64u + (uint32_t)b;
+          else on = decide_pixel64<DS>(J, row0 + r, (int64_t)w * 64 + b);
+        }
+        half[q] = __ballot_sync(0xffffffffu, on);
+      }
+      if (lane == 0) out[t] = ((uint64_t)half[1] << 32) | half[0];
+    }
+    __syncthreads();
+    // ---- phase 5: the collected pixels in FP64, into the words stored above
+    const int npend = min(s_np, kPendCap);
+    for (int q = threadIdx.x; q < npend; q += nthr) {
+      const int k = (int)(plist[q] >> 6), b = (int)(plist[q] & 63u);
+      const int t = t0 + k, r = row_of(t), w = t - r * row_words;
+      if (decide_pixel64<DS>(J, row0 + r, (int64_t)w * 64 + b))
+        atomicOr(reinterpret_cast<unsigned long long*>(out + t), 1ull << b);
+    }
+    if (t0 + kPass < nwords) {
+      __syncthreads();
+      if (threadIdx.x == 0) s_n = s_npx = s_nre = s_np = 0;
+      __syncthreads();
     }
   }
 }
@@ -745,7 +789,7 @@ plot_corner_kernel(const CornerJob* __restrict__ jobs, int njobs, int64_t total_
           f = run_expr(J.prog, J.nops, J.consts, x);
         } else {
           const double* cp = J.coeffs;
-          f = nest_rows(J.arity - 1, J.degree, cp, x);
+          f = nest_rows<double>(J.arity - 1, J.degree, cp, x);
         }
         n |= (decide64(f, J.kind, J.eps, J.strict) ? 1u : 0u) << j;
         pp |= ((isfinite(f) && f > 0.0) ? 1u : 0u) << j;
@@ -771,15 +815,15 @@ void launch_plot_corner(const CornerJob* d_jobs, int njobs, int64_t total_words,
 
 // Blocks of the plot kernel (of this degree) that the GPU holds at once:
 // per SM as the occupancy calculator gives it for 256 threads and a typical
-// 16 KB of shared memory (registers are the limit), times the SMs.  Cached;
-// 3 x 152 when the device cannot be asked.
+// 4 KB of row polynomials (registers are the limit), times the SMs.  Cached;
+// 4 x 152 when the device cannot be asked.
 int plot_resident_blocks(int common_degree) {
   static std::mutex mu;
   static std::map<std::pair<int, int>, int> cache;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) {
     cudaGetLastError();
-    return 3 * 152;
+    return 4 * 152;
   }
   const std::pair<int, int> key(dev, common_degree);
   {
@@ -796,9 +840,9 @@ int plot_resident_blocks(int common_degree) {
     default: fn = reinterpret_cast<const void*>(plot_kernel<-1>); break;
   }
   int sms = 0, per = 0;
-  int v = 3 * 152;
+  int v = 4 * 152;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, kPlotThreads, 16 * 1024) ==
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, kPlotThreads, 4 * 1024) ==
           cudaSuccess &&
       sms > 0 && per > 0)
     v = sms * per;
@@ -815,34 +859,17 @@ cudaError_t probe_kernel_image() {
 }
 
 void launch_plot(const PlotJob* d_jobs, int njobs, int64_t total_tiles, int max_rows_per_tile,
-                 int max_degree, int common_degree, int max_res_last, int64_t max_tile_words,
-                 const ZeroRange* d_zero, int nzero, int64_t zero_words, cudaStream_t s) {
+                 int max_degree, int common_degree, const ZeroRange* d_zero, int nzero,
+                 int64_t zero_words, cudaStream_t s) {
   if (total_tiles <= 0) return;
-  const int ycap = max_res_last <= kYTabCap ? max_res_last : 0;
-  const int gstride = max_degree + 1, rmax = max_rows_per_tile;
-  // thresholds, centre table, then the list of undecided words (one int per
-  // word of the largest tile)
-  const size_t smem = plot_thr_offset(rmax, gstride) + (size_t)rmax * 16 +
-                      (size_t)(ycap + ycap / 64 + 1) * sizeof(float) +
-                      (size_t)max_tile_words * sizeof(int);
+  const int gstride = max_degree + 1;
+  const size_t smem = (size_t)max_rows_per_tile * gstride * sizeof(float);
   const unsigned grid = (unsigned)total_tiles;
-  // programmatic dependent launch: the blocks may start while the centre
-  // tables are being computed and wait for them after their row set-up
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(kPlotThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
 #define PA_PLOT(DD)                                                                          \
   do {                                                                                       \
     smem_limit(reinterpret_cast<const void*>(plot_kernel<DD>), smem);                        \
-    cudaLaunchKernelEx(&cfg, plot_kernel<DD>, d_jobs, njobs, ycap, gstride, rmax, d_zero,    \
-                       nzero, zero_words);                                                   \
+    plot_kernel<DD><<<grid, kPlotThreads, smem, s>>>(d_jobs, njobs, gstride, d_zero, nzero,  \
+                                                     zero_words);                            \
   } while (0)
   switch (common_degree) {
     case 1: PA_PLOT(1); break;
