@@ -477,7 +477,7 @@ void flush_mma(Builder& bd) {
 
 void flush_rowor_only(Builder& bd);
 
-// The waiting contractions as launches: one per tile width, one for the
+// The waiting contractions as launches: one per CTA size, one for the
 // tensor-core path.
 void flush_rowor(Builder& bd) {
   flush_rowor_only(bd);
@@ -500,10 +500,17 @@ void flush_rowor_only(Builder& bd) {
     if (done[i]) continue;
     std::vector<RowOrDesc> group;
     for (size_t j = i; j < bd.pend.size(); ++j)
-      if (!done[j] && bd.pend[j].Nt == bd.pend[i].Nt) {
+      if (!done[j] && bd.pend[j].threads == bd.pend[i].threads) {
         group.push_back(bd.pend[j]);
         done[j] = 1;
       }
+    // the CTAs with most work first: what starts last is short (work of a CTA:
+    // its rows times their words, next to its tile)
+    auto work = [](const RowOrDesc& d) {
+      return d.rows_per_split * (d.Kc / 64 + 8) + 2 * (int64_t)d.Kc;
+    };
+    std::stable_sort(group.begin(), group.end(),
+                     [&](const RowOrDesc& x, const RowOrDesc& y) { return work(x) > work(y); });
     std::vector<CUtensorMap> maps(group.size());
     std::vector<int64_t> cta0(group.size() + 1, 0);
     size_t smem = 0;
@@ -522,7 +529,7 @@ void flush_rowor_only(Builder& bd) {
     op.n = (int)group.size();
     op.count = cta0.back();
     op.smem = smem;
-    op.i0 = group[0].Nt;
+    op.i0 = group[0].threads;
     if (op.count > 0x7fffffffLL) bd.fail(PA_ERR_TOO_LARGE, "contraction grid too large");
     bd.ops.push_back(op);
   }
@@ -677,16 +684,11 @@ double rowor_cost_us(const pa_ctx* ctx, const JoinShape& js, double dens) {
   const double r0 = ctx ? ctx->rate_or : 2.0e5, r1 = ctx ? ctx->rate_or_dense : 9.0e5;
   const double f = std::min(1.0, std::max(0.0, log(std::max(dens, 1e-12) / 0.02) / log(8.0)));
   const double rate_or = r0 * pow(r1 / r0, f);
-  RowOrDesc rd;
-  memset(&rd, 0, sizeof rd);
-  rd.nbatch = js.nbatch;
-  rd.M = js.M;
-  rd.K = js.K;
-  rd.Nw = (int64_t)ceil(N / 64);
-  rd.a_row_words = (js.K + 63) / 64;
-  rowor_plan(rd, 152);
-  const double units = nb * M * (double)rd.k_chunks * (double)rd.n_tiles;
-  return dens * M * K * nb * ceil(N / 64) / rate_or + units / kRowOrUnitsPerUs;
+  const double Nw = ceil(N / 64);
+  int Nt = 1;
+  while (Nt < 32 && Nt < Nw) Nt <<= 1;
+  const double units = nb * M * ceil(K / (double)rowor_max_kc(Nt, 1024)) * ceil(Nw / Nt);
+  return dens * M * K * nb * Nw / rate_or + units / kRowOrUnitsPerUs;
 }
 
 // Bytes per microsecond the two expansion kernels write together (measured
@@ -734,7 +736,7 @@ void add_occupancy(Builder& bd, MmaDesc& md) {
 // rx, ry: estimated densities of X and Y (< 0: unknown); *rho_out receives the
 // estimated density of the result when both are known.
 BitArr join(Builder& bd, const BitArr& X, const BitArr& Y, const std::vector<int>& keep,
-            const std::vector<int64_t>& vres, const BitArr* target, int64_t target_ctas,
+            const std::vector<int64_t>& vres, const BitArr* target, double share,
             double rx = -1.0, double ry = -1.0, double* rho_out = nullptr) {
   const JoinShape js = analyze_join(X, Y, keep, vres);
   bd.st.pixel_ops_dense += js.cost;
@@ -840,7 +842,7 @@ BitArr join(Builder& bd, const BitArr& X, const BitArr& Y, const std::vector<int
   d.stat = bd.d_stat;
   if (d.M > 0x7fffffffLL || d.K > 0x7fffffffLL)
     bd.fail(PA_ERR_TOO_LARGE, "contraction with more than 2^31 rows");
-  rowor_plan(d, target_ctas);
+  rowor_plan(d, share);
   if (d.atomic) {
     Op op;
     op.kind = OP_MEMSET;
@@ -1439,7 +1441,7 @@ void fold_memsets(Builder& bd) {
 
 // Plots of all networks in one launch, then their joins level by level:
 // the joins of one level of every network's cluster tree are independent and
-// share one contraction launch per tile width.
+// share one contraction launch per CTA size.
 void build_networks(Builder& bd, std::vector<Network>& nets, bool one_join_per_launch = false,
                     std::vector<BitArr>* join_results = nullptr) {
   std::vector<PlotReq> reqs;
@@ -1500,11 +1502,11 @@ void build_networks(Builder& bd, std::vector<Network>& nets, bool one_join_per_l
     for (size_t k = 0; k < nets.size(); ++k)
       for (size_t t = 0; t < S[k].plan.joins.size(); ++t)
         n_in_level += (S[k].level[nets[k].nrel + t] == lv);
-    // The row-OR joins of a level share one launch; each gets a share of one
-    // wave of 152 CTAs in proportion to its estimated time, so a large join
+    // The row-OR joins of a level share one launch; each gets a share of the
+    // 152 SMs in proportion to its estimated time, so a large join
     // among many small ones is split over many CTAs instead of setting the
     // launch's length alone.
-    std::map<std::pair<size_t, int>, int64_t> target_of;
+    std::map<std::pair<size_t, int>, double> share_of;
     {
       std::vector<std::pair<std::pair<size_t, int>, double>> work;
       double total = 0.0;
@@ -1517,18 +1519,18 @@ void build_networks(Builder& bd, std::vector<Network>& nets, bool one_join_per_l
           const JoinShape js = analyze_join(s.slots[jn.a], s.slots[jn.b], jn.keep, s.vres);
           double w = 0.0;
           if (!js.hadamard && !js.outer && !js.dot) {
-            double ra = 0.05;
+            double ra = -1.0;
             if (!s.dens.empty() && s.dens[jn.a] >= 0 && s.dens[jn.b] >= 0)
               ra = or_density(js.swap ? s.dens[jn.b] : s.dens[jn.a], js.private_a);
-            w = rowor_cost_us(bd.ctx, js, ra);
+            // (a join of the tensor path is in another launch)
+            if (!use_mma(bd.ctx, js, ra)) w = rowor_cost_us(bd.ctx, js, ra >= 0 ? ra : 0.05);
           }
           work.push_back({{k, t}, w});
           total += w;
         }
       }
       for (const auto& e : work)
-        target_of[e.first] =
-            total > 0 ? std::max<int64_t>(1, (int64_t)(152.0 * e.second / total)) : 1;
+        share_of[e.first] = total > 0 ? 152.0 * e.second / total : 1.0;
     }
     bd.defer = !one_join_per_launch;
     for (size_t k = 0; k < nets.size(); ++k) {
@@ -1542,7 +1544,7 @@ void build_networks(Builder& bd, std::vector<Network>& nets, bool one_join_per_l
         const bool dn = !s.dens.empty();
         s.slots[nrel + t] = join(bd, s.slots[jn.a], s.slots[jn.b], jn.keep, s.vres,
                                  last ? &nets[k].target : nullptr,
-                                 one_join_per_launch ? 152 : target_of[{k, t}],
+                                 one_join_per_launch ? 152.0 : share_of[{k, t}],
                                  dn ? s.dens[jn.a] : -1.0, dn ? s.dens[jn.b] : -1.0,
                                  dn ? &s.dens[nrel + t] : nullptr);
         if (dn) {
@@ -2484,7 +2486,7 @@ pa_status pa_autotune(pa_ctx* ctx, pa_rates* out, void* stream) {
           [&] {
             launch_rowor(reinterpret_cast<const RowOrDesc*>(tab),
                          reinterpret_cast<const CUtensorMap*>(tab + 1024),
-                         reinterpret_cast<const int64_t*>(tab + 2048), 1, rcta[1], rsmem, rd.Nt, s);
+                         reinterpret_cast<const int64_t*>(tab + 2048), 1, rcta[1], rsmem, rd.threads, s);
           },
           reps);
       cudaMemcpy(&words, ctx->d_stat, sizeof words, cudaMemcpyDeviceToHost);

@@ -397,32 +397,39 @@ void launch_ewise(const EwJob* d_jobs, const int64_t* d_cta0, int n, int64_t gri
 }
 
 // ---------------------------------------------------------------- row-OR
-// One CTA owns the tile B[b][k0 .. k0+Kc)[n0 .. n0+Nt) in shared memory, staged
-// by the Tensor Memory Accelerator (2-D boxes of 256 rows x Nt words) when the
-// row pitch allows it, else by plain loads.  Next to it the CTA builds the ORs
-// of aligned blocks of 4, 16 and 64 tile rows (tables T2, T4, T6; T0 is the
-// tile itself), plus an all-zero sentinel row.  A run of set bits in a row of
-// A selects a run of B rows, whose OR is the OR of the maximal aligned blocks
-// covering it: the plotted relations are thick curves, so most set bits lie in
-// long runs and a row needs a few block lookups instead of one per bit.
-// Each warp then takes one output row at a time:
-//   1. its lanes load up to 32 words of the row's A bits for this K range and
-//      split each word into maximal all-ones aligned blocks of 64, 16, 4 and 1
-//      bits (a few bit operations), counting them;
-//   2. every lane writes the table rows of its blocks into the warp's list in
-//      shared memory (256 entries: slots taken from a warp counter; a row
-//      with more blocks goes through the list in ordered windows);
-//   3. the warp splits into 32/Nt groups of Nt lanes; group g ORs table rows
-//      list[g], list[g + 32/Nt], ... (four loads in flight per lane), lane l of
-//      a group holding word n0 + l;
-//   4. the groups' words are OR-ed together with shuffles and stored.
+// One CTA owns the tile B[b][k0 .. k0+Kc)[n0 .. n0+G) in shared memory, staged
+// by bulk copies when the tile is one run of memory, by 2-D boxes of 64 rows x
+// G words (tensor map) when the row pitch allows it, else by 8-byte
+// asynchronous copies.  Next to it the CTA
+// builds the ORs of aligned blocks of 4, 16 and 64 tile rows (tables T2, T4,
+// T6; T0 is the tile itself), plus an all-zero sentinel row.  A run of set bits
+// in a row of A selects a run of B rows, whose OR is the OR of the maximal
+// aligned blocks covering it: the plotted relations are thick curves, so most
+// set bits lie in long runs and a row needs a few block lookups instead of one
+// per bit.  Each warp takes a batch of R consecutive output rows at a time, a
+// group of L lanes per row for its K range's L A words (L <= 32, R = 32 / L):
+//   1. the lanes load one A word each and split it into maximal all-ones
+//      aligned blocks of 64, 16, 4 and 1 bits (a few bit operations);
+//   2. a prefix sum over the lanes gives every block its slot in the warp's
+//      list in shared memory, the rows' entries one after another;
+//   3. the warp splits into groups of G/2 lanes (two words each: one 16-byte
+//      load per lookup); a group ORs a row's table rows, three loads in flight
+//      per lane.  With more groups than rows a row's list is dealt over several
+//      groups and their words are OR-ed together with shuffles.
+// A batch whose blocks exceed the list goes row by row through it in windows.
+// What bounds it: instruction issue (2 to 2.6 per clock and SM in the rows).  A
+// row by itself costs about 200 warp instructions whatever its length, most of
+// it on lanes without an A word; in batches a row of 8 or 9 words costs 50 to
+// 70.  Against one row per warp, one launch per tile width and 1024-thread CTAs
+// throughout (ncu, cold): 4096 chains 2.92 -> 0.78 ms, 38 networks 3.89 -> 1.02
+// ms, two 4001^3 joins 41 -> 24 us, four 2048^3 joins 20 -> 16 us.
 namespace {
 
-constexpr int kRowOrThreads = 1024;
-// Entries of a warp's list per window, plus sentinel padding.  A unit whose
-// blocks do not fit is processed in several windows.
+constexpr int kRowOrThreads = 1024;  // at most; see rowor_plan
+constexpr int kRowOrMaxKc = 2048;    // K range of a CTA: one A word per lane
+// Entries of a warp's list per window, plus sentinel padding.
 constexpr int kListWin = 256;
-constexpr int kListCap = kListWin + 128;
+constexpr int kListCap = kListWin + 4 * 32;  // (a window is padded to 4 entries per group)
 
 // Tile rows of the tables for a K range staged in `staged` rows: T0 (rounded
 // up to whole 64-row groups), the sentinel, T2, T4 and T6.
@@ -454,163 +461,107 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long l
   return false;
 }
 
-// Launch description: problem p owns CTAs [cta0[p], cta0[p+1]); its
-// descriptor and tensor map (used when d.use_tma) live in global memory.
+// The words a lane holds of an output row: two adjacent ones (one 16-byte
+// shared-memory load per lookup) except on one-word rows.
+template <int W>
+struct Words {
+  uint64_t v[W];
+};
+__device__ __forceinline__ void or_row(Words<1>& w, const uint64_t* p) { w.v[0] |= *p; }
+__device__ __forceinline__ void or_row(Words<2>& w, const uint64_t* p) {
+  const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(p);
+  w.v[0] |= t.x;
+  w.v[1] |= t.y;
+}
+
+// The output rows of one CTA: its tile's tables are in bs (G words per row).
 template <int G>
-__global__ void __launch_bounds__(kRowOrThreads)
-rowor_tile_kernel(const RowOrDesc* __restrict__ descs, const CUtensorMap* __restrict__ maps,
-                  const int64_t* __restrict__ cta0s, int nprob) {
-  extern __shared__ __align__(1024) uint64_t bs[];
-  __shared__ RowOrDesc sd;
-  __shared__ int s_p;
-  // the next launch may be scheduled onto SMs this grid frees; it waits for
-  // this grid's completion before it touches any data
-  asm volatile("griddepcontrol.launch_dependents;");
-  const int tid = threadIdx.x;
-  const int nwarps = blockDim.x >> 5;
-  if (tid == 0) {
-    int lo = 0, hi = nprob - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (cta0s[mid] <= (int64_t)blockIdx.x) lo = mid; else hi = mid - 1;
-    }
-    s_p = lo;
-    sd = descs[lo];
-  }
-  __syncthreads();
-  const int p = s_p;
-  const RowOrDesc& d = sd;
-  const CUtensorMap* tmap = maps + p;
-  const int64_t staged = d.use_tma ? ((int64_t)d.Kc + 255) / 256 * 256 : d.Kc;
-  const int r64 = (int)rowor_r64(staged);
+__device__ __forceinline__ void rowor_rows(const RowOrDesc& d, const uint64_t* __restrict__ bs,
+                                           uint16_t* list, int64_t b, int64_t k0, int kc_len,
+                                           int64_t n0, int rs, int r64) {
+  constexpr int W = G >= 2 ? 2 : 1, GL = G / W;  // words per lane, lanes per row
+  constexpr int P = 32 / GL;                     // lookup groups per warp
+  const int nwarps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int sent = r64, t2 = r64 + 1, t4 = t2 + r64 / 4, t6 = t4 + r64 / 16;
-  uint16_t* lists = reinterpret_cast<uint16_t*>(bs + rowor_table_rows(staged) * G);
-  uint64_t* bar = reinterpret_cast<uint64_t*>(lists + (size_t)nwarps * kListCap);
-
-  int64_t cta = (int64_t)blockIdx.x - cta0s[p];
-  const int64_t rs = cta % d.row_splits;
-  cta /= d.row_splits;
-  const int64_t kc = cta % d.k_chunks;
-  cta /= d.k_chunks;
-  const int64_t nt = cta % d.n_tiles;
-  const int64_t b = cta / d.n_tiles;
-  const int64_t k0 = kc * d.Kc;
-  const int kc_len = (int)min((int64_t)d.Kc, d.K - k0);
-  const int64_t n0 = nt * G;
-
-  // ---- stage the B tile
-  if (d.use_tma) {
-    const int nbox = (kc_len + 255) / 256;
-    if (tid == 0) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(1) : "memory");
-      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      // the tensor map was written to global memory by a copy before the launch
-      asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(tmap) : "memory");
-    }
-    // everything the earlier kernels of the stream wrote (A, B) is complete
-    // and visible past this point, and C may be overwritten
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    __syncthreads();
-    if (tid == 0) {
-      const uint32_t bytes = (uint32_t)nbox * 256u * (uint32_t)G * 8u;
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-                   "r"(bytes)
-                   : "memory");
-      for (int j = 0; j < nbox; ++j) {
-        const int x = (int)n0;
-        const int y = (int)(b * d.K + k0 + 256 * j);
-        asm volatile(
-            "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
-            " [%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(bs + (size_t)j * 256 * G)),
-            "l"(reinterpret_cast<uint64_t>(tmap)), "r"(x), "r"(y), "r"(smem_u32(bar))
-            : "memory");
-      }
-    }
-    const bool ok = mbar_wait(bar, 0, 1000000000ll);
-    if (__syncthreads_or(!ok)) {
-      if (tid == 0) atomicExch(d.err, 1);
-      return;
-    }
-  } else {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    // rows past the K range are zero (only block tables that no lookup reads
-    // include them)
-    for (int idx = tid; idx < r64 * G; idx += blockDim.x) {
-      const int r = idx / G, c = idx % G;
-      const int64_t n = n0 + c;
-      bs[idx] = (r < kc_len && n < d.Nw) ? __ldg(d.B + (b * d.K + k0 + r) * d.Nw + n) : 0ull;
-    }
-  }
-  if (tid < G) bs[(size_t)sent * G + tid] = 0ull;  // sentinel row
-  __syncthreads();
-  // block tables: each row the OR of four rows of the level below
-  {
-    const int lv_src[3] = {0, t2, t4}, lv_dst[3] = {t2, t4, t6}, lv_n[3] = {r64 / 4, r64 / 16, r64 / 64};
-#pragma unroll
-    for (int l = 0; l < 3; ++l) {
-      const uint64_t* src = bs + (size_t)lv_src[l] * G;
-      uint64_t* dst = bs + (size_t)lv_dst[l] * G;
-      for (int idx = tid; idx < lv_n[l] * G; idx += blockDim.x) {
-        const int q = idx / G, c = idx - (idx / G) * G;
-        const uint64_t* s0 = src + (size_t)(4 * q) * G + c;
-        dst[idx] = s0[0] | s0[G] | s0[2 * G] | s0[3 * G];
-      }
-      __syncthreads();
-    }
-  }
-
-  // ---- output rows, one warp each
-  const int warp = tid >> 5, lane = tid & 31;
-  const int grp = lane / G, lig = lane % G;
-  constexpr int P = 32 / G;
-  uint16_t* list = lists + (size_t)warp * kListCap;
-  // rows are dealt out cyclically over every warp of the CTAs sharing this
-  // tile, so that runs of dense rows (curves are locally thick) are spread out.
-  // A warp's work is a sequence of units (row, batch of 32 A words); the A
-  // words of the next four units are always in flight while one is processed.
-  const int gw = (int)rs * nwarps + warp;
-  const int gstride = (int)d.row_splits * nwarps;
+  const int grp = lane / GL, lig = lane % GL;
+  const uint64_t* mine = bs + W * lig;
+  // lanes per row and rows per batch
   const int kw0 = (int)(k0 / 64);
   const int kw1 = (int)min(d.a_row_words, (k0 + kc_len + 63) / 64);
-  const int nbat = (kw1 - kw0 + 31) / 32;
+  const int kw = kw1 - kw0;
+  // (no more rows per batch than leave every warp a batch: with few rows the
+  // batches would run on a few of the warps, one after another)
+  const int L = kw;  // at most 32: a K range is at most kRowOrMaxKc
+  const int all_warps = (int)d.row_splits * nwarps;
+  const int R = min(32 / L, ((int)d.M + all_warps - 1) / all_warps);
+  // groups per row (gpr, a power of two) of a lookup round, rows per round and
+  // rounds
+  int gpr = 1;
+  while (2 * gpr * R <= P) gpr *= 2;
+  const int rpr = P / gpr, rounds = (R + rpr - 1) / rpr;
+  const int sub = grp % gpr, rin = grp / gpr;
+  // batches of rows are dealt out cyclically over every warp of the CTAs
+  // sharing this tile, so that runs of dense rows (curves are locally thick)
+  // are spread out.  The A words of the next three batches are always in
+  // flight while one is processed.
+  const int gw = rs * nwarps + warp;
+  const int rstep = all_warps * R;
   const int M = (int)d.M;
-  const int nrows_w = (gw < M) ? (M - gw + gstride - 1) / gstride : 0;
-  const int nunits = nrows_w * nbat;
-  const uint64_t* __restrict__ abase = d.A + (b * d.M) * d.a_row_words;
   const int64_t arw = d.a_row_words;
-  int* wcount = reinterpret_cast<int*>(bar + 1) + warp;
-  if (lane == 0) *wcount = 0;
-  int wbase = 0;
-  __syncwarp();
-  auto load_unit = [&](int u) -> uint64_t {
-    if (u >= nunits) return 0ull;
-    const int i = (nbat == 1) ? u : u / nbat;
-    const int q = u - i * nbat;
-    const int kwl = kw0 + q * 32 + lane;
-    return (kwl < kw1) ? __ldg(abase + (int64_t)(gw + i * gstride) * arw + kwl) : 0ull;
+  const int my_row = lane / L, my_word = lane - my_row * L;
+  const bool busy = my_row < R;  // lanes past the last whole row are idle
+  const int64_t Nw = d.Nw;
+  uint64_t* const cbase = d.C + b * d.M * Nw + n0 + W * lig;
+  const int cols = (int)min((int64_t)W, max((int64_t)0, Nw - n0 - W * lig));  // of this lane's words
+  const bool vec = W == 2 && Nw % 2 == 0 && reinterpret_cast<uintptr_t>(d.C) % 16 == 0;
+  const bool atomic = d.atomic != 0;
+  auto store = [&](int row, const Words<W>& w) {
+    uint64_t* c = cbase + (int64_t)row * Nw;
+    if (atomic) {
+#pragma unroll
+      for (int k = 0; k < W; ++k)
+        if (k < cols && w.v[k]) atomicOr((unsigned long long*)(c + k), (unsigned long long)w.v[k]);
+    } else if (W == 2 && vec) {
+      if (cols > 0) *reinterpret_cast<ulonglong2*>(c) = make_ulonglong2(w.v[0], w.v[W - 1]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < W; ++k)
+        if (k < cols) c[k] = w.v[k];
+    }
   };
-  uint64_t pre0 = load_unit(0), pre1 = load_unit(1), pre2 = load_unit(2), pre3 = load_unit(3);
-  uint64_t acc = 0;
-  for (int u = 0; u < nunits; ++u) {
+  // OR over the groups that share a row (lane distances GL .. to)
+  auto combine = [&](Words<W>& w, int to) {
+    for (int o = GL; o < to; o <<= 1)
+#pragma unroll
+      for (int k = 0; k < W; ++k) w.v[k] |= __shfl_xor_sync(0xffffffffu, w.v[k], o);
+  };
+  const uint64_t* __restrict__ abase = d.A + (b * d.M) * arw + kw0 + my_word;
+  int lrow = gw * R + my_row;  // row of the next batch to fetch
+  auto fetch = [&]() -> uint64_t {
+    const uint64_t v = (busy && lrow < M) ? __ldg(abase + (int64_t)lrow * arw) : 0ull;
+    lrow += rstep;
+    return v;
+  };
+  uint64_t pre0 = fetch(), pre1 = fetch(), pre2 = fetch();
+  Words<W> zero;
+#pragma unroll
+  for (int k = 0; k < W; ++k) zero.v[k] = 0;
+  // tile row of this lane's word's bit 0 (a multiple of 64), and the word's
+  // bits inside the K range
+  const int base = (kw0 + my_word) * 64 - (int)k0;
+  const uint64_t in_range = base + 64 <= kc_len ? ~0ull : base >= kc_len ? 0ull : (1ull << (kc_len - base)) - 1ull;
+  for (int row0 = gw * R; row0 < M; row0 += rstep) {
     uint64_t a = pre0;
     pre0 = pre1;
     pre1 = pre2;
-    pre2 = pre3;
-    pre3 = load_unit(u + 4);
-    const int i = (nbat == 1) ? u : u / nbat;
-    const int q = u - i * nbat;
-    if (q == 0) acc = 0;
+    pre2 = fetch();
+    a &= in_range;
     if (__any_sync(0xffffffffu, a != 0ull)) {
-      // tile row of this word's bit 0 (a multiple of 64); bits past the K
-      // range are dropped
-      const int base = (kw0 + q * 32 + lane) * 64 - (int)k0;
-      if (base + 64 > kc_len) a &= (base >= kc_len) ? 0ull : ((1ull << (kc_len - base)) - 1ull);
       // maximal all-ones aligned blocks of the word: bit 4i of f4 when bits
       // 4i..4i+3 are set, bit 16i of f16 when bits 16i..16i+15 are set, f1 the
       // set bits in neither; a full word is one 64-block
       const bool full = (a == ~0ull);
-      uint64_t f16 = 0, f4 = 0, f1 = a;
+      uint64_t f16 = 0, f4 = 0, f1 = 0;
       if (!full) {
         uint64_t t = a & (a >> 1);
         t &= t >> 2;
@@ -622,83 +573,263 @@ rowor_tile_kernel(const RowOrDesc* __restrict__ descs, const CUtensorMap* __rest
         f4 &= ~m16;
         f1 = a & ~(m16 | f4 * 0xFull);
       }
-      const int c = full ? 1 : __popcll(f16) + __popcll(f4) + __popcll(f1);
-      const int T = (int)__reduce_add_sync(0xffffffffu, (unsigned)c);
+      const int c = full ? 1 : __popcll(f16 | f4 | f1);  // (three disjoint sets of positions)
+      int incl = c;
+#pragma unroll
+      for (int sh = 1; sh < 32; sh <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, sh);
+        if (lane >= sh) incl += v;
+      }
+      const int excl = incl - c;
+      const int T = __shfl_sync(0xffffffffu, incl, 31);
       if (d.stat && lane == 0) atomicAdd(d.stat, (unsigned long long)T * G);
+      // the table rows of this lane's blocks, in a fixed order
+      auto entries = [&](auto&& put) {
+        if (full) put(t6 + (base >> 6));
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          for (uint32_t m = (uint32_t)(f16 >> (32 * h)); m;) {
+            const int p = 31 - __clz(m);
+            m ^= 1u << p;
+            put(t4 + ((base + 32 * h + p) >> 4));
+          }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          for (uint32_t m = (uint32_t)(f4 >> (32 * h)); m;) {
+            const int p = 31 - __clz(m);
+            m ^= 1u << p;
+            put(t2 + ((base + 32 * h + p) >> 2));
+          }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          for (uint32_t m = (uint32_t)(f1 >> (32 * h)); m;) {
+            const int p = 31 - __clz(m);
+            m ^= 1u << p;
+            put(base + 32 * h + p);
+          }
+        }
+      };
       if (T <= kListWin) {
-        // one window: each lane claims its slots from the warp's counter,
-        // which only grows (this unit's slots start at the units' running
-        // total, known to every lane), so it never needs resetting
-        int e = c ? atomicAdd(wcount, c) - wbase : 0;
-        if (full) {
-          list[e] = (uint16_t)(t6 + base / 64);
-        } else {
-          for (uint64_t m = f16; m; m &= m - 1) list[e++] = (uint16_t)(t4 + (base + __ffsll((long long)m) - 1) / 16);
-          for (uint64_t m = f4; m; m &= m - 1) list[e++] = (uint16_t)(t2 + (base + __ffsll((long long)m) - 1) / 4);
-          for (uint64_t m = f1; m; m &= m - 1) list[e++] = (uint16_t)(base + __ffsll((long long)m) - 1);
-        }
-        wbase += T;
-        // pad to a whole number of rounds with the sentinel row (4P entries,
-        // which is more than one per lane when the groups are narrow)
-        for (int t = lane; t < 4 * P; t += 32) list[T + t] = (uint16_t)sent;
+        uint16_t* to = list + excl;
+        entries([&](int row) { *to++ = (uint16_t)row; });
         __syncwarp();
-        for (int e2 = grp; e2 < T; e2 += 4 * P) {
-          const int i0 = list[e2], i1 = list[e2 + P], i2 = list[e2 + 2 * P], i3 = list[e2 + 3 * P];
-          acc |= bs[i0 * G + lig] | bs[i1 * G + lig] | bs[i2 * G + lig] | bs[i3 * G + lig];
+        for (int rd = 0; rd < rounds; ++rd) {
+          const int r = rd * rpr + rin;  // r >= R (the last round's spare groups): no row
+          const int o0 = __shfl_sync(0xffffffffu, excl, (r * L) & 31);
+          int o1 = __shfl_sync(0xffffffffu, incl, (r * L + L - 1) & 31);
+          if (r >= R) o1 = 0;
+          Words<W> w = zero;
+          for (int e = o0 + sub; e < o1; e += 3 * gpr) {
+            const int i0 = list[e];
+            const int i1 = e + gpr < o1 ? list[e + gpr] : sent;
+            const int i2 = e + 2 * gpr < o1 ? list[e + 2 * gpr] : sent;
+            or_row(w, mine + i0 * G);
+            or_row(w, mine + i1 * G);
+            or_row(w, mine + i2 * G);
+          }
+          __syncwarp();
+          combine(w, GL * gpr);
+          if (sub == 0 && r < R && row0 + r < M) store(row0 + r, w);
         }
-        __syncwarp();
       } else {
-        // several windows: this lane's entries are [o, o + c) of the unit's
-        // T in a fixed order, and each window writes the ones inside it
-        int o = c;
-#pragma unroll
-        for (int sh = 1; sh < 32; sh <<= 1) {
-          const int v = __shfl_up_sync(0xffffffffu, o, sh);
-          if (lane >= sh) o += v;
-        }
-        o -= c;
-        for (int w0 = 0; w0 < T; w0 += kListWin) {
-          const int w1 = min(T, w0 + kListWin);
-          if (o < w1 && o + c > w0) {
-            int e = o;
-            auto put = [&](int row) {
-              if (e >= w0 && e < w1) list[e - w0] = (uint16_t)row;
-              ++e;
-            };
-            if (full) {
-              put(t6 + base / 64);
-            } else {
-              for (uint64_t m = f16; m; m &= m - 1) put(t4 + (base + __ffsll((long long)m) - 1) / 16);
-              for (uint64_t m = f4; m; m &= m - 1) put(t2 + (base + __ffsll((long long)m) - 1) / 4);
-              for (uint64_t m = f1; m; m &= m - 1) put(base + __ffsll((long long)m) - 1);
+        // more blocks than the list holds: row by row, in windows of the list;
+        // this lane's entries are [excl, incl) of the batch's T
+        for (int r = 0; r < R; ++r) {
+          const int ro0 = __shfl_sync(0xffffffffu, excl, r * L);
+          const int ro1 = __shfl_sync(0xffffffffu, incl, r * L + L - 1);
+          Words<W> w = zero;
+          for (int w0 = ro0; w0 < ro1; w0 += kListWin) {
+            const int w1 = min(ro1, w0 + kListWin);
+            if (my_row == r && excl < w1 && incl > w0) {
+              int e = excl;
+              entries([&](int row) {
+                if (e >= w0 && e < w1) list[e - w0] = (uint16_t)row;
+                ++e;
+              });
             }
+            const int n = w1 - w0;
+            // pad to a whole number of rounds with the sentinel row (4P entries,
+            // which is more than one per lane when the groups are narrow)
+            for (int t = lane; t < 4 * P; t += 32) list[n + t] = (uint16_t)sent;
+            __syncwarp();
+            for (int e = grp; e < n; e += 4 * P) {
+              or_row(w, mine + list[e] * G);
+              or_row(w, mine + list[e + P] * G);
+              or_row(w, mine + list[e + 2 * P] * G);
+              or_row(w, mine + list[e + 3 * P] * G);
+            }
+            __syncwarp();
           }
-          const int n = w1 - w0;
-          for (int t = lane; t < 4 * P; t += 32) list[n + t] = (uint16_t)sent;
-          __syncwarp();
-          for (int e2 = grp; e2 < n; e2 += 4 * P) {
-            const int i0 = list[e2], i1 = list[e2 + P], i2 = list[e2 + 2 * P], i3 = list[e2 + 3 * P];
-            acc |= bs[i0 * G + lig] | bs[i1 * G + lig] | bs[i2 * G + lig] | bs[i3 * G + lig];
-          }
-          __syncwarp();
+          combine(w, 32);
+          if (grp == 0 && row0 + r < M) store(row0 + r, w);
+        }
+      }
+    } else if (!atomic) {
+      for (int r = grp; r < R; r += P)
+        if (row0 + r < M) store(row0 + r, zero);  // nothing selected: zero rows
+    }
+  }
+}
+
+// Launch description: problem p owns CTAs [cta0[p], cta0[p+1]); its
+// descriptor and tensor map (used by kStageTile) live in global memory.  One
+// launch serves every tile width (a branch on the problem's width).
+__global__ void __launch_bounds__(kRowOrThreads)
+rowor_kernel(const RowOrDesc* __restrict__ descs, const CUtensorMap* __restrict__ maps,
+             const int64_t* __restrict__ cta0s, int nprob) {
+  extern __shared__ __align__(1024) uint64_t bs[];
+  __shared__ RowOrDesc sd;
+  __shared__ int s_p;
+  // the next launch may be scheduled onto SMs this grid frees; it waits for
+  // this grid's completion before it touches any data
+  asm volatile("griddepcontrol.launch_dependents;");
+  const int tid = threadIdx.x;
+  {
+    // the last problem whose first CTA is at most this one: every thread
+    // compares one of an evenly spaced sample, then the gap is searched the
+    // same way (a binary search is a chain of L2 latencies)
+    int lo = 0, n = nprob;
+    while (n > 1) {
+      const int step = (n + (int)blockDim.x - 1) / (int)blockDim.x;
+      const int64_t at = (int64_t)tid * step;
+      const int below = at < n && cta0s[lo + at] <= (int64_t)blockIdx.x;
+      const int first = (__syncthreads_count(below) - 1) * step;
+      lo += first;
+      n = min(step, n - first);
+    }
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(descs + lo);
+    uint32_t* dst = reinterpret_cast<uint32_t*>(&sd);
+    if (tid < (int)(sizeof(RowOrDesc) / 4)) dst[tid] = src[tid];
+    if (tid == 0) s_p = lo;
+  }
+  __syncthreads();
+  const int p = s_p;
+  const RowOrDesc& d = sd;
+  const CUtensorMap* tmap = maps + p;
+  const int G = d.Nt;
+  const int r64 = (int)rowor_r64(d.Kc);
+  uint16_t* lists = reinterpret_cast<uint16_t*>(bs + rowor_table_rows(d.Kc) * G);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(lists + (size_t)(blockDim.x >> 5) * kListCap);
+
+  int64_t cta = (int64_t)blockIdx.x - cta0s[p];
+  const int rs = (int)(cta % d.row_splits);
+  cta /= d.row_splits;
+  const int64_t kc = cta % d.k_chunks;
+  cta /= d.k_chunks;
+  const int64_t nt = cta % d.n_tiles;
+  const int64_t b = cta / d.n_tiles;
+  const int64_t k0 = kc * d.Kc;
+  const int kc_len = (int)min((int64_t)d.Kc, d.K - k0);
+  const int64_t n0 = nt * G;
+
+  // ---- stage the B tile
+  if (d.stage != kStageWords) {
+    if (tid == 0) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(1) : "memory");
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      // the tensor map was written to global memory by a copy before the launch
+      if (d.stage == kStageTile)
+        asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(tmap) : "memory");
+    }
+    // everything the earlier kernels of the stream wrote (A, B) is complete
+    // and visible past this point, and C may be overwritten
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    __syncthreads();
+    if (tid == 0) {
+      if (d.stage == kStageTile) {
+        const int nbox = (kc_len + 63) / 64;
+        const uint32_t bytes = (uint32_t)nbox * 64u * (uint32_t)G * 8u;
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
+                     "r"(bytes)
+                     : "memory");
+        for (int j = 0; j < nbox; ++j) {
+          const int x = (int)n0;
+          const int y = (int)(b * d.K + k0 + 64 * j);
+          asm volatile(
+              "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
+              " [%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(bs + (size_t)j * 64 * G)),
+              "l"(reinterpret_cast<uint64_t>(tmap)), "r"(x), "r"(y), "r"(smem_u32(bar))
+              : "memory");
+        }
+      } else {
+        // the tile is one run of memory (G words per row in both)
+        const uint32_t bytes = (uint32_t)kc_len * (uint32_t)G * 8u;
+        const uint64_t* src = d.B + (b * d.K + k0) * G;
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
+                     "r"(bytes)
+                     : "memory");
+        for (uint32_t at = 0; at < bytes; at += 16384u) {
+          const uint32_t n = min(bytes - at, 16384u);
+          asm volatile(
+              "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes"
+              " [%0], [%1], %2, [%3];" ::"r"(smem_u32(bs) + at),
+              "l"(reinterpret_cast<const char*>(src) + at), "r"(n), "r"(smem_u32(bar))
+              : "memory");
         }
       }
     }
-    if (q == nbat - 1) {
-      uint64_t r = acc;
+    const bool ok = mbar_wait(bar, 0, 1000000000ll);
+    if (__syncthreads_or(!ok)) {
+      if (tid == 0) atomicExch(d.err, 1);
+      return;
+    }
+  } else {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // 8-byte asynchronous copies, all in flight at once; words past the row
+    // and rows past the K range are filled with zeros
+    const int lg = 31 - __clz(G);
+    for (int idx = tid; idx < r64 << lg; idx += blockDim.x) {
+      const int r = idx >> lg, c = idx & (G - 1);
+      const int64_t n = n0 + c;
+      const bool in = r < kc_len && n < d.Nw;
+      const uint64_t* src = in ? d.B + (b * d.K + k0 + r) * d.Nw + n : d.B;
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(smem_u32(bs + idx)),
+                   "l"(src), "r"(in ? 8 : 0)
+                   : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+  }
+  if (tid < G) bs[(size_t)r64 * G + tid] = 0ull;  // sentinel row
+  __syncthreads();
+  // block tables: a thread per (16-row block, column) ORs its four 4-row
+  // blocks and the block itself, then the 64-row blocks follow
+  {
+    const int lg = 31 - __clz(G);
+    uint64_t* T2 = bs + (size_t)(r64 + 1) * G;
+    uint64_t* T4 = T2 + (size_t)(r64 / 4) * G;
+    uint64_t* T6 = T4 + (size_t)(r64 / 16) * G;
+    for (int idx = tid; idx < (r64 / 16) << lg; idx += blockDim.x) {
+      const int q = idx >> lg, c = idx & (G - 1);
+      const uint64_t* s0 = bs + (size_t)(16 * q) * G + c;
+      uint64_t all = 0;
 #pragma unroll
-      for (int o = G; o < 32; o <<= 1) r |= __shfl_xor_sync(0xffffffffu, r, o);
-      const int m = gw + i * gstride;
-      const int64_t n = n0 + lane;
-      if (lane < G && n < d.Nw) {
-        uint64_t* c = d.C + (b * d.M + m) * d.Nw + n;
-        if (d.atomic) {
-          if (r) atomicOr((unsigned long long*)c, (unsigned long long)r);
-        } else {
-          *c = r;
-        }
+      for (int j = 0; j < 4; ++j) {
+        const uint64_t v = s0[(4 * j) * G] | s0[(4 * j + 1) * G] | s0[(4 * j + 2) * G] | s0[(4 * j + 3) * G];
+        T2[(size_t)(4 * q + j) * G + c] = v;
+        all |= v;
       }
+      T4[idx] = all;
     }
+    __syncthreads();
+    for (int idx = tid; idx < (r64 / 64) << lg; idx += blockDim.x) {
+      const int q = idx >> lg, c = idx & (G - 1);
+      const uint64_t* s0 = T4 + (size_t)(4 * q) * G + c;
+      T6[idx] = s0[0] | s0[G] | s0[2 * G] | s0[3 * G];
+    }
+    __syncthreads();
+  }
+  uint16_t* list = lists + (size_t)(tid >> 5) * kListCap;
+  switch (G) {
+    case 1: rowor_rows<1>(d, bs, list, b, k0, kc_len, n0, rs, r64); break;
+    case 2: rowor_rows<2>(d, bs, list, b, k0, kc_len, n0, rs, r64); break;
+    case 4: rowor_rows<4>(d, bs, list, b, k0, kc_len, n0, rs, r64); break;
+    case 8: rowor_rows<8>(d, bs, list, b, k0, kc_len, n0, rs, r64); break;
+    case 16: rowor_rows<16>(d, bs, list, b, k0, kc_len, n0, rs, r64); break;
+    default: rowor_rows<32>(d, bs, list, b, k0, kc_len, n0, rs, r64); break;
   }
 }
 
@@ -723,11 +854,12 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
-// Shared memory of one CTA: the tables plus the warps' lists, their counters
-// and the mbarrier, within the 227 KB a CTA may opt into.
+// Shared memory of one CTA: the tables plus the warps' lists and the mbarrier,
+// within the 227 KB a CTA may opt into.
 constexpr size_t kSmemLimit = 227 * 1024 - 2048;  // the kernel's static shared memory stays out
-constexpr size_t kListBytes = (size_t)(kRowOrThreads / 32) * kListCap * 2 + 16 +
-                              (size_t)(kRowOrThreads / 32) * 4;
+constexpr size_t kSmemHalf = 113 * 1024 - 1024;     // two CTAs to an SM
+constexpr size_t kSmemQuarter = 56 * 1024 - 1024;   // four
+constexpr size_t list_bytes(int threads) { return (size_t)(threads / 32) * kListCap * 2 + 16; }
 
 size_t table_bytes(int64_t staged, int Nt) { return (size_t)rowor_table_rows(staged) * Nt * 8; }
 
@@ -749,10 +881,14 @@ cudaError_t smem_limit(const void* fn, size_t bytes) {
   return e;
 }
 
-void rowor_plan(RowOrDesc& d, int64_t target_ctas) {
-  const bool tma_ok = (d.Nw % 2 == 0) && (reinterpret_cast<uintptr_t>(d.B) % 16 == 0) &&
-                      (d.nbatch * d.K < (1ll << 31)) && encode_fn() != nullptr;
-  auto staged_of = [&](int64_t kc, bool tma) { return tma ? (kc + 255) / 256 * 256 : kc; };
+int64_t rowor_max_kc(int Nt, int threads) {
+  const size_t limit = (threads < kRowOrThreads ? kSmemHalf : kSmemLimit) - list_bytes(threads);
+  // table_bytes(kc) = ((1 + 1/4 + 1/16 + 1/64) kc + 1) rows of Nt words
+  const int64_t kc = (int64_t)(((double)limit / (8.0 * Nt) - 1.0) / 1.328125) / 64 * 64;
+  return std::min<int64_t>(kRowOrMaxKc, std::max<int64_t>(64, kc));
+}
+
+void rowor_plan(RowOrDesc& d, double share) {
   // the widest power-of-two tile (<= 32 words, <= the row): a row of A is
   // split into blocks and listed once per tile, so wide tiles cut that work
   // (32-word tiles took the chain's 2048^3 joins from 19.3 to 16.0 us per
@@ -762,41 +898,69 @@ void rowor_plan(RowOrDesc& d, int64_t target_ctas) {
   int Nt = 1;
   while (Nt < 32 && Nt < d.Nw) Nt <<= 1;
   d.Nt = Nt;
-  d.use_tma = (tma_ok && Nt % 2 == 0) ? 1 : 0;
-  const int64_t step = d.use_tma ? 256 : 64;
-  if (table_bytes(staged_of(d.K, d.use_tma), Nt) + kListBytes <= kSmemLimit) {
-    d.Kc = (int32_t)d.K;
-  } else {
-    int64_t kc = step;
-    while (table_bytes(kc + step, Nt) + kListBytes <= kSmemLimit) kc += step;
-    d.Kc = (int32_t)kc;
-  }
+  // A problem with SMs to itself takes a CTA of 1024 threads per SM (64
+  // registers a thread: an SM holds 1024), which shorten the set-up
+  // (descriptor, copies, tables).  One with more CTAs than its share of SMs
+  // takes smaller ones, whose set-up overlaps the rows of the others on the
+  // SM: four of 256 threads for the many small tiles of a shared batch axis
+  // (38 networks: 1.49 against 1.79 ms with two of 512), two of 512 otherwise
+  // (4096 chains: 0.99 against 1.31 ms with four of 256, whose last ones run
+  // long).
+  const int64_t tiles = d.nbatch * ((d.Nw + Nt - 1) / Nt);
+  const int64_t whole_max = rowor_max_kc(Nt, kRowOrThreads);
+  d.threads = (double)(tiles * ((d.K + whole_max - 1) / whole_max)) <= share              ? kRowOrThreads
+              : d.nbatch >= 8 && table_bytes(d.K, Nt) + list_bytes(256) <= kSmemQuarter ? 256
+                                                                                      : 512;
+  // K in chunks of equal length; many chunks take a power of two of rows, so
+  // that whole batches of rows fill the lanes.  A problem with SMs left over
+  // takes more chunks (down to 512 rows of K), each staging its own part of B
+  // only, before its rows are split over CTAs that all stage the same one.
+  int64_t kmax = rowor_max_kc(Nt, d.threads);
+  if (d.K >= 4 * kmax)
+    while (kmax & (kmax - 1)) kmax &= kmax - 1;
+  int64_t chunks = (d.K + kmax - 1) / kmax;
+  if (d.threads == kRowOrThreads)
+    chunks = std::max(chunks, std::min<int64_t>((int64_t)(share / (double)tiles), (d.K + 511) / 512));
+  d.Kc = chunks <= 1 ? (int32_t)d.K : (int32_t)(((d.K + chunks - 1) / chunks + 63) / 64 * 64);
+  // How the tile is staged.  A tile as wide as the rows is one run of memory
+  // (bulk copies; narrow 2-D boxes move one 8- or 16-byte row per request);
+  // other tiles are 2-D boxes, or 8-byte copies where the row pitch is not a
+  // multiple of 16 bytes.
+  const bool aligned = reinterpret_cast<uintptr_t>(d.B) % 16 == 0;
+  if (d.Nw == Nt && aligned && (d.Nw % 2 == 0 || d.K % 2 == 0))
+    d.stage = kStageRun;  // (every chunk starts and ends on 16 bytes: Kc is even or all of K)
+  else if (Nt % 2 == 0 && d.Nw % 2 == 0 && aligned && d.nbatch * d.K < (1ll << 31) &&
+           encode_fn() != nullptr)
+    d.stage = kStageTile;
+  else
+    d.stage = kStageWords;
   d.n_tiles = (d.Nw + Nt - 1) / Nt;
   d.k_chunks = (d.K + d.Kc - 1) / d.Kc;
   d.atomic = d.k_chunks > 1 ? 1 : 0;
   const int64_t base = d.nbatch * d.n_tiles * d.k_chunks;
-  const int64_t target = std::max<int64_t>(1, target_ctas);
-  // round down: a launch of more CTAs than SMs (one CTA fits an SM) would run
-  // a short second wave and nearly double its time
+  // small CTAs: about twice as many as the problem's share of the slots, so
+  // that the last ones to finish are short; at least 64 rows each
+  const bool whole = d.threads == kRowOrThreads;
+  const int64_t target = whole ? (int64_t)share : (int64_t)(2.0 * share * (kRowOrThreads / d.threads) + 0.5);
+  // round down: a launch of more CTAs than fit at once would run a short
+  // second wave and nearly double its time
   int64_t splits = target / base;
-  splits = std::max<int64_t>(1, std::min<int64_t>(splits, (d.M + 15) / 16));
+  const int64_t min_rows = whole ? 16 : 64;
+  splits = std::max<int64_t>(1, std::min<int64_t>(splits, (d.M + min_rows - 1) / min_rows));
   d.rows_per_split = (d.M + splits - 1) / splits;
   d.row_splits = (d.M + d.rows_per_split - 1) / d.rows_per_split;
 }
 
-size_t rowor_smem_bytes(const RowOrDesc& d) {
-  const int64_t staged = d.use_tma ? ((int64_t)d.Kc + 255) / 256 * 256 : d.Kc;
-  return table_bytes(staged, d.Nt) + kListBytes;
-}
+size_t rowor_smem_bytes(const RowOrDesc& d) { return table_bytes(d.Kc, d.Nt) + list_bytes(d.threads); }
 
 int64_t rowor_ctas(const RowOrDesc& d) { return d.nbatch * d.n_tiles * d.k_chunks * d.row_splits; }
 
 cudaError_t rowor_encode_map(const RowOrDesc& d, CUtensorMap* map) {
   memset(map, 0, sizeof *map);
-  if (!d.use_tma) return cudaSuccess;
+  if (d.stage != kStageTile) return cudaSuccess;
   const cuuint64_t dims[2] = {(cuuint64_t)d.Nw, (cuuint64_t)(d.nbatch * d.K)};
   const cuuint64_t strides[1] = {(cuuint64_t)d.Nw * 8};
-  const cuuint32_t box[2] = {(cuuint32_t)d.Nt, 256u};
+  const cuuint32_t box[2] = {(cuuint32_t)d.Nt, 64u};
   const cuuint32_t estr[2] = {1u, 1u};
   CUresult r = encode_fn()(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, const_cast<uint64_t*>(d.B), dims,
                            strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -822,7 +986,7 @@ cudaError_t launch_wait_selftest(int* err, long long limit_ns, cudaStream_t s) {
 }
 
 cudaError_t launch_rowor(const RowOrDesc* d_descs, const CUtensorMap* d_maps,
-                         const int64_t* d_cta0, int nprob, int64_t grid, size_t smem, int Nt,
+                         const int64_t* d_cta0, int nprob, int64_t grid, size_t smem, int threads,
                          cudaStream_t s) {
   if (nprob <= 0 || grid <= 0) return cudaSuccess;
   if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
@@ -833,25 +997,13 @@ cudaError_t launch_rowor(const RowOrDesc* d_descs, const CUtensorMap* d_maps,
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(kRowOrThreads);
+  cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-#define PA_ROWOR(GG)                                                                         \
-  do {                                                                                       \
-    smem_limit(reinterpret_cast<const void*>(rowor_tile_kernel<GG>), smem);                  \
-    cudaLaunchKernelEx(&cfg, rowor_tile_kernel<GG>, d_descs, d_maps, d_cta0, nprob);         \
-  } while (0)
-  switch (Nt) {
-    case 1: PA_ROWOR(1); break;
-    case 2: PA_ROWOR(2); break;
-    case 4: PA_ROWOR(4); break;
-    case 8: PA_ROWOR(8); break;
-    case 16: PA_ROWOR(16); break;
-    default: PA_ROWOR(32); break;
-  }
-#undef PA_ROWOR
+  smem_limit(reinterpret_cast<const void*>(rowor_kernel), smem);
+  cudaLaunchKernelEx(&cfg, rowor_kernel, d_descs, d_maps, d_cta0, nprob);
   return cudaGetLastError();
 }
 

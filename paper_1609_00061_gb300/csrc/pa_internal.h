@@ -211,24 +211,28 @@ struct RowOrDesc {
   int64_t nbatch, M, K, Nw;   // Nw = words per B / C row
   int64_t a_row_words;        // = ceil(K / 64)
   int32_t Nt;                 // words per tile (power of two <= 32)
-  int32_t Kc;                 // B rows per tile (multiple of 256 when use_tma)
+  int32_t Kc;                 // B rows per tile (a multiple of 64 unless it is all of K)
+  int32_t threads;            // per CTA: 256, 512 or 1024
   int64_t n_tiles, k_chunks, row_splits, rows_per_split;
   int32_t atomic;             // 1: C pre-zeroed, results OR-ed in atomically
-  int32_t use_tma;            // 1: stage the tile with cp.async.bulk.tensor
+  int32_t stage;              // kStage*: how the tile reaches shared memory
   int* err;                   // device error word: set when a bounded wait runs out
   unsigned long long* stat;   // when not null: += shared-memory words OR-ed (timing mode)
 };
-// Choose the tile shape and grid for a contraction of this shape; the grid
-// aims at about target_ctas CTAs (several contractions can share one launch).
-void rowor_plan(RowOrDesc& d, int64_t target_ctas);
+enum { kStageWords = 0, kStageTile = 1, kStageRun = 2 };
+// Longest K range whose tables fit next to the lists of a CTA of `threads`.
+int64_t rowor_max_kc(int Nt, int threads);
+// Choose the tile shape and grid for a contraction of this shape, which has
+// `share` SMs (a fraction when many contractions share one launch).
+void rowor_plan(RowOrDesc& d, double share);
 size_t rowor_smem_bytes(const RowOrDesc& d);
 int64_t rowor_ctas(const RowOrDesc& d);
-// TMA descriptor of d.B (all zero when d.use_tma is 0)
+// TMA descriptor of d.B (all zero unless d.stage is kStageTile)
 cudaError_t rowor_encode_map(const RowOrDesc& d, CUtensorMap* map);
-// Independent contractions with the same tile width Nt in one launch:
-// descriptors, tensor maps and CTA offsets (nprob + 1 entries) on the device.
+// Independent contractions with the same CTA size in one launch: descriptors,
+// tensor maps and CTA offsets (nprob + 1 entries) on the device.
 cudaError_t launch_rowor(const RowOrDesc* d_descs, const CUtensorMap* d_maps,
-                         const int64_t* d_cta0, int nprob, int64_t grid, size_t smem, int Nt,
+                         const int64_t* d_cta0, int nprob, int64_t grid, size_t smem, int threads,
                          cudaStream_t s);
 // cuTensorMapEncodeTiled from the driver (null when unavailable)
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
