@@ -262,9 +262,7 @@ pa_status pa_profile_read(pa_ctx* ctx, int32_t max_kernels, char* names, int64_t
 /* How a matrix-form cluster (Sec. 3.5) is contracted.  Both give the same
  * bits.  PA_PATH_ROWOR: bit-packed row-OR on the CUDA cores (work follows the
  * set bits of A).  PA_PATH_MMA: 0/1 E4M3 matrix product on the tensor cores
- * (tcgen05, FP32 accumulation, thresholded at > 0; work follows M x N x K;
- * both operands are first expanded once into E4M3 byte arrays in the
- * workspace, (M + N) x K bytes per batch entry).
+ * (tcgen05, FP32 accumulation, thresholded at > 0; work follows M x N x K).
  * PA_PATH_AUTO (default): per cluster, the faster by the context's rates and
  * the operands' estimated densities. */
 typedef enum { PA_PATH_AUTO = 0, PA_PATH_ROWOR = 1, PA_PATH_MMA = 2 } pa_path;
@@ -275,8 +273,8 @@ pa_status pa_set_contract_path(pa_ctx* ctx, int32_t path);
  * contraction of random operands through each path, five runs timed with CUDA
  * events on `stream` after one warm-up run) and keeps them for later calls.
  * The row-OR rate depends on the density of A and is measured at 2 % and 16 %
- * (log-linear in between); the tensor-core rate includes the expansion of both
- * operands.  Blocks the host; allocates and frees about 10 MB of device memory. */
+ * (log-linear in between).  Blocks the host; allocates and frees about 2 MB of
+ * device memory. */
 typedef struct {
   double rowor_words_per_us;        /* 64-bit words OR-ed by the row-OR kernel, A 2 % dense */
   double rowor_words_per_us_dense;  /* the same, A 16 % dense */

@@ -59,9 +59,9 @@ struct pa_ctx {
   // contraction path (pa_set_contract_path) and the rates its automatic
   // choice compares (defaults measured on a GB300; pa_autotune re-measures)
   int path = PA_PATH_AUTO;
-  double rate_or = 2.0e5;      // row-OR: B words OR-ed per microsecond, A 2 % dense
-  double rate_or_dense = 9.0e5;  // the same, A 16 % dense
-  double rate_mma = 4.4e8;     // tensor path (with operand expansion): multiply-adds per microsecond
+  double rate_or = 2.9e5;      // row-OR: B words OR-ed per microsecond, A 2 % dense
+  double rate_or_dense = 1.39e6;  // the same, A 16 % dense
+  double rate_mma = 5.5e8;     // tensor path: multiply-adds per microsecond
   std::unordered_map<uint64_t, double> dens_cache;  // relation key -> estimated plot density
   std::unordered_map<uint64_t, double> obs_dens;    // subtree key -> density measured by pa_join_log
   std::unordered_map<uint64_t, double> obs_time;    // subtree key -> join microseconds measured by pa_join_log
@@ -93,7 +93,7 @@ pa_status set_err(pa_ctx* ctx, pa_status st, const std::string& msg) {
 bool has(const std::vector<int>& v, int x) { return std::find(v.begin(), v.end(), x) != v.end(); }
 
 // ------------------------------------------------------------ program
-enum OpKind { OP_PLOT, OP_MEMSET, OP_RESHAPE, OP_ROWOR, OP_UNPACK,
+enum OpKind { OP_PLOT, OP_MEMSET, OP_RESHAPE, OP_ROWOR,
               OP_MMA, OP_PLOT_EXPR, OP_PLOT_CORNER, OP_PERMUTE, OP_EWISE };
 
 struct Op {
@@ -123,10 +123,17 @@ const char* op_name(const Op& op) {
       return op.i0 == kRsTranspose ? "reshape_transpose_kernel"
              : (op.i0 == kRsWords32 || op.i0 == kRsWords64) ? "reshape_words_kernel"
                                                             : "reshape_kernel";
-    case OP_UNPACK: return "unpack_kernels";
-    case OP_MMA: return "mma_bool_kernel";
+    case OP_MMA: return "mma_bits_kernel";
     default: return "rowor_kernel";
   }
+}
+
+// Kernels and memsets of a program (a tensor-core op with occupancy bitmaps
+// is two kernels).
+int32_t count_launches(const std::vector<Op>& ops) {
+  int32_t n = 0;
+  for (const Op& op : ops) n += op.kind == OP_MMA && op.m > 0 ? 2 : 1;
+  return n;
 }
 
 // A planned call kept for reuse: its key (arguments and planning state), its
@@ -443,34 +450,20 @@ BitArr make_arr(const std::vector<int>& vars, const std::vector<int64_t>& vres, 
 void flush_mma(Builder& bd) {
   if (bd.pend_mma.empty()) return;
   const size_t n = bd.pend_mma.size();
-  std::vector<CUtensorMap> maps(2 * n);
-  std::vector<int64_t> cta0(n + 1, 0);
+  std::vector<int64_t> cta0(n + 1, 0), occ0(n + 1, 0);
   for (size_t p = 0; p < n; ++p) {
-    if (bd.dry) memset(&maps[2 * p], 0, 2 * sizeof(CUtensorMap));
-    else if (mma_encode_maps(bd.pend_mma[p], &maps[2 * p]) != cudaSuccess)
-      bd.fail(PA_ERR_CUDA, "cuTensorMapEncodeTiled failed (tensor-core path)");
     cta0[p + 1] = cta0[p] + mma_ctas(bd.pend_mma[p]);
+    occ0[p + 1] = occ0[p] + (bd.pend_mma[p].occ ? mma_occ_blocks(bd.pend_mma[p]) : 0);
   }
-  // one launch per operand kind expands every problem's operands, then one
-  // launch contracts them all
-  Op up;
-  up.kind = OP_UNPACK;
-  up.off0 = bd.put(bd.pend_mma.data(), n, 64);
-  up.n = (int)n;
-  for (const MmaDesc& d : bd.pend_mma) {
-    up.m = std::max<int64_t>(up.m, unpack_blocks_a(d));
-    up.nw = std::max<int64_t>(up.nw, unpack_blocks_b(d));
-  }
-  if (n > 65535) bd.fail(PA_ERR_TOO_LARGE, "more than 65535 tensor-core problems in one level");
-  bd.ops.push_back(up);
   Op op;
   op.kind = OP_MMA;
-  op.off0 = up.off0;
-  op.off1 = bd.put(maps.data(), maps.size(), 128);
+  op.off0 = bd.put(bd.pend_mma.data(), n, 64);
+  op.off1 = bd.put(occ0.data(), occ0.size(), 16);
   op.off2 = bd.put(cta0.data(), cta0.size(), 16);
   op.n = (int)n;
   op.count = cta0.back();
-  if (op.count > 0x7fffffffLL) bd.fail(PA_ERR_TOO_LARGE, "contraction grid too large");
+  op.m = occ0.back();
+  if (op.count > 0x7fffffffLL || op.m > 0x7fffffffLL) bd.fail(PA_ERR_TOO_LARGE, "contraction grid too large");
   bd.ops.push_back(op);
   bd.pend_mma.clear();
 }
@@ -664,26 +657,42 @@ double or_density(double rho, double n);
 
 // Tensor-core path or row-OR for a matrix-form cluster?  Forced by
 // pa_set_contract_path, else the faster by the context's measured rates: the
-// row-OR is costed as (set bits of A) x (words per B row) word ORs at the rate
-// measured on random operands (runs of set bits make it faster than that)
-// plus a fixed cost per (row, K chunk, tile) unit; the tensor path as every
-// multiply-add of its padded 128 x BN x 128 tiles (its rate includes the
-// expansion of both operands; tile pairs it skips because one operand's tile
-// is empty are not credited, so the estimate errs towards the row-OR).  `ra`
-// is A's estimated density (< 0: unknown).
-constexpr double kRowOrUnitsPerUs = 3.0e3;
+// row-OR is costed as (set bits of A) x (words per B row) word ORs plus a fixed
+// cost per (row, K chunk, tile) unit; the tensor path as a fixed cost and every
+// multiply-add of its padded 128 x BN x 128 tiles (tile pairs it skips because
+// one operand's tile is empty are not credited, so the estimate errs towards
+// the row-OR).  `ra` is A's estimated density (< 0: unknown).
+//
+// The rates are measured on random bits.  The set bits of plotted relations
+// and of their joins come in runs, which the row-OR takes several bits at a
+// time: where densities are known (a network's own plots) its rate counts
+// kRowOrRuns times.  Measured on whole cases with factors 1 / 2.5 / 3.5: chain of 8 at
+// 2048 px 64 / 62 / 54 us, of 4 at 4001 px 70 / 57 / 57 us, 38 networks 7.84 /
+// 7.45 / 7.42 ms.  Operands of unknown density (pa_contract) are taken as random and 16 %
+// dense.
+constexpr double kRowOrRuns = 3.5;
+constexpr double kUnknownDensity = 0.16;
+
+// Fixed cost of a unit, about 60 warp instructions (ncu, chain joins) at half
+// the issue rate of 152 SMs x 4 schedulers x 2 GHz: some 1e10 units per second
+// (at 3e3 per us 4096 chains took 2.36 ms, at 1e4 1.99).
+constexpr double kRowOrUnitsPerUs = 1.0e4;
+// Fixed cost of a tensor-core problem among the others of its launch (set-up,
+// first block, read-back): 0 sends 540 joins of 4096 chains there (1.89 ms per
+// replay), 0.5 sends 24 (1.60), 1 none (1.58).
+constexpr double kMmaFixedUs = 0.5;
 
 // Estimated microseconds of a matrix-form cluster on the row-OR path when A
-// has density `dens`: its word ORs at the context's measured rate (log-linear
-// in the density between the two measured points) plus every (row, K chunk,
-// tile) unit's fixed bookkeeping, about 200 warp instructions (ncu, chain
-// joins) at half the issue rate of 152 SMs x 4 schedulers x 2 GHz, some 3e9
-// units per second.
+// has density `dens` (< 0: unknown): its word ORs at the context's measured
+// rate (log-linear in the density between the two measured points) plus every
+// (row, K chunk, tile) unit's fixed cost.
 double rowor_cost_us(const pa_ctx* ctx, const JoinShape& js, double dens) {
   const double M = (double)js.M, N = js.nbits, K = (double)js.K, nb = (double)js.nbatch;
-  const double r0 = ctx ? ctx->rate_or : 2.0e5, r1 = ctx ? ctx->rate_or_dense : 9.0e5;
+  const double r0 = ctx ? ctx->rate_or : 2.9e5, r1 = ctx ? ctx->rate_or_dense : 1.39e6;
+  const double runs = dens >= 0 ? kRowOrRuns : 1.0;
+  if (dens < 0) dens = kUnknownDensity;
   const double f = std::min(1.0, std::max(0.0, log(std::max(dens, 1e-12) / 0.02) / log(8.0)));
-  const double rate_or = r0 * pow(r1 / r0, f);
+  const double rate_or = r0 * pow(r1 / r0, f) * runs;
   const double Nw = ceil(N / 64);
   int Nt = 1;
   while (Nt < 32 && Nt < Nw) Nt <<= 1;
@@ -691,46 +700,19 @@ double rowor_cost_us(const pa_ctx* ctx, const JoinShape& js, double dens) {
   return dens * M * K * nb * Nw / rate_or + units / kRowOrUnitsPerUs;
 }
 
-// Bytes per microsecond the two expansion kernels write together (measured
-// on 2048 x 2048 operands of a GB300: 8.4 MB in 12 us).
-constexpr double kExpandBytesPerUs = 7.0e5;
-
 bool use_mma(const pa_ctx* ctx, const JoinShape& js, double ra) {
-  // no context (pa_solve_network_static): the row-OR, which needs no byte copies
-  if (!ctx || ctx->path == PA_PATH_ROWOR || tensor_map_encoder() == nullptr) return false;
+  // no context (pa_solve_network_static): the row-OR
+  if (!ctx || ctx->path == PA_PATH_ROWOR) return false;
   const double M = (double)js.M, N = js.nbits, K = (double)js.K, nb = (double)js.nbatch;
   if (nb * M >= 2147483647.0 || N >= 2147483647.0 || nb >= 2147483647.0) return false;
-  if (nb * (M + N) * (ceil(K / 128) * 128) > 4e9) return false;  // byte copies of the operands
+  if (nb * (M + N) * (ceil(K / 128) * 128) > 4e9) return false;  // operands of more than 500 MB
   if (ctx->path == PA_PATH_MMA) return true;
-  const double BN = N <= 64 ? 64 : N <= 128 ? 128 : 256;
+  const double BN = N <= 128 ? 128 : 256;
   const double macs = nb * ceil(M / 128) * 128 * ceil(N / BN) * BN * ceil(K / 128) * 128;
   if (macs < 134217728.0) return false;  // small clusters: the row-OR's launch is cheaper
-  const double dens = ra >= 0 ? ra : 0.05;
-  const double t_or = rowor_cost_us(ctx, js, dens);
-  // rate_mma is measured on a 2048^3 product, expansion of both operands
-  // included (2 x 2048^2 bytes for 2048^3 multiply-adds); a cluster whose
-  // operands are larger relative to its products (few rows and columns,
-  // many summed values) pays the bytes beyond that share at the expansion
-  // kernels' rate
-  const double bytes = nb * (M + N) * (ceil(K / 128) * 128);
-  const double extra = std::max(0.0, bytes - macs * (2.0 / 2048.0));
-  const double t_mma = macs / ctx->rate_mma + extra / kExpandBytesPerUs;
+  const double t_or = rowor_cost_us(ctx, js, ra);
+  const double t_mma = macs / ctx->rate_mma + kMmaFixedUs;
   return t_mma < t_or;
-}
-
-// The occupancy bitmaps of a tensor-core problem (one bit per 128 x 128 tile
-// of each operand), cleared before its expansion kernels set them.
-void add_occupancy(Builder& bd, MmaDesc& md) {
-  const int64_t w32 = mma_occ_words(md);
-  const int64_t w64 = (w32 + 1) / 2;
-  uint32_t* occ = static_cast<uint32_t*>(bd.alloc((size_t)w64 * 8));
-  md.occ_a = occ;
-  md.occ_b = occ + md.nbatch * md.m_tiles * md.kb_words;
-  Op op;
-  op.kind = OP_MEMSET;
-  op.p = reinterpret_cast<uint64_t*>(occ);
-  op.count = w64;
-  bd.emit(op);
 }
 
 // rx, ry: estimated densities of X and Y (< 0: unknown); *rho_out receives the
@@ -811,9 +793,7 @@ BitArr join(Builder& bd, const BitArr& X, const BitArr& Y, const std::vector<int
     md.nbatch = js.nbatch;
     md.err = bd.d_err;
     mma_plan(md);
-    md.Ab = static_cast<uint8_t*>(bd.alloc((size_t)(md.nbatch * md.M * md.Kp)));
-    md.Bb = static_cast<uint8_t*>(bd.alloc((size_t)(md.nbatch * md.N * md.Kp)));
-    add_occupancy(bd, md);
+    if (mma_wants_occ(md)) md.occ = static_cast<uint8_t*>(bd.alloc((size_t)mma_occ_blocks(md)));
     if (md.ksplit > 1) {
       // the CTAs of one tile OR their partial results into C
       Op z;
@@ -871,7 +851,6 @@ void join_count(Builder& bd, const BitArr& X, const BitArr& Y, const std::vector
   if (js.private_a != 1.0 || js.private_b != 1.0)
     bd.fail(PA_ERR_UNSUPPORTED, "counting: every summed variable must be shared by A and B");
   if (js.K > (1 << 24)) bd.fail(PA_ERR_UNSUPPORTED, "counting: more than 2^24 summed values");
-  if (tensor_map_encoder() == nullptr) bd.fail(PA_ERR_UNSUPPORTED, "counting needs the tensor maps");
   const double M = (double)js.M, N = js.nbits, nb = (double)js.nbatch;
   if (nb * M >= 2147483647.0 || N >= 2147483647.0 ||
       nb * (M + N) * (ceil((double)js.K / 128) * 128) > 4e9)
@@ -900,9 +879,7 @@ void join_count(Builder& bd, const BitArr& X, const BitArr& Y, const std::vector
   md.nbatch = js.nbatch;
   md.err = bd.d_err;
   mma_plan(md);
-  md.Ab = static_cast<uint8_t*>(bd.alloc((size_t)(md.nbatch * md.M * md.Kp)));
-  md.Bb = static_cast<uint8_t*>(bd.alloc((size_t)(md.nbatch * md.N * md.Kp)));
-  add_occupancy(bd, md);
+  if (mma_wants_occ(md)) md.occ = static_cast<uint8_t*>(bd.alloc((size_t)mma_occ_blocks(md)));
   bd.pend_mma.push_back(md);
   bd.st.mma_macs += nb * M * N * (double)js.K;
   bd.st.n_mma++;
@@ -1627,15 +1604,12 @@ void run_ops(pa_ctx* ctx, const std::vector<Op>& ops, char* blob, cudaStream_t s
         launch_reshape(reinterpret_cast<const ReshapeDesc*>(blob + op.off0),
                        reinterpret_cast<const int64_t*>(blob + op.off1), op.n, op.i0, op.count, s);
         break;
-      case OP_UNPACK:
-        launch_unpack(reinterpret_cast<const MmaDesc*>(blob + op.off0), op.n, op.m, op.nw, s);
-        break;
       case OP_MMA:
         check_cuda(ctx,
                    launch_mma(reinterpret_cast<const MmaDesc*>(blob + op.off0),
-                              reinterpret_cast<const CUtensorMap*>(blob + op.off1),
-                              reinterpret_cast<const int64_t*>(blob + op.off2), op.n, op.count, s),
-                   "mma_bool_kernel");
+                              reinterpret_cast<const int64_t*>(blob + op.off2),
+                              reinterpret_cast<const int64_t*>(blob + op.off1), op.n, op.count, op.m, s),
+                   "mma_bits_kernel");
         break;
       case OP_ROWOR:
         check_cuda(ctx,
@@ -1733,7 +1707,7 @@ pa_status run_call(pa_ctx* ctx, cudaStream_t s, pa_stats* stats, F&& body,
     upload_blob(ctx, bd.blob, s);
     run_ops(ctx, bd.ops, ctx->arena, s, ctx->prof);
     bd.st.workspace_bytes = (int64_t)bd.used;
-    bd.st.n_launches = (int32_t)bd.ops.size();
+    bd.st.n_launches = count_launches(bd.ops);
     if (stats) *stats = bd.st;
     if (memo_key) {
       // a new program: the old one's graph goes with it (an executable graph
@@ -2398,7 +2372,6 @@ pa_status pa_autotune(pa_ctx* ctx, pa_rates* out, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   constexpr int64_t R = 2048, W = R / 64;
   uint64_t *A = nullptr, *B = nullptr, *C = nullptr;
-  uint8_t *Ab = nullptr, *Bb = nullptr;
   char* tab = nullptr;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   pa_status st = PA_OK;
@@ -2420,7 +2393,6 @@ pa_status pa_autotune(pa_ctx* ctx, pa_rates* out, void* stream) {
   do {
     if (cudaMalloc(&A, R * W * 8) != cudaSuccess || cudaMalloc(&B, R * W * 8) != cudaSuccess ||
         cudaMalloc(&C, R * W * 8) != cudaSuccess || cudaMalloc(&tab, 4096) != cudaSuccess ||
-        cudaMalloc(&Ab, R * R) != cudaSuccess || cudaMalloc(&Bb, R * R) != cudaSuccess ||
         cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
       fail("device allocation failed");
       break;
@@ -2458,21 +2430,13 @@ pa_status pa_autotune(pa_ctx* ctx, pa_rates* out, void* stream) {
     md.nbatch = 1;
     md.err = ctx->d_err;
     mma_plan(md);
-    md.Ab = Ab;
-    md.Bb = Bb;
-    CUtensorMap mmaps[2];
-    if (mma_encode_maps(md, mmaps) != cudaSuccess) {
-      fail("tensor maps (tensor-core path)");
-      break;
-    }
-    const int64_t mcta[2] = {0, mma_ctas(md)};
+    const int64_t mcta[2] = {0, mma_ctas(md)};  // (16 K blocks: no occupancy bitmaps)
     // pageable sources: each copy returns once the driver has taken the bytes
     cudaMemcpyAsync(tab, &rd, sizeof rd, cudaMemcpyHostToDevice, s);
     cudaMemcpyAsync(tab + 1024, &rmap, sizeof rmap, cudaMemcpyHostToDevice, s);
     cudaMemcpyAsync(tab + 2048, rcta, sizeof rcta, cudaMemcpyHostToDevice, s);
     cudaMemcpyAsync(tab + 3072, &md, sizeof md, cudaMemcpyHostToDevice, s);
     cudaMemcpyAsync(tab + 2048 + 64, mcta, sizeof mcta, cudaMemcpyHostToDevice, s);
-    cudaMemcpyAsync(tab + 1024 + 128, mmaps, sizeof mmaps, cudaMemcpyHostToDevice, s);
     const size_t rsmem = rowor_smem_bytes(rd);
     const int reps = 5;
     // row-OR at two densities of A (words OR-ed counted by the kernel)
@@ -2493,14 +2457,11 @@ pa_status pa_autotune(pa_ctx* ctx, pa_rates* out, void* stream) {
       cudaMemset(ctx->d_stat, 0, sizeof words);
       if (t_or > 0 && words > 0) rate_or[i] = (double)words / (reps + 1) / t_or;
     }
-    // the tensor path's rate includes expanding both operands
     const double t_mma = time_us(
         [&] {
-          launch_unpack(reinterpret_cast<const MmaDesc*>(tab + 3072), 1, unpack_blocks_a(md),
-                        unpack_blocks_b(md), s);
           launch_mma(reinterpret_cast<const MmaDesc*>(tab + 3072),
-                     reinterpret_cast<const CUtensorMap*>(tab + 1024 + 128),
-                     reinterpret_cast<const int64_t*>(tab + 2048 + 64), 1, mcta[1], s);
+                     reinterpret_cast<const int64_t*>(tab + 2048 + 64),
+                     nullptr, 1, mcta[1], 0, s);
         },
         reps);
     if (cudaGetLastError() != cudaSuccess || rate_or[0] <= 0 || rate_or[1] <= 0 || t_mma <= 0) {
@@ -2522,7 +2483,7 @@ pa_status pa_autotune(pa_ctx* ctx, pa_rates* out, void* stream) {
   if (st == PA_OK && out) pa_get_rates(ctx, out);
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
-  for (void* p : {(void*)A, (void*)B, (void*)C, (void*)Ab, (void*)Bb, (void*)tab})
+  for (void* p : {(void*)A, (void*)B, (void*)C, (void*)tab})
     if (p) cudaFree(p);
   return st;
 }
@@ -2838,7 +2799,7 @@ pa_status pa_batch_create(pa_ctx* ctx, int32_t nsys, const pa_system* systems, p
     bt->ops = bd.ops;
     bt->st = bd.st;
     bt->st.workspace_bytes = (int64_t)bd.used;
-    bt->st.n_launches = (int32_t)bd.ops.size();
+    bt->st.n_launches = count_launches(bd.ops);
     bt->blob_size = bd.blob.size();
     check_cuda(ctx, cudaMallocHost(reinterpret_cast<void**>(&bt->h_blob),
                                    std::max<size_t>(1, bt->blob_size)),
@@ -3265,7 +3226,7 @@ extern "C" pa_status pa_solve_network_static(int32_t nvars, const pa_axis* axes,
                "cudaMemcpyAsync");
     run_ops(ctx, bd.ops, work, s, false);
     bd.st.workspace_bytes = (int64_t)(kStaticHeader + bd.used);
-    bd.st.n_launches = (int32_t)bd.ops.size() + 2;
+    bd.st.n_launches = count_launches(bd.ops) + 2;
     if (stats) *stats = bd.st;
     return PA_OK;
   } catch (const Fail& f) {

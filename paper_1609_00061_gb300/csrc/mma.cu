@@ -1,29 +1,54 @@
 // Tensor-core path of the Boolean contraction (Eq. GAM of Sec. 3.3 for one
 // cluster of Sec. 3.5): C[b][m][n] = OR_k A[b][m][k] AND B[b][k][n] computed as
-// the 0/1 matrix product sum_k A[b][m][k] * B[b][k][n] on the 5th-generation
-// tensor cores, then thresholded at > 0.
+// a matrix product of operands that are 0 or a power of two on the
+// 5th-generation tensor cores, then thresholded at > 0.
 //
-// Exactness: the operands hold only 0.0 and 1.0 (exact in E4M3), every product
-// is 0 or 1 and the FP32 accumulator only ever adds non-negative values, so the
-// sum is positive exactly when some product is 1 (a positive FP32 sum can round
-// but never back to zero).  The result bits are therefore the Boolean product
-// for any K.
+// Exactness: the operands' non-zero values are exact in E4M3, every product is
+// 0 or at least 2^-18 and the FP32 accumulator only ever adds non-negative
+// values, so the sum is positive exactly when some product is not 0 (a positive
+// FP32 sum can round but never back to zero).  The result bits are therefore the
+// Boolean product for any K.  The counting semiring uses 2.0 throughout: sums
+// are multiples of 4 up to 2^26, exact.
 //
-// Data path: each operand is expanded once from its bit-packed row-OR layout
-// into E4M3 bytes, K-major (A as [b][m][k]: unpack_rows_kernel; B as
-// [b][n][k]: unpack_transpose_kernel, through 64 x 64 bit transposes in
-// registers).  mma_bool_kernel stages 128-byte-wide K slices of both with TMA
-// (128-byte swizzle) into a 4-deep ring, one elected thread issues
-// tcgen05.mma kind::f8f6f4 (M = 128, N = BN, K = 32 per instruction) into a
-// TMEM accumulator of 128 lanes x BN FP32 columns, and four epilogue warps read
-// it back with tcgen05.ld, compare with zero and store bit-packed rows.  A
-// product with few output tiles and a long K splits K over several CTAs per
-// tile, whose bits are OR-ed into C (cleared beforehand): partial sums combine
-// by OR because each is positive exactly when one of its products is.  Every
-// wait on an mbarrier is bounded (about 1 s); on expiry the kernel sets the
-// error word, finishes without storing and frees its TMEM.  (Expanding inside
-// the contraction kernel instead re-expands every A tile once per column tile
-// and every B tile once per row tile, and measured 2.4x slower.)
+// Data path.  Both operands are read as the bit-packed arrays the row-OR reads
+// and expanded to E4M3 bytes in shared memory by the CTA that multiplies them;
+// nothing but bits moves between HBM, L2 and the SMs.  (Expanding both
+// operands into byte arrays first, in two launches, and fetching those with TMA
+// cost 11 us of a 2048^3 product's 23, and 8 times the traffic.)  Two choices
+// make the expansion cheap:
+//   - four bytes come from a 32-bit word by one mask: bits r, r + 8, r + 16 and
+//     r + 24 stay where they are, bit r of four bytes.  A byte with one of the
+//     bits 0 .. 6 set is a power of two in E4M3 (2^-9 .. 2), and only whether a
+//     product is positive matters; bit 7 (the sign) moves to bit 6, and for
+//     counts every bit does (0x40 is 2.0).  The bytes of a word are thereby
+//     permuted; for K that does not matter as long as B's K rows are stored in
+//     the same order, for N it permutes the accumulator's columns, which the
+//     epilogue undoes with constant indexes;
+//   - B stays N-major (tcgen05 reads 8-bit operands in either orientation), so
+//     no bit transposes.
+// Per 128-value K block four producer warps fill one of four 16 + 32 KB stages
+// (128-byte swizzle); four such groups work on four blocks at a time, because a
+// group's chain of loads, masks and stores is longer than the tensor core's time
+// for a block (one group of eight warps measured 1900 cycles per block).  One
+// thread issues tcgen05.mma kind::f8f6f4 (M = 128, N = BN, K = 32 per
+// instruction) into a TMEM accumulator of 128 lanes x BN FP32 columns, and the
+// producer warps read it back with tcgen05.ld and store bit-packed rows.  K
+// blocks in which the A rows or the B columns of the tile hold no bit are
+// skipped: a group sees it in the words it has loaded, and where a CTA has many
+// blocks two bitmaps name the occupied ones (occupancy_kernel, one pass over the
+// bits first).  A product with few output tiles and a long K splits K over
+// several CTAs per tile, whose bits are OR-ed into C (cleared beforehand):
+// partial sums combine by OR because each is positive exactly when one of its
+// products is.  Every wait on an mbarrier is bounded (about 1 s); on expiry the
+// kernel sets the error word, finishes without storing and frees its TMEM.
+//
+// What bounds it (clock64 stamps, dense 2048^3, 128 CTAs): 2.7 k cycles of
+// set-up, 5.1 k until the first of the four stages is full, 1060 per block, 3 k
+// of read-back, 27.9 k in all.  Without the shared stores a block takes 930
+// cycles and without the products 825, so both sides are near their limit (an
+// N-major B halves the rate of a K-major one, 560 per block, which would need
+// bit transposes).  Against the byte-array version: 8192^3 of two cubic plots
+// 100 -> 80 us per call, the 2048^3 count 55 -> 48 us, ternary 256 78 -> 71 us.
 #include <cuda.h>
 #include <string.h>
 
@@ -36,14 +61,16 @@ namespace pa {
 namespace {
 
 constexpr int kMmaBM = 128;                   // rows of A per tile (TMEM lanes)
-constexpr int kMmaBK = 128;                   // K bytes per stage = one 128-byte swizzle row
-constexpr int kMmaStages = 4;
+constexpr int kMmaBK = 128;                   // K values per stage = one 128-byte swizzle row
 constexpr int kMmaATile = kMmaBM * kMmaBK;    // 16 KB
-constexpr int kMmaMaxBN = 256;
-constexpr int kMmaStageMax = kMmaATile + kMmaMaxBN * kMmaBK;  // 48 KB
+constexpr int kMmaNBlock = 128 * kMmaBK;      // 16 KB: 128 columns of B
+constexpr int kMmaStage = kMmaATile + 2 * kMmaNBlock;  // 48 KB
+constexpr int kMmaStages = 4;                 // one per producer group
 constexpr int kMmaTmemCols = 256;
-constexpr int kMmaThreads = 256;
-constexpr size_t kMmaSmem = (size_t)kMmaStages * kMmaStageMax + 1024 + 256;
+constexpr int kMmaProducers = 4 * kMmaStages;  // warps; the last warp issues the products
+constexpr int kMmaThreads = 32 * (kMmaProducers + 1);
+constexpr size_t kMmaSmem = (size_t)kMmaStages * kMmaStage + 1024;
+constexpr int kOccBlocks = 8;                 // K blocks per block of occupancy_kernel
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -66,25 +93,25 @@ __device__ __forceinline__ bool bar_wait(uint64_t* bar, uint32_t parity) {
   return false;
 }
 
-// Shared-memory matrix descriptor of a K-major operand tile in the canonical
-// 128-byte swizzled layout: 8-row x 128-byte atoms stacked every 1024 bytes
-// (stride byte offset), descriptor version 1, swizzle mode 2 (128 B).  The
-// leading byte offset is unused because a stage is exactly one atom wide in K.
-__device__ __forceinline__ uint64_t sw128_kmajor_desc(uint32_t saddr) {
+// Shared-memory matrix descriptor, 128-byte swizzle (mode 2), version 1; lbo and
+// sbo in bytes.  A (K-major): 8-row x 128-byte atoms every sbo bytes.  B
+// (N-major): 8 K rows of 128 columns per atom, the next 8 K rows sbo bytes on,
+// the next 128 columns lbo bytes on.
+__device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
   uint64_t d = 0;
   d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-  d |= (uint64_t)1 << 16;
-  d |= (uint64_t)(1024 >> 4) << 32;
+  d |= (uint64_t)(lbo >> 4) << 16;
+  d |= (uint64_t)(sbo >> 4) << 32;
   d |= (uint64_t)1 << 46;
   d |= (uint64_t)2 << 61;
   return d;
 }
 
 // Instruction descriptor of kind::f8f6f4: FP32 accumulator (bits 4-5 = 1),
-// A and B E4M3 (bits 7-9, 10-12 = 0), both K-major (bits 15, 16 = 0),
-// N >> 3 in bits 17-22, M >> 4 in bits 24-28.
+// A and B E4M3 (bits 7-9, 10-12 = 0), A K-major (bit 15 = 0), B N-major (bit
+// 16 = 1), N >> 3 in bits 17-22, M >> 4 in bits 24-28.
 __device__ __forceinline__ uint32_t f8_idesc(int M, int N) {
-  return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+  return (1u << 4) | (1u << 16) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* v) {
@@ -99,215 +126,288 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* v) {
       : "r"(taddr));
 }
 
-// 16 bits -> 16 bytes: byte j = E4M3 1.0 (0x38) when bit j is set, else 0.
-// For a nibble n, n * 0x00204081 places bit j of n at bit 8j (the four shifted
-// copies occupy disjoint bit ranges, so nothing carries); masking keeps those
-// bits and the final multiply turns each 0/1 byte into 0/0x38.
-__device__ __forceinline__ uint32_t expand4(uint32_t n) {
-  return ((n * 0x00204081u) & 0x01010101u) * 0x38u;
-}
-__device__ __forceinline__ uint4 expand16(uint32_t bits) {
-  return make_uint4(expand4(bits & 0xFu), expand4((bits >> 4) & 0xFu), expand4((bits >> 8) & 0xFu),
-                    expand4((bits >> 12) & 0xFu));
-}
+// Byte position p of a 32-value group holds value 8 (p % 4) + p / 4 (of K in an A
+// row, of N in a B row; B's K rows are placed by the same map).
+__device__ __forceinline__ int pos_value(int p) { return 8 * (p & 3) + (p >> 2); }
 
-// In-register transpose of a 64 x 64 bit block held by one warp: lane l holds
-// rows l (lo) and l + 32 (hi), bit c of a row being column c; afterwards lane
-// l holds columns l and l + 32.  Recursive block swap: for block size s the
-// rows r and r + s (r & s == 0) exchange the columns c + s of row r with the
-// columns c of row r + s (c & s == 0).
-__device__ __forceinline__ void transpose64(uint64_t& lo, uint64_t& hi, int lane) {
-  uint64_t t = ((lo >> 32) ^ hi) & 0x00000000FFFFFFFFull;
-  hi ^= t;
-  lo ^= t << 32;
-  const uint64_t masks[5] = {0x0000FFFF0000FFFFull, 0x00FF00FF00FF00FFull, 0x0F0F0F0F0F0F0F0Full,
-                             0x3333333333333333ull, 0x5555555555555555ull};
-#pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    const int s = 16 >> i;
-    const uint64_t m = masks[i];
-    const uint64_t plo = __shfl_xor_sync(0xffffffffu, lo, s);
-    const uint64_t phi = __shfl_xor_sync(0xffffffffu, hi, s);
-    if (lane & s) {
-      lo ^= ((plo >> s) ^ lo) & m;
-      hi ^= ((phi >> s) ^ hi) & m;
-    } else {
-      lo ^= (((lo >> s) ^ plo) & m) << s;
-      hi ^= (((hi >> s) ^ phi) & m) << s;
-    }
+// Byte positions 16 part .. 16 part + 15 of a 32-bit word: register t holds the
+// word's bits 4 part + t + 8 j (byte j).  Boolean products keep the bit where it
+// is; counts move it to bit 6.
+template <bool COUNT>
+__device__ __forceinline__ uint4 expand16(uint32_t x, int part) {
+  if (COUNT) {
+    const uint32_t y = x >> (4 * part);
+    return make_uint4((y << 6) & 0x40404040u, (y << 5) & 0x40404040u, (y << 4) & 0x40404040u,
+                      (y << 3) & 0x40404040u);
   }
+  return part == 0 ? make_uint4(x & 0x01010101u, x & 0x02020202u, x & 0x04040404u, x & 0x08080808u)
+                   : make_uint4(x & 0x10101010u, x & 0x20202020u, x & 0x40404040u,
+                                (x >> 1) & 0x40404040u);
 }
 
-// A operand: out[r][64 w .. 64 w + 63] = E4M3 bytes of word w of bit row r
-// (zero past the row's words).  One thread per input word; a warp's 32 words
-// are written as 128 16-byte chunks, four stores of 512 contiguous bytes each
-// (chunk c takes its 16 bits from the word of lane c / 4 by a shuffle).
-// Problem blockIdx.y of the table.
-__global__ void unpack_rows_kernel(const MmaDesc* __restrict__ descs) {
-  const MmaDesc& d = descs[blockIdx.y];
-  const uint64_t* __restrict__ in = d.A;
-  uint8_t* __restrict__ out = d.Ab;
-  const int64_t rows = d.nbatch * d.M, row_words = d.a_row_words, Kp = d.Kp;
-  const int64_t wpr = Kp / 64;  // output words of 64 bytes per row (even)
-  const int64_t total = rows * wpr;
-  const int lane = threadIdx.x & 31;
-  // the trip count is the same for every lane of a warp (total rounded up to
-  // whole warps), so the shuffles and ballots see all 32 lanes
-  const int64_t total_w = (total + 31) / 32 * 32;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total_w;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    uint64_t word = 0;
-    int64_t r = 0, w = 0;
-    if (i < total) {
-      r = i / wpr;
-      w = i - r * wpr;
-      word = w < row_words ? __ldg(in + r * row_words + w) : 0ull;
-    }
-    // chunk c = 32 j + lane of the warp's 128 is bits 16 (c % 4) .. of the
-    // word of lane c / 4; it lands at byte 16 c past the warp's first output
-    // byte, since the warp's words are consecutive in the output
-    const int64_t i0 = i - lane;
+__device__ __forceinline__ void st_shared16(uint32_t addr, uint4 v) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z),
+               "r"(v.w)
+               : "memory");
+}
+
+struct MmaShared {
+  uint64_t full[kMmaStages], empty[kMmaStages], accum;
+  uint32_t occ[kMmaStages][2];       // per group, by turns: a byte per warp, 1 A words, 2 B words
+  volatile int skip[kMmaStages];     // the stage's block is to be skipped
+  volatile int issued;               // blocks multiplied
+  uint32_t tmem;
+  volatile int fail;
+};
+
+// The last entry of the ascending table at[0 .. n) that is at most `block`, by
+// every thread of the block (evenly spaced samples, then the gap).
+__device__ __forceinline__ int find_problem(const int64_t* __restrict__ at0, int n, int64_t block) {
+  int p = 0;
+  while (n > 1) {
+    const int step = (n + (int)blockDim.x - 1) / (int)blockDim.x;
+    const int64_t at = (int64_t)threadIdx.x * step;
+    const int below = at < n && at0[p + at] <= block;
+    const int first = (__syncthreads_count(below) - 1) * step;
+    p += first;
+    n = min(step, n - first);
+  }
+  return p;
+}
+
+// Occupancy bitmaps of a problem's tiles: bit kb of a row tile of A (of a column
+// tile of B) when its K values 128 kb .. hold a set bit.  One block per tile and
+// eight K blocks, a warp each; the block writes one byte.  (Reads every bit of
+// the operands once: HBM or L2 bound, a few us of launch on small products.)
+__global__ void __launch_bounds__(32 * kOccBlocks)
+occupancy_kernel(const MmaDesc* __restrict__ descs, const int64_t* __restrict__ block0s, int nprob) {
+  asm volatile("griddepcontrol.launch_dependents;");
+  const int p = find_problem(block0s, nprob, (int64_t)blockIdx.x);
+  const MmaDesc& d = descs[p];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int64_t t = (int64_t)blockIdx.x - block0s[p];
+  const int64_t bytes = d.kb_words * 4;
+  const int64_t byte = t % bytes;
+  t /= bytes;
+  const int64_t ntile = d.m_tiles + d.n_tiles;
+  const int64_t b = t / ntile, tile = t - b * ntile;
+  const int64_t kb = byte * kOccBlocks + warp;
+  uint64_t any = 0;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (kb * kMmaBK < d.K) {
+    if (tile < d.m_tiles) {
+      const int64_t w = 2 * kb + (lane & 1), m0 = tile * kMmaBM + (lane >> 1);
+      const uint64_t* src = d.A + (b * d.M + m0) * d.a_row_words + w;
+      if (w < d.a_row_words) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int c = 32 * j + lane;
-      const uint64_t src = __shfl_sync(0xffffffffu, word, c >> 2);
-      if (i0 + (c >> 2) < total)
-        reinterpret_cast<uint4*>(out)[(i0 * 64 + 16 * (int64_t)c) / 16] =
-            expand16((uint32_t)(src >> ((c & 3) * 16)) & 0xFFFFu);
-    }
-    // occupancy: the lanes whose word holds a set bit OR their (row tile,
-    // K block) bits together per bitmap word, and one lane per word issues
-    // the atomic (a warp covering one row of K <= 4096 issues one), skipped
-    // when the bits are already set: every row of a tile sets the same bits,
-    // and same-address atomics queue at L2
-    if (d.occ_a) {
-      const bool nzl = word != 0;
-      const uint32_t nz = __ballot_sync(0xffffffffu, nzl);
-      if (nzl) {
-        const int64_t tile = (r / d.M) * d.m_tiles + (r % d.M) / 128, kb = w / 2;
-        const int64_t widx = tile * d.kb_words + kb / 32;
-        const uint32_t peers = __match_any_sync(nz, (unsigned long long)widx);
-        const uint32_t bits = __reduce_or_sync(peers, 1u << (kb % 32));
-        if (lane == __ffs(peers) - 1) {
-          uint32_t* o = d.occ_a + widx;
-          if ((__ldcg(o) & bits) != bits) atomicOr(o, bits);
-        }
+        for (int i = 0; i < 8; ++i)
+          if (m0 + 16 * i < d.M) any |= __ldg(src + (int64_t)(16 * i) * d.a_row_words);
+      }
+    } else {
+      // BN / 64 words of 128 rows, lanes along a row's words
+      const int wl = d.BN / 64, rows = 32 / wl;  // 4 and 8, or 2 and 16
+      const int64_t w = (tile - d.m_tiles) * wl + lane % wl;
+      const int64_t k0 = kb * kMmaBK + lane / wl;
+      const uint64_t* src = d.B + (b * d.K + k0) * d.Nw + w;
+      if (w < d.Nw) {
+#pragma unroll 8
+        for (int i = 0; i < kMmaBK; i += rows)
+          if (k0 + i < d.K) any |= __ldg(src + (int64_t)i * d.Nw);
       }
     }
   }
-}
-
-// B operand: in [nb][K][Nw] bits (N packed) -> out [nb][N][Kp] bytes
-// (K-major).  One warp per 64 x 64 bit block (batch, 64 K rows, 64 columns):
-// lanes load K rows l and l + 32 and transpose in registers (lane l then holds
-// columns l and l + 32, 64 K bits each); the 64 output rows of 64 bytes are
-// written 8 rows per instruction, 4 lanes per row, words passed by shuffles.
-// K rows >= K give zeros.
-// Problem blockIdx.y of the table.
-__global__ void unpack_transpose_kernel(const MmaDesc* __restrict__ descs) {
-  // the contraction launch that follows may start its set-up now; it waits
-  // for this grid to finish before it reads anything written here
-  asm volatile("griddepcontrol.launch_dependents;");
-  const MmaDesc& d = descs[blockIdx.y];
-  const uint64_t* __restrict__ in = d.B;
-  uint8_t* __restrict__ out = d.Bb;
-  const int64_t nb = d.nbatch, K = d.K, N = d.N, Nw = d.Nw, Kp = d.Kp;
-  const int lane = threadIdx.x & 31;
-  const int64_t kblk = Kp / 64, nblk = Nw;
-  const int64_t total = nb * kblk * nblk;
-  const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t it = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); it < total;
-       it += nwarps) {
-    const int64_t nbk = it % nblk, rest = it / nblk;
-    const int64_t kb = rest % kblk, b = rest / kblk;
-    const int64_t k0 = kb * 64 + lane;
-    const uint64_t* src = in + b * K * Nw + nbk;
-    uint64_t lo = k0 < K ? __ldg(src + k0 * Nw) : 0ull;
-    uint64_t hi = k0 + 32 < K ? __ldg(src + (k0 + 32) * Nw) : 0ull;
-    // a 64 x 64 block lies inside one (column tile, K block) pair
-    if (d.occ_b && __any_sync(0xffffffffu, (lo | hi) != 0ull) && lane == 0) {
-      const int64_t nt = (nbk * 64) / d.BN, kblock = (kb * 64) / 128;
-      uint32_t* o = d.occ_b + (b * d.n_tiles + nt) * d.kb_words + kblock / 32;
-      const uint32_t bit = 1u << (kblock % 32);
-      if (!(__ldcg(o) & bit)) atomicOr(o, bit);
-    }
-    transpose64(lo, hi, lane);
-    uint8_t* dst = out + (b * N) * Kp + kb * 64;
-    const int sub = lane >> 2, c = lane & 3;
+  __shared__ uint32_t bits[kOccBlocks];
+  const bool on = __any_sync(0xffffffffu, any != 0ull);
+  if (lane == 0) bits[warp] = on ? 1u : 0u;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    uint32_t v = 0;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int r = 8 * (j & 3) + sub;  // row within the half
-      const uint64_t v = __shfl_sync(0xffffffffu, j < 4 ? lo : hi, r);
-      const int64_t n = nbk * 64 + (j < 4 ? 0 : 32) + r;
-      if (n < N)
-        *reinterpret_cast<uint4*>(dst + n * Kp + c * 16) =
-            expand16((uint32_t)(v >> (16 * c)) & 0xFFFFu);
-    }
+    for (int i = 0; i < kOccBlocks; ++i) v |= bits[i] << i;
+    d.occ[(b * ntile + tile) * bytes + byte] = (uint8_t)v;
   }
 }
 
-// One CTA per (problem, batch, 128-row tile of A, BN-column tile of B).
-// Warp 0 lane 0: TMA producer.  Warp 1 lane 0: MMA issuer.  Warp 2: TMEM
-// allocation.  Warps 4-7: epilogue (warp 4 + j reads TMEM lanes 32j..32j+31).
-//
-// Start-up: the launch may begin while the expansion kernel that writes the
-// operands and occupancy bitmaps is still running (programmatic dependent
-// launch).  Thread 0 reads the descriptor, initialises the barriers and
-// signals the other warps through a named barrier, then waits for the
-// expansion to finish (griddepcontrol.wait) and issues its first copies at
-// once, while warp 2 allocates TMEM; no role reads the operands, the bitmaps
-// or C before its own griddepcontrol.wait.
+// Walks the K blocks of a CTA: those in [kb0, kb1) that both bitmaps hold, or
+// all of them without bitmaps.
+struct ActiveBlocks {
+  const uint32_t* occa;
+  const uint32_t* occb;
+  int kb0, kb1, w;
+  uint32_t m;
+  __device__ __forceinline__ uint32_t word(int i) const {
+    const int lo = max(kb0 - 32 * i, 0), hi = min(kb1 - 32 * i, 32);
+    if (hi <= lo) return 0u;
+    const uint32_t m = occa ? __ldcg(occa + i) & __ldcg(occb + i) : 0xffffffffu;
+    return m & (hi == 32 ? 0xffffffffu : (1u << hi) - 1u) &
+           ~((1u << lo) - 1u);
+  }
+  __device__ __forceinline__ void start() {
+    w = kb0 / 32;
+    m = word(w);
+  }
+  // the next active block, or -1
+  __device__ __forceinline__ int next() {
+    while (!m) {
+      if (32 * (w + 1) >= kb1) return -1;
+      m = word(++w);
+    }
+    const int kb = 32 * w + __ffs((int)m) - 1;
+    m &= m - 1;
+    return kb;
+  }
+};
+
+// A producer warp's blocks: the group's share (every kMmaStages-th) of the
+// CTA's, into the group's stage.  BN = 128 or 256.  A thread holds two A
+// words and BN / 64 B words of a block, loaded one block of its group ahead.
+// The thread-to-word maps make the loads 16- and 32-byte runs of a row and the
+// 16-byte shared stores free of conflicts (eight chunks of distinct bank groups
+// per quarter warp).
+template <int BN, bool COUNT>
+__device__ __forceinline__ void produce(const MmaDesc& d, MmaShared& sh, uint32_t ring,
+                                        ActiveBlocks act, int64_t b, int64_t m0, int64_t w0) {
+  constexpr int NB = BN / 64;               // B words per thread
+  constexpr int kPosStep = BN == 256 ? 8 : 16;  // K positions between a thread's B words
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int group = warp >> 2, wg = warp & 3;
+  // A: rows arow and arow + 16, word ahalf of the block's two
+  const int arow = wg * 32 + (lane >> 1), ahalf = lane & 1;
+  const uint64_t* ap = d.A + (b * d.M + m0 + arow) * d.a_row_words + ahalf;
+  const int64_t a_step = 16 * d.a_row_words;
+  const bool ain0 = m0 + arow < d.M, ain1 = m0 + arow + 16 < d.M;
+  // B: K positions pos + kPosStep i (rows krow + kPosStep / 4 i), word bword of
+  // the tile's BN / 64
+  const int q = lane >> 3;
+  const int bword = BN == 256 ? lane & 3 : lane & 1;
+  const int pos = wg * 32 + (BN == 256 ? (q & 1) + 4 * (q >> 1) + 2 * ((lane >> 2) & 1) : lane >> 1);
+  const int krow = (pos & ~31) + pos_value(pos & 31);
+  const uint64_t* bp = d.B + (b * d.K + krow) * d.Nw + w0 + bword;
+  const int64_t b_step = (kPosStep / 4) * d.Nw;
+  const bool bin = w0 + bword < d.Nw;
+  // shared-memory offsets of the four chunks of a word
+  uint32_t aoff[4], boff[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    aoff[c] = (uint32_t)arow * 128u + (((uint32_t)(4 * ahalf + c) ^ (uint32_t)(arow & 7)) << 4);
+    // the second column block holds a word's halves in opposite order (its rows
+    // share banks with the first's)
+    const uint32_t chunk = (uint32_t)(4 * (bword & 1) + 2 * (c >> 1) + ((c & 1) ^ (bword >> 1)));
+    boff[c] = (uint32_t)(kMmaATile + (bword >> 1) * kMmaNBlock) + (uint32_t)pos * 128u +
+              ((chunk ^ (uint32_t)(pos & 7)) << 4);
+  }
+  const uint32_t at = ring + (uint32_t)group * kMmaStage;
+  auto load = [&](int kb, uint64_t (&aw)[2], uint64_t (&bw)[NB]) {
+    const bool aw_in = kb >= 0 && 2 * (int64_t)kb + ahalf < d.a_row_words;
+    const uint64_t* p = ap + 2 * (int64_t)kb;
+    aw[0] = aw_in && ain0 ? __ldg(p) : 0ull;
+    aw[1] = aw_in && ain1 ? __ldg(p + a_step) : 0ull;
+    const int64_t left = kb >= 0 && bin ? d.K - (int64_t)kb * kMmaBK : 0;
+    const int kleft = (int)min((int64_t)kMmaBK, left) - krow;  // rows past krow in range
+    const uint64_t* r = bp + (int64_t)kb * kMmaBK * d.Nw;
+#pragma unroll
+    for (int i = 0; i < NB; ++i) bw[i] = i * (kPosStep / 4) < kleft ? __ldg(r + i * b_step) : 0ull;
+  };
+  act.start();
+  int kb = act.next();
+  for (int i = 0; i < group && kb >= 0; ++i) kb = act.next();
+  uint64_t aw[2], bw[NB];
+  load(kb, aw, bw);
+  bool dead = false;
+  for (int it = 0; kb >= 0; ++it) {
+    uint64_t a[2], bb[NB];
+    a[0] = aw[0];
+    a[1] = aw[1];
+#pragma unroll
+    for (int i = 0; i < NB; ++i) bb[i] = bw[i];
+    for (int i = 0; i < kMmaStages && kb >= 0; ++i) kb = act.next();
+    load(kb, aw, bw);
+    bool use = true;
+    if (!act.occa) {
+      // does the block hold a bit of A and of B?  (the group's four warps
+      // agree; they have all passed the last reading of this slot when they
+      // meet here for the other one)
+      uint64_t bor = bb[0];
+#pragma unroll
+      for (int i = 1; i < NB; ++i) bor |= bb[i];
+      const bool na = __any_sync(0xffffffffu, (a[0] | a[1]) != 0ull);
+      const bool nb = __any_sync(0xffffffffu, bor != 0ull);
+      if (lane == 0)
+        reinterpret_cast<volatile uint8_t*>(&sh.occ[group][it & 1])[wg] = (uint8_t)((na ? 1 : 0) | (nb ? 2 : 0));
+      asm volatile("bar.sync %0, 128;" ::"r"(1 + group) : "memory");
+      const uint32_t o = *reinterpret_cast<volatile uint32_t*>(&sh.occ[group][it & 1]);
+      use = (o & 0x01010101u) && (o & 0x02020202u);
+    }
+    // (a warp whose wait ran out goes on without storing or arriving: the
+    // group's barriers need it)
+    if (dead || (it > 0 && !bar_wait(&sh.empty[group], (uint32_t)(it - 1) & 1u))) {
+      sh.fail = 1;
+      dead = true;
+      continue;
+    }
+    if (use) {
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          st_shared16(at + aoff[c] + i * (16 * 128),
+                      expand16<COUNT>((uint32_t)(a[i] >> (32 * (c >> 1))), c & 1));
+#pragma unroll
+      for (int i = 0; i < NB; ++i)
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          st_shared16(at + boff[c] + i * (kPosStep * 128),
+                      expand16<COUNT>((uint32_t)(bb[i] >> (32 * (c >> 1))), c & 1));
+      // the stores become visible to the tensor core's proxy, then the warp
+      // arrives
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (wg == 0 && lane == 0) sh.skip[group] = use ? 0 : 1;
+    __syncwarp();
+    if (lane == 0)
+      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&sh.full[group])) : "memory");
+  }
+}
+
+// One CTA per (problem, batch, 128-row tile of A, BN-column tile of B, K
+// chunk).  Warps 0-15: producers, then the epilogue (warp w reads TMEM lanes
+// 32 (w % 4) .. and columns BN / 4 (w / 4) ..).  Warp 16: TMEM allocation and,
+// in one lane, the products.
 __global__ void __launch_bounds__(kMmaThreads, 1)
-mma_bool_kernel(const MmaDesc* __restrict__ descs, const CUtensorMap* __restrict__ maps,
-                const int64_t* __restrict__ cta0s, int nprob) {
+mma_bits_kernel(const MmaDesc* __restrict__ descs, const int64_t* __restrict__ cta0s, int nprob) {
   extern __shared__ uint8_t mma_raw[];
   uint8_t* smem =
       reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(mma_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + (size_t)kMmaStages * kMmaStageMax);
-  uint64_t* empty = full + kMmaStages;
-  uint64_t* accum = empty + kMmaStages;
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(accum + 1);
-  volatile int* sfail = reinterpret_cast<volatile int*>(tslot + 1);
-  int* sp = const_cast<int*>(sfail) + 1;
+  __shared__ MmaShared sh;
   __shared__ MmaDesc sd;
+  asm volatile("griddepcontrol.launch_dependents;");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  uint32_t tmem = 0;  // warps 1-7 (the producer never touches TMEM)
-
-  if (warp == 0) {
-    if (lane == 0) {
-      int lo = 0, hi = nprob - 1;
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (cta0s[mid] <= (int64_t)blockIdx.x) lo = mid; else hi = mid - 1;
-      }
-      *sp = lo;
-      sd = descs[lo];
-      for (int s = 0; s < kMmaStages; ++s) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&full[s])) : "memory");
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&empty[s])) : "memory");
-      }
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(accum)) : "memory");
-      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      *sfail = 0;
-    }
-    __syncwarp();
-    // descriptor, barriers and failure word are ready for warps 1-7
-    asm volatile("bar.arrive 1, %0;" ::"r"(kMmaThreads) : "memory");
-  } else {
-    if (warp == 2) {
-      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                       smem_addr(tslot)),
-                   "r"(kMmaTmemCols)
-                   : "memory");
-      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    asm volatile("bar.sync 1, %0;" ::"r"(kMmaThreads) : "memory");
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    tmem = *tslot;
+  const int p = find_problem(cta0s, nprob, (int64_t)blockIdx.x);
+  {
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(descs + p);
+    uint32_t* dst = reinterpret_cast<uint32_t*>(&sd);
+    if (threadIdx.x < (int)(sizeof(MmaDesc) / 4)) dst[threadIdx.x] = src[threadIdx.x];
   }
-  const int p = *sp;
+  if (warp == kMmaProducers) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_addr(&sh.tmem)),
+                 "r"(kMmaTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  } else if (threadIdx.x == 0) {
+    for (int s = 0; s < kMmaStages; ++s) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;" ::"r"(smem_addr(&sh.full[s])) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&sh.empty[s])) : "memory");
+    }
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 2;" ::"r"(smem_addr(&sh.accum)) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    sh.fail = 0;
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = sh.tmem;
   const MmaDesc& d = sd;
   int64_t t = (int64_t)blockIdx.x - cta0s[p];
   const int kc = (int)(t % d.ksplit);
@@ -317,202 +417,138 @@ mma_bool_kernel(const MmaDesc* __restrict__ descs, const CUtensorMap* __restrict
   const int64_t mt = t % d.m_tiles;
   const int64_t b = t / d.m_tiles;
   const int BN = d.BN;
-  const int stage_bytes = kMmaATile + BN * kMmaBK;
-  const int nk = (int)(d.Kp / kMmaBK);
-  // the K blocks where both this CTA's A row tile and B column tile hold a set
-  // bit (every block when the problem has no occupancy bitmaps); producer and
-  // issuer walk the same sequence, the j-th active block using ring slot j
-  const uint32_t* occa = d.occ_a ? d.occ_a + (b * d.m_tiles + mt) * d.kb_words : nullptr;
-  const uint32_t* occb = d.occ_b ? d.occ_b + (b * d.n_tiles + nt) * d.kb_words : nullptr;
-  // this CTA's K blocks [kb0, kb1) and the bitmap words that hold them
-  const int kb0 = kc * d.kchunk, kb1 = min(nk, kb0 + d.kchunk);
-  const int w0 = kb0 / 32, w1 = (kb1 + 31) / 32;
+  const int nk = (int)((d.K + kMmaBK - 1) / kMmaBK);
   const bool split = d.ksplit > 1;
-  auto active = [&](int w) -> uint32_t {
-    uint32_t m = 0xffffffffu;
-    if (occa) m &= __ldcg(occa + w);
-    if (occb) m &= __ldcg(occb + w);
-    const int lo = max(kb0 - 32 * w, 0), hi = min(kb1 - 32 * w, 32);
-    if (hi <= lo) return 0u;
-    m &= (hi == 32 ? 0xffffffffu : (1u << hi) - 1u) & ~((1u << lo) - 1u);
-    return m;
-  };
+  // every role walks the same sequence of K blocks, the j-th in stage
+  // j % kMmaStages
+  ActiveBlocks act;
+  const uint32_t* occ = reinterpret_cast<const uint32_t*>(d.occ) + b * (d.m_tiles + d.n_tiles) * d.kb_words;
+  act.occa = d.occ ? occ + mt * d.kb_words : nullptr;
+  act.occb = d.occ ? occ + (d.m_tiles + nt) * d.kb_words : nullptr;
+  act.kb0 = kc * d.kchunk;
+  act.kb1 = min(nk, act.kb0 + d.kchunk);
+  // the operands, the bitmaps and C belong to the earlier kernels of the
+  // stream until here
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 
-  // the operands, the bitmaps and C belong to the expansion kernel until it
-  // has finished: each role waits for it (griddepcontrol.wait) right before
-  // its first access to them
-  if (warp == 0) {
+  if (warp == kMmaProducers) {
     if (lane == 0) {
-      const CUtensorMap* ma = maps + 2 * p;
-      const CUtensorMap* mb = ma + 1;
-      // the tensor maps were written to global memory by a copy before the launch
-      asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(ma) : "memory");
-      asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(mb) : "memory");
-      asm volatile("griddepcontrol.wait;" ::: "memory");
-      int j = 0;
-      bool failed = false;
-      for (int w = w0; w < w1 && !failed; ++w) {
-        for (uint32_t m = active(w); m; m &= m - 1) {
-          const int k = w * 32 + __ffs(m) - 1;
-          const int s = j % kMmaStages;
-          const uint32_t ph = (uint32_t)(j / kMmaStages) & 1u;
-          if (j >= kMmaStages && !bar_wait(&empty[s], ph ^ 1u)) {
-            *sfail = 1;
-            failed = true;
-            break;
-          }
-          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(
-                           smem_addr(&full[s])),
-                       "r"(stage_bytes)
-                       : "memory");
-          const uint32_t dst_a = smem_addr(smem + (size_t)s * kMmaStageMax);
-          const uint32_t dst_b = dst_a + kMmaATile;
-          asm volatile(
-              "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
-              " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst_a),
-              "l"(reinterpret_cast<uint64_t>(ma)), "r"(k * kMmaBK), "r"((int)(mt * kMmaBM)),
-              "r"((int)b), "r"(smem_addr(&full[s]))
-              : "memory");
-          asm volatile(
-              "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
-              " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst_b),
-              "l"(reinterpret_cast<uint64_t>(mb)), "r"(k * kMmaBK), "r"((int)(nt * BN)),
-              "r"((int)b), "r"(smem_addr(&full[s]))
-              : "memory");
-          ++j;
-        }
-      }
-      // after a failure anywhere, wait (bounded) for the copies still in
-      // flight before the CTA's shared memory is released
-      if (*sfail)
-        for (int q = j > kMmaStages ? j - kMmaStages : 0; q < j; ++q)
-          bar_wait(&full[q % kMmaStages], (uint32_t)(q / kMmaStages) & 1u);
-    }
-    __syncwarp();
-  } else if (warp == 1) {
-    if (lane == 0) {
-      asm volatile("griddepcontrol.wait;" ::: "memory");
       const uint32_t idesc = f8_idesc(kMmaBM, BN);
-      int j = 0;
-      bool failed = false;
-      for (int w = w0; w < w1 && !failed; ++w) {
-        for (uint32_t m = active(w); m; m &= m - 1) {
-          const int s = j % kMmaStages;
-          const uint32_t ph = (uint32_t)(j / kMmaStages) & 1u;
-          if (!bar_wait(&full[s], ph)) {
-            *sfail = 1;
-            failed = true;
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t a0 = smem_addr(smem + (size_t)s * kMmaStageMax), b0 = a0 + kMmaATile;
-#pragma unroll
-          for (int kk = 0; kk < kMmaBK / 32; ++kk) {
-            const uint64_t ad = sw128_kmajor_desc(a0 + kk * 32), bd = sw128_kmajor_desc(b0 + kk * 32);
-            const uint32_t acc = (j > 0 || kk > 0) ? 1u : 0u;
-            asm volatile(
-                "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                " tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-                "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
-                : "memory");
-          }
-          asm volatile(
-              "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                  smem_addr(&empty[s]))
-              : "memory");
-          ++j;
+      act.start();
+      int issued = 0;
+      for (int j = 0; act.next() >= 0; ++j) {
+        const int s = j % kMmaStages;
+        if (!bar_wait(&sh.full[s], (uint32_t)(j / kMmaStages) & 1u)) {
+          sh.fail = 1;
+          break;
         }
+        if (sh.skip[s]) {
+          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&sh.empty[s])) : "memory");
+          continue;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t a0 = smem_addr(smem + (size_t)s * kMmaStage), b0 = a0 + kMmaATile;
+#pragma unroll
+        for (int kk = 0; kk < kMmaBK / 32; ++kk) {
+          const uint64_t ad = sw128_desc(a0 + kk * 32, 16, 1024);
+          const uint64_t bd = sw128_desc(b0 + kk * 4096, kMmaNBlock, 1024);
+          const uint32_t acc = (issued > 0 || kk > 0) ? 1u : 0u;
+          asm volatile(
+              "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+              " tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
+              "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
+              : "memory");
+        }
+        asm volatile(
+            "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                smem_addr(&sh.empty[s]))
+            : "memory");
+        ++issued;
       }
-      // arrives once every MMA issued above has completed (also on failure)
+      sh.issued = issued;
+      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&sh.accum)) : "memory");
+      // arrives once every product issued above has completed (also on failure)
       asm volatile(
           "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-              smem_addr(accum))
+              smem_addr(&sh.accum))
           : "memory");
     }
     __syncwarp();
-  } else if (warp >= 4) {
-    const int ew = warp - 4;
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    // no K block in common: nothing was accumulated, every sum is zero
-    // (decided while the products run)
-    bool none = true;
-    for (int w = w0; w < w1 && none; ++w) none = (active(w) == 0);
-    const bool ok = bar_wait(accum, 0);
+  } else {
+    const int64_t m0 = mt * kMmaBM, w0 = nt * (BN / 64);
+    const uint32_t ring = smem_addr(smem);
+    if (d.counts) {
+      if (BN == 256) produce<256, true>(d, sh, ring, act, b, m0, w0);
+      else produce<128, true>(d, sh, ring, act, b, m0, w0);
+    } else {
+      if (BN == 256) produce<256, false>(d, sh, ring, act, b, m0, w0);
+      else produce<128, false>(d, sh, ring, act, b, m0, w0);
+    }
+    const bool ok = bar_wait(&sh.accum, 0);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    // with K split, a CTA that summed nothing leaves C as it is (other CTAs
-    // OR their bits into the same words)
-    const bool store = ok && !*sfail && !(split && none);
-    const int64_t m = mt * kMmaBM + ew * 32 + lane;
-    // up to 128 columns per round: every TMEM load of the round is in flight
-    // before the one wait
-    const int G = BN < 128 ? BN : 128;
-    for (int c0 = 0; c0 < BN; c0 += G) {
-      uint32_t v[128];
+    // no block multiplied: nothing was accumulated, every sum is zero; with K
+    // split such a CTA leaves C as it is (others OR their bits into it)
+    const bool none = sh.issued == 0;
+    const bool store = ok && !sh.fail && !(split && none);
+    const int ew = warp & 3, part = warp >> 2;
+    const int64_t m = m0 + ew * 32 + lane;
+    // a warp's columns, 32 at a time: the bits of half a result word
+    for (int c0 = part * (BN / 4); c0 < (part + 1) * (BN / 4); c0 += 32) {
+      uint32_t v[32];
       const uint32_t ta = tmem + ((uint32_t)(ew * 32) << 16) + (uint32_t)c0;
       if (none) {
 #pragma unroll
-        for (int q = 0; q < 128; ++q) v[q] = 0u;
+        for (int k = 0; k < 32; ++k) v[k] = 0u;
       } else {
         tmem_ld32(ta, v);
-        tmem_ld32(ta + 32u, v + 32);
-        if (G == 128) {
-          tmem_ld32(ta + 64u, v + 64);
-          tmem_ld32(ta + 96u, v + 96);
-        }
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
       }
+      const int64_t n0 = w0 * 64 + c0;  // first result column
+      const int swap = c0 >= 128 ? 4 : 0;  // the second column block's halves are swapped
+      if (d.counts) {
+        // counting semiring: every sum is 4 x an integer <= K <= 2^24, exact in
+        // FP32.  The warp's 32 x 32 counts go through shared memory (the ring
+        // is idle once every product is done; rows padded to 33 words against
+        // bank conflicts) so that each store writes 32 consecutive counts of
+        // one row.
+        if (store) {
+          uint32_t* st = reinterpret_cast<uint32_t*>(smem) + warp * (32 * 33);
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        if (h * 64 >= G) break;
-        const uint32_t* vh = v + 64 * h;
-        const int c = (c0 >> 6) + h;  // 64-column chunk of the tile
-        if (d.counts) {
-          // counting semiring: every sum is an integer <= K <= 2^24, exact in
-          // FP32.  The warp's 32 rows x 64 counts go through shared memory (the
-          // operand ring is idle once every product is done; rows padded to 65
-          // words against bank conflicts) so that each store writes 32
-          // consecutive counts of one row.
-          if (store) {
-            uint32_t* st = reinterpret_cast<uint32_t*>(smem) + ew * (32 * 65);
-#pragma unroll
-            for (int q = 0; q < 64; ++q) st[lane * 65 + q] = (uint32_t)__uint_as_float(vh[q]);
-            __syncwarp();
-            const int64_t n0 = nt * BN + c * 64;
-            for (int rr = 0; rr < 32; ++rr) {
-              const int64_t mm = mt * kMmaBM + ew * 32 + rr;
-              if (mm >= d.M) break;
-              uint32_t* row = d.counts + (b * d.M + mm) * d.N;
-              if (n0 + lane < d.N) row[n0 + lane] = st[rr * 65 + lane];
-              if (n0 + 32 + lane < d.N) row[n0 + 32 + lane] = st[rr * 65 + 32 + lane];
-            }
-            __syncwarp();
-          }
-          continue;
+          for (int k = 0; k < 32; ++k)
+            st[lane * 33 + 8 * (k & 3) + ((k >> 2) ^ swap)] = (uint32_t)(__uint_as_float(v[k]) * 0.25f);
+          __syncwarp();
+          const int64_t rows = min((int64_t)32, d.M - (m0 + ew * 32));
+          uint32_t* dst = d.counts + (b * d.M + m0 + ew * 32) * d.N + n0 + lane;
+          if (n0 + lane < d.N)
+            for (int rr = 0; rr < rows; ++rr) dst[(int64_t)rr * d.N] = st[rr * 33 + lane];
+          __syncwarp();
         }
-        uint64_t word = 0;
+        continue;
+      }
+      uint32_t bits = 0;
 #pragma unroll
-        for (int q = 0; q < 64; ++q) word |= (uint64_t)(__uint_as_float(vh[q]) > 0.0f) << q;
-        const int64_t w = nt * (BN / 64) + c;
-        if (store && m < d.M && w < d.Nw) {
-          const int64_t rem = d.N - w * 64;
-          if (rem < 64) word &= (1ull << rem) - 1ull;
-          uint64_t* dst = d.C + (b * d.M + m) * d.Nw + w;
-          if (!split) *dst = word;
-          else if (word) atomicOr(reinterpret_cast<unsigned long long*>(dst), (unsigned long long)word);
-        }
+      for (int k = 0; k < 32; ++k) bits |= (v[k] != 0u ? 1u : 0u) << (8 * (k & 3) + (k >> 2));  // pos_value(k)
+      if (swap) bits = ((bits & 0x0f0f0f0fu) << 4) | ((bits >> 4) & 0x0f0f0f0fu);
+      const int64_t w = n0 >> 6;
+      if (store && m < d.M && w < d.Nw) {
+        const int64_t rem = d.N - n0;
+        if (rem < 32) bits &= rem <= 0 ? 0u : (1u << rem) - 1u;
+        uint32_t* dst = reinterpret_cast<uint32_t*>(d.C + (b * d.M + m) * d.Nw + w) + ((n0 >> 5) & 1);
+        if (!split) *dst = bits;
+        else if (bits) atomicOr(dst, bits);
       }
     }
     if (!ok && lane == 0) atomicExch(d.err, 1);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (warp == 2) {
+  if (warp == kMmaProducers) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                  "r"(kMmaTmemCols)
                  : "memory");
   }
-  if (threadIdx.x == 0 && *sfail) atomicExch(d.err, 1);
+  if (threadIdx.x == 0 && sh.fail) atomicExch(d.err, 1);
 }
 
 // Random bits for autotuning: bit j of word i is set when the SplitMix64 mix
@@ -572,12 +608,11 @@ void launch_random_bits(uint64_t* w, int64_t nwords, int64_t row_words, int64_t 
 }
 
 void mma_plan(MmaDesc& d) {
-  d.BN = d.N <= 64 ? 64 : d.N <= 128 ? 128 : 256;
+  d.BN = d.N <= 128 ? 128 : 256;
   d.Nw = (d.N + 63) / 64;
-  d.Kp = (d.K + kMmaBK - 1) / kMmaBK * kMmaBK;
   d.m_tiles = (d.M + kMmaBM - 1) / kMmaBM;
   d.n_tiles = (d.N + d.BN - 1) / d.BN;
-  const int64_t nk = d.Kp / kMmaBK;
+  const int64_t nk = (d.K + kMmaBK - 1) / kMmaBK;
   d.kb_words = (nk + 31) / 32;
   // Few output tiles and a long K (a cluster that sums many variables into a
   // small result) would leave most SMs idle: split K over up to one CTA per
@@ -596,81 +631,40 @@ void mma_plan(MmaDesc& d) {
   }
 }
 
-int64_t mma_occ_words(const MmaDesc& d) {
-  return d.nbatch * (d.m_tiles + d.n_tiles) * d.kb_words;
-}
-
 int64_t mma_ctas(const MmaDesc& d) { return d.nbatch * d.m_tiles * d.n_tiles * d.ksplit; }
 
-size_t mma_smem_bytes() { return kMmaSmem; }
+// Bitmaps pay where a CTA walks many K blocks: writing them takes a launch of
+// about 4 us, seeing an empty block in its loaded words about 200 cycles (a
+// CTA of 16 blocks gains 1.6 us at most, one of 64 sparse ones 6).
+bool mma_wants_occ(const MmaDesc& d) { return d.kchunk >= 32; }
 
-cudaError_t mma_encode_maps(const MmaDesc& d, CUtensorMap* maps2) {
-  memset(maps2, 0, 2 * sizeof(CUtensorMap));
-  EncodeTiledFn enc = tensor_map_encoder();
-  if (!enc) return cudaErrorNotSupported;
-  const int64_t rows[2] = {d.M, d.N};
-  const uint8_t* base[2] = {d.Ab, d.Bb};
-  const cuuint32_t box_rows[2] = {(cuuint32_t)kMmaBM, (cuuint32_t)d.BN};
-  for (int i = 0; i < 2; ++i) {
-    const cuuint64_t dims[3] = {(cuuint64_t)d.Kp, (cuuint64_t)rows[i], (cuuint64_t)d.nbatch};
-    const cuuint64_t strides[2] = {(cuuint64_t)d.Kp, (cuuint64_t)(d.Kp * rows[i])};
-    const cuuint32_t box[3] = {(cuuint32_t)kMmaBK, box_rows[i], 1u};
-    const cuuint32_t estr[3] = {1u, 1u, 1u};
-    CUresult r = enc(&maps2[i], CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<uint8_t*>(base[i]), dims,
-                     strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
-  }
-  return cudaSuccess;
+int64_t mma_occ_blocks(const MmaDesc& d) {
+  return d.nbatch * (d.m_tiles + d.n_tiles) * d.kb_words * 4;  // one byte per block
 }
 
-int64_t unpack_blocks_a(const MmaDesc& d) {
-  return std::min<int64_t>((d.nbatch * d.M * (d.Kp / 64) + 255) / 256, 152 * 16);
-}
-
-int64_t unpack_blocks_b(const MmaDesc& d) {
-  return std::min<int64_t>((d.nbatch * (d.Kp / 64) * d.Nw + 7) / 8, 152 * 16);
-}
-
-void launch_unpack(const MmaDesc* d_descs, int nprob, int64_t blocks_a, int64_t blocks_b,
-                   cudaStream_t s) {
-  if (nprob <= 0) return;
-  // the expansion kernels use no shared memory; asking for the largest
-  // shared-memory carveout anyway keeps the SMs in the configuration the
-  // contraction kernel that follows needs, so that no reconfiguration sits
-  // between the two launches
-  static bool carveout = [] {
-    cudaFuncSetAttribute(reinterpret_cast<const void*>(unpack_rows_kernel),
-                         cudaFuncAttributePreferredSharedMemoryCarveout,
-                         cudaSharedmemCarveoutMaxShared);
-    cudaFuncSetAttribute(reinterpret_cast<const void*>(unpack_transpose_kernel),
-                         cudaFuncAttributePreferredSharedMemoryCarveout,
-                         cudaSharedmemCarveoutMaxShared);
-    return true;
-  }();
-  (void)carveout;
-  if (blocks_a > 0) unpack_rows_kernel<<<dim3((unsigned)blocks_a, (unsigned)nprob), 256, 0, s>>>(d_descs);
-  if (blocks_b > 0)
-    unpack_transpose_kernel<<<dim3((unsigned)blocks_b, (unsigned)nprob), 256, 0, s>>>(d_descs);
-}
-
-cudaError_t launch_mma(const MmaDesc* d_descs, const CUtensorMap* d_maps, const int64_t* d_cta0,
-                       int nprob, int64_t grid, cudaStream_t s) {
+cudaError_t launch_mma(const MmaDesc* d_descs, const int64_t* d_cta0, const int64_t* d_occ0, int nprob,
+                       int64_t grid, int64_t occ_grid, cudaStream_t s) {
   if (nprob <= 0 || grid <= 0) return cudaSuccess;
-  if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  smem_limit(reinterpret_cast<const void*>(mma_bool_kernel), kMmaSmem);
-  // programmatic dependent launch: the set-up overlaps the expansion kernel
+  if (grid > 0x7fffffffLL || occ_grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+  smem_limit(reinterpret_cast<const void*>(mma_bits_kernel), kMmaSmem);
+  // programmatic dependent launches: the set-up overlaps the previous kernel
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(kMmaThreads);
-  cfg.dynamicSmemBytes = kMmaSmem;
+  cfg.gridDim = dim3((unsigned)occ_grid);
+  cfg.blockDim = dim3(32 * kOccBlocks);
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, mma_bool_kernel, d_descs, d_maps, d_cta0, nprob);
+  if (occ_grid > 0) {
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, occupancy_kernel, d_descs, d_occ0, nprob);
+    if (e != cudaSuccess) return e;
+  }
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(kMmaThreads);
+  cfg.dynamicSmemBytes = kMmaSmem;
+  return cudaLaunchKernelEx(&cfg, mma_bits_kernel, d_descs, d_cta0, nprob);
 }
 
 }  // namespace pa

@@ -242,49 +242,38 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 EncodeTiledFn tensor_map_encoder();
 
 // Tensor-core contraction (mma.cu): the same problem as RowOrDesc, from the
-// same bit-packed layouts, as a 0/1 E4M3 matrix product thresholded at > 0.
-// The operands are first expanded into the byte arrays Ab and Bb.
+// same bit-packed layouts, as a 0/1 matrix product on E4M3 operands thresholded
+// at > 0.
 struct MmaDesc {
   const uint64_t* A;          // [nbatch][M][a_row_words], K bits per row
   const uint64_t* B;          // [nbatch][K][Nw], N bits per row
   uint64_t* C;                // [nbatch][M][Nw]
-  uint8_t* Ab;                // [nbatch][M][Kp] E4M3 bytes
-  uint8_t* Bb;                // [nbatch][N][Kp] E4M3 bytes
-  int64_t M, N, K, Kp, Nw, a_row_words, nbatch;
+  int64_t M, N, K, Nw, a_row_words, nbatch;
   int64_t m_tiles, n_tiles;
-  int32_t BN;                 // columns per tile: 64, 128 or 256
-  int* err;                   // device error word: set when a bounded wait runs out
-  uint32_t* counts;           // when not null: the sums themselves, [nbatch][M][N]
-                              // (counting semiring), and C is not written
-  // Occupancy bitmaps of the 128 x 128 tiles (cleared before the expansion,
-  // set by it): bit kb of occ_a[(b * m_tiles + mt) * kb_words + kb / 32] when
-  // A's rows 128 mt.. and K values 128 kb.. hold a set bit, likewise occ_b per
-  // BN-column tile.  The contraction multiplies only the K blocks both hold.
-  uint32_t* occ_a;
-  uint32_t* occ_b;
+  // Occupancy bitmaps, kb_words 32-bit words for every row tile of A and then
+  // every column tile of B, per batch value: bit kb when K values 128 kb ..
+  // hold a set bit.  The product skips the K blocks either one lacks.  Null: the
+  // product looks at the words themselves.
+  uint8_t* occ;
   int64_t kb_words;
+  int32_t BN;                 // columns per tile: 128 or 256
   // K split: ksplit CTAs per output tile, each summing kchunk consecutive
   // 128-value K blocks and OR-ing its bits into C, which starts at zero
   // (Boolean products only; 1 when every tile is summed by one CTA)
   int32_t ksplit, kchunk;
+  int* err;                   // device error word: set when a bounded wait runs out
+  uint32_t* counts;           // when not null: the sums themselves, [nbatch][M][N]
+                              // (counting semiring), and C is not written
 };
-// 32-bit words of the two occupancy bitmaps of a planned problem
-int64_t mma_occ_words(const MmaDesc& d);
-void mma_plan(MmaDesc& d);    // BN, Nw, Kp and the tile counts from M, N, K, nbatch
+void mma_plan(MmaDesc& d);    // BN, Nw and the tile counts from M, N, K, nbatch
 int64_t mma_ctas(const MmaDesc& d);
-size_t mma_smem_bytes();
-// TMA descriptors of Ab and Bb (needs d.Ab, d.Bb set)
-cudaError_t mma_encode_maps(const MmaDesc& d, CUtensorMap* maps2);
-// Expand A and B of every problem of a table into Ab and Bb (two launches;
-// blocks per problem from unpack_blocks_a / _b, the largest over the table).
-int64_t unpack_blocks_a(const MmaDesc& d);
-int64_t unpack_blocks_b(const MmaDesc& d);
-void launch_unpack(const MmaDesc* d_descs, int nprob, int64_t blocks_a, int64_t blocks_b,
-                   cudaStream_t s);
-// Independent problems in one launch: descriptors, two tensor maps per problem
-// and CTA offsets (nprob + 1 entries) on the device.
-cudaError_t launch_mma(const MmaDesc* d_descs, const CUtensorMap* d_maps, const int64_t* d_cta0,
-                       int nprob, int64_t grid, cudaStream_t s);
+bool mma_wants_occ(const MmaDesc& d);      // occupancy bitmaps for this problem?
+int64_t mma_occ_blocks(const MmaDesc& d);  // their bytes, and the blocks that write them
+// Independent problems in one launch, or two when some want occupancy bitmaps
+// (occ_grid > 0): descriptors, CTA offsets and bitmap block offsets (nprob + 1
+// entries each; no blocks for problems without) on the device.
+cudaError_t launch_mma(const MmaDesc* d_descs, const int64_t* d_cta0, const int64_t* d_occ0, int nprob,
+                       int64_t grid, int64_t occ_grid, cudaStream_t s);
 // out[i] = in[src(i)] for a row-major array whose axes are a permutation of
 // the input's: out axis a has extent d_ext[a] and steps d_stride[a] elements
 // of the input (one thread per output element; d_ext and d_stride are DEVICE

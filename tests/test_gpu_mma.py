@@ -135,3 +135,27 @@ def test_autotune_and_auto_path(orc):
     want = orc.solve(sysm.axes, sysm.rels, sysm.exposed).data
     check_same(out, want, sysm.name)
     e.close()
+
+
+@pytest.mark.parametrize("M,K,N", [(1, 128, 64), (127, 129, 128), (129, 100, 129), (130, 640, 257),
+                                   (300, 4200, 200), (257, 4500, 700), (40, 9000, 2100)])
+@pytest.mark.parametrize("kind", ["blocks", "dense"])
+def test_tile_edges(eng, orc, M, K, N, kind):
+    """Rows, columns and K around the tile sizes, odd row pitches, and operands
+    whose 128 x 128 blocks are mostly empty (skipped by the words a CTA has
+    loaded, or by bitmaps where it walks 32 blocks or more); counts too."""
+    rng = np.random.default_rng(9000 + M + K + N)
+    X, Y = rand_bits(rng, (M, K), 0.3), rand_bits(rng, (K, N), 0.3)
+    if kind == "blocks":
+        for a in (X, Y):
+            for i in range(0, a.shape[0], 128):
+                for j in range(0, a.shape[1], 128):
+                    if rng.random() < 0.7:
+                        a[i:i + 128, j:j + 128] = 0
+    vres = [M, K, N]
+    got = eng.contract(pack(X, (0, 1)), pack(Y, (1, 2)), (0, 2))
+    cnt = eng.contract_count(pack(X, (0, 1)), pack(Y, (1, 2)), (0, 2))
+    eng.sync()
+    check_same(got, orc.contract(orc.Arr(X, (0, 1)), orc.Arr(Y, (1, 2)), (0, 2), vres).data, f"{vres}")
+    want = orc.contract_count(orc.Arr(X, (0, 1)), orc.Arr(Y, (1, 2)), (0, 2), vres)
+    assert np.array_equal(cnt.cpu().numpy(), want.astype(np.int64)), f"counts {vres}"
