@@ -20,16 +20,18 @@ struct Mlp {
   float* loss = nullptr;        // device scalar: loss of the last backward()
   int64_t step = 0;
   int cap = 0;                  // samples the activation buffers hold
-  std::vector<float*> acts, pres;
-  float* dbuf0 = nullptr;
-  float* dbuf1 = nullptr;
+  std::vector<float*> acts;     // per hidden layer its output, [l + 1]
+  std::vector<float*> deltas;   // per layer the loss's derivative by its sums
+  float* scratch = nullptr;     // blocks' squared errors [cap], parts of the gradients
 
   Mlp(int nin, int hidden, int nlayers);
   ~Mlp();
   cudaError_t alloc_params();
   cudaError_t reserve(int n);
   void free_acts();
-  // y[n] = net(x[n][nin]) (device pointers; y may be null to keep only acts)
+  // parts the samples of a gradient may be split into (bounded scratch)
+  int max_parts() const;
+  // y[n] = net(x[n][nin]) (device pointers)
   cudaError_t forward(const float* x, int n, float* y, cudaStream_t s);
   // forward, loss 0.5 mean (y - t)^2 into *loss, gradient into g
   cudaError_t backward(const float* x, const float* t, int n, cudaStream_t s);

@@ -169,3 +169,33 @@ def test_learned_batch_matches_greedy_batch(eng):
     for a, b in zip(outs_l, outs_g):
         assert np.array_equal(a.to_numpy(), b.to_numpy())
     m.close()
+
+
+@pytest.mark.parametrize("hidden,nlayers,n", [(1, 1, 1), (5, 2, 3), (33, 8, 600), (100, 1, 609),
+                                              (600, 2, 70), (128, 0, 90), (128, 3, 2433),
+                                              (128, 3, 5000)])
+def test_forward_backward_shapes(eng, hidden, nlayers, n):
+    """Widths that are not multiples of the vector and tile sizes, more units
+    than threads, no hidden layer, and sample counts around the changes of the
+    samples per block and of the split of the gradients; against the oracle in
+    FP64 with the bounds of test_forward_backward_match_oracle."""
+    import torch
+    from oracle import mlp as M
+    m = pa.CostModel(eng, hidden=hidden, nlayers=nlayers, seed=11)
+    rng = np.random.default_rng(hidden + 7 * n)
+    p = (rng.normal(size=m.n_params) * 0.5 / np.sqrt(max(hidden, 16))).astype(np.float32)
+    m.set_params(p)
+    X = rng.normal(size=(n, pa.N_FEATURES)).astype(np.float32)
+    T = rng.normal(size=n).astype(np.float32)
+    xd, td = torch.from_numpy(X).cuda(), torch.from_numpy(T).cuda()
+    y = m.forward(xd).cpu().numpy()
+    y_ref = M.forward(p.astype(np.float64), sizes_of(m), X)
+    assert np.max(np.abs(y - y_ref)) <= 1e-4 * (1 + np.max(np.abs(y_ref)))
+    loss = m.backward(xd, td)
+    g = m.get_grads()
+    L_ref, g_ref = M.loss_and_grad(p.astype(np.float64), sizes_of(m), X, T)
+    assert abs(loss - L_ref) <= 1e-4 * (1 + abs(L_ref))
+    assert np.max(np.abs(g - g_ref)) <= 2e-4 * np.max(np.abs(g_ref)) + 1e-7
+    m.backward(xd, td)
+    assert np.array_equal(g, m.get_grads())
+    m.close()
