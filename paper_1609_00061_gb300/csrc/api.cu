@@ -1086,7 +1086,7 @@ std::vector<BitArr> plot_all(Builder& bd, const std::vector<PlotReq>& reqs) {
   std::vector<PlotReq> poly, corner;
   std::vector<size_t> poly_at, corner_at;
   std::vector<ExprJob> ejobs;
-  std::vector<size_t> prog_off, const_off;
+  std::vector<size_t> prog_off, const_off, c32_off;
   int64_t words = 0;
   for (size_t i = 0; i < reqs.size(); ++i) {
     const pa_relation& r = *reqs[i].rel;
@@ -1133,6 +1133,14 @@ std::vector<BitArr> plot_all(Builder& bd, const std::vector<PlotReq>& reqs) {
     words += a.words();
     prog_off.push_back(bd.put(r.expr->ops, (size_t)r.expr->nops));
     const_off.push_back(bd.put(r.expr->consts, (size_t)r.expr->nconsts));
+    std::vector<float2> c32((size_t)r.expr->nconsts);
+    for (int k = 0; k < r.expr->nconsts; ++k) {
+      const double c = r.expr->consts[k];
+      const float f = (float)c;
+      c32[k] = make_float2((double)f > c ? nextafterf(f, -INFINITY) : f,
+                           (double)f < c ? nextafterf(f, INFINITY) : f);
+    }
+    c32_off.push_back(bd.put(c32.data(), c32.size()));
     ejobs.push_back(J);
     bd.st.pixels_plotted += (double)a.bits();
     bd.st.n_plots++;
@@ -1142,6 +1150,7 @@ std::vector<BitArr> plot_all(Builder& bd, const std::vector<PlotReq>& reqs) {
     for (size_t k = 0; k < ejobs.size(); ++k) {
       ejobs[k].prog = reinterpret_cast<const int32_t*>(bd.dev(prog_off[k]));
       ejobs[k].consts = reinterpret_cast<const double*>(bd.dev(const_off[k]));
+      ejobs[k].c32 = reinterpret_cast<const float2*>(bd.dev(c32_off[k]));
     }
     Op op;
     op.kind = OP_PLOT_EXPR;

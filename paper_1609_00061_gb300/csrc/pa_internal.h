@@ -58,6 +58,7 @@ struct PlotJob {
 struct ExprJob {
   const int32_t* prog;
   const double* consts;
+  const float2* c32;                // per constant an FP32 interval that holds it
   uint64_t* out;
   double lo[kMaxDim];
   double delta[kMaxDim];
@@ -67,8 +68,7 @@ struct ExprJob {
   int32_t res[kMaxDim];
   int32_t port_axis[kMaxDim];
 };
-// Every expression plot of a call in one launch, one thread per pixel (a
-// warp per 32-pixel half of an output word).
+// Every expression plot of a call in one launch.
 void launch_plot_expr(const ExprJob* d_jobs, int njobs, int64_t total_words, cudaStream_t s);
 
 // One relation plotted by the corner rule (pa.h, pa_rule): a polynomial

@@ -254,3 +254,47 @@ def test_butterfly_no_false_negative(eng, orc):
         iw, iz = int((p[0] + 3.0) / d), int((p[3] + 3.0) / d)
         assert got[iw, iz] == 1, p
     assert np.array_equal(got, orc.solve(sy2.axes, sy2.rels, sy2.exposed).data)
+
+
+EDGES = [
+    lambda x, y: tan_(x * 3.0) - y,                        # poles inside runs of pixels
+    lambda x, y: 1.0 / (x - y) - 2.0,                      # a pole along the diagonal
+    lambda x, y: log_(x) * y + sqrt_(y - 0.5) - 0.3,       # undefined for half the box
+    lambda x, y: abs_(x) ** (y * 1.5) - 1.0,               # pow with exponents of both signs
+    lambda x, y: (x - 1.0) ** 3 - (y + 0.25) ** 2,         # odd and even powers over 0
+    lambda x, y: x ** -3 + y ** -2 - 4.0,                  # negative powers over 0
+    lambda x, y: exp_(x * 60.0) - exp_(y * 55.0),          # beyond the FP32 range
+    lambda x, y: exp_(x * 400.0) / exp_(y * 400.0) - 1.0,  # beyond the FP64 range: inf / inf
+    lambda x, y: atan_(1.0 / x) + tanh_(1.0 / y) - 0.4,    # bounded functions of a pole
+    lambda x, y: (log_(x) ** 0) * 0.5 + y,                 # NaN to the power 0
+    lambda x, y: sin_(x * 1e5) * cos_(y * 40.0) - 0.2,     # fast oscillation
+    lambda x, y: cosh_(x * 3.0) - sinh_(y * 3.0) - 2.0,
+]
+
+
+@pytest.mark.parametrize("case", range(len(EDGES)))
+@pytest.mark.parametrize("kind", [W.KIND_EQ, W.KIND_LE, W.KIND_LT])
+def test_runs_of_pixels(eng, orc, case, kind):
+    """Grids on which whole words and 8-pixel pieces are decided by intervals:
+    poles, domain edges, overflow and both signs inside them."""
+    x, y = Ex.port(0), Ex.port(1)
+    for axes in ([(-2.0, 2.0, 130), (-2.0, 2.0, 700)], [(-1.0, 3.0, 64), (-3.0, 1.0, 333)]):
+        for eps in (0.02, 0.5, 3.0):
+            rel = W.expr_relation((0, 1), EDGES[case](x, y), kind=kind, eps=eps)
+            got = eng.plot(rel, axes)
+            eng.sync()
+            check_plot_band(orc, rel, axes, got, f"case {case} eps {eps}")
+
+
+@pytest.mark.parametrize("seed", range(12))
+def test_random_expressions_fine(eng, orc, seed):
+    """Random programs on fine last axes (ragged and whole words)."""
+    rng = np.random.default_rng(9700 + seed)
+    arity = 2 + seed % 2
+    res = [40, 600] if arity == 2 else [9, 13, 515]
+    axes = [(-2.5, 2.0, r) for r in res]
+    e = random_expr(rng, arity, 4)
+    rel = W.expr_relation(tuple(range(arity)), e, kind=seed % 3, eps=float(rng.choice([0.01, 0.3])))
+    got = eng.plot(rel, axes)
+    eng.sync()
+    check_plot_band(orc, rel, axes, got, f"seed {seed}")
