@@ -30,11 +30,7 @@ struct RsCtx {
 };
 __device__ __forceinline__ RsCtx rs_pick(const ReshapeDesc* __restrict__ descs,
                                          const int64_t* __restrict__ cta0, int n, ReshapeDesc* sd) {
-  int lo = 0, hi = n - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (cta0[mid] <= (int64_t)blockIdx.x) lo = mid; else hi = mid - 1;
-  }
+  const int lo = find_entry([&](int i) { return cta0[i]; }, n, (int64_t)blockIdx.x);
   const int64_t* src = reinterpret_cast<const int64_t*>(descs + lo);
   int64_t* dst = reinterpret_cast<int64_t*>(sd);
   for (int i = threadIdx.x; i < (int)(sizeof(ReshapeDesc) / 8); i += blockDim.x) dst[i] = src[i];
@@ -46,12 +42,75 @@ __device__ __forceinline__ RsCtx rs_pick(const ReshapeDesc* __restrict__ descs,
 // 64 bits).  Every bit is decoded and gathered on its own, OR-ed over the
 // reduced axes with an early exit.  With row_any set, every packed input axis
 // is reduced and red_* hold only the reduced row axes: a bit is then the OR of
-// whole input rows, scanned by words (padding bits are zero).
+// whole input rows, scanned by words (padding bits are zero).  When those rows
+// are long together (kAnyScan words or more per bit) a block takes an output
+// word and its warps one bit after another, a bit's words dealt over the lanes:
+// a lane scanning them alone is a chain of as many loads.
+constexpr int64_t kAnyScan = 64;
+__device__ void any_rows(const ReshapeDesc& d, int64_t bid, int64_t nblk) {
+  __shared__ uint32_t s_bits[2];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const int64_t total = d.out_nrows * d.out_row_words;
+  const int outer = d.out_ndim - d.out_inner;
+  int64_t red_total = 1;
+  for (int q = 0; q < d.nred; ++q) red_total *= d.red_res[q];
+  const int64_t scan = red_total * d.in_row_words;
+  for (int64_t ow = bid; ow < total; ow += nblk) {
+    if (threadIdx.x < 2) s_bits[threadIdx.x] = 0;
+    __syncthreads();
+    const int64_t orow = ow / d.out_row_words, w = ow % d.out_row_words;
+    int64_t brow = 0, rest = orow;
+    for (int a = outer - 1; a >= 0; --a) {
+      brow += rest % d.out_res[a] * d.row_stride[a];
+      rest /= d.out_res[a];
+    }
+    for (int bit = warp; bit < 64; bit += nwarps) {
+      const int64_t ocol = w * 64 + bit;
+      if (ocol >= d.out_rowlen) break;
+      int64_t row = brow, rest2 = ocol;
+      for (int a = d.out_ndim - 1; a >= outer; --a) {
+        row += rest2 % d.out_res[a] * d.row_stride[a];
+        rest2 /= d.out_res[a];
+      }
+      bool any = false;
+      for (int64_t s0 = 0; s0 < scan && !any; s0 += 32) {
+        const int64_t s = s0 + lane;
+        uint64_t v = 0;
+        if (s < scan) {
+          int64_t r = row, srest = s / d.in_row_words;
+          const int64_t k = s - srest * d.in_row_words;
+          for (int q = d.nred - 1; q >= 0; --q) {
+            r += srest % d.red_res[q] * d.red_row_stride[q];
+            srest /= d.red_res[q];
+          }
+          v = __ldg(d.in + r * d.in_row_words + k);
+        }
+        any = __any_sync(0xffffffffu, v != 0ull);
+      }
+      if (any && lane == 0) atomicOr(&s_bits[bit >> 5], 1u << (bit & 31));
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) d.out[ow] = (uint64_t)s_bits[0] | ((uint64_t)s_bits[1] << 32);
+    __syncthreads();
+  }
+}
+
+// Words scanned per output bit of a row_any reshape.
+__host__ __device__ __forceinline__ int64_t any_scan(const ReshapeDesc& d) {
+  int64_t n = d.in_row_words;
+  for (int q = 0; q < d.nred; ++q) n *= d.red_res[q];
+  return n;
+}
+
 __global__ void reshape_kernel(const ReshapeDesc* __restrict__ descs, const int64_t* __restrict__ cta0,
                                int n) {
   __shared__ ReshapeDesc sd;
   const RsCtx rc = rs_pick(descs, cta0, n, &sd);
   const ReshapeDesc& d = sd;
+  if (d.row_any && any_scan(d) >= kAnyScan) {
+    any_rows(d, rc.bid, rc.nblk);
+    return;
+  }
   const int lane = threadIdx.x & 31;
   const int64_t total = d.out_nrows * d.out_row_words;
   const int outer = d.out_ndim - d.out_inner;
@@ -107,97 +166,161 @@ __global__ void reshape_kernel(const ReshapeDesc* __restrict__ descs, const int6
 }
 
 // Words mode: output word index -> input word index through the mixed-radix
-// decomposition (u_res, u_in), then an OR over the reduced axes.  Index type I
-// is 32-bit when every word index fits.
-template <class I>
-__global__ void reshape_words_kernel(const ReshapeDesc* __restrict__ descs,
-                                     const int64_t* __restrict__ cta0, int n) {
-  __shared__ ReshapeDesc sd;
-  const RsCtx rc = rs_pick(descs, cta0, n, &sd);
-  const ReshapeDesc& d = sd;
-  const I total = (I)(d.out_nrows * d.out_row_words);
-  I red_total = 1;
-  for (int q = 0; q < d.nred; ++q) red_total *= (I)d.red_res[q];
-  auto src_of = [&](I ow) -> I {
-    I rest = ow, src = 0;
-    for (int a = d.nu - 1; a >= 0; --a) {
-      const I r = (I)d.u_res[a];
-      const I q = rest / r;
+// decomposition (u_res, u_in), then an OR over the reduced axes.  A thread takes
+// V = 4, 2 or 1 consecutive words (the last axis runs along the words of both
+// sides), which spreads the divisions of the decomposition over them; a
+// reduction over many values with few output words is dealt over the lanes of a
+// warp.  Index type I is 32-bit when every word index fits.  Bound by HBM and the
+// index arithmetic: 38 networks' word reshapes 0.96 -> 0.28 ms, a reduction of
+// 75^2 values into 2 words each 47 -> 6 us (ncu, cold; a thread per word before).
+template <int V>
+struct WordRun {
+  uint64_t v[V];
+};
+template <int V>
+__device__ __forceinline__ WordRun<V> load_run(const uint64_t* __restrict__ p) {
+  WordRun<V> r;
+  if constexpr (V == 1) {
+    r.v[0] = *p;
+  } else {
+#pragma unroll
+    for (int k = 0; k < V; k += 2) {
+      const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(p + k);
+      r.v[k] = t.x;
+      r.v[k + 1] = t.y;
+    }
+  }
+  return r;
+}
+template <int V>
+__device__ __forceinline__ void store_run(uint64_t* p, const WordRun<V>& r) {
+  if constexpr (V == 1) {
+    *p = r.v[0];
+  } else {
+#pragma unroll
+    for (int k = 0; k < V; k += 2)
+      *reinterpret_cast<ulonglong2*>(p + k) = make_ulonglong2(r.v[k], r.v[k + 1]);
+  }
+}
+
+template <class I, int V>
+__device__ __forceinline__ void reshape_words(const ReshapeDesc& d, I bid, I nblk) {
+  const I units = (I)(d.out_nrows * d.out_row_words) / V;
+  const int last = d.nu - 1;
+  auto src_of = [&](I u) -> I {
+    I r = (I)d.u_res[last] / V;
+    I q = u / r;
+    I src = (u - q * r) * V;  // (u_in[last] is 1)
+    I rest = q;
+    for (int a = last - 1; a >= 0; --a) {
+      r = (I)d.u_res[a];
+      q = rest / r;
       src += (rest - q * r) * (I)d.u_in[a];
       rest = q;
     }
     return src;
   };
+  I red_total = 1;
+  for (int q = 0; q < d.nred; ++q) red_total *= (I)d.red_res[q];
+  const I gid = bid * blockDim.x + threadIdx.x, gthreads = nblk * blockDim.x;
   if (red_total == 1) {
-    // a pure permutation of words: four loads in flight per thread
-    const I stride = (I)rc.nblk * blockDim.x;
-    I ow = (I)rc.bid * blockDim.x + threadIdx.x;
-    for (; ow + 3 * stride < total; ow += 4 * stride) {
-      uint64_t v[4];
+    // a pure permutation: 4 words in flight per thread
+    constexpr int U = 4 / V;
+    I u = gid;
+    for (; u + (U - 1) * gthreads < units; u += U * gthreads) {
+      WordRun<V> v[U];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) v[k] = d.in[src_of(ow + (I)k * stride)];
+      for (int k = 0; k < U; ++k) v[k] = load_run<V>(d.in + src_of(u + (I)k * gthreads));
 #pragma unroll
-      for (int k = 0; k < 4; ++k) d.out[ow + (I)k * stride] = v[k];
+      for (int k = 0; k < U; ++k) store_run<V>(d.out + (u + (I)k * gthreads) * V, v[k]);
     }
-    for (; ow < total; ow += stride) d.out[ow] = d.in[src_of(ow)];
+    for (; u < units; u += gthreads) store_run<V>(d.out + u * V, load_run<V>(d.in + src_of(u)));
     return;
   }
-  for (I ow = (I)rc.bid * blockDim.x + threadIdx.x; ow < total; ow += (I)rc.nblk * blockDim.x) {
-    I rest = ow, src = 0;
-    for (int a = d.nu - 1; a >= 0; --a) {
-      const I r = (I)d.u_res[a];
-      const I q = rest / r;
-      src += (rest - q * r) * (I)d.u_in[a];
-      rest = q;
-    }
-    uint64_t word = 0;
-    I cnt[2 * kMaxDim] = {};
-    for (I s = 0; s < red_total; ++s) {
-      word |= d.in[src];
-      for (int q = d.nred - 1; q >= 0; --q) {
-        src += (I)d.red_in_w[q];
-        if (++cnt[q] < (I)d.red_res[q]) break;
-        src -= (I)d.red_in_w[q] * (I)d.red_res[q];
-        cnt[q] = 0;
+  // lanes per unit: a power of two, as long as there are values and idle threads
+  int g = 1;
+  while (g < 32 && (I)(2 * g) <= red_total && units * (I)(2 * g) <= (I)(152 * 2048)) g *= 2;
+  const int sub = threadIdx.x & (g - 1);
+  // (whole warps run the loop: the lanes of a unit combine with shuffles)
+  const I uend = (units + 32 / g - 1) / (32 / g) * (32 / g);
+  for (I u = gid / g; u < uend; u += gthreads / g) {
+    WordRun<V> acc;
+#pragma unroll
+    for (int k = 0; k < V; ++k) acc.v[k] = 0;
+    if (u < units) {
+      const I src = src_of(u);
+#pragma unroll 4
+      for (I s = sub; s < red_total; s += g) {
+        I at = src, rest = s;
+        for (int q = d.nred - 1; q > 0; --q) {
+          const I r = (I)d.red_res[q], t = rest / r;
+          at += (rest - t * r) * (I)d.red_in_w[q];
+          rest = t;
+        }
+        at += rest * (I)d.red_in_w[0];
+        const WordRun<V> v = load_run<V>(d.in + at);
+#pragma unroll
+        for (int k = 0; k < V; ++k) acc.v[k] |= v.v[k];
       }
     }
-    d.out[ow] = word;
+    for (int o = 1; o < g; o <<= 1)
+#pragma unroll
+      for (int k = 0; k < V; ++k) acc.v[k] |= __shfl_xor_sync(0xffffffffu, acc.v[k], o);
+    if (u < units && sub == 0) store_run<V>(d.out + u * V, acc);
   }
 }
 
-// In-register transpose of a 64 x 64 bit block held by one warp: lane l holds
-// rows l (lo) and l + 32 (hi), bit c of a row being column c.  Afterwards lane l
-// holds columns l and l + 32 as rows.  Recursive block swap (halves, quarters,
-// ... single bits): for block size s the rows r and r + s (r & s == 0) exchange
-// the columns c + s of row r with the columns c of row r + s (c & s == 0).
-__device__ __forceinline__ void transpose64(uint64_t& lo, uint64_t& hi, int lane) {
-  uint64_t t = ((lo >> 32) ^ hi) & 0x00000000FFFFFFFFull;
-  hi ^= t;
-  lo ^= t << 32;
-  const uint64_t masks[5] = {0x0000FFFF0000FFFFull, 0x00FF00FF00FF00FFull, 0x0F0F0F0F0F0F0F0Full,
-                             0x3333333333333333ull, 0x5555555555555555ull};
+template <class I>
+__global__ void __launch_bounds__(256)
+reshape_words_kernel(const ReshapeDesc* __restrict__ descs, const int64_t* __restrict__ cta0, int n) {
+  __shared__ ReshapeDesc sd;
+  const RsCtx rc = rs_pick(descs, cta0, n, &sd);
+  const ReshapeDesc& d = sd;
+  const bool aligned = ((reinterpret_cast<uintptr_t>(d.in) | reinterpret_cast<uintptr_t>(d.out)) & 15) == 0;
+  if (d.vec == 4 && aligned) reshape_words<I, 4>(d, (I)rc.bid, (I)rc.nblk);
+  else if (d.vec >= 2 && aligned) reshape_words<I, 2>(d, (I)rc.bid, (I)rc.nblk);
+  else reshape_words<I, 1>(d, (I)rc.bid, (I)rc.nblk);
+}
+
+// In-register transpose of 32 x 32 bit blocks held by one warp: lane l holds row
+// l; afterwards column l.  Recursive block swap: for block size s the rows r and
+// r + s (r & s == 0) exchange the columns c + s of row r with the columns c of
+// row r + s (c & s == 0).  Each step is one shuffle, one rotation and one select:
+// a lane keeps the columns of `keep` and takes the others from its partner's
+// row, rotated by s (rows without s) or back (rows with s); no kept column wraps.
+struct Transpose32 {
+  uint32_t keep[5];
+  uint32_t rot[5];
+  __device__ __forceinline__ explicit Transpose32(int lane) {
+    const uint32_t masks[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
 #pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    const int s = 16 >> i;
-    const uint64_t m = masks[i];
-    const uint64_t plo = __shfl_xor_sync(0xffffffffu, lo, s);
-    const uint64_t phi = __shfl_xor_sync(0xffffffffu, hi, s);
-    if (lane & s) {
-      lo ^= ((plo >> s) ^ lo) & m;
-      hi ^= ((phi >> s) ^ hi) & m;
-    } else {
-      lo ^= (((lo >> s) ^ plo) & m) << s;
-      hi ^= (((hi >> s) ^ phi) & m) << s;
+    for (int i = 0; i < 5; ++i) {
+      const int s = 16 >> i;
+      keep[i] = (lane & s) ? ~masks[i] : masks[i];
+      rot[i] = (lane & s) ? 32 - s : s;
     }
   }
-}
+  __device__ __forceinline__ uint32_t operator()(uint32_t x) const {
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+      const uint32_t y = __shfl_xor_sync(0xffffffffu, x, 16 >> i);
+      x = (x & keep[i]) | (__funnelshift_l(y, y, rot[i]) & ~keep[i]);
+    }
+    return x;
+  }
+};
 
 // Transpose mode.  A CTA tile is 256 values of L (4 output words) x 256 values
 // of J (4 input words) at one value of the other axes: coalesced 32-byte loads
-// of 256 input rows into shared memory, 16 warp transposes of 64 x 64 blocks,
+// of 256 input rows into shared memory, 64 warp transposes of 32 x 32 blocks,
 // coalesced 32-byte stores of 256 output rows.  Rows of the shared tiles are
-// padded to 5 words so the column reads of a block are free of bank conflicts.
+// padded to 5 words.
+// Index type I is 32-bit when every word and tile index fits.  Bound by the
+// latency of 32-byte accesses at the arrays' pitches (1.7 TB/s); 64-bit divisions
+// (two thirds of 8570 warp instructions per tile) and branching 64 x 64 block
+// transposes bound it before: 38 networks' transposes 1.88 -> 1.28 ms.
 constexpr int kTrPad = 5;
+template <class I>
 __global__ void __launch_bounds__(256)
 reshape_transpose_kernel(const ReshapeDesc* __restrict__ descs, const int64_t* __restrict__ cta0, int n) {
   __shared__ ReshapeDesc sd;
@@ -206,102 +329,119 @@ reshape_transpose_kernel(const ReshapeDesc* __restrict__ descs, const int64_t* _
   __shared__ uint64_t s_in[256 * kTrPad];
   __shared__ uint64_t s_out[256 * kTrPad];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t nJT = (d.tQ + 255) / 256, nLT = (d.tR + 255) / 256;
-  const int64_t tiles = d.n_other * nJT * nLT;
+  const Transpose32 tr(lane);
+  const I tQ = (I)d.tQ, tR = (I)d.tR, t_in_L = (I)d.t_in_L, t_out_J = (I)d.t_out_J;
+  const I nJT = (tQ + 255) / 256, nLT = (tR + 255) / 256;
+  const I tiles = (I)d.n_other * nJT * nLT;
+  const I nblk = (I)rc.nblk;
   // tile -> (L tile, J tile, first input and output word of its other axes)
-  auto locate = [&](int64_t tile, int64_t& lt, int64_t& jt, int64_t& base_in, int64_t& base_out) {
-    lt = tile % nLT;
-    const int64_t r = tile / nLT;
-    jt = r % nJT;
-    int64_t rest = r / nJT;
+  auto locate = [&](I tile, I& lt, I& jt, I& base_in, I& base_out) {
+    const I r = tile / nLT;
+    lt = tile - r * nLT;
+    I rest = r / nJT;
+    jt = r - rest * nJT;
     base_in = 0;
     base_out = 0;
     for (int a = d.nu - 1; a >= 0; --a) {
-      const int64_t v = rest % d.u_res[a];
-      rest /= d.u_res[a];
-      base_in += v * d.u_in[a];
-      base_out += v * d.u_out[a];
+      const I res = (I)d.u_res[a], q = rest / res, v = rest - q * res;
+      rest = q;
+      base_in += v * (I)d.u_in[a];
+      base_out += v * (I)d.u_out[a];
     }
   };
   // the four input words this thread loads for a tile
-  auto load = [&](int64_t lt, int64_t jt, int64_t base_in, uint64_t* v) {
+  auto load = [&](I lt, I jt, I base_in, uint64_t* v) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int idx = tid + 256 * i, b = idx >> 2, c = idx & 3;
-      const int64_t L = lt * 256 + b, jb = jt * 4 + c;
-      v[i] = (L < d.tR && jb * 64 < d.tQ) ? d.in[base_in + L * d.t_in_L + jb] : 0ull;
+      const I L = lt * 256 + b, jb = jt * 4 + c;
+      v[i] = (L < tR && jb * 64 < tQ) ? d.in[base_in + L * t_in_L + jb] : 0ull;
     }
   };
   // the next tile's loads are issued before the current tile is transposed
   // and stored, so that their latency overlaps that work
-  int64_t lt = 0, jt = 0, base_in = 0, base_out = 0;
+  I lt = 0, jt = 0, base_in = 0, base_out = 0;
   uint64_t nv[4] = {0, 0, 0, 0};
-  if (rc.bid < tiles) {
-    locate(rc.bid, lt, jt, base_in, base_out);
+  if ((I)rc.bid < tiles) {
+    locate((I)rc.bid, lt, jt, base_in, base_out);
     load(lt, jt, base_in, nv);
   }
-  for (int64_t tile = rc.bid; tile < tiles; tile += rc.nblk) {
+  for (I tile = (I)rc.bid; tile < tiles; tile += nblk) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int idx = tid + 256 * i, b = idx >> 2, c = idx & 3;
       s_in[b * kTrPad + c] = nv[i];
     }
-    const int64_t clt = lt, cjt = jt, cbase_out = base_out;
-    if (tile + rc.nblk < tiles) {
-      locate(tile + rc.nblk, lt, jt, base_in, base_out);
+    const I clt = lt, cjt = jt, cbase_out = base_out;
+    if (tile + nblk < tiles) {
+      locate(tile + nblk, lt, jt, base_in, base_out);
       load(lt, jt, base_in, nv);
     }
     __syncthreads();
+    // warp w: the 32 columns w of J, all eight 32-row blocks of L
+    if ((cjt * 8 + warp) * 32 < tQ) {
+      const uint32_t* in32 = reinterpret_cast<const uint32_t*>(s_in) + lane * (2 * kTrPad) + warp;
+      uint32_t* out32 = reinterpret_cast<uint32_t*>(s_out) + (warp * 32 + lane) * (2 * kTrPad);
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int k = warp * 2 + i, cw = k >> 2, lw = k & 3;
-      if ((cjt * 4 + cw) * 64 < d.tQ && clt * 256 + lw * 64 < d.tR) {
-        uint64_t lo = s_in[(lw * 64 + lane) * kTrPad + cw];
-        uint64_t hi = s_in[(lw * 64 + lane + 32) * kTrPad + cw];
-        transpose64(lo, hi, lane);
-        s_out[(cw * 64 + lane) * kTrPad + lw] = lo;
-        s_out[(cw * 64 + lane + 32) * kTrPad + lw] = hi;
-      }
+      for (int i = 0; i < 8; ++i) out32[i] = tr(in32[i * 32 * (2 * kTrPad)]);
     }
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int idx = tid + 256 * i, t = idx >> 2, w = idx & 3;
-      const int64_t J = cjt * 256 + t, lw = clt * 4 + w;
-      if (J < d.tQ && lw * 64 < d.tR) d.out[cbase_out + J * d.t_out_J + lw] = s_out[t * kTrPad + w];
+      const I J = cjt * 256 + t, lw = clt * 4 + w;
+      if (J < tQ && lw * 64 < tR) d.out[cbase_out + J * t_out_J + lw] = s_out[t * kTrPad + w];
     }
     __syncthreads();
   }
 }
 
+constexpr int64_t kMaxReshapeBlocks = 152 * 16;
+
 int reshape_kind(const ReshapeDesc& d) {
-  if (d.mode == kReshapeTranspose) return kRsTranspose;
-  if (d.mode == kReshapeWords) {
-    const int64_t total = d.out_nrows * d.out_row_words;
-    const int64_t blocks = reshape_blocks(d);
-    int64_t in_max = 0;  // largest input word index + 1 (bounded by the sum below)
-    for (int a = 0; a < d.nu; ++a) in_max += (d.u_res[a] - 1) * d.u_in[a];
-    for (int q = 0; q < d.nred; ++q) in_max += (d.red_res[q] - 1) * d.red_in_w[q];
-    return (total + 256 * blocks < (1ll << 31) && in_max < (1ll << 31)) ? kRsWords32 : kRsWords64;
+  if (d.mode == kReshapeBits) return kRsBits;
+  const int64_t total = d.out_nrows * d.out_row_words, blocks = kMaxReshapeBlocks;
+  int64_t in_max = 0;  // largest input word index + 1 (bounded by the sums below)
+  for (int a = 0; a < d.nu; ++a) in_max += (d.u_res[a] - 1) * d.u_in[a];
+  if (d.mode == kReshapeTranspose) {
+    in_max += (d.tR + 255) * d.t_in_L + d.tQ / 64 + 4;
+    const int64_t tiles = d.n_other * ((d.tQ + 255) / 256) * ((d.tR + 255) / 256);
+    return (in_max < (1ll << 31) && total < (1ll << 31) && tiles + blocks < (1ll << 31)) ? kRsTranspose32
+                                                                                        : kRsTranspose64;
   }
-  return kRsBits;
+  for (int q = 0; q < d.nred; ++q) in_max += (d.red_res[q] - 1) * d.red_in_w[q];
+  return (total + 1024 * blocks < (1ll << 31) && in_max < (1ll << 31)) ? kRsWords32 : kRsWords64;
 }
 
-int64_t reshape_blocks(const ReshapeDesc& d) {
+int64_t reshape_units(const ReshapeDesc& d) {
   const int64_t total = d.out_nrows * d.out_row_words;
   if (total <= 0) return 0;
-  if (d.mode == kReshapeTranspose)
-    return std::min<int64_t>(d.n_other * ((d.tQ + 255) / 256) * ((d.tR + 255) / 256), 152 * 8);
-  if (d.mode == kReshapeWords) return std::min<int64_t>((total + 255) / 256, 152 * 16);
-  return std::min<int64_t>((total + 7) / 8, 152 * 16);  // one warp per word
+  if (d.mode == kReshapeTranspose) return d.n_other * ((d.tQ + 255) / 256) * ((d.tR + 255) / 256);
+  if (d.mode == kReshapeWords) {
+    // a thread per run of words, or more for a reduction (see the kernel)
+    int64_t red = 1;
+    for (int q = 0; q < d.nred; ++q) red *= d.red_res[q];
+    const int64_t threads = total / d.vec * std::min<int64_t>(32, red);
+    return (threads + 255) / 256;
+  }
+  if (d.row_any && any_scan(d) >= kAnyScan) return total;
+  return (total + 7) / 8;  // one warp per word
+}
+
+int64_t reshape_blocks(const ReshapeDesc& d, int64_t per) {
+  const int64_t n = reshape_units(d);
+  return n <= 0 ? 0 : std::min<int64_t>((n + per - 1) / per, kMaxReshapeBlocks);
 }
 
 void launch_reshape(const ReshapeDesc* d_descs, const int64_t* d_cta0, int n, int kind,
                     int64_t grid, cudaStream_t s) {
   if (n <= 0 || grid <= 0) return;
   switch (kind) {
-    case kRsTranspose:
-      reshape_transpose_kernel<<<(unsigned)grid, 256, 0, s>>>(d_descs, d_cta0, n);
+    case kRsTranspose32:
+      reshape_transpose_kernel<uint32_t><<<(unsigned)grid, 256, 0, s>>>(d_descs, d_cta0, n);
+      break;
+    case kRsTranspose64:
+      reshape_transpose_kernel<uint64_t><<<(unsigned)grid, 256, 0, s>>>(d_descs, d_cta0, n);
       break;
     case kRsWords32:
       reshape_words_kernel<uint32_t><<<(unsigned)grid, 256, 0, s>>>(d_descs, d_cta0, n);
@@ -321,43 +461,62 @@ constexpr int64_t kDotRun = 256;
 // ------------------------------------------- outer / dot / and, batched
 // Every such cluster of one tree level in one launch: job p owns blocks
 // [cta0[p], cta0[p+1]) and runs the loop of its kind over them.
+// Index type I is 32-bit when every word and row index of the launch's jobs
+// fits (a 64-bit division is 100 instructions, and an outer product's element
+// takes two: 38 networks 0.73 -> 0.54 ms).
+template <class I>
 __global__ void __launch_bounds__(256)
 ewise_kernel(const EwJob* __restrict__ jobs, const int64_t* __restrict__ cta0, int n) {
-  int lo = 0, hi = n - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (cta0[mid] <= (int64_t)blockIdx.x) lo = mid; else hi = mid - 1;
-  }
+  const int lo = find_entry([&](int k) { return cta0[k]; }, n, (int64_t)blockIdx.x);
   const EwJob& j = jobs[lo];
-  const int64_t bid = (int64_t)blockIdx.x - cta0[lo], nblk = cta0[lo + 1] - cta0[lo];
+  const I bid = (I)((int64_t)blockIdx.x - cta0[lo]), nblk = (I)(cta0[lo + 1] - cta0[lo]);
   const int lane = threadIdx.x & 31;
-  const int64_t gwarp = bid * (blockDim.x >> 5) + (threadIdx.x >> 5), nwarps = nblk * (blockDim.x >> 5);
+  const I gwarp = bid * (blockDim.x >> 5) + (threadIdx.x >> 5), nwarps = nblk * (blockDim.x >> 5);
+  const I rows = (I)j.rows, m = (I)j.m, nw = (I)j.nw;
   const uint64_t* __restrict__ A = j.a;
   const uint64_t* __restrict__ B = j.b;
   uint64_t* __restrict__ C = j.c;
-  if (j.kind == kEwAnd) {
-    for (int64_t i = bid * blockDim.x + threadIdx.x; i < j.rows; i += nblk * blockDim.x) C[i] = A[i] & B[i];
-  } else if (j.kind == kEwOuter) {
-    // C[r][w] = bit r of A ? B[r / M][w] : 0
-    const int64_t total = j.rows * j.nw;
-    for (int64_t i = bid * blockDim.x + threadIdx.x; i < total; i += nblk * blockDim.x) {
-      const int64_t r = i / j.nw, w = i - r * j.nw;
-      const uint64_t bit = (A[r >> 6] >> (r & 63)) & 1ull;
-      C[i] = bit ? B[(r / j.m) * j.nw + w] : 0ull;
+  const int kind = j.kind;
+  if (kind == kEwAnd) {
+    // two words at a time, four loads in flight, where the arrays allow it
+    const bool vec = ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B) |
+                       reinterpret_cast<uintptr_t>(C)) & 15) == 0;
+    const I pairs = vec ? rows / 2 : 0;
+    const ulonglong2* A2 = reinterpret_cast<const ulonglong2*>(A);
+    const ulonglong2* B2 = reinterpret_cast<const ulonglong2*>(B);
+    ulonglong2* C2 = reinterpret_cast<ulonglong2*>(C);
+    const I step = nblk * blockDim.x;
+    for (I i = bid * blockDim.x + threadIdx.x; i < pairs; i += step) {
+      const ulonglong2 a = A2[i], b = B2[i];
+      C2[i] = make_ulonglong2(a.x & b.x, a.y & b.y);
     }
-  } else if (j.kind == kEwDot) {
+    for (I i = 2 * pairs + bid * blockDim.x + threadIdx.x; i < rows; i += step) C[i] = A[i] & B[i];
+  } else if (kind == kEwOuter) {
+    // C[r][w] = bit r of A ? B[r / M][w] : 0
+    const I total = rows * nw;
+    for (I i = bid * blockDim.x + threadIdx.x; i < total; i += nblk * blockDim.x) {
+      const I r = i / nw, w = i - r * nw;
+      const uint64_t bit = (A[r >> 6] >> (r & 63)) & 1ull;
+      C[i] = bit ? B[(r / m) * nw + w] : 0ull;
+    }
+  } else if (kind == kEwDot) {
     // one warp per word of C: lanes take bits r and r + 32
-    const int64_t words = (j.rows + 63) / 64;
-    for (int64_t cw = gwarp; cw < words; cw += nwarps) {
+    const I words = (rows + 63) / 64;
+    for (I cw = gwarp; cw < words; cw += nwarps) {
       uint32_t half[2];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const int64_t r = cw * 64 + h * 32 + lane;
+        const I r = cw * 64 + h * 32 + lane;
         uint64_t acc = 0;
-        if (r < j.rows) {
-          const uint64_t* a = A + r * j.nw;
-          const uint64_t* b = B + (r / j.m) * j.nw;
-          for (int64_t w = 0; w < j.nw && !acc; ++w) acc = a[w] & b[w];
+        if (r < rows) {
+          const uint64_t* a = A + r * nw;
+          const uint64_t* b = B + (r / m) * nw;
+          // (four words at a time: the loads of a run are in flight together)
+          for (I w = 0; w < nw && !acc; w += 4) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              if (w + k < nw) acc |= a[w + k] & b[w + k];
+          }
         }
         half[h] = __ballot_sync(0xffffffffu, acc != 0);
       }
@@ -365,15 +524,15 @@ ewise_kernel(const EwJob* __restrict__ jobs, const int64_t* __restrict__ cta0, i
     }
   } else {
     // long rows: one warp per (row, run of 256 words) into the cleared C
-    const int64_t nruns = (j.nw + kDotRun - 1) / kDotRun;
-    const int64_t items = j.rows * nruns;
-    for (int64_t it = gwarp; it < items; it += nwarps) {
-      const int64_t r = it / nruns, w0 = (it - r * nruns) * kDotRun;
-      const int64_t w1 = min(j.nw, w0 + kDotRun);
-      const uint64_t* a = A + r * j.nw;
-      const uint64_t* b = B + (r / j.m) * j.nw;
+    const I nruns = (nw + (I)kDotRun - 1) / (I)kDotRun;
+    const I items = rows * nruns;
+    for (I it = gwarp; it < items; it += nwarps) {
+      const I r = it / nruns, w0 = (it - r * nruns) * (I)kDotRun;
+      const I w1 = min(nw, w0 + (I)kDotRun);
+      const uint64_t* a = A + r * nw;
+      const uint64_t* b = B + (r / m) * nw;
       uint64_t acc = 0;
-      for (int64_t w = w0 + lane; w < w1; w += 32) acc |= a[w] & b[w];
+      for (I w = w0 + lane; w < w1; w += 32) acc |= a[w] & b[w];
       if (__any_sync(0xffffffffu, acc != 0) && lane == 0)
         atomicOr(reinterpret_cast<unsigned long long*>(&C[r >> 6]), 1ull << (r & 63));
     }
@@ -383,7 +542,7 @@ ewise_kernel(const EwJob* __restrict__ jobs, const int64_t* __restrict__ cta0, i
 int64_t ewise_blocks(const EwJob& j) {
   int64_t items;
   switch (j.kind) {
-    case kEwAnd: items = (j.rows + 255) / 256; break;
+    case kEwAnd: items = (j.rows / 2 + 255) / 256 + 1; break;
     case kEwOuter: items = (j.rows * j.nw + 255) / 256; break;
     case kEwDot: items = ((j.rows + 63) / 64 + 7) / 8; break;
     default: items = (j.rows * ((j.nw + kDotRun - 1) / kDotRun) + 7) / 8; break;
@@ -391,9 +550,16 @@ int64_t ewise_blocks(const EwJob& j) {
   return std::min<int64_t>(items, 152 * 16);
 }
 
-void launch_ewise(const EwJob* d_jobs, const int64_t* d_cta0, int n, int64_t grid, cudaStream_t s) {
+bool ewise_fits32(const EwJob& j) {
+  // (word indexes of every array, and a grid-stride past the end)
+  return j.rows * std::max<int64_t>(1, j.nw) < (1ll << 31) - (1ll << 24) && j.m < (1ll << 31);
+}
+
+void launch_ewise(const EwJob* d_jobs, const int64_t* d_cta0, int n, int64_t grid, bool wide,
+                  cudaStream_t s) {
   if (n <= 0 || grid <= 0) return;
-  ewise_kernel<<<(unsigned)grid, 256, 0, s>>>(d_jobs, d_cta0, n);
+  if (wide) ewise_kernel<uint64_t><<<(unsigned)grid, 256, 0, s>>>(d_jobs, d_cta0, n);
+  else ewise_kernel<uint32_t><<<(unsigned)grid, 256, 0, s>>>(d_jobs, d_cta0, n);
 }
 
 // ---------------------------------------------------------------- row-OR
@@ -687,18 +853,7 @@ rowor_kernel(const RowOrDesc* __restrict__ descs, const CUtensorMap* __restrict_
   asm volatile("griddepcontrol.launch_dependents;");
   const int tid = threadIdx.x;
   {
-    // the last problem whose first CTA is at most this one: every thread
-    // compares one of an evenly spaced sample, then the gap is searched the
-    // same way (a binary search is a chain of L2 latencies)
-    int lo = 0, n = nprob;
-    while (n > 1) {
-      const int step = (n + (int)blockDim.x - 1) / (int)blockDim.x;
-      const int64_t at = (int64_t)tid * step;
-      const int below = at < n && cta0s[lo + at] <= (int64_t)blockIdx.x;
-      const int first = (__syncthreads_count(below) - 1) * step;
-      lo += first;
-      n = min(step, n - first);
-    }
+    const int lo = find_entry([&](int i) { return cta0s[i]; }, nprob, (int64_t)blockIdx.x);
     const uint32_t* src = reinterpret_cast<const uint32_t*>(descs + lo);
     uint32_t* dst = reinterpret_cast<uint32_t*>(&sd);
     if (tid < (int)(sizeof(RowOrDesc) / 4)) dst[tid] = src[tid];

@@ -160,21 +160,6 @@ struct MmaShared {
   volatile int fail;
 };
 
-// The last entry of the ascending table at[0 .. n) that is at most `block`, by
-// every thread of the block (evenly spaced samples, then the gap).
-__device__ __forceinline__ int find_problem(const int64_t* __restrict__ at0, int n, int64_t block) {
-  int p = 0;
-  while (n > 1) {
-    const int step = (n + (int)blockDim.x - 1) / (int)blockDim.x;
-    const int64_t at = (int64_t)threadIdx.x * step;
-    const int below = at < n && at0[p + at] <= block;
-    const int first = (__syncthreads_count(below) - 1) * step;
-    p += first;
-    n = min(step, n - first);
-  }
-  return p;
-}
-
 // Occupancy bitmaps of a problem's tiles: bit kb of a row tile of A (of a column
 // tile of B) when its K values 128 kb .. hold a set bit.  One block per tile and
 // eight K blocks, a warp each; the block writes one byte.  (Reads every bit of
@@ -182,7 +167,7 @@ __device__ __forceinline__ int find_problem(const int64_t* __restrict__ at0, int
 __global__ void __launch_bounds__(32 * kOccBlocks)
 occupancy_kernel(const MmaDesc* __restrict__ descs, const int64_t* __restrict__ block0s, int nprob) {
   asm volatile("griddepcontrol.launch_dependents;");
-  const int p = find_problem(block0s, nprob, (int64_t)blockIdx.x);
+  const int p = find_entry([&](int i) { return block0s[i]; }, nprob, (int64_t)blockIdx.x);
   const MmaDesc& d = descs[p];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int64_t t = (int64_t)blockIdx.x - block0s[p];
@@ -382,7 +367,7 @@ mma_bits_kernel(const MmaDesc* __restrict__ descs, const int64_t* __restrict__ c
   __shared__ MmaDesc sd;
   asm volatile("griddepcontrol.launch_dependents;");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int p = find_problem(cta0s, nprob, (int64_t)blockIdx.x);
+  const int p = find_entry([&](int i) { return cta0s[i]; }, nprob, (int64_t)blockIdx.x);
   {
     const uint32_t* src = reinterpret_cast<const uint32_t*>(descs + p);
     uint32_t* dst = reinterpret_cast<uint32_t*>(&sd);

@@ -21,6 +21,27 @@ cudaError_t smem_limit(const void* fn, size_t bytes);
 constexpr int kMaxDim = PA_MAX_DIM;
 constexpr int kMaxDeg = PA_MAX_DEGREE;
 
+#ifdef __CUDACC__
+// The last entry of an ascending table (entry i at first(i), i < n, first(0) <=
+// block) that is at most `block`, found by every thread of the block together:
+// each compares one of an evenly spaced sample, then the gap is searched the
+// same way.  (Two rounds of independent loads up to 65536 entries; a binary
+// search is a chain of as many L2 latencies as log2(n).)
+template <class F>
+__device__ __forceinline__ int find_entry(F&& first, int n, int64_t block) {
+  int p = 0;
+  while (n > 1) {
+    const int step = (n + (int)blockDim.x - 1) / (int)blockDim.x;
+    const int64_t at = (int64_t)threadIdx.x * step;
+    const int below = at < n && first(p + (int)at) <= block;
+    const int skip = (__syncthreads_count(below) - 1) * step;
+    p += skip;
+    n = min(step, n - skip);
+  }
+  return p;
+}
+#endif
+
 // ------------------------------------------------------------------ plotting
 // One relation to plot.  Coefficients are in "nest order": the order in which
 // the nested evaluation visits the monomials (last port outermost, every
@@ -169,6 +190,7 @@ struct ReshapeDesc {
   int64_t u_in[2 * kMaxDim];         // input words per step of the axis
   int64_t u_out[2 * kMaxDim];        // output words per step (transpose mode)
   int64_t red_in_w[2 * kMaxDim];     // words mode: input words per reduced step
+  int64_t vec;                       // words mode: consecutive words that stay together (1, 2, 4)
   int64_t tQ, tR;                    // transpose: resolutions of J and L
   int64_t t_in_L, t_out_J;           // input words per L step, output words per J step
   int64_t n_other;                   // transpose: product of u_res
@@ -176,9 +198,10 @@ struct ReshapeDesc {
 // Kernel variant of a reshape (kRs*) and its block count; a launch runs a
 // table of n descriptors of one kind, problem p on blocks [cta0[p], cta0[p+1])
 // (device arrays), grid = cta0[n].
-enum { kRsBits = 0, kRsWords32 = 1, kRsWords64 = 2, kRsTranspose = 3 };
+enum { kRsBits = 0, kRsWords32, kRsWords64, kRsTranspose32, kRsTranspose64, kRsKinds };
 int reshape_kind(const ReshapeDesc& d);
-int64_t reshape_blocks(const ReshapeDesc& d);
+int64_t reshape_units(const ReshapeDesc& d);   // block-sized pieces of its work
+int64_t reshape_blocks(const ReshapeDesc& d, int64_t per);  // blocks of `per` pieces each
 void launch_reshape(const ReshapeDesc* d_descs, const int64_t* d_cta0, int n, int kind,
                     int64_t grid, cudaStream_t s);
 
@@ -199,7 +222,9 @@ struct EwJob {
   int32_t kind;
 };
 int64_t ewise_blocks(const EwJob& j);
-void launch_ewise(const EwJob* d_jobs, const int64_t* d_cta0, int n, int64_t grid, cudaStream_t s);
+bool ewise_fits32(const EwJob& j);  // 32-bit indexes suffice (else launch with wide)
+void launch_ewise(const EwJob* d_jobs, const int64_t* d_cta0, int n, int64_t grid, bool wide,
+                  cudaStream_t s);
 
 // C[b*M + m, :] |= B[b*K + k, :] for every set bit k of A[b*M + m, :].
 // One CTA owns a tile of B (Kc rows x Nt words of batch b) in shared memory and

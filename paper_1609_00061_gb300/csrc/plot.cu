@@ -330,24 +330,6 @@ __device__ __forceinline__ void clear_ranges(const ZeroRange* __restrict__ zr, i
   }
 }
 
-// The last job whose first tile is at most this block's: every thread compares
-// one job of an evenly spaced sample, then the gap is searched the same way (two
-// rounds of independent loads up to 65536 jobs; a binary search by one thread
-// is a chain of as many L2 latencies as log2(jobs)).
-__device__ __forceinline__ int find_job(const PlotJob* __restrict__ jobs, int njobs) {
-  int lo = 0, n = njobs;  // the job is in [lo, lo + n)
-  while (n > 1) {
-    const int step = (n + (int)blockDim.x - 1) / (int)blockDim.x;
-    const int64_t at = (int64_t)threadIdx.x * step;
-    const int below = at < n && jobs[lo + at].tile0 <= (int64_t)blockIdx.x;
-    const int c = __syncthreads_count(below);  // tile0 ascends, job lo is below
-    const int first = (c - 1) * step;
-    lo += first;
-    n = min(step, n - first);
-  }
-  return lo;
-}
-
 // Taylor coefficients about yc of the polynomial in a (in place, synthetic
 // division).
 template <int DS, int N>
@@ -440,7 +422,7 @@ plot_kernel(const PlotJob* __restrict__ jobs, int njobs, int gstride,
   __shared__ uint32_t plist[kPendCap];
   __shared__ int s_n, s_npx, s_nre, s_np;
   {
-    const int job = find_job(jobs, njobs);
+    const int job = find_entry([&](int i) { return jobs[i].tile0; }, njobs, (int64_t)blockIdx.x);
     const uint32_t* src = reinterpret_cast<const uint32_t*>(jobs + job);
     uint32_t* dst = reinterpret_cast<uint32_t*>(&sJ);
     for (int i = threadIdx.x; i < (int)(sizeof(PlotJob) / 4); i += blockDim.x) dst[i] = src[i];

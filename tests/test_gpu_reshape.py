@@ -1,0 +1,57 @@
+"""Reshapes into matrix form at the edges of their kernels: permutations whose
+last axis is a run of 1, 2, 3 or 4 words, transposes around the 256-value
+tiles, reductions over few and many values (by words, by whole rows, and
+together with a permutation), through clusters against the oracle."""
+import numpy as np
+import pytest
+
+import paper_1609_00061_gb300 as pa
+
+from test_gpu_parity import check_same, pack, rand_bits
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def eng():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    e = pa.Engine(0)
+    e.set_path("rowor")
+    yield e
+    e.close()
+
+
+CASES = [
+    # (X vars, Y vars, keep, res by var)
+    ((1, 0), (1, 2), (0, 2), [65, 300, 70]),                 # A transposed
+    ((1, 0), (2, 1), (0, 2), [257, 255, 513]),               # both transposed
+    ((1, 0, 3), (1, 2), (0, 3, 2), [64, 70, 66, 128]),       # words moved, runs of 2
+    ((1, 0, 3), (1, 2), (0, 3, 2), [33, 40, 66, 192]),       # runs of 3
+    ((1, 0, 3), (1, 2), (0, 3, 2), [20, 30, 66, 512]),       # runs of 4
+    ((0, 4, 1), (1, 2), (0, 2), [50, 64, 70, 1, 300]),       # a private axis in the middle
+    ((1, 4, 0), (1, 2), (0, 2), [128, 64, 70, 1, 300]),      # the same, then transposed
+    ((1, 0, 4), (1, 2), (0, 2), [128, 96, 70, 1, 300]),      # the packed axis private, transposed
+    ((0, 1, 4, 5), (1, 2), (0, 2), [9, 64, 70, 1, 60, 200]),  # two private axes, rows of words
+    ((4, 0, 1), (1, 2), (0, 2), [3, 64, 70, 1, 4000]),       # few results, long reduction
+    ((4, 1), (1, 2), (2,), [1, 64, 70, 1, 5000]),
+    ((0, 1), (2, 0), (1, 2), [300, 520, 290]),
+    ((0, 1, 2), (0, 1, 2), (2, 0, 1), [70, 64, 65]),         # Hadamard, permuted
+    ((0, 1), (0, 2), (0, 1, 2), [65, 130, 66]),              # outer product per batch value
+    ((0, 1), (0, 1), (0,), [500, 1000]),                     # dots of short and long rows
+    ((0, 1), (0, 1), (0,), [70, 5000]),
+]
+
+
+@pytest.mark.parametrize("case", range(len(CASES)))
+@pytest.mark.parametrize("density", [0.004, 0.3])
+def test_reshaped_clusters(eng, orc, case, density):
+    xv, yv, keep, vres = CASES[case]
+    rng = np.random.default_rng(8800 + 10 * case + int(100 * density))
+    X = rand_bits(rng, tuple(vres[v] for v in xv), density)
+    Y = rand_bits(rng, tuple(vres[v] for v in yv), density)
+    want = orc.contract(orc.Arr(X, xv), orc.Arr(Y, yv), keep, vres).data
+    got = eng.contract(pack(X, xv), pack(Y, yv), keep)
+    eng.sync()
+    check_same(got, want, str(CASES[case]))
