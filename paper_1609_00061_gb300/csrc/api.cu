@@ -69,6 +69,7 @@ struct pa_ctx {
   // next call's arguments and planning state are the same byte for byte
   uint64_t plan_epoch = 0;  // changes with every setting or measurement that steers planning
   pa::Memo* memo = nullptr;
+  std::vector<pa::Memo*> old_memos;  // replaced ones whose last launch may still be running (at most 4)
 };
 
 namespace pa {
@@ -143,14 +144,22 @@ struct Memo {
   std::vector<Op> ops;
   std::vector<char> blob;
   pa_stats st{};
-  // the launches captured as one CUDA graph on the second call with the key
-  // (the descriptor upload stays a copy of its own before each launch)
+  // The upload and the launches captured as one CUDA graph on the second call
+  // with the key.  The graph copies from a pinned image of the blob of its own,
+  // which nothing changes, so calls need no staging slot; `done` follows each
+  // launch, because the image has to outlive the copies.
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
+  char* h_blob = nullptr;
+  cudaEvent_t done = nullptr;
   bool capture_failed = false;
+  bool idle() const { return !done || cudaEventQuery(done) != cudaErrorNotReady; }
   ~Memo() {
+    if (done) cudaEventSynchronize(done);
     if (exec) cudaGraphExecDestroy(exec);
     if (graph) cudaGraphDestroy(graph);
+    if (h_blob) cudaFreeHost(h_blob);
+    if (done) cudaEventDestroy(done);
   }
 };
 
@@ -1734,6 +1743,18 @@ void upload_blob(pa_ctx* ctx, const std::vector<char>& blob, cudaStream_t s) {
 
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
+// Free the replaced programs that are done, and the oldest others beyond `keep`
+// (waiting for them).
+void retire_memos(pa_ctx* ctx, size_t keep) {
+  std::vector<Memo*>& old = ctx->old_memos;
+  size_t n = 0;
+  for (size_t i = 0; i < old.size(); ++i) {
+    if (old.size() - i <= keep && !old[i]->idle()) old[n++] = old[i];
+    else delete old[i];
+  }
+  old.resize(n);
+}
+
 // Size, build and run one call on the context's arena.
 template <class F>
 pa_status run_call(pa_ctx* ctx, cudaStream_t s, pa_stats* stats, F&& body,
@@ -1760,9 +1781,11 @@ pa_status run_call(pa_ctx* ctx, cudaStream_t s, pa_stats* stats, F&& body,
     bd.st.n_launches = count_launches(bd.ops);
     if (stats) *stats = bd.st;
     if (memo_key) {
-      // a new program: the old one's graph goes with it (an executable graph
-      // still running is freed when it completes)
-      delete ctx->memo;
+      // a new program: the old one goes when its last launch is done (a few are
+      // kept until then, so that the host need not wait here)
+      if (ctx->memo) ctx->old_memos.push_back(ctx->memo);
+      ctx->memo = nullptr;
+      retire_memos(ctx, 4);
       ctx->memo = new Memo();
       Memo& m = *ctx->memo;
       m.key.swap(*memo_key);
@@ -1835,6 +1858,40 @@ std::vector<char> solve_key(pa_ctx* ctx, int32_t nvars, const pa_axis* axes, int
   return k;
 }
 
+// Capture the upload of a kept program's descriptors and its launches as one
+// graph, on a stream of their own.  False when something does not capture.
+bool capture_memo(pa_ctx* ctx, Memo& m) {
+  if (cudaEventCreateWithFlags(&m.done, cudaEventDisableTiming) != cudaSuccess ||
+      cudaMallocHost(reinterpret_cast<void**>(&m.h_blob), std::max<size_t>(1, m.blob.size())) !=
+          cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  memcpy(m.h_blob, m.blob.data(), m.blob.size());
+  cudaStream_t cs = nullptr;
+  bool ok = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) == cudaSuccess &&
+            cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+  if (ok) {
+    ok = cudaMemcpyAsync(ctx->arena, m.h_blob, m.blob.size(), cudaMemcpyHostToDevice, cs) == cudaSuccess;
+    try {
+      if (ok) run_ops(ctx, m.ops, ctx->arena, cs, false);
+    } catch (const Fail&) {
+      ok = false;
+    }
+    cudaGraph_t g = nullptr;
+    ok = (cudaStreamEndCapture(cs, &g) == cudaSuccess) && ok;
+    m.graph = g;
+    ok = ok && g && cudaGraphInstantiate(&m.exec, g, 0) == cudaSuccess;
+  }
+  if (cs) cudaStreamDestroy(cs);
+  if (!ok) {
+    cudaGetLastError();
+    if (m.exec) cudaGraphExecDestroy(m.exec);
+    m.exec = nullptr;
+  }
+  return ok;
+}
+
 // Relaunch the kept program.  Its blob is uploaded again like any call's: the
 // coefficients are host inputs of every call, and another call may have
 // replaced the blob region of the arena since.
@@ -1845,39 +1902,14 @@ pa_status run_memo(pa_ctx* ctx, cudaStream_t s, pa_stats* stats) {
       return set_err(ctx, PA_ERR_CUDA, "cudaSetDevice failed");
     }
     Memo& m = *ctx->memo;
-    upload_blob(ctx, m.blob, s);
-    if (ctx->prof || m.capture_failed) {
-      // per-launch timing needs the launches one by one
+    // per-launch timing needs the launches one by one
+    if (!ctx->prof && !m.exec && !m.capture_failed) m.capture_failed = !capture_memo(ctx, m);
+    if (ctx->prof || !m.exec) {
+      upload_blob(ctx, m.blob, s);
       run_ops(ctx, m.ops, ctx->arena, s, ctx->prof);
     } else {
-      if (!m.exec) {
-        // capture the launches once, on a stream of their own
-        cudaStream_t cs = nullptr;
-        bool ok = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) == cudaSuccess &&
-                  cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-        if (ok) {
-          try {
-            run_ops(ctx, m.ops, ctx->arena, cs, false);
-          } catch (const Fail&) {
-            ok = false;
-          }
-          cudaGraph_t g = nullptr;
-          ok = (cudaStreamEndCapture(cs, &g) == cudaSuccess) && ok;
-          m.graph = g;
-          ok = ok && g && cudaGraphInstantiate(&m.exec, g, 0) == cudaSuccess;
-        }
-        if (cs) cudaStreamDestroy(cs);
-        if (!ok) {
-          cudaGetLastError();
-          if (m.exec) cudaGraphExecDestroy(m.exec);
-          m.exec = nullptr;
-          m.capture_failed = true;
-          run_ops(ctx, m.ops, ctx->arena, s, false);
-          if (stats) *stats = m.st;
-          return PA_OK;
-        }
-      }
       check_cuda(ctx, cudaGraphLaunch(m.exec, s), "cudaGraphLaunch");
+      check_cuda(ctx, cudaEventRecord(m.done, s), "cudaEventRecord");
     }
     if (stats) *stats = m.st;
     return PA_OK;
@@ -2371,6 +2403,7 @@ void pa_destroy(pa_ctx* ctx) {
     if (ctx->stage_pending[i]) cudaEventSynchronize(ctx->stage_done[i]);
   delete ctx->memo;  // its graph before the arena it points into
   ctx->memo = nullptr;
+  retire_memos(ctx, 0);
   if (ctx->arena) cudaFree(ctx->arena);
   if (ctx->d_err) cudaFree(ctx->d_err);
   if (ctx->d_stat) cudaFree(ctx->d_stat);
