@@ -769,8 +769,9 @@ bool use_mma(const pa_ctx* ctx, const JoinShape& js, double ra) {
 // estimated density of the result when both are known.
 BitArr join(Builder& bd, const BitArr& X, const BitArr& Y, const std::vector<int>& keep,
             const std::vector<int64_t>& vres, const BitArr* target, double share,
-            double rx = -1.0, double ry = -1.0, double* rho_out = nullptr) {
-  const JoinShape js = analyze_join(X, Y, keep, vres);
+            double rx = -1.0, double ry = -1.0, double* rho_out = nullptr,
+            const JoinShape* shape = nullptr) {
+  const JoinShape js = shape ? *shape : analyze_join(X, Y, keep, vres);
   bd.st.pixel_ops_dense += js.cost;
   bd.st.n_joins++;
   double ra = -1.0;
@@ -1295,6 +1296,7 @@ std::vector<BitArr> plot_poly(Builder& bd, const std::vector<PlotReq>& reqs) {
   }
   int64_t tiles = 0;
   int max_rows = 1, max_deg = 0, common_deg = reqs[0].rel->degree;
+  std::map<std::pair<int, int>, std::vector<int64_t>> orders;  // by arity and degree
   std::vector<double> nc;
   std::vector<float> nc32;
   for (int i = 0; i < nrel; ++i) {
@@ -1311,7 +1313,8 @@ std::vector<BitArr> plot_poly(Builder& bd, const std::vector<PlotReq>& reqs) {
     a.w = reqs[i].direct ? reqs[i].direct : bd.alloc_words(a.words());
     plots.push_back(a);
     // coefficients in nest order
-    std::vector<int64_t> ord = nest_order(r.arity, r.degree);
+    std::vector<int64_t>& ord = orders[{r.arity, r.degree}];
+    if (ord.empty()) ord = nest_order(r.arity, r.degree);
     nc.resize(ord.size());
     nc32.resize(ord.size());
     for (size_t k = 0; k < ord.size(); ++k) {
@@ -1383,6 +1386,8 @@ struct Network {
   std::vector<uint64_t> slot_keys;  // per slot: key of the relations and kept variables below it
   Plan plan;                        // the join order, planned once for both passes of a call
   bool planned = false;
+  std::vector<JoinShape> shapes;    // per join, likewise (layouts do not depend on addresses;
+  std::vector<char> shaped;         // finding one costs some 2 us of vectors)
 };
 
 // Run f(i) for i in [0, n) on up to `threads` host threads (contiguous
@@ -1552,7 +1557,16 @@ void build_networks(Builder& bd, std::vector<Network>& nets, bool one_join_per_l
         for (int t = 0; t < (int)s.plan.joins.size(); ++t) {
           if (s.level[nrel + t] != lv) continue;
           const Join& jn = s.plan.joins[t];
-          const JoinShape js = analyze_join(s.slots[jn.a], s.slots[jn.b], jn.keep, s.vres);
+          Network& net = nets[k];
+          if (net.shapes.empty()) {
+            net.shapes.resize(s.plan.joins.size());
+            net.shaped.assign(s.plan.joins.size(), 0);
+          }
+          if (!net.shaped[t]) {
+            net.shapes[t] = analyze_join(s.slots[jn.a], s.slots[jn.b], jn.keep, s.vres);
+            net.shaped[t] = 1;
+          }
+          const JoinShape& js = net.shapes[t];
           double w = 0.0;
           if (!js.hadamard && !js.outer && !js.dot) {
             double ra = -1.0;
@@ -1582,7 +1596,7 @@ void build_networks(Builder& bd, std::vector<Network>& nets, bool one_join_per_l
                                  last ? &nets[k].target : nullptr,
                                  one_join_per_launch ? 152.0 : share_of[{k, t}],
                                  dn ? s.dens[jn.a] : -1.0, dn ? s.dens[jn.b] : -1.0,
-                                 dn ? &s.dens[nrel + t] : nullptr);
+                                 dn ? &s.dens[nrel + t] : nullptr, &nets[k].shapes[t]);
         if (dn) {
           // a density measured by pa_join_log beats the independence estimate
           auto it = bd.ctx->obs_dens.find(nets[k].slot_keys[nrel + t]);
