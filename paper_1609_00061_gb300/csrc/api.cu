@@ -121,7 +121,7 @@ const char* op_name(const Op& op) {
     case OP_EWISE: return "ewise_kernel";
     case OP_MEMSET: return "memset";
     case OP_RESHAPE:
-      return op.i0 == kRsTranspose32 || op.i0 == kRsTranspose64 ? "reshape_transpose_kernel"
+      return op.i0 >= kRsTranspose32 ? "reshape_transpose_kernel"
              : (op.i0 == kRsWords32 || op.i0 == kRsWords64) ? "reshape_words_kernel"
                                                             : "reshape_kernel";
     case OP_MMA: return "mma_bits_kernel";
@@ -433,8 +433,8 @@ void flush_reshapes(Builder& bd) {
     // 369 us for the first level of 38 networks; the other kinds lost 16 %)
     int64_t total = 0, per = 1;
     for (const ReshapeDesc& d : group) total += reshape_units(d);
-    if (kind == kRsTranspose32 || kind == kRsTranspose64)
-      per = std::max<int64_t>(1, std::min<int64_t>(8, total / (152 * 8)));
+    if (kind >= kRsTranspose32)
+      per = std::max<int64_t>(1, std::min<int64_t>(8, total / (152 * (kind == kRsTranspose32Wide ? 3 : 8))));
     for (const ReshapeDesc& d : group) cta0.push_back(cta0.back() + reshape_blocks(d, per));
     if (group.empty()) continue;
     if (cta0.back() > 0x7fffffffLL) bd.fail(PA_ERR_TOO_LARGE, "reshape grid too large");

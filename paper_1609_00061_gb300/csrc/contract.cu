@@ -310,28 +310,31 @@ struct Transpose32 {
   }
 };
 
-// Transpose mode.  A CTA tile is 256 values of L (4 output words) x 256 values
-// of J (4 input words) at one value of the other axes: coalesced 32-byte loads
-// of 256 input rows into shared memory, 64 warp transposes of 32 x 32 blocks,
-// coalesced 32-byte stores of 256 output rows.  Rows of the shared tiles are
-// padded to 5 words.
-// Index type I is 32-bit when every word and tile index fits.  Bound by the
-// latency of 32-byte accesses at the arrays' pitches (1.7 TB/s); 64-bit divisions
-// (two thirds of 8570 warp instructions per tile) and branching 64 x 64 block
-// transposes bound it before: 38 networks' transposes 1.88 -> 1.28 ms.
-constexpr int kTrPad = 5;
-template <class I>
-__global__ void __launch_bounds__(256)
+// Transpose mode.  A CTA tile is 64 TW values of L (TW output words) x 64 TW
+// values of J (TW input words) at one value of the other axes: its input rows
+// are loaded into shared memory, transposed by warps in 32 x 32 blocks, and its
+// output rows stored.  TW = 4 (256 x 256), or 8 where both axes have more than
+// 256 values: rows of 512 bits are then read and written whole, 32 KB in one run
+// where the rows are neighbours, instead of in 32-byte halves.  Rows of the
+// shared tiles are padded by a word.  Index type I is 32-bit when every word and
+// tile index fits.  Bound by the latency of short accesses at the arrays'
+// pitches; 64-bit divisions (two thirds of 8570 warp instructions per tile) and
+// branching 64 x 64 block transposes bound it before: 38 networks' transposes
+// 1.88 -> 1.28 ms, with the wide tiles 1.12.
+template <class I, int TW>
+__global__ void __launch_bounds__(64 * TW)
 reshape_transpose_kernel(const ReshapeDesc* __restrict__ descs, const int64_t* __restrict__ cta0, int n) {
+  constexpr int kThreads = 64 * TW, kPad = TW + 1;  // a thread per value of an axis
+  extern __shared__ uint64_t tr_smem[];
+  uint64_t* s_in = tr_smem;
+  uint64_t* s_out = tr_smem + 64 * TW * kPad;
   __shared__ ReshapeDesc sd;
   const RsCtx rc = rs_pick(descs, cta0, n, &sd);
   const ReshapeDesc& d = sd;
-  __shared__ uint64_t s_in[256 * kTrPad];
-  __shared__ uint64_t s_out[256 * kTrPad];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const Transpose32 tr(lane);
   const I tQ = (I)d.tQ, tR = (I)d.tR, t_in_L = (I)d.t_in_L, t_out_J = (I)d.t_out_J;
-  const I nJT = (tQ + 255) / 256, nLT = (tR + 255) / 256;
+  const I nJT = (tQ + 64 * TW - 1) / (64 * TW), nLT = (tR + 64 * TW - 1) / (64 * TW);
   const I tiles = (I)d.n_other * nJT * nLT;
   const I nblk = (I)rc.nblk;
   // tile -> (L tile, J tile, first input and output word of its other axes)
@@ -349,28 +352,28 @@ reshape_transpose_kernel(const ReshapeDesc* __restrict__ descs, const int64_t* _
       base_out += v * (I)d.u_out[a];
     }
   };
-  // the four input words this thread loads for a tile
+  // the TW input words this thread loads for a tile
   auto load = [&](I lt, I jt, I base_in, uint64_t* v) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int idx = tid + 256 * i, b = idx >> 2, c = idx & 3;
-      const I L = lt * 256 + b, jb = jt * 4 + c;
+    for (int i = 0; i < TW; ++i) {
+      const int idx = tid + kThreads * i, b = idx / TW, c = idx % TW;
+      const I L = lt * (64 * TW) + b, jb = jt * TW + c;
       v[i] = (L < tR && jb * 64 < tQ) ? d.in[base_in + L * t_in_L + jb] : 0ull;
     }
   };
   // the next tile's loads are issued before the current tile is transposed
   // and stored, so that their latency overlaps that work
   I lt = 0, jt = 0, base_in = 0, base_out = 0;
-  uint64_t nv[4] = {0, 0, 0, 0};
+  uint64_t nv[TW];
   if ((I)rc.bid < tiles) {
     locate((I)rc.bid, lt, jt, base_in, base_out);
     load(lt, jt, base_in, nv);
   }
   for (I tile = (I)rc.bid; tile < tiles; tile += nblk) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int idx = tid + 256 * i, b = idx >> 2, c = idx & 3;
-      s_in[b * kTrPad + c] = nv[i];
+    for (int i = 0; i < TW; ++i) {
+      const int idx = tid + kThreads * i;
+      s_in[idx / TW * kPad + idx % TW] = nv[i];
     }
     const I clt = lt, cjt = jt, cbase_out = base_out;
     if (tile + nblk < tiles) {
@@ -378,22 +381,30 @@ reshape_transpose_kernel(const ReshapeDesc* __restrict__ descs, const int64_t* _
       load(lt, jt, base_in, nv);
     }
     __syncthreads();
-    // warp w: the 32 columns w of J, all eight 32-row blocks of L
-    if ((cjt * 8 + warp) * 32 < tQ) {
-      const uint32_t* in32 = reinterpret_cast<const uint32_t*>(s_in) + lane * (2 * kTrPad) + warp;
-      uint32_t* out32 = reinterpret_cast<uint32_t*>(s_out) + (warp * 32 + lane) * (2 * kTrPad);
+    // warp w: the 32 columns w of J, all 32-row blocks of L
+    if ((cjt * (2 * TW) + warp) * 32 < tQ) {
+      const uint32_t* in32 = reinterpret_cast<const uint32_t*>(s_in) + lane * (2 * kPad) + warp;
+      uint32_t* out32 = reinterpret_cast<uint32_t*>(s_out) + (warp * 32 + lane) * (2 * kPad);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) out32[i] = tr(in32[i * 32 * (2 * kTrPad)]);
+      for (int i = 0; i < 2 * TW; ++i) out32[i] = tr(in32[i * 32 * (2 * kPad)]);
     }
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int idx = tid + 256 * i, t = idx >> 2, w = idx & 3;
-      const I J = cjt * 256 + t, lw = clt * 4 + w;
-      if (J < tQ && lw * 64 < tR) d.out[cbase_out + J * t_out_J + lw] = s_out[t * kTrPad + w];
+    for (int i = 0; i < TW; ++i) {
+      const int idx = tid + kThreads * i, t = idx / TW, w = idx % TW;
+      const I J = cjt * (64 * TW) + t, lw = clt * TW + w;
+      if (J < tQ && lw * 64 < tR) d.out[cbase_out + J * t_out_J + lw] = s_out[t * kPad + w];
     }
     __syncthreads();
   }
+}
+
+// Words of a transpose's tile per side, and the bytes of its two shared tiles.
+int transpose_tw(const ReshapeDesc& d) { return d.tQ > 256 && d.tR > 256 ? 8 : 4; }
+constexpr size_t transpose_smem(int tw) { return (size_t)2 * 64 * tw * (tw + 1) * 8; }
+int64_t transpose_tiles(const ReshapeDesc& d) {
+  const int64_t side = 64 * transpose_tw(d);
+  return d.n_other * ((d.tQ + side - 1) / side) * ((d.tR + side - 1) / side);
 }
 
 constexpr int64_t kMaxReshapeBlocks = 152 * 16;
@@ -404,10 +415,10 @@ int reshape_kind(const ReshapeDesc& d) {
   int64_t in_max = 0;  // largest input word index + 1 (bounded by the sums below)
   for (int a = 0; a < d.nu; ++a) in_max += (d.u_res[a] - 1) * d.u_in[a];
   if (d.mode == kReshapeTranspose) {
-    in_max += (d.tR + 255) * d.t_in_L + d.tQ / 64 + 4;
-    const int64_t tiles = d.n_other * ((d.tQ + 255) / 256) * ((d.tR + 255) / 256);
-    return (in_max < (1ll << 31) && total < (1ll << 31) && tiles + blocks < (1ll << 31)) ? kRsTranspose32
-                                                                                        : kRsTranspose64;
+    in_max += (d.tR + 511) * d.t_in_L + d.tQ / 64 + 8;
+    const bool fits = in_max < (1ll << 31) && total < (1ll << 31) &&
+                      transpose_tiles(d) + blocks < (1ll << 31);
+    return !fits ? kRsTranspose64 : transpose_tw(d) == 8 ? kRsTranspose32Wide : kRsTranspose32;
   }
   for (int q = 0; q < d.nred; ++q) in_max += (d.red_res[q] - 1) * d.red_in_w[q];
   return (total + 1024 * blocks < (1ll << 31) && in_max < (1ll << 31)) ? kRsWords32 : kRsWords64;
@@ -416,7 +427,7 @@ int reshape_kind(const ReshapeDesc& d) {
 int64_t reshape_units(const ReshapeDesc& d) {
   const int64_t total = d.out_nrows * d.out_row_words;
   if (total <= 0) return 0;
-  if (d.mode == kReshapeTranspose) return d.n_other * ((d.tQ + 255) / 256) * ((d.tR + 255) / 256);
+  if (d.mode == kReshapeTranspose) return transpose_tiles(d);
   if (d.mode == kReshapeWords) {
     // a thread per run of words, or more for a reduction (see the kernel)
     int64_t red = 1;
@@ -438,10 +449,17 @@ void launch_reshape(const ReshapeDesc* d_descs, const int64_t* d_cta0, int n, in
   if (n <= 0 || grid <= 0) return;
   switch (kind) {
     case kRsTranspose32:
-      reshape_transpose_kernel<uint32_t><<<(unsigned)grid, 256, 0, s>>>(d_descs, d_cta0, n);
+      reshape_transpose_kernel<uint32_t, 4>
+          <<<(unsigned)grid, 256, transpose_smem(4), s>>>(d_descs, d_cta0, n);
+      break;
+    case kRsTranspose32Wide:
+      smem_limit(reinterpret_cast<const void*>(reshape_transpose_kernel<uint32_t, 8>), transpose_smem(8));
+      reshape_transpose_kernel<uint32_t, 8>
+          <<<(unsigned)grid, 512, transpose_smem(8), s>>>(d_descs, d_cta0, n);
       break;
     case kRsTranspose64:
-      reshape_transpose_kernel<uint64_t><<<(unsigned)grid, 256, 0, s>>>(d_descs, d_cta0, n);
+      reshape_transpose_kernel<uint64_t, 4>
+          <<<(unsigned)grid, 256, transpose_smem(4), s>>>(d_descs, d_cta0, n);
       break;
     case kRsWords32:
       reshape_words_kernel<uint32_t><<<(unsigned)grid, 256, 0, s>>>(d_descs, d_cta0, n);

@@ -198,7 +198,8 @@ struct ReshapeDesc {
 // Kernel variant of a reshape (kRs*) and its block count; a launch runs a
 // table of n descriptors of one kind, problem p on blocks [cta0[p], cta0[p+1])
 // (device arrays), grid = cta0[n].
-enum { kRsBits = 0, kRsWords32, kRsWords64, kRsTranspose32, kRsTranspose64, kRsKinds };
+enum { kRsBits = 0, kRsWords32, kRsWords64, kRsTranspose32, kRsTranspose32Wide, kRsTranspose64,
+       kRsKinds };
 int reshape_kind(const ReshapeDesc& d);
 int64_t reshape_units(const ReshapeDesc& d);   // block-sized pieces of its work
 int64_t reshape_blocks(const ReshapeDesc& d, int64_t per);  // blocks of `per` pieces each
