@@ -1872,11 +1872,23 @@ std::vector<char> solve_key(pa_ctx* ctx, int32_t nvars, const pa_axis* axes, int
   return k;
 }
 
+// A small blob is fetched from pinned host memory by a kernel instead of a copy
+// node: a copy engine's hand-over to the first kernel costs more than the copy,
+// and the plot launch that follows is scheduled while this one runs (chain of 8 at
+// 2048 px 59 -> 53 us per solve, circle and parabola at 256 px 28.4 -> 26.7).
+constexpr size_t kFetchBytes = 64 * 1024;
+__global__ void __launch_bounds__(256)
+fetch_kernel(uint4* __restrict__ dst, const uint4* __restrict__ src, int n) {
+  asm volatile("griddepcontrol.launch_dependents;");
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i < n) dst[i] = src[i];
+}
+
 // Capture the upload of a kept program's descriptors and its launches as one
 // graph, on a stream of their own.  False when something does not capture.
 bool capture_memo(pa_ctx* ctx, Memo& m) {
   if (cudaEventCreateWithFlags(&m.done, cudaEventDisableTiming) != cudaSuccess ||
-      cudaMallocHost(reinterpret_cast<void**>(&m.h_blob), std::max<size_t>(1, m.blob.size())) !=
+      cudaMallocHost(reinterpret_cast<void**>(&m.h_blob), round_up(m.blob.size() + 16, 16)) !=
           cudaSuccess) {
     cudaGetLastError();
     return false;
@@ -1886,7 +1898,14 @@ bool capture_memo(pa_ctx* ctx, Memo& m) {
   bool ok = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) == cudaSuccess &&
             cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
   if (ok) {
-    ok = cudaMemcpyAsync(ctx->arena, m.h_blob, m.blob.size(), cudaMemcpyHostToDevice, cs) == cudaSuccess;
+    // (whole 16-byte pieces: the blob's region is larger than the blob)
+    const int n16 = (int)((m.blob.size() + 15) / 16);
+    if (m.blob.size() <= kFetchBytes && n16 > 0)
+      fetch_kernel<<<(unsigned)((n16 + 255) / 256), 256, 0, cs>>>(
+          reinterpret_cast<uint4*>(ctx->arena), reinterpret_cast<const uint4*>(m.h_blob), n16);
+    else
+      cudaMemcpyAsync(ctx->arena, m.h_blob, m.blob.size(), cudaMemcpyHostToDevice, cs);
+    ok = cudaGetLastError() == cudaSuccess;
     try {
       if (ok) run_ops(ctx, m.ops, ctx->arena, cs, false);
     } catch (const Fail&) {

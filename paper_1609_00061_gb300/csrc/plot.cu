@@ -416,6 +416,10 @@ __global__ void __launch_bounds__(kPlotThreads, 4)
 plot_kernel(const PlotJob* __restrict__ jobs, int njobs, int gstride,
             const ZeroRange* __restrict__ zr, int nzero, int64_t zero_words) {
   extern __shared__ __align__(16) float g32s[];  // [rows][gstride] row polynomials
+  // the launch before this one may be the upload of the descriptors; those after
+  // it read theirs before they wait for this grid, so they may only start when
+  // that upload is complete
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;");
   __shared__ PlotJob sJ;
   __shared__ uint16_t list[kPass], list_px[kPass], list_re[kPass];
@@ -846,12 +850,23 @@ void launch_plot(const PlotJob* d_jobs, int njobs, int64_t total_tiles, int max_
   if (total_tiles <= 0) return;
   const int gstride = max_degree + 1;
   const size_t smem = (size_t)max_rows_per_tile * gstride * sizeof(float);
-  const unsigned grid = (unsigned)total_tiles;
+  // programmatic dependent launch: the blocks are scheduled while the launch
+  // before them (the upload of a kept program) runs
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)total_tiles);
+  cfg.blockDim = dim3(kPlotThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
 #define PA_PLOT(DD)                                                                          \
   do {                                                                                       \
     smem_limit(reinterpret_cast<const void*>(plot_kernel<DD>), smem);                        \
-    plot_kernel<DD><<<grid, kPlotThreads, smem, s>>>(d_jobs, njobs, gstride, d_zero, nzero,  \
-                                                     zero_words);                            \
+    cudaLaunchKernelEx(&cfg, plot_kernel<DD>, d_jobs, njobs, gstride, d_zero, nzero,         \
+                       zero_words);                                                          \
   } while (0)
   switch (common_degree) {
     case 1: PA_PLOT(1); break;
