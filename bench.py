@@ -251,7 +251,7 @@ def kernel_rooflines(kernels, stats_step, steps, sysm, pk):
                           "work_per_launch": f"{hb:.4g} bytes: A, B read and C written once, "
                                             f"{joins / launches:.3g} joins of {r}^3",
                           "share": share})
-        elif name == "mma_bool_kernel":
+        elif name == "mma_bits_kernel":
             # 2 flops per multiply-add of the unpadded clusters (M x N x K each)
             macs = stats_step.get("mma_macs", 0.0) * steps / launches
             ach = 2.0 * macs / t / 1e12

@@ -1010,20 +1010,23 @@ rowor_kernel(const RowOrDesc* __restrict__ descs, const CUtensorMap* __restrict_
 
 namespace {
 
+// cuTensorMapEncodeTiled from the driver (null when unavailable)
+typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
+                                  const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
+                                  const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
 EncodeTiledFn encode_fn() {
-  static EncodeTiledFn fn = nullptr;
-  static bool tried = false;
-  if (!tried) {
-    tried = true;
+  static const EncodeTiledFn fn = [] {  // looked up once, whatever thread comes first
     void* p = nullptr;
     cudaDriverEntryPointQueryResult q;
     if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
                                          &q) == cudaSuccess &&
         q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(p);
-    else
-      cudaGetLastError();
-  }
+      return reinterpret_cast<EncodeTiledFn>(p);
+    cudaGetLastError();
+    return EncodeTiledFn(nullptr);
+  }();
   return fn;
 }
 
@@ -1037,8 +1040,6 @@ constexpr size_t list_bytes(int threads) { return (size_t)(threads / 32) * kList
 size_t table_bytes(int64_t staged, int Nt) { return (size_t)rowor_table_rows(staged) * Nt * 8; }
 
 }  // namespace
-
-EncodeTiledFn tensor_map_encoder() { return encode_fn(); }
 
 cudaError_t smem_limit(const void* fn, size_t bytes) {
   static std::mutex mu;

@@ -260,12 +260,6 @@ cudaError_t rowor_encode_map(const RowOrDesc& d, CUtensorMap* map);
 cudaError_t launch_rowor(const RowOrDesc* d_descs, const CUtensorMap* d_maps,
                          const int64_t* d_cta0, int nprob, int64_t grid, size_t smem, int threads,
                          cudaStream_t s);
-// cuTensorMapEncodeTiled from the driver (null when unavailable)
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
-                                  const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
-                                  const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn tensor_map_encoder();
 
 // Tensor-core contraction (mma.cu): the same problem as RowOrDesc, from the
 // same bit-packed layouts, as a 0/1 matrix product on E4M3 operands thresholded
