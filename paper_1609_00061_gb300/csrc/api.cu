@@ -167,6 +167,9 @@ struct Memo {
 struct Builder {
   pa_ctx* ctx;
   bool dry;
+  // Set when the layout would not fit the memory there is: no array that only
+  // makes a reshape faster (conform).
+  bool compact = false;
   char* base = nullptr;     // device memory the layout lives in (null in the sizing pass)
   size_t used = 0;          // bytes of `base` in use
   size_t blob_cap = 0;      // bytes reserved for the blob at the start of `base`
@@ -462,7 +465,7 @@ BitArr conform(Builder& bd, const BitArr& x, BitArr want) {
   // reduced value and bit: 276 us for three 512^3 arrays).  It is a reduction in
   // x's own axis order, by words or whole rows, and a transpose of the much
   // smaller result; a level's transposes are launched after its reductions.
-  if (make_reshape(x, want).mode == kReshapeBits) {
+  if (!bd.compact && make_reshape(x, want).mode == kReshapeBits) {
     BitArr mid;
     for (int a = 0; a < x.ndim; ++a)
       if (axis_of(want, x.vars[a]) >= 0) {
@@ -1771,6 +1774,24 @@ void retire_memos(pa_ctx* ctx, size_t keep) {
   old.resize(n);
 }
 
+// Size a program: the bytes `body` needs next to `extra`, its blob's region in
+// *blob_cap; *compact when only the compact layout stays within `limit` (0: none).
+template <class F>
+size_t size_program(pa_ctx* ctx, F&& body, size_t limit, size_t extra, size_t* blob_cap,
+                    bool* compact, pa_stats* st = nullptr) {
+  for (*compact = false;; *compact = true) {
+    Builder dry(ctx, true, nullptr, 0);
+    dry.compact = *compact;
+    body(dry);
+    *blob_cap = round_up(dry.blob.size() + 64, kAlign);
+    const size_t need = extra + dry.used + *blob_cap + kAlign;
+    if (*compact || !limit || need <= limit) {
+      if (st) *st = dry.st;
+      return need;
+    }
+  }
+}
+
 // Size, build and run one call on the context's arena.
 template <class F>
 pa_status run_call(pa_ctx* ctx, cudaStream_t s, pa_stats* stats, F&& body,
@@ -1780,13 +1801,13 @@ pa_status run_call(pa_ctx* ctx, cudaStream_t s, pa_stats* stats, F&& body,
       cudaGetLastError();
       return set_err(ctx, PA_ERR_CUDA, "cudaSetDevice failed");
     }
-    Builder dry(ctx, true, nullptr, 0);
-    body(dry);
-    const size_t blob_cap = round_up(dry.blob.size() + 64, kAlign);
-    const size_t need = dry.used + blob_cap + kAlign;
+    size_t blob_cap = 0;
+    bool compact = false;
+    const size_t need = size_program(ctx, body, ctx->cap, 0, &blob_cap, &compact);
     pa_status st = ensure_arena(ctx, need);
     if (st != PA_OK) return st;
     Builder bd(ctx, false, ctx->arena, blob_cap);
+    bd.compact = compact;
     bd.d_err = ctx->d_err;
     bd.d_stat = ctx->prof ? ctx->d_stat : nullptr;
     body(bd);
@@ -2900,10 +2921,10 @@ pa_status pa_batch_create(pa_ctx* ctx, int32_t nsys, const pa_system* systems, p
   cudaStream_t cs = nullptr;
   try {
     check_cuda(ctx, cudaSetDevice(ctx->device), "cudaSetDevice");
-    Builder dry(ctx, true, nullptr, 0);
-    build_networks(dry, nets);
-    const size_t blob_cap = round_up(dry.blob.size() + 64, kAlign);
-    bt->mem_size = dry.used + blob_cap + kAlign;
+    size_t blob_cap = 0;
+    bool compact = false;
+    bt->mem_size = size_program(ctx, [&](Builder& b) { build_networks(b, nets); }, ctx->cap, 0,
+                                &blob_cap, &compact);
     if (ctx->cap && bt->mem_size > ctx->cap)
       throw Fail{set_err(ctx, PA_ERR_OOM, "batch workspace exceeds the context's cap")};
     if (cudaMalloc(reinterpret_cast<void**>(&bt->mem), bt->mem_size) != cudaSuccess) {
@@ -2912,6 +2933,7 @@ pa_status pa_batch_create(pa_ctx* ctx, int32_t nsys, const pa_system* systems, p
       throw Fail{set_err(ctx, PA_ERR_OOM, "cudaMalloc of the batch workspace failed")};
     }
     Builder bd(ctx, false, bt->mem, blob_cap);
+    bd.compact = compact;
     bd.d_err = ctx->d_err;
     build_networks(bd, nets);
     bt->ops = bd.ops;
@@ -3127,12 +3149,13 @@ pa_status pa_join_log(pa_ctx* ctx, const pa_system* sys, const pa_options* opts,
   std::vector<cudaEvent_t> evs;
   try {
     check_cuda(ctx, cudaSetDevice(ctx->device), "cudaSetDevice");
-    Builder dry(ctx, true, nullptr, 0);
-    build_networks(dry, nets, true);
-    const size_t blob_cap = round_up(dry.blob.size() + 64, kAlign);
-    st = ensure_arena(ctx, dry.used + blob_cap + kAlign);
+    size_t blob_cap = 0;
+    bool compact = false;
+    st = ensure_arena(ctx, size_program(ctx, [&](Builder& b) { build_networks(b, nets, true); },
+                                        ctx->cap, 0, &blob_cap, &compact));
     if (st != PA_OK) return st;
     Builder bd(ctx, false, ctx->arena, blob_cap);
+    bd.compact = compact;
     bd.d_err = ctx->d_err;
     std::vector<BitArr> results;
     build_networks(bd, nets, true, &results);
@@ -3321,19 +3344,22 @@ extern "C" pa_status pa_solve_network_static(int32_t nvars, const pa_axis* axes,
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   try {
-    Builder dry(ctx, true, nullptr, 0);
-    build_networks(dry, nets);
-    const size_t blob_cap = round_up(dry.blob.size() + 64, kAlign);
-    const size_t need = kStaticHeader + dry.used + blob_cap + kAlign;
+    size_t blob_cap = 0;
+    bool compact = false;
+    pa_stats dry_st{};
+    const size_t need = size_program(ctx, [&](Builder& b) { build_networks(b, nets); },
+                                     PA_STATIC_SCRATCH_BYTES, kStaticHeader, &blob_cap, &compact,
+                                     &dry_st);
     if (need > PA_STATIC_SCRATCH_BYTES) {
       if (stats) {
-        *stats = dry.st;
+        *stats = dry_st;
         stats->workspace_bytes = (int64_t)need;
       }
       return PA_ERR_TOO_LARGE;
     }
     char* work = base + kStaticHeader;
     Builder bd(ctx, false, work, blob_cap);
+    bd.compact = compact;
     bd.d_err = reinterpret_cast<int*>(base);
     build_networks(bd, nets);
     if (bd.blob.size() > blob_cap) return PA_ERR_CUDA;
