@@ -27,7 +27,8 @@
 //   - B stays N-major (tcgen05 reads 8-bit operands in either orientation), so
 //     no bit transposes.
 // Per 128-value K block four producer warps fill one of four 16 + 32 KB stages
-// (128-byte swizzle); four such groups work on four blocks at a time, because a
+// (128-byte swizzle); four such groups work on four blocks of an SM at a time (of
+// one CTA, or two each of two CTAs where there are more tiles than SMs), because a
 // group's chain of loads, masks and stores is longer than the tensor core's time
 // for a block (one group of eight warps measured 1900 cycles per block).  One
 // thread issues tcgen05.mma kind::f8f6f4 (M = 128, N = BN, K = 32 per
@@ -48,7 +49,8 @@
 // cycles and without the products 825, so both sides are near their limit (an
 // N-major B halves the rate of a K-major one, 560 per block, which would need
 // bit transposes).  Against the byte-array version: 8192^3 of two cubic plots
-// 100 -> 80 us per call, the 2048^3 count 55 -> 48 us, ternary 256 78 -> 71 us.
+// 100 -> 58 us per call, the 2048^3 count 55 -> 46 us, ternary 256 (256 products of
+// 256^3) 78 -> 62 us.
 #include <cuda.h>
 #include <string.h>
 
@@ -65,11 +67,11 @@ constexpr int kMmaBK = 128;                   // K values per stage = one 128-by
 constexpr int kMmaATile = kMmaBM * kMmaBK;    // 16 KB
 constexpr int kMmaNBlock = 128 * kMmaBK;      // 16 KB: 128 columns of B
 constexpr int kMmaStage = kMmaATile + 2 * kMmaNBlock;  // 48 KB
-constexpr int kMmaStages = 4;                 // one per producer group
+constexpr int kMmaMaxStages = 4;              // one per producer group
 constexpr int kMmaTmemCols = 256;
-constexpr int kMmaProducers = 4 * kMmaStages;  // warps; the last warp issues the products
-constexpr int kMmaThreads = 32 * (kMmaProducers + 1);
-constexpr size_t kMmaSmem = (size_t)kMmaStages * kMmaStage + 1024;
+// Four producer warps to a stage; the last warp issues the products.
+constexpr int mma_threads(int stages) { return 32 * (4 * stages + 1); }
+constexpr size_t mma_smem(int stages) { return (size_t)stages * kMmaStage + 1024; }
 constexpr int kOccBlocks = 8;                 // K blocks per block of occupancy_kernel
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
@@ -152,9 +154,9 @@ __device__ __forceinline__ void st_shared16(uint32_t addr, uint4 v) {
 }
 
 struct MmaShared {
-  uint64_t full[kMmaStages], empty[kMmaStages], accum;
-  uint32_t occ[kMmaStages][2];       // per group, by turns: a byte per warp, 1 A words, 2 B words
-  volatile int skip[kMmaStages];     // the stage's block is to be skipped
+  uint64_t full[kMmaMaxStages], empty[kMmaMaxStages], accum;
+  uint32_t occ[kMmaMaxStages][2];    // per group, by turns: a byte per warp, 1 A words, 2 B words
+  volatile int skip[kMmaMaxStages];  // the stage's block is to be skipped
   volatile int issued;               // blocks multiplied
   uint32_t tmem;
   volatile int fail;
@@ -243,13 +245,13 @@ struct ActiveBlocks {
   }
 };
 
-// A producer warp's blocks: the group's share (every kMmaStages-th) of the
+// A producer warp's blocks: the group's share (every STAGES-th) of the
 // CTA's, into the group's stage.  BN = 128 or 256.  A thread holds two A
 // words and BN / 64 B words of a block, loaded one block of its group ahead.
 // The thread-to-word maps make the loads 16- and 32-byte runs of a row and the
 // 16-byte shared stores free of conflicts (eight chunks of distinct bank groups
 // per quarter warp).
-template <int BN, bool COUNT>
+template <int STAGES, int BN, bool COUNT>
 __device__ __forceinline__ void produce(const MmaDesc& d, MmaShared& sh, uint32_t ring,
                                         ActiveBlocks act, int64_t b, int64_t m0, int64_t w0) {
   constexpr int NB = BN / 64;               // B words per thread
@@ -305,7 +307,7 @@ __device__ __forceinline__ void produce(const MmaDesc& d, MmaShared& sh, uint32_
     a[1] = aw[1];
 #pragma unroll
     for (int i = 0; i < NB; ++i) bb[i] = bw[i];
-    for (int i = 0; i < kMmaStages && kb >= 0; ++i) kb = act.next();
+    for (int i = 0; i < STAGES && kb >= 0; ++i) kb = act.next();
     load(kb, aw, bw);
     bool use = true;
     if (!act.occa) {
@@ -355,11 +357,16 @@ __device__ __forceinline__ void produce(const MmaDesc& d, MmaShared& sh, uint32_
 }
 
 // One CTA per (problem, batch, 128-row tile of A, BN-column tile of B, K
-// chunk).  Warps 0-15: producers, then the epilogue (warp w reads TMEM lanes
-// 32 (w % 4) .. and columns BN / 4 (w / 4) ..).  Warp 16: TMEM allocation and,
-// in one lane, the products.
-__global__ void __launch_bounds__(kMmaThreads, 1)
+// chunk).  The first 4 STAGES warps: producers, then the epilogue (warp w reads
+// TMEM lanes 32 (w % 4) .. and columns BN / STAGES (w / 4) ..).  The last warp:
+// TMEM allocation and, in one lane, the products.
+// STAGES = 4: one CTA to an SM.  STAGES = 2: two, each with half the producers,
+// half the ring and half of TMEM, so that one's set-up, first block and
+// read-back (some 11K cycles, ten K blocks' worth) run under the other's.
+template <int STAGES>
+__global__ void __launch_bounds__(mma_threads(STAGES), 4 / STAGES)
 mma_bits_kernel(const MmaDesc* __restrict__ descs, const int64_t* __restrict__ cta0s, int nprob) {
+  constexpr int kProducers = 4 * STAGES;
   extern __shared__ uint8_t mma_raw[];
   uint8_t* smem =
       reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(mma_raw) + 1023) & ~uintptr_t(1023));
@@ -373,14 +380,14 @@ mma_bits_kernel(const MmaDesc* __restrict__ descs, const int64_t* __restrict__ c
     uint32_t* dst = reinterpret_cast<uint32_t*>(&sd);
     if (threadIdx.x < (int)(sizeof(MmaDesc) / 4)) dst[threadIdx.x] = src[threadIdx.x];
   }
-  if (warp == kMmaProducers) {
+  if (warp == kProducers) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_addr(&sh.tmem)),
                  "r"(kMmaTmemCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   } else if (threadIdx.x == 0) {
-    for (int s = 0; s < kMmaStages; ++s) {
+    for (int s = 0; s < STAGES; ++s) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;" ::"r"(smem_addr(&sh.full[s])) : "memory");
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&sh.empty[s])) : "memory");
     }
@@ -405,7 +412,7 @@ mma_bits_kernel(const MmaDesc* __restrict__ descs, const int64_t* __restrict__ c
   const int nk = (int)((d.K + kMmaBK - 1) / kMmaBK);
   const bool split = d.ksplit > 1;
   // every role walks the same sequence of K blocks, the j-th in stage
-  // j % kMmaStages
+  // j % STAGES
   ActiveBlocks act;
   const uint32_t* occ = reinterpret_cast<const uint32_t*>(d.occ) + b * (d.m_tiles + d.n_tiles) * d.kb_words;
   act.occa = d.occ ? occ + mt * d.kb_words : nullptr;
@@ -416,14 +423,14 @@ mma_bits_kernel(const MmaDesc* __restrict__ descs, const int64_t* __restrict__ c
   // stream until here
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
-  if (warp == kMmaProducers) {
+  if (warp == kProducers) {
     if (lane == 0) {
       const uint32_t idesc = f8_idesc(kMmaBM, BN);
       act.start();
       int issued = 0;
       for (int j = 0; act.next() >= 0; ++j) {
-        const int s = j % kMmaStages;
-        if (!bar_wait(&sh.full[s], (uint32_t)(j / kMmaStages) & 1u)) {
+        const int s = j % STAGES;
+        if (!bar_wait(&sh.full[s], (uint32_t)(j / STAGES) & 1u)) {
           sh.fail = 1;
           break;
         }
@@ -463,11 +470,11 @@ mma_bits_kernel(const MmaDesc* __restrict__ descs, const int64_t* __restrict__ c
     const int64_t m0 = mt * kMmaBM, w0 = nt * (BN / 64);
     const uint32_t ring = smem_addr(smem);
     if (d.counts) {
-      if (BN == 256) produce<256, true>(d, sh, ring, act, b, m0, w0);
-      else produce<128, true>(d, sh, ring, act, b, m0, w0);
+      if (BN == 256) produce<STAGES, 256, true>(d, sh, ring, act, b, m0, w0);
+      else produce<STAGES, 128, true>(d, sh, ring, act, b, m0, w0);
     } else {
-      if (BN == 256) produce<256, false>(d, sh, ring, act, b, m0, w0);
-      else produce<128, false>(d, sh, ring, act, b, m0, w0);
+      if (BN == 256) produce<STAGES, 256, false>(d, sh, ring, act, b, m0, w0);
+      else produce<STAGES, 128, false>(d, sh, ring, act, b, m0, w0);
     }
     const bool ok = bar_wait(&sh.accum, 0);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -478,7 +485,7 @@ mma_bits_kernel(const MmaDesc* __restrict__ descs, const int64_t* __restrict__ c
     const int ew = warp & 3, part = warp >> 2;
     const int64_t m = m0 + ew * 32 + lane;
     // a warp's columns, 32 at a time: the bits of half a result word
-    for (int c0 = part * (BN / 4); c0 < (part + 1) * (BN / 4); c0 += 32) {
+    for (int c0 = part * (BN / STAGES); c0 < (part + 1) * (BN / STAGES); c0 += 32) {
       uint32_t v[32];
       const uint32_t ta = tmem + ((uint32_t)(ew * 32) << 16) + (uint32_t)c0;
       if (none) {
@@ -527,7 +534,7 @@ mma_bits_kernel(const MmaDesc* __restrict__ descs, const int64_t* __restrict__ c
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (warp == kMmaProducers) {
+  if (warp == kProducers) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                  "r"(kMmaTmemCols)
@@ -631,7 +638,15 @@ cudaError_t launch_mma(const MmaDesc* d_descs, const int64_t* d_cta0, const int6
                        int64_t grid, int64_t occ_grid, cudaStream_t s) {
   if (nprob <= 0 || grid <= 0) return cudaSuccess;
   if (grid > 0x7fffffffLL || occ_grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  smem_limit(reinterpret_cast<const void*>(mma_bits_kernel), kMmaSmem);
+  // More CTAs than SMs: two to an SM (see the kernel).  Two against one, whole
+  // calls: an 8192^3 product of sparse plots (2048 CTAs) 82.6 -> 58.1 us, ternary 256
+  // (512 CTAs of two K blocks) 62.8 -> 53.8, 38 random networks 5660 -> 5560, 4096
+  // chains the same.  Up to 152 CTAs have an SM each, and all four producer groups
+  // serve one ring: a CTA's own chain is what such a launch waits for.
+  const bool pairs = grid > 152;
+  const auto kernel = pairs ? mma_bits_kernel<2> : mma_bits_kernel<4>;
+  const int stages = pairs ? 2 : 4;
+  smem_limit(reinterpret_cast<const void*>(kernel), mma_smem(stages));
   // programmatic dependent launches: the set-up overlaps the previous kernel
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -647,9 +662,9 @@ cudaError_t launch_mma(const MmaDesc* d_descs, const int64_t* d_cta0, const int6
     if (e != cudaSuccess) return e;
   }
   cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(kMmaThreads);
-  cfg.dynamicSmemBytes = kMmaSmem;
-  return cudaLaunchKernelEx(&cfg, mma_bits_kernel, d_descs, d_cta0, nprob);
+  cfg.blockDim = dim3(mma_threads(stages));
+  cfg.dynamicSmemBytes = mma_smem(stages);
+  return cudaLaunchKernelEx(&cfg, kernel, d_descs, d_cta0, nprob);
 }
 
 }  // namespace pa

@@ -159,3 +159,24 @@ def test_tile_edges(eng, orc, M, K, N, kind):
     check_same(got, orc.contract(orc.Arr(X, (0, 1)), orc.Arr(Y, (1, 2)), (0, 2), vres).data, f"{vres}")
     want = orc.contract_count(orc.Arr(X, (0, 1)), orc.Arr(Y, (1, 2)), (0, 2), vres)
     assert np.array_equal(cnt.cpu().numpy(), want.astype(np.int64)), f"counts {vres}"
+
+
+@pytest.mark.parametrize("nb,M,K,N", [(153, 1, 70, 64), (80, 129, 128, 100), (39, 130, 257, 300),
+                                      (20, 513, 400, 257), (80, 200, 4300, 129)])
+def test_more_tiles_than_sms(eng, orc, nb, M, K, N):
+    """Batched products of more tiles than the GPU has SMs, which run two to an
+    SM: one, two and more K blocks, ragged tiles, empty blocks; counts too."""
+    rng = np.random.default_rng(9500 + M + K + N)
+    density = 0.3 if K < 1000 else 0.02
+    X, Y = rand_bits(rng, (nb, M, K), density), rand_bits(rng, (nb, K, N), density)
+    X[::3, :, : K // 2] = 0
+    Y[1::3, K // 2:] = 0
+    X[2::9] = 0
+    vres = [M, K, N, nb]
+    xv, yv, keep = (3, 0, 1), (3, 1, 2), (3, 0, 2)
+    got = eng.contract(pack(X, xv), pack(Y, yv), keep)
+    cnt = eng.contract_count(pack(X, xv), pack(Y, yv), keep)
+    eng.sync()
+    want = np.matmul(X.astype(np.float32), Y.astype(np.float32))
+    check_same(got, (want > 0).astype(np.uint8), f"{vres}")
+    assert np.array_equal(cnt.cpu().numpy(), want.astype(np.int64)), f"counts {vres}"
