@@ -282,6 +282,103 @@ reshape_words_kernel(const ReshapeDesc* __restrict__ descs, const int64_t* __res
   else reshape_words<I, 1>(d, (I)rc.bid, (I)rc.nblk);
 }
 
+// Transpose of a 32 x 32 bit block in a thread's registers: x[i] is row i,
+// afterwards column i.  Recursive block swap: for block size s the rows k and
+// k + s (k & s == 0) exchange the columns c + s of row k with the columns c of
+// row k + s (c & s == 0); whole bytes by permutes, the rest by a shift and a
+// select each: 256 instructions for 32 blocks of a warp.
+__device__ __forceinline__ void transpose32(uint32_t (&x)[32]) {
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const uint32_t a = x[k], b = x[k + 16];
+    x[k] = __byte_perm(a, b, 0x5410);
+    x[k + 16] = __byte_perm(a, b, 0x7632);
+  }
+#pragma unroll
+  for (int k = 0; k < 32; ++k)
+    if (!(k & 8)) {
+      const uint32_t a = x[k], b = x[k + 8];
+      x[k] = __byte_perm(a, b, 0x6240);
+      x[k + 8] = __byte_perm(a, b, 0x7351);
+    }
+#pragma unroll
+  for (int s = 4; s >= 1; s >>= 1) {
+    const uint32_t m = s == 4 ? 0x0F0F0F0Fu : s == 2 ? 0x33333333u : 0x55555555u;
+#pragma unroll
+    for (int k = 0; k < 32; ++k)
+      if (!(k & s)) {
+        const uint32_t a = x[k], b = x[k + s];
+        x[k] = (a & m) | ((b << s) & ~m);
+        x[k + s] = ((a >> s) & m) | (b & ~m);
+      }
+  }
+}
+
+// Transpose mode.  A CTA tile is 64 TW values of L (TW output words) x 64 TW
+// values of J (TW input words) at one value of the other axes.  A thread takes a
+// 32 x 32 block: its 32 rows come straight from the input (a tile row is read by
+// 2 TW neighbouring lanes), are transposed in its registers and go to a shared
+// tile, from which the output rows are stored whole.  TW = 4 (256 x 256), or 8
+// where both axes have more than 256 values: rows of 512 bits are then read and
+// written whole instead of in 32-byte halves.  The shared tile is skewed by 16 / TW
+// words per 32 rows, which makes the block stores (32 rows apart) and the row
+// loads free of conflicts.  Index type I is 32-bit when every word and tile index
+// fits.  Bound by short accesses at the arrays' pitches.  With 32 x 32 blocks
+// transposed across a warp's lanes (five shuffles each) between two shared tiles,
+// L1 and shared memory were 77-82 % busy; 38
+// networks' whole replay 5.60 -> 5.21 ms.
+template <class I, int TW>
+__global__ void __launch_bounds__(4 * TW * TW)
+reshape_transpose_kernel(const ReshapeDesc* __restrict__ descs, const int64_t* __restrict__ cta0, int n) {
+  constexpr int kThreads = 4 * TW * TW, kSkew = 16 / TW;
+  __shared__ __align__(16) uint32_t tile32[64 * TW * 2 * TW + 2 * TW * kSkew];
+  __shared__ ReshapeDesc sd;
+  const RsCtx rc = rs_pick(descs, cta0, n, &sd);
+  const ReshapeDesc& d = sd;
+  const int tid = threadIdx.x;
+  const int c = tid % (2 * TW), br = tid / (2 * TW);  // 32 columns of J, 32 rows of L
+  const I tQ = (I)d.tQ, tR = (I)d.tR, t_in_L = (I)d.t_in_L, t_out_J = (I)d.t_out_J;
+  const I nJT = (tQ + 64 * TW - 1) / (64 * TW), nLT = (tR + 64 * TW - 1) / (64 * TW);
+  const I tiles = (I)d.n_other * nJT * nLT;
+  const I nblk = (I)rc.nblk;
+  for (I tile = (I)rc.bid; tile < tiles; tile += nblk) {
+    // (L tile, J tile, first input and output word of the other axes)
+    const I r = tile / nLT;
+    const I lt = tile - r * nLT;
+    I rest = r / nJT;
+    const I jt = r - rest * nJT;
+    I base_in = 0, base_out = 0;
+    for (int a = d.nu - 1; a >= 0; --a) {
+      const I res = (I)d.u_res[a], q = rest / res, v = rest - q * res;
+      rest = q;
+      base_in += v * (I)d.u_in[a];
+      base_out += v * (I)d.u_out[a];
+    }
+    const I jb = jt * TW + c / 2, L0 = lt * (64 * TW) + br * 32;
+    const bool in = jb * 64 < tQ;
+    uint32_t x[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i)
+      x[i] = in && L0 + i < tR
+                 ? __ldg(reinterpret_cast<const uint32_t*>(d.in + (base_in + (L0 + i) * t_in_L + jb)) + (c & 1))
+                 : 0u;
+    transpose32(x);
+    uint32_t* st = tile32 + c * (32 * 2 * TW + kSkew) + br;
+#pragma unroll
+    for (int i = 0; i < 32; ++i) st[i * (2 * TW)] = x[i];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const int idx = tid + kThreads * i, t = idx / TW, w = idx % TW;
+      const I J = jt * (64 * TW) + t, lw = lt * TW + w;
+      if (J < tQ && lw * 64 < tR)
+        d.out[base_out + J * t_out_J + lw] =
+            *reinterpret_cast<const uint64_t*>(tile32 + t * (2 * TW) + (t / 32) * kSkew + 2 * w);
+    }
+    __syncthreads();
+  }
+}
+
 // In-register transpose of 32 x 32 bit blocks held by one warp: lane l holds row
 // l; afterwards column l.  Recursive block swap: for block size s the rows r and
 // r + s (r & s == 0) exchange the columns c + s of row r with the columns c of
@@ -310,24 +407,14 @@ struct Transpose32 {
   }
 };
 
-// Transpose mode.  A CTA tile is 64 TW values of L (TW output words) x 64 TW
-// values of J (TW input words) at one value of the other axes: its input rows
-// are loaded into shared memory, transposed by warps in 32 x 32 blocks, and its
-// output rows stored.  TW = 4 (256 x 256), or 8 where both axes have more than
-// 256 values: rows of 512 bits are then read and written whole, 32 KB in one run
-// where the rows are neighbours, instead of in 32-byte halves.  Rows of the
-// shared tiles are padded by a word.  Index type I is 32-bit when every word and
-// tile index fits.  Bound by the latency of short accesses at the arrays'
-// pitches; 64-bit divisions (two thirds of 8570 warp instructions per tile) and
-// branching 64 x 64 block transposes bound it before: 38 networks' transposes
-// 1.88 -> 1.28 ms, with the wide tiles 1.12.
-template <class I, int TW>
-__global__ void __launch_bounds__(64 * TW)
-reshape_transpose_kernel(const ReshapeDesc* __restrict__ descs, const int64_t* __restrict__ cta0, int n) {
-  constexpr int kThreads = 64 * TW, kPad = TW + 1;  // a thread per value of an axis
-  extern __shared__ uint64_t tr_smem[];
-  uint64_t* s_in = tr_smem;
-  uint64_t* s_out = tr_smem + 64 * TW * kPad;
+// Transposes of few 256 x 256 tiles: a tile's 32 x 32 blocks go to warps, a lane
+// per row, so that 256 threads share a tile's loads and stores and no thread has
+// a chain of 32 rows of its own.
+__global__ void __launch_bounds__(256)
+reshape_transpose_few_kernel(const ReshapeDesc* __restrict__ descs, const int64_t* __restrict__ cta0, int n) {
+  using I = uint32_t;
+  constexpr int TW = 4, kThreads = 64 * TW, kPad = TW + 1;  // a thread per value of an axis
+  __shared__ uint64_t s_in[64 * TW * kPad], s_out[64 * TW * kPad];
   __shared__ ReshapeDesc sd;
   const RsCtx rc = rs_pick(descs, cta0, n, &sd);
   const ReshapeDesc& d = sd;
@@ -399,9 +486,13 @@ reshape_transpose_kernel(const ReshapeDesc* __restrict__ descs, const int64_t* _
   }
 }
 
-// Words of a transpose's tile per side, and the bytes of its two shared tiles.
+// Up to two tiles per SM the launch lasts as long as one tile does (75^3 arrays, 75
+// tiles: 56.0 us per solve against 56.8); more tiles are bound by L1 and shared
+// memory, where a block per thread is the cheaper way.
+constexpr int64_t kFewTiles = 304;
+
+// Words of a transpose's tile per side.
 int transpose_tw(const ReshapeDesc& d) { return d.tQ > 256 && d.tR > 256 ? 8 : 4; }
-constexpr size_t transpose_smem(int tw) { return (size_t)2 * 64 * tw * (tw + 1) * 8; }
 int64_t transpose_tiles(const ReshapeDesc& d) {
   const int64_t side = 64 * transpose_tw(d);
   return d.n_other * ((d.tQ + side - 1) / side) * ((d.tR + side - 1) / side);
@@ -449,17 +540,20 @@ void launch_reshape(const ReshapeDesc* d_descs, const int64_t* d_cta0, int n, in
   if (n <= 0 || grid <= 0) return;
   switch (kind) {
     case kRsTranspose32:
+      if (grid <= kFewTiles) {
+        reshape_transpose_few_kernel<<<(unsigned)grid, 256, 0, s>>>(d_descs, d_cta0, n);
+        break;
+      }
       reshape_transpose_kernel<uint32_t, 4>
-          <<<(unsigned)grid, 256, transpose_smem(4), s>>>(d_descs, d_cta0, n);
+          <<<(unsigned)grid, 64, 0, s>>>(d_descs, d_cta0, n);
       break;
     case kRsTranspose32Wide:
-      smem_limit(reinterpret_cast<const void*>(reshape_transpose_kernel<uint32_t, 8>), transpose_smem(8));
       reshape_transpose_kernel<uint32_t, 8>
-          <<<(unsigned)grid, 512, transpose_smem(8), s>>>(d_descs, d_cta0, n);
+          <<<(unsigned)grid, 256, 0, s>>>(d_descs, d_cta0, n);
       break;
     case kRsTranspose64:
       reshape_transpose_kernel<uint64_t, 4>
-          <<<(unsigned)grid, 256, transpose_smem(4), s>>>(d_descs, d_cta0, n);
+          <<<(unsigned)grid, 64, 0, s>>>(d_descs, d_cta0, n);
       break;
     case kRsWords32:
       reshape_words_kernel<uint32_t><<<(unsigned)grid, 256, 0, s>>>(d_descs, d_cta0, n);

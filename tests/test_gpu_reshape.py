@@ -55,3 +55,16 @@ def test_reshaped_clusters(eng, orc, case, density):
     got = eng.contract(pack(X, xv), pack(Y, yv), keep)
     eng.sync()
     check_same(got, want, str(CASES[case]))
+
+
+@pytest.mark.parametrize("vres", [(310, 70, 65), (320, 33, 257), (305, 256, 64), (306, 1, 130),
+                                  (40, 300, 800)])
+def test_many_transposes(eng, orc, vres):
+    """Transposes of more tiles than the GPU takes at once (a 32 x 32 block per
+    thread), and of wide tiles: every edge of blocks, words and tiles."""
+    rng = np.random.default_rng(8900 + sum(vres))
+    X, Y = rand_bits(rng, vres, 0.4), rand_bits(rng, vres, 0.6)
+    want = orc.contract(orc.Arr(X, (0, 1, 2)), orc.Arr(Y, (0, 1, 2)), (0, 2, 1), list(vres)).data
+    got = eng.contract(pack(X, (0, 1, 2)), pack(Y, (0, 1, 2)), (0, 2, 1))
+    eng.sync()
+    check_same(got, want, str(vres))
