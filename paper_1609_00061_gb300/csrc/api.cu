@@ -432,8 +432,8 @@ void flush_reshapes(Builder& bd) {
       if (reshape_kind(d) == kind && reshape_units(d) > 0) group.push_back(d);
     // Pieces of work per block: one, but up to 8 transpose tiles when the launch
     // has many, so that a block's start (finding its problem, the descriptor, the
-    // first loads) is paid once and a tile's loads overlap the tile before (426 ->
-    // 369 us for the first level of 38 networks; the other kinds lost 16 %)
+    // first loads) is paid once (426 -> 369 us for the first level of 38 networks,
+    // with a row per lane; the other kinds lost 16 %)
     int64_t total = 0, per = 1;
     for (const ReshapeDesc& d : group) total += reshape_units(d);
     if (kind >= kRsTranspose32)

@@ -325,8 +325,8 @@ __device__ __forceinline__ void transpose32(uint32_t (&x)[32]) {
 // loads free of conflicts.  Index type I is 32-bit when every word and tile index
 // fits.  Bound by short accesses at the arrays' pitches.  With 32 x 32 blocks
 // transposed across a warp's lanes (five shuffles each) between two shared tiles,
-// L1 and shared memory were 77-82 % busy; 38
-// networks' whole replay 5.60 -> 5.21 ms.
+// L1 and shared memory were 77-82 % busy (ncu); 38 networks' whole replay 5.60 ->
+// 5.21 ms.
 template <class I, int TW>
 __global__ void __launch_bounds__(4 * TW * TW)
 reshape_transpose_kernel(const ReshapeDesc* __restrict__ descs, const int64_t* __restrict__ cta0, int n) {
