@@ -22,15 +22,13 @@ struct Mlp {
   int cap = 0;                  // samples the activation buffers hold
   std::vector<float*> acts;     // per hidden layer its output, [l + 1]
   std::vector<float*> deltas;   // per layer the loss's derivative by its sums
-  float* scratch = nullptr;     // blocks' squared errors [cap], parts of the gradients
+  float* sq_err = nullptr;      // the samples' squared errors [cap]
 
   Mlp(int nin, int hidden, int nlayers);
   ~Mlp();
   cudaError_t alloc_params();
   cudaError_t reserve(int n);
   void free_acts();
-  // parts the samples of a gradient may be split into (bounded scratch)
-  int max_parts() const;
   // y[n] = net(x[n][nin]) (device pointers)
   cudaError_t forward(const float* x, int n, float* y, cudaStream_t s);
   // forward, loss 0.5 mean (y - t)^2 into *loss, gradient into g
