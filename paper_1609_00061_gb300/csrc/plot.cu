@@ -19,8 +19,11 @@
 // (a_k scaled by delta^k, D fused multiply-adds per pixel).
 //
 // Error bound.  u = 2^-24, X_p >= |x_p| on port p's range (widened by three
-// pixels on the last port, which covers |y_c| + |t| for every word), and
+// pixels on the last port), and
 //   A = sum_e |c_e| prod_p X_p^e_p   (all exponents, the last port's included).
+// Every expansion is about the middle pixel (nb >> 1) of the nb pixels it serves,
+// so y_c +- t stays within one pixel of them, and |y_c| + |t| <= X of the last port
+// for every pixel that is decided.
 // Every quantity the kernel computes is a sum of rounded products of the
 // coefficients' monomials, so its error is at most (roundings on a monomial's
 // path) u A.  A monomial of total degree at most D meets: the rounding of c_e
@@ -644,10 +647,9 @@ plot_kernel(const PlotJob* __restrict__ jobs, int njobs, int gstride,
         const int nb = min(C == 1 ? 64 : 8, res_last - i0);  // <= 0: padding past the row
         uint64_t bits = 0;
         if (nb > 0) {
-          // expansion about a pixel of the row near the piece's middle; a piece
-          // cut by the row's end is also evaluated past it, those bits dropped
-          const int half = C == 1 ? 32 : 4;
-          const int ic = nb > half ? half : C == 1 && nb > 16 ? 16 : nb >> 1;
+          // expanded about the piece's own middle, as the bound assumes; the
+          // offsets run past a piece that the row's end cuts, those bits dropped
+          const int ic = nb >> 1;
           float a[kG];
           expand(r, i0 + ic, a);
           float closest = INFINITY;
@@ -660,13 +662,13 @@ plot_kernel(const PlotJob* __restrict__ jobs, int njobs, int gstride,
               lo = eval_pixels<DS, false, 32, -32>(a, D, eps, &closest);
               hi = eval_pixels<DS, false, 32, 0>(a, D, eps, &closest);
             }
-            bits = ((uint64_t)hi << 32) | lo;
+            bits = (((uint64_t)hi << 32) | lo) >> (32 - ic);
           } else if (C == 1 && nb > 16) {
-            bits = eq ? eval_pixels<DS, true, 32, -16>(a, D, eps, &closest)
-                      : eval_pixels<DS, false, 32, -16>(a, D, eps, &closest);
+            bits = (eq ? eval_pixels<DS, true, 32, -16>(a, D, eps, &closest)
+                       : eval_pixels<DS, false, 32, -16>(a, D, eps, &closest)) >> (16 - ic);
           } else if (C == 8 && nb > 4) {
-            bits = eq ? eval_pixels<DS, true, 8, -4>(a, D, eps, &closest)
-                      : eval_pixels<DS, false, 8, -4>(a, D, eps, &closest);
+            bits = (eq ? eval_pixels<DS, true, 8, -4>(a, D, eps, &closest)
+                       : eval_pixels<DS, false, 8, -4>(a, D, eps, &closest)) >> (4 - ic);
           } else {
             closest = 0.0f;  // few pixels: left to phase 4
           }

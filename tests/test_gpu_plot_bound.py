@@ -1,0 +1,57 @@
+"""The plot kernel's FP32 error bound where it is widest against what the kernel
+evaluates.  Every plot equals the oracle's bit for bit (the FP64 decision has no
+tolerance)."""
+import itertools
+
+import numpy as np
+import pytest
+
+import paper_1609_00061_gb300 as pa
+from paper_1609_00061_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def eng():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    e = pa.Engine(0)
+    yield e
+    e.close()
+
+
+def check(eng, orc, rel, axes, what):
+    got = eng.plot(rel, axes)
+    want = orc.plot_relation(rel, axes).data
+    diff = int((got.to_numpy() != want).sum())
+    assert diff == 0, f"{what}: {diff} of {want.size} pixels differ"
+    assert got.padding_clean(), what
+
+
+# Rows that end inside a word, in plots with more undecided words per block than
+# threads take piece by piece: the word's pixels are evaluated about its middle.
+@pytest.mark.parametrize("res", [17, 20, 31, 33, 36, 40, 48, 63, 81, 97])
+@pytest.mark.parametrize("degree", [3, 6, 8, 12, 16])
+def test_partial_words_at_high_degree(eng, orc, res, degree):
+    rng = W.SplitMix64(8000 + 32 * res + degree)
+    for box, eps in ((3.0, 0.05), (1.0, 0.05), (1.0, 0.01)):
+        for one_sided in (False, True):
+            axes = [(-box, box, 256), (0.0 if one_sided else -box, box, res)]
+            for kind in (W.KIND_EQ, W.KIND_LE, W.KIND_LT):
+                rel = W.Relation((0, 1), degree, rng.normal(W.coeff_count(2, degree)), kind, eps)
+                check(eng, orc, rel, axes, f"box {box} one-sided {one_sided} kind {kind}")
+
+
+# The same in pieces of 8 pixels, the last of which ends inside (few rows).
+@pytest.mark.parametrize("res", [5, 6, 7, 13, 21, 38, 71])
+@pytest.mark.parametrize("degree", [3, 8, 16])
+def test_partial_pieces_at_high_degree(eng, orc, res, degree):
+    rng = W.SplitMix64(8100 + 32 * res + degree)
+    for rows in (3, 24):
+        for box in (1.0, 3.0):
+            axes = [(-box, box, rows), (-box, box, res)]
+            for kind in (W.KIND_EQ, W.KIND_LT):
+                rel = W.Relation((0, 1), degree, rng.normal(W.coeff_count(2, degree)), kind, 0.05)
+                check(eng, orc, rel, axes, f"rows {rows} box {box} kind {kind}")
