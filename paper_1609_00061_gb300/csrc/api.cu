@@ -1243,8 +1243,9 @@ void plot_filter(PlotJob& J, const pa_relation& r, const pa_axis* axes,
     ok = ok && X[p] < 1e18 && d > 1e-18;
   }
   // A = sum |c_e| prod X_p^e_p over the monomials in nest order (the last port
-  // outermost, exponents ascending)
-  double A = 0.0;
+  // outermost, exponents ascending).  The same with max(X_p, 1) bounds every
+  // partial sum and coefficient on the way to f.
+  double A = 0.0, reach = 0.0;
   size_t at = 0;
   int e[kMaxDim] = {};
   for (;;) {
@@ -1259,16 +1260,20 @@ void plot_filter(PlotJob& J, const pa_relation& r, const pa_axis* axes,
       ++e[p + 1];
       continue;
     }
-    double m = fabs(r.coeffs[ord[at++]]);
+    double m = fabs(r.coeffs[ord[at++]]), big = m;
     for (int p = 0; p < n; ++p)
-      for (int k = 0; k < e[p]; ++k) m *= X[p];
+      for (int k = 0; k < e[p]; ++k) {
+        m *= X[p];
+        big *= fmax(X[p], 1.0);
+      }
     A += m;
+    reach += big;
     ++e[0];
   }
   const double K = 7.0 * D + n * (D + 1.0) + 14.0;
   const double underflow = 0x1p-140 * (double)ord.size() * pow(xmax, D) + 1e-30;
   const double B = 1.05 * K * 0x1p-24 * A + 0x1p-21 * (double)J.eps32 + underflow;
-  ok = ok && at == ord.size() && A < 1e30 && pow(xmax, D) < 1e30 && B < 1e30;
+  ok = ok && at == ord.size() && reach < 1e30 && pow(xmax, D) < 1e30 && B < 1e30;
   J.filter = ok ? 1 : 0;
   J.bound = ok ? (float)(B * (1.0 + 0x1p-20)) : INFINITY;
   J.dabs = (float)(1.01 * J.delta[n - 1]);

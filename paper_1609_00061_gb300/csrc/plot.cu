@@ -40,7 +40,8 @@
 // The whole-word test keeps 3 B.  Pixels within B, some per cent of the band
 // edges on a fine grid, are collected and decided by the FP64 evaluation of
 // pa.h from scratch: the result is the FP64 decision, bit for bit.  A relation
-// whose A is not comfortably inside the FP32 range takes FP64 at every pixel.
+// whose coefficients or partial sums are not comfortably inside the FP32 range
+// takes FP64 at every pixel.
 #include <float.h>
 
 #include <algorithm>
@@ -364,8 +365,16 @@ __device__ __forceinline__ float excess(const float (&a)[N], int D, float s, flo
   return __fsub_rn(EQ ? fabsf(f) : f, eps);
 }
 
+// The smaller of two values, NaN when either is.
+__device__ __forceinline__ float min_nan(float a, float b) {
+  float r;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
 // P pixels (8 or 32) at offsets s0, s0 + 1, ...: bit b of the result is the
-// sign of pixel b's excess (1: on), *closest the smallest |excess|.
+// sign of pixel b's excess (1: on), *closest the smallest |excess|, or NaN (no
+// pixel of the word is taken as decided then).
 template <int DS, bool EQ, int P, int S0, int N>
 __device__ __forceinline__ uint32_t eval_pixels(const float (&a)[N], int D, float eps,
                                                 float* closest) {
@@ -375,7 +384,7 @@ __device__ __forceinline__ uint32_t eval_pixels(const float (&a)[N], int D, floa
   for (int b = P - 1; b >= 0; --b) {
     const float e = excess<DS, EQ>(a, D, (float)(S0 + b), eps);
     m = __funnelshift_l(__float_as_uint(e), m, 1);
-    c = fminf(c, fabsf(e));
+    c = min_nan(c, fabsf(e));
   }
   *closest = c;
   return m;

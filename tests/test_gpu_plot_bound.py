@@ -55,3 +55,32 @@ def test_partial_pieces_at_high_degree(eng, orc, res, degree):
             for kind in (W.KIND_EQ, W.KIND_LT):
                 rel = W.Relation((0, 1), degree, rng.normal(W.coeff_count(2, degree)), kind, 0.05)
                 check(eng, orc, rel, axes, f"rows {rows} box {box} kind {kind}")
+
+
+def small_box(rng, box, degree, shape, kind, eps):
+    """N(0,1) coefficients in units of the box: every monomial counts on it."""
+    n = len(shape)
+    c = rng.normal(W.coeff_count(n, degree))
+    axes = [(-box, box, r) for r in shape]
+    return W.Relation(tuple(range(n)), degree, c / box ** total_degrees(n, degree), kind, eps), axes
+
+
+def total_degrees(n, degree):
+    """Total degree of every coefficient (graded order)."""
+    out = []
+    for d in range(degree + 1):
+        out += [d] * (W.coeff_count(n, d) - (W.coeff_count(n, d - 1) if d else 0))
+    return np.array(out, dtype=np.float64)
+
+
+# Coefficients beyond FP32's range on a box so small that f is of order one.
+@pytest.mark.parametrize("box,degree", [(1e-10, 4), (1e-12, 3), (1e-20, 2), (1e-3, 16), (1e-40, 1)])
+def test_coefficients_beyond_fp32(eng, orc, box, degree):
+    rng = W.SplitMix64(8200 + degree)
+    for kind in (W.KIND_EQ, W.KIND_LE, W.KIND_LT):
+        for shape in ((300, 333), (31, 2000)):
+            for eps in (-1.0, 0.01):
+                rel, axes = small_box(rng, box, degree, shape, kind, eps)
+                check(eng, orc, rel, axes, f"{shape} kind {kind} eps {eps}")
+    rel, axes = small_box(rng, box, degree, (17, 19, 70), W.KIND_EQ, -1.0)
+    check(eng, orc, rel, axes, "3 ports")
