@@ -1220,15 +1220,22 @@ std::vector<BitArr> plot_all(Builder& bd, const std::vector<PlotReq>& reqs) {
   return plots;
 }
 
-// The FP32 filter of one plot job (plot.cu): its error bound B, or no filter
-// when a port shares its variable with another, an axis is too long for exact
-// FP32 pixel indices or the magnitudes leave FP32's comfortable range.
+// The FP32 filter of one plot job (plot.cu): its scaled ports and coefficients (c32,
+// nest order) and its error bound B, or no filter when a port shares its variable
+// with another, an axis is too long for exact FP32 pixel indices or the magnitudes
+// leave the range in which the FP64 evaluation itself neither overflows nor loses
+// anything by underflow.
+//
+// Everything is in units of powers of two, which changes no rounding: port p in
+// 2^k_p >= X_p, the greatest coordinate that an expansion reaches, and f in 2^q
+// >= A = sum |c_e| prod X_p^e_p.  Coordinates are at most 1, coefficients at most
+// 2^D and A at most 1 then, whatever the box and the coefficients are.
 void plot_filter(PlotJob& J, const pa_relation& r, const pa_axis* axes,
-                 const std::vector<int64_t>& ord) {
+                 const std::vector<int64_t>& ord, std::vector<float>& c32) {
   const int n = r.arity, D = r.degree;
-  J.eps32 = (float)J.eps;
-  bool ok = J.ndim == n && isfinite(J.eps32);
+  bool ok = J.ndim == n;
   double X[kMaxDim], xmax = 1.0;
+  int k[kMaxDim];
   for (int p = 0; p < n; ++p) {
     const pa_axis& ax = axes[r.vars[p]];
     const double d = J.delta[p];
@@ -1236,16 +1243,19 @@ void plot_filter(PlotJob& J, const pa_relation& r, const pa_axis* axes,
     // the last port's expansions reach a few pixels past the range
     X[p] = fmax(fabs(ax.lo), fabs(ax.hi)) * (1.0 + 0x1p-20) + (p == n - 1 ? 3.0 * d : 0.0);
     xmax = fmax(xmax, X[p]);
-    J.lo_hi[p] = (float)ax.lo;
-    J.lo_lo[p] = (float)(ax.lo - (double)J.lo_hi[p]);
-    J.d_hi[p] = (float)d;
-    J.d_lo[p] = (float)(d - (double)J.d_hi[p]);
-    ok = ok && X[p] < 1e18 && d > 1e-18;
+    frexp(X[p], &k[p]);
+    const double lo = ldexp(ax.lo, -k[p]), ds = ldexp(d, -k[p]);
+    J.lo_hi[p] = (float)lo;
+    J.lo_lo[p] = (float)(lo - (double)J.lo_hi[p]);
+    J.d_hi[p] = (float)ds;
+    J.d_lo[p] = (float)(ds - (double)J.d_hi[p]);
+    ok = ok && X[p] < 1e18 && ds > 0x1p-60;
   }
-  // A = sum |c_e| prod X_p^e_p over the monomials in nest order (the last port
-  // outermost, exponents ascending).  The same with max(X_p, 1) bounds every
-  // partial sum and coefficient on the way to f.
+  // A over the monomials in nest order (the last port outermost, exponents
+  // ascending).  The same with max(X_p, 1) bounds every partial sum of the FP64
+  // evaluation.
   double A = 0.0, reach = 0.0;
+  std::vector<int> unit(ord.size());  // per coefficient: sum of e_p k_p
   size_t at = 0;
   int e[kMaxDim] = {};
   for (;;) {
@@ -1260,23 +1270,35 @@ void plot_filter(PlotJob& J, const pa_relation& r, const pa_axis* axes,
       ++e[p + 1];
       continue;
     }
-    double m = fabs(r.coeffs[ord[at++]]), big = m;
+    double m = fabs(r.coeffs[ord[at]]), big = m;
+    int u = 0;
     for (int p = 0; p < n; ++p)
-      for (int k = 0; k < e[p]; ++k) {
+      for (int j = 0; j < e[p]; ++j) {
         m *= X[p];
         big *= fmax(X[p], 1.0);
+        u += k[p];
       }
+    unit[at++] = u;
     A += m;
     reach += big;
     ++e[0];
   }
+  // FP64: nothing overflows, and what underflows (2^-1074 each of up to 2^22
+  // operations, times at most reach and the powers of a coordinate) stays below
+  // 2^-60 A
+  ok = ok && at == ord.size() && reach < 1e300 &&
+       (reach == 0.0 || fmax(reach, 1.0) * 0x1p-990 * pow(xmax, D) <= A);
+  int q = 0;
+  frexp(A, &q);
+  c32.assign(ord.size(), 0.0f);
+  for (size_t j = 0; ok && j < ord.size(); ++j) c32[j] = (float)ldexp(r.coeffs[ord[j]], unit[j] - q);
+  J.eps32 = (float)ldexp(J.eps, -q);
   const double K = 7.0 * D + n * (D + 1.0) + 14.0;
-  const double underflow = 0x1p-140 * (double)ord.size() * pow(xmax, D) + 1e-30;
-  const double B = 1.05 * K * 0x1p-24 * A + 0x1p-21 * (double)J.eps32 + underflow;
-  ok = ok && at == ord.size() && reach < 1e30 && pow(xmax, D) < 1e30 && B < 1e30;
+  const double B = 1.05 * K * 0x1p-24 * ldexp(A, -q) + 0x1p-21 * (double)J.eps32 + 0x1p-48;
+  ok = ok && isfinite(J.eps32);
   J.filter = ok ? 1 : 0;
   J.bound = ok ? (float)(B * (1.0 + 0x1p-20)) : INFINITY;
-  J.dabs = (float)(1.01 * J.delta[n - 1]);
+  J.dabs = (float)(1.01 * ldexp(J.delta[n - 1], -k[n - 1]));
 }
 
 // The polynomial relations' plots in one launch.
@@ -1324,13 +1346,8 @@ std::vector<BitArr> plot_poly(Builder& bd, const std::vector<PlotReq>& reqs) {
     std::vector<int64_t>& ord = orders[{r.arity, r.degree}];
     if (ord.empty()) ord = nest_order(r.arity, r.degree);
     nc.resize(ord.size());
-    nc32.resize(ord.size());
-    for (size_t k = 0; k < ord.size(); ++k) {
-      nc[k] = r.coeffs[ord[k]];
-      nc32[k] = (float)nc[k];
-    }
+    for (size_t k = 0; k < ord.size(); ++k) nc[k] = r.coeffs[ord[k]];
     coeff_off[i] = bd.put(nc.data(), nc.size());
-    c32_off[i] = bd.put(nc32.data(), nc32.size());
 
     PlotJob& J = jobs[i];
     memset(&J, 0, sizeof J);
@@ -1350,7 +1367,8 @@ std::vector<BitArr> plot_poly(Builder& bd, const std::vector<PlotReq>& reqs) {
     J.nrows = a.nrows();
     J.row_words = a.row_words();
     J.eps = relation_eps(r, axes);
-    plot_filter(J, r, axes, ord);
+    plot_filter(J, r, axes, ord, nc32);
+    c32_off[i] = bd.put(nc32.data(), nc32.size());
     J.rows_per_tile = (int32_t)std::max<int64_t>(
         1, std::min<int64_t>(1024, (tile_words + J.row_words - 1) / J.row_words));
     J.tile0 = tiles;

@@ -52,11 +52,12 @@ __device__ __forceinline__ int find_entry(F&& first, int n, int64_t block) {
 // rounded on both, so the value is the one pa.h defines).
 struct PlotJob {
   const double* coeffs;             // device, nest order
-  const float* c32;                 // the same rounded to FP32 (filtered jobs)
+  // filtered jobs: ports in units of 2^k_p and f in units of 2^q (plot.cu)
+  const float* c32;                 // the coefficients in those units, rounded to FP32
   uint64_t* out;                    // device, pa_array layout
   double lo[kMaxDim];               // per port: range start of its variable
   double delta[kMaxDim];            // per port: pixel width of its variable
-  float lo_hi[kMaxDim], lo_lo[kMaxDim];  // lo and delta as sums of two floats
+  float lo_hi[kMaxDim], lo_lo[kMaxDim];  // lo and delta in units of the port, as sums of two floats
   float d_hi[kMaxDim], d_lo[kMaxDim];
   int64_t nrows;                    // rows = product of all but the last array axis
   int64_t row_words;                // ceil(res_last / 64)
@@ -68,9 +69,9 @@ struct PlotJob {
   int32_t res[kMaxDim];             // array axis resolutions
   int32_t port_axis[kMaxDim];       // port -> array axis
   double eps;
-  float eps32;                      // eps rounded to FP32
+  float eps32;                      // eps in units of f, rounded to FP32
   float bound;                      // B: FP32 against FP64, eps rounding included (plot.cu)
-  float dabs;                       // 1.01 x the last port's pixel width
+  float dabs;                       // 1.01 x the last port's pixel width in its unit
 };
 
 // One expression relation to plot (expr.cu): the postfix program and its

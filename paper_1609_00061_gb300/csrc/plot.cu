@@ -18,6 +18,12 @@
 // evaluates its pixels as polynomials in the integer offset s = (y - y_c) / delta
 // (a_k scaled by delta^k, D fused multiply-adds per pixel).
 //
+// Units.  The filter holds coordinates in units of powers of two, x_p = 2^k_p z_p
+// with 2^k_p >= X_p, and f in units of 2^q >= A (X and A below), folded into the
+// coefficients on the host.  No rounding changes by that, but |z_p| <= 1 and
+// |c_e| <= 2^D whatever the box and the coefficients are, so that nothing leaves
+// FP32's range.
+//
 // Error bound.  u = 2^-24, X_p >= |x_p| on port p's range (widened by three
 // pixels on the last port), and
 //   A = sum_e |c_e| prod_p X_p^e_p   (all exponents, the last port's included).
@@ -32,16 +38,20 @@
 // most D + 1 roundings of sums per port, D + 1 in the synthetic division, one
 // per factor in the scaling by delta^k and D + 1 in the final Horner sum.
 // Together less than K = 7 D + n (D + 1) + 14 for n ports.  The FP64 value's own error
-// (the same counts of 2^-53) is covered by the factor 1.05, so with
-//   B = 1.05 K u A + 2^-21 eps + underflow
-// (eps is rounded to FP32; a product that underflows loses at most 2^-149,
-// times powers of the X_p) the FP64 decision equals the sign of |f32| - eps
+// (the same counts of 2^-53) is covered by the factor 1.05.
+// Underflow: a product that underflows loses at most 2^-150.  Coordinates being at
+// most 1, a loss before the expansion grows by no more than 2^D (coefficients) and
+// 3^D (expansion and offsets), so the up to 2^22 of them stay below 2^-80.  One in
+// delta^k is multiplied by a_k <= 2^D and, in the Horner sum, by s^k <= 33^k: below
+// 2^-51 for D = 16.  With f in units of 2^q (A between 1/2 and 1) and
+//   B = 1.05 K u A + 2^-21 eps + 2^-48
+// (eps is rounded to FP32) the FP64 decision equals the sign of |f32| - eps
 // (f32 - eps for PA_LE / PA_LT) whenever that value exceeds B in magnitude.
 // The whole-word test keeps 3 B.  Pixels within B, some per cent of the band
 // edges on a fine grid, are collected and decided by the FP64 evaluation of
 // pa.h from scratch: the result is the FP64 decision, bit for bit.  A relation
-// whose coefficients or partial sums are not comfortably inside the FP32 range
-// takes FP64 at every pixel.
+// for which FP64 itself might overflow or underflow on the way takes FP64 at every
+// pixel.
 #include <float.h>
 
 #include <algorithm>

@@ -84,3 +84,47 @@ def test_coefficients_beyond_fp32(eng, orc, box, degree):
                 check(eng, orc, rel, axes, f"{shape} kind {kind} eps {eps}")
     rel, axes = small_box(rng, box, degree, (17, 19, 70), W.KIND_EQ, -1.0)
     check(eng, orc, rel, axes, "3 ports")
+
+
+# Large coefficients within FP32's range on small boxes: powers of the pixel width
+# and of the coordinates fall below it.
+@pytest.mark.parametrize("box,degree", [(1e-9, 4), (1e-6, 5), (1e-2, 16), (0.1, 16), (1e-4, 8),
+                                        (1e-1, 12), (1e-7, 3)])
+def test_powers_below_fp32(eng, orc, box, degree):
+    rng = W.SplitMix64(8300 + degree)
+    for kind in (W.KIND_EQ, W.KIND_LE):
+        for shape in ((500, 333), (500, 64), (90, 1500)):
+            for eps in (-1.0, 0.01, 1e-4):
+                rel, axes = small_box(rng, box, degree, shape, kind, eps)
+                check(eng, orc, rel, axes, f"{shape} kind {kind} eps {eps}")
+    rel, axes = small_box(rng, box, min(degree, 6), (17, 19, 70), W.KIND_EQ, -1.0)
+    check(eng, orc, rel, axes, "3 ports")
+
+
+# Boxes of very different sizes on the ports, coefficients to match; values of f
+# far from one; plots in which every pixel, or none, is on.
+@pytest.mark.parametrize("boxes", [(1e-12, 1e6), (1e6, 1e-12), (1e15, 1e-15), (1e-3, 3e5, 1e-8), (1e17, 1e17)])
+@pytest.mark.parametrize("scale", [1.0, 1e-40, 1e60, 1e-200])
+def test_uneven_boxes_and_scales(eng, orc, boxes, scale):
+    n, degree = len(boxes), 3
+    rng = W.SplitMix64(8400 + int(np.log10(scale)))
+    c = rng.normal(W.coeff_count(n, degree)) * scale
+    for e in itertools.product(range(degree + 1), repeat=n):
+        if sum(e) <= degree:
+            c[orc.coeff_index(e, degree)] /= np.prod([b ** float(k) for b, k in zip(boxes, e)])
+    shape = (61, 190) if n == 2 else (9, 11, 140)
+    axes = [(-b, 0.9 * b, r) for b, r in zip(boxes, shape)]
+    for kind in (W.KIND_EQ, W.KIND_LT):
+        for eps in (-1.0, 0.0, 0.02 * scale, 1e30 * scale):
+            rel = W.Relation(tuple(range(n)), degree, c, kind, eps)
+            check(eng, orc, rel, axes, f"kind {kind} eps {eps}")
+
+
+# FP64 sums that overflow on the way make the pixel's value infinite: off.
+def test_fp64_overflow_on_the_way(eng, orc):
+    # port 0 innermost: c x0 overflows before the tiny x1 brings it back
+    axes = [(1e10, 2e10, 70), (1e-20, 2e-20, 70)]
+    c = np.zeros(W.coeff_count(2, 2))
+    c[orc.coeff_index((1, 1), 2)] = 1e300
+    for kind, eps in ((W.KIND_LE, 1e300), (W.KIND_EQ, 1e300), (W.KIND_LT, 2e290)):
+        check(eng, orc, W.Relation((0, 1), 2, c, kind, eps), axes, f"kind {kind}")
