@@ -17,6 +17,7 @@
 #include <mutex>
 
 #include "pa_internal.h"
+#include "row_walk.h"
 
 namespace pa {
 
@@ -771,7 +772,8 @@ __device__ __forceinline__ void rowor_rows(const RowOrDesc& d, const uint64_t* _
   // batches would run on a few of the warps, one after another)
   const int L = kw;  // at most 32: a K range is at most kRowOrMaxKc
   const int all_warps = (int)d.row_splits * nwarps;
-  const int R = min(32 / L, ((int)d.M + all_warps - 1) / all_warps);
+  const RowWalk walk(d.M, all_warps, L);
+  const int R = (int)walk.batch;
   // groups per row (gpr, a power of two) of a lookup round, rows per round and
   // rounds
   int gpr = 1;
@@ -783,8 +785,7 @@ __device__ __forceinline__ void rowor_rows(const RowOrDesc& d, const uint64_t* _
   // are spread out.  The A words of the next three batches are always in
   // flight while one is processed.
   const int gw = rs * nwarps + warp;
-  const int rstep = all_warps * R;
-  const int M = (int)d.M;
+  const uint32_t rstep = walk.step, M = walk.M;
   const int64_t arw = d.a_row_words;
   const int my_row = lane / L, my_word = lane - my_row * L;
   const bool busy = my_row < R;  // lanes past the last whole row are idle
@@ -793,7 +794,7 @@ __device__ __forceinline__ void rowor_rows(const RowOrDesc& d, const uint64_t* _
   const int cols = (int)min((int64_t)W, max((int64_t)0, Nw - n0 - W * lig));  // of this lane's words
   const bool vec = W == 2 && Nw % 2 == 0 && reinterpret_cast<uintptr_t>(d.C) % 16 == 0;
   const bool atomic = d.atomic != 0;
-  auto store = [&](int row, const Words<W>& w) {
+  auto store = [&](uint32_t row, const Words<W>& w) {
     uint64_t* c = cbase + (int64_t)row * Nw;
     if (atomic) {
 #pragma unroll
@@ -814,7 +815,7 @@ __device__ __forceinline__ void rowor_rows(const RowOrDesc& d, const uint64_t* _
       for (int k = 0; k < W; ++k) w.v[k] |= __shfl_xor_sync(0xffffffffu, w.v[k], o);
   };
   const uint64_t* __restrict__ abase = d.A + (b * d.M) * arw + kw0 + my_word;
-  int lrow = gw * R + my_row;  // row of the next batch to fetch
+  uint32_t lrow = (uint32_t)(gw * R + my_row);  // row of the next batch to fetch
   auto fetch = [&]() -> uint64_t {
     const uint64_t v = (busy && lrow < M) ? __ldg(abase + (int64_t)lrow * arw) : 0ull;
     lrow += rstep;
@@ -828,7 +829,8 @@ __device__ __forceinline__ void rowor_rows(const RowOrDesc& d, const uint64_t* _
   // bits inside the K range
   const int base = (kw0 + my_word) * 64 - (int)k0;
   const uint64_t in_range = base + 64 <= kc_len ? ~0ull : base >= kc_len ? 0ull : (1ull << (kc_len - base)) - 1ull;
-  for (int row0 = gw * R; row0 < M; row0 += rstep) {
+  for (uint32_t row0 = (uint32_t)(gw * R); row0 < M; row0 += rstep) {
+    const int live = (int)min((uint32_t)R, M - row0);  // rows of this batch
     uint64_t a = pre0;
     pre0 = pre1;
     pre1 = pre2;
@@ -909,7 +911,7 @@ __device__ __forceinline__ void rowor_rows(const RowOrDesc& d, const uint64_t* _
           }
           __syncwarp();
           combine(w, GL * gpr);
-          if (sub == 0 && r < R && row0 + r < M) store(row0 + r, w);
+          if (sub == 0 && r < live) store(row0 + r, w);
         }
       } else {
         // more blocks than the list holds: row by row, in windows of the list;
@@ -941,12 +943,11 @@ __device__ __forceinline__ void rowor_rows(const RowOrDesc& d, const uint64_t* _
             __syncwarp();
           }
           combine(w, 32);
-          if (grp == 0 && row0 + r < M) store(row0 + r, w);
+          if (grp == 0 && r < live) store(row0 + r, w);
         }
       }
     } else if (!atomic) {
-      for (int r = grp; r < R; r += P)
-        if (row0 + r < M) store(row0 + r, zero);  // nothing selected: zero rows
+      for (int r = grp; r < live; r += P) store(row0 + r, zero);  // nothing selected: zero rows
     }
   }
 }
