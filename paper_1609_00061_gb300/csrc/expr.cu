@@ -20,11 +20,12 @@
 //     it give and set a flag; the others are NaN, which stays NaN through every
 //     operation but pow (then: any value) and turns the pixel off.  A run is only
 //     decided "on" without the flag.
-// Blocks test whole words (64 pixels), then the 8-pixel pieces of the words left,
+// Blocks test whole words (64 pixels; not on small grids), then the 8-pixel pieces of
+// the words left,
 // then evaluate the pieces left with eight lanes each.  What bounds it: the FP64
-// pipe on the pieces left, and the interpreter's instructions.  Three 2048^2
-// plots of the butterfly system 1456 -> 85 us, three 75^3 plots 185 -> 34 us
-// (ncu, cold; FP64 at every pixel before).
+// pipe on the pieces left, and the interpreter's instructions.  Whole solves against
+// FP64 at every pixel: butterfly at 2048 px 1523 -> 113 us, 3-D arrays at 75 px
+// 248 -> 55.
 #include <float.h>
 #include <math.h>
 
@@ -270,19 +271,25 @@ __device__ __forceinline__ int decide_run(const Place& P, int i0, int i1) {
   return (!bad && hi < J.eps) ? 2 : 0;
 }
 
-constexpr int kExprThreads = 256;
-constexpr int kExprWords = 256;  // most words per block
+constexpr int kExprThreads = 128;
+constexpr int kExprWords = 128;  // most words per block
 
+// by_words: whole words are tested first; else the 8-pixel pieces of every word.
 __global__ void __launch_bounds__(kExprThreads)
-plot_expr_kernel(const ExprJob* __restrict__ jobs, int njobs, int64_t total_words, int words) {
+plot_expr_kernel(const ExprJob* __restrict__ jobs, int njobs, int64_t total_words, int words, bool by_words) {
   __shared__ uint16_t wlist[kExprWords], plist[8 * kExprWords];
   __shared__ int s_w, s_p;
   const int tid = threadIdx.x;
-  if (tid == 0) s_w = s_p = 0;
-  __syncthreads();
   const int64_t w0 = (int64_t)blockIdx.x * words;
-  // whole words
-  if (tid < words && w0 + tid < total_words) {
+  const int mine = (int)min((int64_t)words, total_words - w0);  // words of this block
+  if (tid == 0) {
+    s_w = by_words ? 0 : mine;
+    s_p = 0;
+  }
+  __syncthreads();
+  if (!by_words) {
+    if (tid < mine) wlist[tid] = (uint16_t)tid;
+  } else if (tid < mine) {
     Place P;
     locate(jobs, njobs, w0 + tid, P);
     const int i0 = P.wi * 64, nb = min(64, P.J->res[P.J->ndim - 1] - i0);
@@ -340,13 +347,19 @@ plot_expr_kernel(const ExprJob* __restrict__ jobs, int njobs, int64_t total_word
 
 void launch_plot_expr(const ExprJob* d_jobs, int njobs, int64_t total_words, cudaStream_t s) {
   if (njobs <= 0 || total_words <= 0) return;
-  // words per block: up to one per thread, fewer while the blocks do not fill
-  // the GPU four times over (the undecided pieces of neighbouring words end up
-  // in one block)
-  int64_t words = 32;
-  while (words < kExprWords && total_words / words > 152 * 16) words *= 2;
+  // Words per block: the largest power of two, up to one per thread, that leaves the
+  // GPU the 12 blocks an SM holds: the undecided pixels of a curve lie in few words,
+  // and FP64 is done by the SMs those words are on.  (Butterfly, whole solves, against
+  // at least 32 words in blocks of 256 threads: 125 px 69 -> 47 us, 300 px 65 -> 51,
+  // 2048 px 119 -> 113; FP64 at every pixel 55, 73 and 1523.)
+  // Small grids start with the 8-pixel pieces: while a piece per thread fills no more
+  // than half the GPU, testing whole words first only lengthens the chain (500 px 58.0
+  // against 53.7 us; from 900 px on it saves, 79.9 against 80.6, 75^3 55.7 against 61.9).
+  int64_t words = 1;
+  while (words < kExprWords && total_words / (2 * words) >= 152 * 12) words *= 2;
+  const bool by_words = 8 * total_words > 152 * 1024;
   plot_expr_kernel<<<(unsigned)((total_words + words - 1) / words), kExprThreads, 0, s>>>(
-      d_jobs, njobs, total_words, (int)words);
+      d_jobs, njobs, total_words, (int)words, by_words);
 }
 
 }  // namespace pa

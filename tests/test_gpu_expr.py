@@ -298,3 +298,19 @@ def test_random_expressions_fine(eng, orc, seed):
     got = eng.plot(rel, axes)
     eng.sync()
     check_plot_band(orc, rel, axes, got, f"seed {seed}")
+
+
+# Word counts around the launch's choices: a block's words (powers of two up to 128, a
+# partial last block) and whether whole words are tested before their pieces.
+@pytest.mark.parametrize("shape", [(2, 3), (2, 70), (40, 40), (3647, 64), (3648, 64), (19456, 33),
+                                   (19457, 64), (19, 65536), (233473, 40), (5, 300001)])
+@pytest.mark.parametrize("case", [0, 2])
+def test_block_shapes(eng, orc, shape, case):
+    rows, cols = shape
+    x, y = Ex.port(0), Ex.port(1)
+    rel = W.expr_relation((0, 1), EDGES[case](x, y), kind=W.KIND_EQ, eps=0.02)
+    axes = [(-2.0, 2.0, rows), (-2.0, 2.0, cols)]
+    got = eng.plot(rel, axes)
+    eng.sync()
+    check_plot_band(orc, rel, axes, got, f"{rows} x {cols}")
+    assert got.padding_clean()
