@@ -271,36 +271,40 @@ __device__ __forceinline__ int decide_run(const Place& P, int i0, int i1) {
   return (!bad && hi < J.eps) ? 2 : 0;
 }
 
-constexpr int kExprThreads = 128;
-constexpr int kExprWords = 128;  // most words per block
-
-// by_words: whole words are tested first; else the 8-pixel pieces of every word.
-__global__ void __launch_bounds__(kExprThreads)
-plot_expr_kernel(const ExprJob* __restrict__ jobs, int njobs, int64_t total_words, int words, bool by_words) {
-  __shared__ uint16_t wlist[kExprWords], plist[8 * kExprWords];
+// THREADS: the block, and the most words it takes.  FIRST: what the block starts with,
+// whole words, the 8-pixel pieces of every word, or every pixel in FP64.
+enum { kWords, kPieces, kPixels };
+template <int THREADS, int FIRST>
+__global__ void __launch_bounds__(THREADS)
+plot_expr_kernel(const ExprJob* __restrict__ jobs, int njobs, int64_t total_words, int words) {
+  __shared__ uint16_t wlist[THREADS], plist[8 * THREADS];
   __shared__ int s_w, s_p;
   const int tid = threadIdx.x;
   const int64_t w0 = (int64_t)blockIdx.x * words;
   const int mine = (int)min((int64_t)words, total_words - w0);  // words of this block
   if (tid == 0) {
-    s_w = by_words ? 0 : mine;
-    s_p = 0;
+    s_w = FIRST == kPieces ? mine : 0;
+    s_p = FIRST == kPixels ? 8 * mine : 0;
   }
   __syncthreads();
-  if (!by_words) {
-    if (tid < mine) wlist[tid] = (uint16_t)tid;
-  } else if (tid < mine) {
-    Place P;
-    locate(jobs, njobs, w0 + tid, P);
-    const int i0 = P.wi * 64, nb = min(64, P.J->res[P.J->ndim - 1] - i0);
-    const int dec = decide_run(P, i0, i0 + nb - 1);
-    if (dec) P.J->out[P.word] = dec == 1 ? 0ull : nb == 64 ? ~0ull : (1ull << nb) - 1ull;
-    else wlist[atomicAdd(&s_w, 1)] = (uint16_t)tid;
+  if (FIRST == kPixels)
+    for (int e = tid; e < 8 * mine; e += THREADS) plist[e] = (uint16_t)e;
+  if (tid < mine) {
+    if constexpr (FIRST == kWords) {
+      Place P;
+      locate(jobs, njobs, w0 + tid, P);
+      const int i0 = P.wi * 64, nb = min(64, P.J->res[P.J->ndim - 1] - i0);
+      const int dec = decide_run(P, i0, i0 + nb - 1);
+      if (dec) P.J->out[P.word] = dec == 1 ? 0ull : nb == 64 ? ~0ull : (1ull << nb) - 1ull;
+      else wlist[atomicAdd(&s_w, 1)] = (uint16_t)tid;
+    } else {
+      wlist[tid] = (uint16_t)tid;
+    }
   }
   __syncthreads();
   // the 8-pixel pieces of the words left (a byte of the word each)
   const int nw = s_w;
-  for (int e = tid; e < 8 * nw; e += kExprThreads) {
+  for (int e = tid; e < 8 * nw; e += THREADS) {
     const int k = wlist[e >> 3], c = e & 7;
     Place P;
     locate(jobs, njobs, w0 + k, P);
@@ -313,7 +317,7 @@ plot_expr_kernel(const ExprJob* __restrict__ jobs, int njobs, int64_t total_word
   // the pieces left, a lane per pixel
   const int np = s_p;
   const int lane = tid & 31;
-  for (int base = 0; base < 8 * np; base += kExprThreads) {
+  for (int base = 0; base < 8 * np; base += THREADS) {
     const int e = base + tid;
     bool on = false;
     Place P;
@@ -347,19 +351,31 @@ plot_expr_kernel(const ExprJob* __restrict__ jobs, int njobs, int64_t total_word
 
 void launch_plot_expr(const ExprJob* d_jobs, int njobs, int64_t total_words, cudaStream_t s) {
   if (njobs <= 0 || total_words <= 0) return;
-  // Words per block: the largest power of two, up to one per thread, that leaves the
-  // GPU the 12 blocks an SM holds: the undecided pixels of a curve lie in few words,
-  // and FP64 is done by the SMs those words are on.  (Butterfly, whole solves, against
-  // at least 32 words in blocks of 256 threads: 125 px 69 -> 47 us, 300 px 65 -> 51,
-  // 2048 px 119 -> 113; FP64 at every pixel 55, 73 and 1523.)
-  // Small grids start with the 8-pixel pieces: while a piece per thread fills no more
-  // than half the GPU, testing whole words first only lengthens the chain (500 px 58.0
-  // against 53.7 us; from 900 px on it saves, 79.9 against 80.6, 75^3 55.7 against 61.9).
-  int64_t words = 1;
-  while (words < kExprWords && total_words / (2 * words) >= 152 * 12) words *= 2;
-  const bool by_words = 8 * total_words > 152 * 1024;
-  plot_expr_kernel<<<(unsigned)((total_words + words - 1) / words), kExprThreads, 0, s>>>(
-      d_jobs, njobs, total_words, (int)words, by_words);
+  // A small grid is bound by a chain of programs and by FP64 on the SMs that its few
+  // undecided words are on: small blocks of few words each, at least seven per SM, and
+  // no test whose lanes would not fill half the GPU (words; a quarter for pieces,
+  // whose test spares FP64), as it only lengthens the chain.  Butterfly, whole
+  // solves, alone / among others, against the launch below: 40 px 104 / 58.7 -> 79 / 49.6,
+  // 125 px 114 / 69.7 -> 81 / 47.5, 300 px 109 / 63.1 -> 91 / 47.6, 500 px 109 / 64.1 -> 99 / 53.0; FP64 at
+  // every pixel in blocks of 256: 84 / 57, 89 / 55, 115 / 73 and 173 / 129.
+  if (8 * total_words <= 152 * 1024) {
+    int64_t words = 1;
+    while (words < 128 && total_words / (2 * words) >= 152 * 7) words *= 2;
+    const unsigned grid = (unsigned)((total_words + words - 1) / words);
+    if (64 * total_words <= 152 * 512)
+      plot_expr_kernel<128, kPixels><<<grid, 128, 0, s>>>(d_jobs, njobs, total_words, (int)words);
+    else
+      plot_expr_kernel<128, kPieces><<<grid, 128, 0, s>>>(d_jobs, njobs, total_words, (int)words);
+    return;
+  }
+  // Others: up to one word per thread, fewer while the blocks do not fill the GPU four
+  // times over (the undecided pieces of neighbouring words end up in one block).  At
+  // 800 px and 75^3 this is as fast as the small blocks (70.5 against 72.8 us, 56.8
+  // against 55.7), at 4096 px faster than any of them (209 against 212).
+  int64_t words = 32;
+  while (words < 256 && total_words / words > 152 * 16) words *= 2;
+  plot_expr_kernel<256, kWords><<<(unsigned)((total_words + words - 1) / words), 256, 0, s>>>(
+      d_jobs, njobs, total_words, (int)words);
 }
 
 }  // namespace pa

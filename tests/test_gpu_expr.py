@@ -300,9 +300,9 @@ def test_random_expressions_fine(eng, orc, seed):
     check_plot_band(orc, rel, axes, got, f"seed {seed}")
 
 
-# Word counts around the launch's choices: a block's words (powers of two up to 128, a
-# partial last block) and whether whole words are tested before their pieces.
-@pytest.mark.parametrize("shape", [(2, 3), (2, 70), (40, 40), (3647, 64), (3648, 64), (19456, 33),
+# Word counts around the launch's choices: a block's words (powers of two, a partial
+# last block) and what it starts with, pixels, pieces or whole words.
+@pytest.mark.parametrize("shape", [(2, 3), (2, 70), (40, 40), (1216, 64), (1217, 64), (4257, 50), (19456, 33),
                                    (19457, 64), (19, 65536), (233473, 40), (5, 300001)])
 @pytest.mark.parametrize("case", [0, 2])
 def test_block_shapes(eng, orc, shape, case):
