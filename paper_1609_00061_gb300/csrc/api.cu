@@ -170,6 +170,9 @@ struct Builder {
   // Set when the layout would not fit the memory there is: no array that only
   // makes a reshape faster (conform).
   bool compact = false;
+  // Set when the program's plot launch clears the results that start at zero
+  // (fold_memsets), so that they cost no launch of their own.
+  bool free_clear = false;
   char* base = nullptr;     // device memory the layout lives in (null in the sizing pass)
   size_t used = 0;          // bytes of `base` in use
   size_t blob_cap = 0;      // bytes reserved for the blob at the start of `base`
@@ -876,7 +879,7 @@ BitArr join(Builder& bd, const BitArr& X, const BitArr& Y, const std::vector<int
   d.stat = bd.d_stat;
   if (d.M > 0x7fffffffLL || d.K > 0x7fffffffLL)
     bd.fail(PA_ERR_TOO_LARGE, "contraction with more than 2^31 rows");
-  rowor_plan(d, share);
+  rowor_plan(d, share, bd.free_clear);
   if (d.atomic) {
     Op op;
     op.kind = OP_MEMSET;
@@ -1515,6 +1518,8 @@ void build_networks(Builder& bd, std::vector<Network>& nets, bool one_join_per_l
   for (auto& n : nets)
     for (int i = 0; i < n.nrel; ++i) reqs.push_back({&n.rels[i], n.axes, n.strict, nullptr});
   std::vector<BitArr> plots = plot_all(bd, reqs);
+  bd.free_clear = !one_join_per_launch &&
+                  std::any_of(bd.ops.begin(), bd.ops.end(), [](const Op& o) { return o.kind == OP_PLOT; });
   plan_networks(nets);
 
   struct State {
@@ -2573,7 +2578,7 @@ pa_status pa_autotune(pa_ctx* ctx, pa_rates* out, void* stream) {
     rd.a_row_words = W;
     rd.err = ctx->d_err;
     rd.stat = ctx->d_stat;
-    rowor_plan(rd, 152);
+    rowor_plan(rd, 152, true);
     CUtensorMap rmap;
     if (rowor_encode_map(rd, &rmap) != cudaSuccess) {
       fail("tensor map (row-OR)");

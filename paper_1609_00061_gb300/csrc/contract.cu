@@ -1157,7 +1157,7 @@ int64_t rowor_max_kc(int Nt, int threads) {
   return std::min<int64_t>(kRowOrMaxKc, std::max<int64_t>(64, kc));
 }
 
-void rowor_plan(RowOrDesc& d, double share) {
+void rowor_plan(RowOrDesc& d, double share, bool free_clear) {
   // the widest power-of-two tile (<= 32 words, <= the row): a row of A is
   // split into blocks and listed once per tile, so wide tiles cut that work
   // (32-word tiles took the chain's 2048^3 joins from 19.3 to 16.0 us per
@@ -1183,12 +1183,14 @@ void rowor_plan(RowOrDesc& d, double share) {
   // K in chunks of equal length; many chunks take a power of two of rows, so
   // that whole batches of rows fill the lanes.  A problem with SMs left over
   // takes more chunks (down to 512 rows of K), each staging its own part of B
-  // only, before its rows are split over CTAs that all stage the same one.
+  // only, before its rows are split over CTAs that all stage the same one; but a
+  // second chunk has C cleared first, which as a launch of its own costs more than
+  // it gains (6611 x 653 x 911, a call among others 39.0 -> 43.1 us).
   int64_t kmax = rowor_max_kc(Nt, d.threads);
   if (d.K >= 4 * kmax)
     while (kmax & (kmax - 1)) kmax &= kmax - 1;
   int64_t chunks = (d.K + kmax - 1) / kmax;
-  if (d.threads == kRowOrThreads)
+  if (d.threads == kRowOrThreads && (free_clear || chunks > 1))
     chunks = std::max(chunks, std::min<int64_t>((int64_t)(share / (double)tiles), (d.K + 511) / 512));
   d.Kc = chunks <= 1 ? (int32_t)d.K : (int32_t)(((d.K + chunks - 1) / chunks + 63) / 64 * 64);
   // How the tile is staged.  A tile as wide as the rows is one run of memory

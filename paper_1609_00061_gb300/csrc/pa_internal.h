@@ -250,8 +250,9 @@ enum { kStageWords = 0, kStageTile = 1, kStageRun = 2 };
 // Longest K range whose tables fit next to the lists of a CTA of `threads`.
 int64_t rowor_max_kc(int Nt, int threads);
 // Choose the tile shape and grid for a contraction of this shape, which has
-// `share` SMs (a fraction when many contractions share one launch).
-void rowor_plan(RowOrDesc& d, double share);
+// `share` SMs (a fraction when many contractions share one launch).  free_clear: a
+// result that has to start at zero costs no launch of its own.
+void rowor_plan(RowOrDesc& d, double share, bool free_clear);
 size_t rowor_smem_bytes(const RowOrDesc& d);
 int64_t rowor_ctas(const RowOrDesc& d);
 // TMA descriptor of d.B (all zero unless d.stage is kStageTile)

@@ -69,3 +69,22 @@ def test_shared_batch_axis(eng, orc, nb, M, K, N):
     for kind in ("runs", "half"):
         x, y = bits(rng, (nb, M, K), kind), bits(rng, (nb, K, N), "runs")
         check(eng, orc, x, y, (0, 1, 2), (0, 2, 3), (0, 1, 3), [nb, M, K, N])
+
+
+# A single cluster whose K range fits one chunk: no second chunk, and so no launch
+# that clears the result, even where CTAs are few.  (Next to tiles of 32 words a chunk
+# has at most 576 rows.)
+@pytest.mark.parametrize("M,K,N,chunks", [(6611, 653, 911, 1), (700, 700, 100, 1), (64, 2048, 64, 1),
+                                          (300, 600, 2100, 2)])
+def test_single_cluster_has_one_launch(eng, orc, M, K, N, chunks):
+    rng = np.random.default_rng(M + K + N)
+    x, y = bits(rng, (M, K), "runs"), bits(rng, (K, N), "runs")
+    pa.pa_profile_enable(eng.ctx)
+    try:
+        pa.pa_profile_read(eng.ctx)
+        check(eng, orc, x, y, (0, 1), (1, 2), (0, 2), [M, K, N])
+        names = pa.pa_profile_read(eng.ctx)
+    finally:
+        pa.pa_profile_enable(eng.ctx, False)
+    names.pop("words_or")  # a counter
+    assert sorted(names) == (["rowor_kernel"] if chunks == 1 else ["memset", "rowor_kernel"]), names
