@@ -724,10 +724,16 @@ double or_density(double rho, double n);
 // time: where densities are known (a network's own plots) its rate counts
 // kRowOrRuns times.  Measured on whole cases with factors 1 / 2.5 / 3.5: chain of 8 at
 // 2048 px 64 / 62 / 54 us, of 4 at 4001 px 70 / 57 / 57 us, 38 networks 7.84 /
-// 7.45 / 7.42 ms.  Operands of unknown density (pa_contract) are taken as random and 16 %
-// dense.
+// 7.45 / 7.42 ms.
+//
+// Of pa_contract's operands nothing is known.  On plots the row-OR is never the slower
+// one, on half-full operands it takes up to three times as long (8192^3: 1363 against
+// 493 us).  So the tensor path is taken where it serves both: where it skips empty
+// blocks by bitmaps and then keeps up on plots (8192^3 53 against 50 us, 4096^3 26
+// against 24, 7100 x 1481 x 2477 26 against 25), if it is the faster one on a dense
+// operand.
 constexpr double kRowOrRuns = 3.5;
-constexpr double kUnknownDensity = 0.16;
+constexpr double kDense = 0.5;
 
 // Fixed cost of a unit, about 60 warp instructions (ncu, chain joins) at half
 // the issue rate of 152 SMs x 4 schedulers x 2 GHz: some 1e10 units per second
@@ -739,14 +745,14 @@ constexpr double kRowOrUnitsPerUs = 1.0e4;
 constexpr double kMmaFixedUs = 0.5;
 
 // Estimated microseconds of a matrix-form cluster on the row-OR path when A
-// has density `dens` (< 0: unknown): its word ORs at the context's measured
+// has density `dens` (< 0: unknown, taken as dense): its word ORs at the context's measured
 // rate (log-linear in the density between the two measured points) plus every
 // (row, K chunk, tile) unit's fixed cost.
 double rowor_cost_us(const pa_ctx* ctx, const JoinShape& js, double dens) {
   const double M = (double)js.M, N = js.nbits, K = (double)js.K, nb = (double)js.nbatch;
   const double r0 = ctx ? ctx->rate_or : 2.9e5, r1 = ctx ? ctx->rate_or_dense : 1.39e6;
   const double runs = dens >= 0 ? kRowOrRuns : 1.0;
-  if (dens < 0) dens = kUnknownDensity;
+  if (dens < 0) dens = kDense;
   const double f = std::min(1.0, std::max(0.0, log(std::max(dens, 1e-12) / 0.02) / log(8.0)));
   const double rate_or = r0 * pow(r1 / r0, f) * runs;
   const double Nw = ceil(N / 64);
@@ -766,6 +772,16 @@ bool use_mma(const pa_ctx* ctx, const JoinShape& js, double ra) {
   const double BN = N <= 128 ? 128 : 256;
   const double macs = nb * ceil(M / 128) * 128 * ceil(N / BN) * BN * ceil(K / 128) * 128;
   if (macs < 134217728.0) return false;  // small clusters: the row-OR's launch is cheaper
+  if (ra < 0) {
+    MmaDesc d;
+    memset(&d, 0, sizeof d);
+    d.M = js.M;
+    d.N = (int64_t)N;
+    d.K = js.K;
+    d.nbatch = js.nbatch;
+    mma_plan(d);
+    if (!mma_wants_occ(d)) return false;
+  }
   const double t_or = rowor_cost_us(ctx, js, ra);
   const double t_mma = macs / ctx->rate_mma + kMmaFixedUs;
   return t_mma < t_or;

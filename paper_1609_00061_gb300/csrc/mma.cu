@@ -625,10 +625,14 @@ void mma_plan(MmaDesc& d) {
 
 int64_t mma_ctas(const MmaDesc& d) { return d.nbatch * d.m_tiles * d.n_tiles * d.ksplit; }
 
-// Bitmaps pay where a CTA walks many K blocks: writing them takes a launch of
-// about 4 us, seeing an empty block in its loaded words about 200 cycles (a
-// CTA of 16 blocks gains 1.6 us at most, one of 64 sparse ones 6).
-bool mma_wants_occ(const MmaDesc& d) { return d.kchunk >= 32; }
+// Bitmaps pay where many K blocks are walked, by a CTA or by an SM's CTAs one after
+// another: writing them takes a launch of about 4 us (8 on dense operands), seeing an
+// empty block in its loaded words about 200 cycles (a CTA of 16 blocks gains 1.6 us at
+// most, one of 64 sparse ones 6).  Plots of 6616 x 3119 x 6140, 205 blocks to an SM
+// but 25 to a CTA, 87 -> 38 us.
+bool mma_wants_occ(const MmaDesc& d) {
+  return d.kchunk >= 32 || (d.kchunk >= 8 && mma_ctas(d) * d.kchunk >= 152 * 24);
+}
 
 int64_t mma_occ_blocks(const MmaDesc& d) {
   return d.nbatch * (d.m_tiles + d.n_tiles) * d.kb_words * 4;  // one byte per block

@@ -180,3 +180,35 @@ def test_more_tiles_than_sms(eng, orc, nb, M, K, N):
     want = np.matmul(X.astype(np.float32), Y.astype(np.float32))
     check_same(got, (want > 0).astype(np.uint8), f"{vres}")
     assert np.array_equal(cnt.cpu().numpy(), want.astype(np.int64)), f"counts {vres}"
+
+
+# Which kernels a single cluster of unknown density takes: the tensor path where it
+# skips empty blocks by bitmaps, whatever the remainders of the sizes are.
+@pytest.mark.parametrize("M,K,N,tensor", [(1000, 1000, 1000, False), (2048, 2048, 2048, False),
+                                          (6611, 653, 911, False), (3000, 1030, 5200, True),
+                                          (8192, 8192, 8192, True), (8000, 8000, 8000, True),
+                                          (4097, 4001, 4000, True), (700, 6000, 64, False)])
+def test_path_of_a_single_cluster(M, K, N, tensor):
+    import torch
+    e = pa.Engine(0)
+    g = torch.Generator(device="cuda").manual_seed(M + K + N)
+    arrays = []
+    for vs, (r, c) in (((0, 1), (M, K)), ((1, 2), (K, N))):
+        w = (c + 63) // 64
+        bits = torch.randint(-2**63, 2**63 - 1, (r, w), generator=g, device="cuda")
+        # empty 512-row bands and 256-column bands, so that blocks are skipped
+        bits[(torch.arange(r, device="cuda") // 512) % 3 == 1] = 0
+        bits[:, (torch.arange(w, device="cuda") // 4) % 4 == 2] = 0
+        bits &= torch.randint(-2**63, 2**63 - 1, (r, w), generator=g, device="cuda")
+        if c % 64:
+            bits[:, -1] &= (1 << (c % 64)) - 1
+        arrays.append(pa.BitArray(bits.reshape(-1), vs, (r, c)))
+    pa.pa_profile_enable(e.ctx)
+    got = e.contract(*arrays, (0, 2))
+    names = pa.pa_profile_read(e.ctx)
+    assert ("mma_bits_kernel" in names) == tensor and ("rowor_kernel" in names) != tensor, names
+    e.set_path("rowor" if tensor else "mma")
+    want = e.contract(*arrays, (0, 2))
+    e.sync()
+    assert torch.equal(got.words, want.words)
+    e.close()
