@@ -492,14 +492,13 @@ reshape_transpose_few_kernel(const ReshapeDesc* __restrict__ descs, const int64_
 // memory, where a block per thread is the cheaper way.
 constexpr int64_t kFewTiles = 304;
 
-// Words of a transpose's tile per side.
-int transpose_tw(const ReshapeDesc& d) { return d.tQ > 256 && d.tR > 256 ? 8 : 4; }
-int64_t transpose_tiles(const ReshapeDesc& d) {
-  const int64_t side = 64 * transpose_tw(d);
+constexpr int64_t kMaxReshapeBlocks = 152 * 16;
+
+// A transpose's tiles of 64 tw x 64 tw values.
+int64_t transpose_tiles(const ReshapeDesc& d, int tw) {
+  const int64_t side = 64 * tw;
   return d.n_other * ((d.tQ + side - 1) / side) * ((d.tR + side - 1) / side);
 }
-
-constexpr int64_t kMaxReshapeBlocks = 152 * 16;
 
 int reshape_kind(const ReshapeDesc& d) {
   if (d.mode == kReshapeBits) return kRsBits;
@@ -509,8 +508,8 @@ int reshape_kind(const ReshapeDesc& d) {
   if (d.mode == kReshapeTranspose) {
     in_max += (d.tR + 511) * d.t_in_L + d.tQ / 64 + 8;
     const bool fits = in_max < (1ll << 31) && total < (1ll << 31) &&
-                      transpose_tiles(d) + blocks < (1ll << 31);
-    return !fits ? kRsTranspose64 : transpose_tw(d) == 8 ? kRsTranspose32Wide : kRsTranspose32;
+                      transpose_tiles(d, 4) + blocks < (1ll << 31);
+    return !fits ? kRsTranspose64 : d.tQ > 256 && d.tR > 256 ? kRsTranspose32Wide : kRsTranspose32;
   }
   for (int q = 0; q < d.nred; ++q) in_max += (d.red_res[q] - 1) * d.red_in_w[q];
   return (total + 1024 * blocks < (1ll << 31) && in_max < (1ll << 31)) ? kRsWords32 : kRsWords64;
@@ -519,7 +518,7 @@ int reshape_kind(const ReshapeDesc& d) {
 int64_t reshape_units(const ReshapeDesc& d) {
   const int64_t total = d.out_nrows * d.out_row_words;
   if (total <= 0) return 0;
-  if (d.mode == kReshapeTranspose) return transpose_tiles(d);
+  if (d.mode == kReshapeTranspose) return transpose_tiles(d, reshape_kind(d) == kRsTranspose32Wide ? 8 : 4);
   if (d.mode == kReshapeWords) {
     // a thread per run of words, or more for a reduction (see the kernel)
     int64_t red = 1;

@@ -68,3 +68,45 @@ def test_many_transposes(eng, orc, vres):
     got = eng.contract(pack(X, (0, 1, 2)), pack(Y, (0, 1, 2)), (0, 2, 1))
     eng.sync()
     check_same(got, want, str(vres))
+
+
+def test_transpose_beyond_32_bit_indexes(eng):
+    """An operand of more than 2^31 words, its last axis moved to the front: the
+    transpose counts words in 64 bits."""
+    import torch
+    M, K, N, T = (1 << 15) + 64, 1 << 16, 64, 64
+    free, _ = torch.cuda.mem_get_info()
+    if free < 80 << 30:
+        pytest.skip("needs 80 GB of device memory")
+    A = pa.BitArray.empty((0, 1, 3), (M, K, T), 0)
+    B = pa.BitArray.empty((1, 2, 3), (K, N, T), 0)
+    a, b = A.words.view(M, K), B.words.view(K, N)
+    a.zero_()
+    b.zero_()
+    rng = np.random.default_rng(1)
+    m = np.concatenate([[0, M - 1, M - 1, 0], rng.integers(0, M, 400)])
+    k = np.concatenate([[0, K - 1, 0, K - 1], rng.integers(0, K, 400)])
+    n = rng.integers(0, N, len(m))
+    av, bv = {}, {}  # one to three values of the last axis per place
+    for i in range(len(m)):
+        t = rng.integers(0, T, 3)
+        av[m[i], k[i]] = av.get((m[i], k[i]), 0) | (1 << int(t[0])) | (1 << int(t[1]))
+        bv[k[i], n[i]] = bv.get((k[i], n[i]), 0) | (1 << int(t[0])) | (1 << int(t[2]))
+
+    def put(dst, values):
+        at = torch.tensor(list(values), device="cuda")
+        dst[at[:, 0], at[:, 1]] = torch.from_numpy(np.array(list(values.values()), np.uint64).view(np.int64)).cuda()
+
+    put(a, av)
+    put(b, bv)
+    want = np.zeros((M, N), np.uint64)
+    for (mi, ki), x in av.items():
+        for (kj, nj), y in bv.items():
+            if ki == kj:
+                want[mi, nj] |= np.uint64(x & y)
+    got = eng.contract(A, B, (0, 2, 3))
+    eng.sync()
+    assert np.array_equal(got.words.view(M, N).cpu().numpy().view(np.uint64), want)
+    assert want.any()
+    del A, B, a, b, got
+    torch.cuda.empty_cache()
