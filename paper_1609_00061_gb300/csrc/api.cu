@@ -1274,6 +1274,14 @@ void plot_filter(PlotJob& J, const pa_relation& r, const pa_axis* axes,
   // ascending).  The same with max(X_p, 1) bounds every partial sum of the FP64
   // evaluation.
   double A = 0.0, reach = 0.0;
+  double pw[kMaxDim][kMaxDeg + 1], pb[kMaxDim][kMaxDeg + 1];  // X^e, max(X, 1)^e
+  for (int p = 0; p < n; ++p) {
+    pw[p][0] = pb[p][0] = 1.0;
+    for (int j = 1; j <= D; ++j) {
+      pw[p][j] = pw[p][j - 1] * X[p];
+      pb[p][j] = pb[p][j - 1] * fmax(X[p], 1.0);
+    }
+  }
   std::vector<int> unit(ord.size());  // per coefficient: sum of e_p k_p
   size_t at = 0;
   int e[kMaxDim] = {};
@@ -1291,12 +1299,11 @@ void plot_filter(PlotJob& J, const pa_relation& r, const pa_axis* axes,
     }
     double m = fabs(r.coeffs[ord[at]]), big = m;
     int u = 0;
-    for (int p = 0; p < n; ++p)
-      for (int j = 0; j < e[p]; ++j) {
-        m *= X[p];
-        big *= fmax(X[p], 1.0);
-        u += k[p];
-      }
+    for (int p = 0; p < n; ++p) {
+      m *= pw[p][e[p]];
+      big *= pb[p][e[p]];
+      u += k[p] * e[p];
+    }
     unit[at++] = u;
     A += m;
     reach += big;
@@ -1386,7 +1393,8 @@ std::vector<BitArr> plot_poly(Builder& bd, const std::vector<PlotReq>& reqs) {
     J.nrows = a.nrows();
     J.row_words = a.row_words();
     J.eps = relation_eps(r, axes);
-    plot_filter(J, r, axes, ord, nc32);
+    if (bd.dry) nc32.assign(ord.size(), 0.0f);
+    else plot_filter(J, r, axes, ord, nc32);
     c32_off[i] = bd.put(nc32.data(), nc32.size());
     J.rows_per_tile = (int32_t)std::max<int64_t>(
         1, std::min<int64_t>(1024, (tile_words + J.row_words - 1) / J.row_words));

@@ -487,9 +487,12 @@ reshape_transpose_few_kernel(const ReshapeDesc* __restrict__ descs, const int64_
   }
 }
 
-// Up to two tiles per SM the launch lasts as long as one tile does (75^3 arrays, 75
-// tiles: 56.0 us per solve against 56.8); more tiles are bound by L1 and shared
-// memory, where a block per thread is the cheaper way.
+// Up to two tiles per SM the launch lasts as long as one tile does; more tiles are
+// bound by L1 and shared memory, where a block per thread is the cheaper way.  Whole
+// solves with the line at 0 / 304 / 608 / 2432 tiles, us: 3-D arrays at 88 px 63.3 /
+// 62.5 / 62.6 / 62.5, at 100 px 81.1 / 80.5 / 80.4 / 80.2; random networks, 2 of them
+// 308 / 300 / 299 / 299, 3: 836 / 826 / 826 / 826, 5: 700 / 698 / 698 / 712, 16: 2466 /
+// 2465 / 2463 / 2508, 38: 5220 / 5215 / 5216 / 5256.
 constexpr int64_t kFewTiles = 304;
 
 constexpr int64_t kMaxReshapeBlocks = 152 * 16;

@@ -48,9 +48,10 @@
 // of read-back, 27.9 k in all.  Without the shared stores a block takes 930
 // cycles and without the products 825, so both sides are near their limit (an
 // N-major B halves the rate of a K-major one, 560 per block, which would need
-// bit transposes).  Against the byte-array version: 8192^3 of two cubic plots
-// 100 -> 58 us per call, the 2048^3 count 55 -> 46 us, ternary 256 (256 products of
-// 256^3) 78 -> 62 us.
+// bit transposes).  Against the byte-array version: plots of 8192^3 102 -> 53 us of
+// device time per call, the 2048^3 count 55 -> 43 per call, ternary 256 (256 products of
+// 256^3) 78 -> 54; half-full operands of 4096^3 94 -> 87, but of 8192^3 450 -> 493 and of
+// 16384^3 3170 -> 3600 (bytes fetched by TMA are K-major).
 #include <cuda.h>
 #include <string.h>
 
