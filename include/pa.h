@@ -264,7 +264,9 @@ pa_status pa_profile_read(pa_ctx* ctx, int32_t max_kernels, char* names, int64_t
  * set bits of A).  PA_PATH_MMA: 0/1 E4M3 matrix product on the tensor cores
  * (tcgen05, FP32 accumulation, thresholded at > 0; work follows M x N x K).
  * PA_PATH_AUTO (default): per cluster, the faster by the context's rates and
- * the operands' estimated densities. */
+ * the operands' estimated densities; pa_contract, which knows no densities, takes
+ * the tensor cores where they are the faster path on dense operands and skip
+ * the empty blocks of sparse ones, the row-OR elsewhere. */
 typedef enum { PA_PATH_AUTO = 0, PA_PATH_ROWOR = 1, PA_PATH_MMA = 2 } pa_path;
 pa_status pa_set_contract_path(pa_ctx* ctx, int32_t path);
 
